@@ -429,7 +429,7 @@ int jet_ctx_create(jet_ctx **out, const jet_hypergraph *hg, const jet_params *p,
     c->cmax = (int32_t)hscal[2];
     c->unit_ewgt = hscal[3] <= 1 ? 1 : 0;
     if ((e = prepare_candidate_kernels(c)) != cudaSuccess || (e = prepare_move_kernels(c)) != cudaSuccess ||
-        (e = prepare_afterburner_kernels(c)) != cudaSuccess) {
+        (e = prepare_state_kernels(c)) != cudaSuccess || (e = prepare_afterburner_kernels(c)) != cudaSuccess) {
       rc = cuda_fail(c, e, "kernel set-up");
       break;
     }

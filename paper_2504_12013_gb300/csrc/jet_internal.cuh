@@ -119,6 +119,7 @@ struct jet_ctx {
   int move_bps[3] = {1, 1, 1};
   int ab_bps[6] = {1, 1, 1, 1, 1, 1};
   int heavy_bps[2] = {1, 1};
+  int pin_bps[2] = {1, 1};  // pin counts: scalar, 16-byte rows
   // compact rebalancing keys: priority gain*c (gain >= 0) or gain*(L/c) (gain < 0), L = lcm(1..cmax),
   // stored as (Pmax - P) << 32 | v when max_wdeg*(cmax + L) < 2^32
   int rb_compact = 0;
@@ -233,6 +234,7 @@ void destroy_refine_graph(jet_ctx *c);
 // state kernels (k_state.cu)
 cudaError_t launch_validate(jet_ctx *c, int64_t *wdeg_tmp, int32_t *degcount_tmp, unsigned long long *scal);
 cudaError_t launch_classify(jet_ctx *c, const int64_t *wdeg);
+cudaError_t prepare_state_kernels(jet_ctx *c);  // pin_bps
 cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int64_t *block_w);
 cudaError_t launch_masks_from_phi(jet_ctx *c, const int32_t *phi);
 cudaError_t launch_connectivity_dense(jet_ctx *c, const int32_t *phi, int64_t *out);

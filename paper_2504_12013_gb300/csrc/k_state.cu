@@ -1,6 +1,7 @@
 // State kernels: input validation, size classes, pin counts phi_e[i] with
 // their connectivity bitmasks, block weights, and the connectivity metric
 // (lambda-1) of Section 2.
+#include <type_traits>
 #include <vector>
 
 #include "jet_internal.cuh"
@@ -95,9 +96,19 @@ __global__ void k_validate_degrees(const int64_t *vptr, const int32_t *inc, cons
   }
   long long tot = block_sum_ll(wsum);
   if (threadIdx.x == 0) atomicAdd(&scal[0], (unsigned long long)tot);
-  atomicMax(&scal[1], wmax);
-  atomicMax(&scal[2], cm);
-  atomicMax(&scal[3], om);
+  // one atomic per warp and maximum: from every thread they serialised on three addresses and the kernel
+  // took 633 us for 1 M vertices
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    wmax = max(wmax, __shfl_xor_sync(kFull, wmax, o));
+    cm = max(cm, __shfl_xor_sync(kFull, cm, o));
+    om = max(om, __shfl_xor_sync(kFull, om, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&scal[1], wmax);
+    atomicMax(&scal[2], cm);
+    atomicMax(&scal[3], om);
+  }
   if (err) atomicOr(&cnt->err, err);
 }
 
@@ -161,64 +172,115 @@ __global__ void k_edge_codes(const int64_t *eptr, int32_t m, uint8_t *code) {
 }
 
 // ---------------------------------------------------------------- pin counts
-// Warp per edge: histogram of the pins' blocks in shared memory, then one
-// coalesced store of the phi row and one ballot per mask word.  An edge longer
-// than one segment (kSegPins pins: the hub rows of a row-net) would hold its
-// warp for thousands of steps; its warp only clears the row, and
-// k_pincounts_seg and k_masks_from_phi complete it.
+// A group of G lanes per edge of at most kWarpEdge pins: the pins' blocks are
+// counted in the group's row in shared memory, which then goes out whole,
+// four counts per lane, with its two mask words.  Bound by the writes of phi
+// (4 k bytes an edge), so the loads must not stand in their way: the offsets
+// of the edge three steps ahead, the pins of the one two ahead and the blocks
+// of the next are in flight while an edge is counted (a warp per edge with
+// nothing in flight took 364 us for 1.1 M edges at k = 128, 563 MB of phi).
+// G = 8 lanes at k <= 32 and 16 at k <= 64: four lanes' counts fill the row
+// in one step, and most edges are that short.  Longer edges are counted by
+// k_pincounts_seg; the rows of those longer than one segment are cleared here.
+template <int KWP>
+constexpr int kPinLanes = KWP == 1 ? 8 : KWP == 2 ? 16 : 32;
+
+template <int KWP, bool VEC>  // VEC: rows are 16-byte aligned (k a multiple of 4, phi aligned)
 __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const int32_t *pins, const int32_t *part,
-                                                   int32_t m, int32_t k, int32_t kwp, int32_t *phi, uint32_t *mask,
+                                                   int32_t m, int32_t k, int32_t *phi, uint32_t *mask,
                                                    Counters *cnt) {
-  extern __shared__ int s_hist[];
-  const int lane = threadIdx.x & 31;
-  int *h = s_hist + (threadIdx.x >> 5) * k;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  constexpr int G = kPinLanes<KWP>, K = 32 * KWP, Q = K / (4 * G);
+  __shared__ __align__(16) int s_h[256 / G][K];
+  const int li = threadIdx.x % G;
+  int *h = s_h[threadIdx.x / G];
+  int4 *h4 = reinterpret_cast<int4 *>(h);
+#pragma unroll
+  for (int q = 0; q < Q; ++q) h4[li + q * G] = make_int4(0, 0, 0, 0);
+  __syncwarp();
+  const int64_t nw = (int64_t)gridDim.x * blockDim.x / G;
+  int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  // the groups of a warp run in lockstep up to the warp's first group; one past the end has no pins
+  int64_t iw = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;
   int err = 0;
-  for (int64_t e = gw; e < m; e += nw) {
-    const int64_t p0 = eptr[e], p1 = eptr[e + 1];
-    if (p1 - p0 > kSegPins) {  // warp-uniform
-      for (int b = lane; b < k; b += 32) phi[e * k + b] = 0;
-      continue;
-    }
-    for (int b = lane; b < k; b += 32) h[b] = 0;
-    __syncwarp();
-    for (int64_t p = p0 + lane; p < p1; p += 32) {
-      int b = part[pins[p]];
-      if ((unsigned)b < (unsigned)k) atomicAdd(&h[b], 1);
+  // stages, named by how many edges ahead they are; sz = 0 and pin = -1 past the end of an edge or the list
+  auto offsets = [&](int64_t e, int64_t &p, int &sz) {
+    p = e < m ? eptr[e] : 0;
+    sz = e < m ? (int)min(eptr[e + 1] - p, (int64_t)kSegPins + 1) : 0;
+  };
+  auto pin_of = [&](int64_t p, int sz) { return li < sz && sz <= kWarpEdge ? pins[p + li] : -1; };
+  int64_t p0, p1, p2, p3;
+  int sz0, sz1, sz2, sz3;
+  offsets(i, p0, sz0);
+  offsets(i + nw, p1, sz1);
+  offsets(i + 2 * nw, p2, sz2);
+  int v0 = pin_of(p0, sz0), v1 = pin_of(p1, sz1);
+  int b0 = v0 >= 0 ? part[v0] : 0;
+  for (; iw < m; i += nw, iw += nw) {
+    offsets(i + 3 * nw, p3, sz3);
+    const int v2 = pin_of(p2, sz2);
+    const int b1 = v1 >= 0 ? part[v1] : 0;
+    const bool store = i < m && sz0 <= kWarpEdge;
+    if (v0 >= 0) {
+      if ((unsigned)b0 < (unsigned)k) atomicAdd(&h[b0], 1);
       else err |= kErrPartRange;
     }
-    __syncwarp();
-    int32_t *row = phi + e * k;
-    for (int q = 0; q < kwp; ++q) {
-      int b = q * 32 + lane;
-      int val = b < k ? h[b] : 0;
-      if (b < k) row[b] = val;
-      const unsigned one = __ballot_sync(kFull, val > 0), two = __ballot_sync(kFull, val > 1);
-      if (lane == 0) {
-        mask[e * 2 * kwp + q] = one;        // Lambda(e)
-        mask[e * 2 * kwp + kwp + q] = two;  // blocks holding >= 2 pins of e
+    if (store) {
+#pragma unroll 4
+      for (int j = G + li; j < sz0; j += G) {
+        const int b = part[pins[p0 + j]];
+        if ((unsigned)b < (unsigned)k) atomicAdd(&h[b], 1);
+        else err |= kErrPartRange;
       }
     }
     __syncwarp();
+    int32_t *row = phi + i * k;
+    if (i < m && sz0 > kSegPins)
+      for (int b = li; b < k; b += G) row[b] = 0;
+    if (!VEC && store)
+      for (int b = li; b < k; b += G) row[b] = h[b];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int4 x = h4[li + q * G];
+      if (VEC && store && 4 * (li + q * G) < k) reinterpret_cast<int4 *>(row)[li + q * G] = x;
+      const int sh = 4 * (li & 7);
+      uint32_t one = ((x.x > 0 ? 1u : 0u) | (x.y > 0 ? 2u : 0u) | (x.z > 0 ? 4u : 0u) | (x.w > 0 ? 8u : 0u)) << sh;
+      uint32_t two = ((x.x > 1 ? 1u : 0u) | (x.y > 1 ? 2u : 0u) | (x.z > 1 ? 4u : 0u) | (x.w > 1 ? 8u : 0u)) << sh;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {  // the eight lanes of one mask word
+        one |= __shfl_xor_sync(kFull, one, o);
+        two |= __shfl_xor_sync(kFull, two, o);
+      }
+      if (store && (li & 7) == 0) {
+        const int w = (li + q * G) >> 3;
+        mask[i * 2 * KWP + w] = one;        // Lambda(e)
+        mask[i * 2 * KWP + KWP + w] = two;  // blocks holding >= 2 pins of e
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) h4[li + q * G] = make_int4(0, 0, 0, 0);
+    __syncwarp();
+    p0 = p1; sz0 = sz1; v0 = v1; b0 = b1;
+    p1 = p2; sz1 = sz2; v1 = v2;
+    p2 = p3; sz2 = sz3;
   }
   if (err) atomicOr(&cnt->err, err);
 }
 
-// The edges longer than one segment: a thread block per segment of at most
-// kSegPins pins (the afterburner's segment list, whose slot field is >= 0 for
-// exactly these edges) counts the blocks of its pins in shared memory and adds
-// the counts into the edge's row, cleared by k_pincounts: one atomic per block
-// of the partition that the segment touches.
+// The edges of more than kWarpEdge pins: a thread block per segment of at most
+// kSegPins pins (the afterburner's segment list) counts the blocks of its pins
+// in shared memory.  An edge of one segment (slot < 0) gets its row and mask
+// words from there; the segments of a longer edge add their counts into the
+// row, cleared by k_pincounts (one atomic per block of the partition that the
+// segment touches), and k_masks_from_phi completes it.
 __global__ void __launch_bounds__(256) k_pincounts_seg(const int64_t *eptr, const int32_t *pins, const int32_t *part,
-                                                       const int4 *seg, int32_t nseg, int32_t k, int32_t *phi,
-                                                       Counters *cnt) {
+                                                       const int4 *seg, int32_t nseg, int32_t k, int32_t kwp,
+                                                       int32_t *phi, uint32_t *mask, Counters *cnt) {
   __shared__ int s_h[kMaxK];
   int err = 0;
   for (int i = blockIdx.x; i < nseg; i += gridDim.x) {
     const int4 sg = seg[i];  // edge, first pin (offset in the edge), pins, slot
-    if (sg.w < 0) continue;  // a one-segment edge: counted by k_pincounts (block-uniform)
-    for (int b = threadIdx.x; b < k; b += blockDim.x) s_h[b] = 0;
+    s_h[threadIdx.x] = 0;    // kMaxK = blockDim.x
     __syncthreads();
     const int64_t p0 = eptr[sg.x] + sg.y;
 #pragma unroll 4
@@ -228,35 +290,60 @@ __global__ void __launch_bounds__(256) k_pincounts_seg(const int64_t *eptr, cons
       else err |= kErrPartRange;
     }
     __syncthreads();
+    const int b = threadIdx.x, val = s_h[b];
     int32_t *row = phi + (int64_t)sg.x * k;
-    for (int b = threadIdx.x; b < k; b += blockDim.x)
-      if (s_h[b]) atomicAdd(&row[b], s_h[b]);
+    if (sg.w >= 0) {
+      if (b < k && val) atomicAdd(&row[b], val);
+    } else {
+      if (b < k) row[b] = val;
+      const unsigned one = __ballot_sync(kFull, val > 0), two = __ballot_sync(kFull, val > 1);
+      if ((b & 31) == 0 && (b >> 5) < kwp) {
+        mask[(int64_t)sg.x * 2 * kwp + (b >> 5)] = one;
+        mask[(int64_t)sg.x * 2 * kwp + kwp + (b >> 5)] = two;
+      }
+    }
     __syncthreads();
   }
   if (err) atomicOr(&cnt->err, err);
 }
 
-// c(V_i) and |V_i|, aggregated per block in shared memory.
-__global__ void k_block_weights(const int32_t *part, const int32_t *vwgt, int32_t n, int32_t k, int64_t *bw,
-                                int32_t *vcount, Counters *cnt) {
-  __shared__ long long s_bw[kMaxK];
+// c(V_i) and |V_i|, aggregated per thread block in shared memory.  Bound by
+// the shared-memory atomics on k addresses, so their number and width count:
+// W = uint32_t when a block's share of the weights cannot leave 32 bits (the
+// launcher checks it against max c(v)), and no weight atomics at all when
+// every c(v) is 1.  Four vertices in flight per thread.
+template <class W, bool UNIT>
+__global__ void __launch_bounds__(256) k_block_weights(const int32_t *part, const int32_t *vwgt, int32_t n, int32_t k,
+                                                       int64_t *bw, int32_t *vcount, Counters *cnt) {
+  __shared__ W s_bw[kMaxK];
   __shared__ int s_cnt[kMaxK];
   for (int b = threadIdx.x; b < k; b += blockDim.x) { s_bw[b] = 0; s_cnt[b] = 0; }
   __syncthreads();
   int err = 0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    int b = part[v];
-    if ((unsigned)b < (unsigned)k) {
-      atomicAdd(reinterpret_cast<unsigned long long *>(&s_bw[b]), (unsigned long long)vwgt[v]);
-      atomicAdd(&s_cnt[b], 1);
-    } else {
-      err |= kErrPartRange;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v0 < n; v0 += 4 * stride) {
+    int b[4], c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t v = v0 + q * stride;
+      b[q] = v < n ? part[v] : -2;
+      c[q] = !UNIT && v < n ? vwgt[v] : 1;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if ((unsigned)b[q] < (unsigned)k) {
+        if constexpr (!UNIT) atomicAdd(&s_bw[b[q]], (W)c[q]);
+        atomicAdd(&s_cnt[b[q]], 1);
+      } else if (v0 + q * stride < n) {
+        err |= kErrPartRange;
+      }
     }
   }
   __syncthreads();
   for (int b = threadIdx.x; b < k; b += blockDim.x) {
-    if (s_bw[b]) add_i64(reinterpret_cast<long long *>(&bw[b]), s_bw[b]);
-    if (s_cnt[b]) atomicAdd(&vcount[b], s_cnt[b]);
+    if (!s_cnt[b]) continue;
+    add_i64(reinterpret_cast<long long *>(&bw[b]), UNIT ? (long long)s_cnt[b] : (long long)s_bw[b]);
+    atomicAdd(&vcount[b], s_cnt[b]);
   }
   if (err) atomicOr(&cnt->err, err);
 }
@@ -283,18 +370,50 @@ __global__ void __launch_bounds__(256) k_masks_from_phi(const int32_t *phi, int3
   }
 }
 
-// (lambda-1) from a dense phi: warp per edge counts the nonzero entries of its row.
+// (lambda-1) from a dense phi, read once: a group of G lanes per row (four
+// entries per lane and load), four rows in flight per group.  A lane adds
+// omega(e) per nonzero entry it sees and the group's first lane takes one
+// omega(e) off if the row has any, so no sum crosses lanes until the end.
+// Bound by the read of phi (a warp per row, one load at a time: 300 us for
+// 563 MB at k = 128).
+template <int G, bool VEC>
 __global__ void __launch_bounds__(256) k_connectivity_dense(const int32_t *phi, const int32_t *ewgt, int32_t m,
                                                             int32_t k, long long *out) {
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  constexpr int kRows = 4;
+  const int lane = threadIdx.x & 31, li = lane % G;
+  const unsigned group = (G == 32 ? kFull : ((1u << (G % 32)) - 1) << (lane - li));
+  const int64_t ng = (int64_t)gridDim.x * blockDim.x / G;
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const int64_t gfirst = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;  // the warp's first group
   long long acc = 0;
-  for (int64_t e = gw; e < m; e += nw) {
-    const int32_t *row = phi + e * k;
-    int lam = 0;
-    for (int b0 = 0; b0 < k; b0 += 32) lam += __popc(__ballot_sync(kFull, b0 + lane < k && row[b0 + lane] > 0));
-    if (lane == 0 && lam > 0) acc += (long long)(lam - 1) * ewgt[e];
+  for (int64_t d = 0; gfirst + d < m; d += kRows * ng) {
+    int c[kRows], w[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int64_t e = g + d + r * ng;
+      c[r] = 0;
+      w[r] = 0;
+      if (e < m) {
+        w[r] = ewgt[e];
+        const int32_t *row = phi + e * k;
+        if constexpr (VEC) {
+          const int4 *row4 = reinterpret_cast<const int4 *>(row);
+#pragma unroll 2
+          for (int x = li; 4 * x < k; x += G) {
+            const int4 y = __ldcs(row4 + x);
+            c[r] += (y.x > 0) + (y.y > 0) + (y.z > 0) + (y.w > 0);
+          }
+        } else {
+#pragma unroll 4
+          for (int x = li; x < k; x += G) c[r] += row[x] > 0;
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const bool any = (__ballot_sync(kFull, c[r] > 0) & group) != 0;
+      acc += (long long)(c[r] - (any && li == 0 ? 1 : 0)) * w[r];
+    }
   }
   long long tot = block_sum_ll(acc);
   if (threadIdx.x == 0 && tot) add_i64(out, tot);
@@ -462,29 +581,66 @@ cudaError_t launch_classify(jet_ctx *c, const int64_t *wdeg) {
   return e;
 }
 
+template <int KWP>
+static void launch_pincounts_kwp(jet_ctx *c, const int32_t *part, int32_t *phi, bool vec) {
+  const int g = grid_for((int64_t)c->m * kPinLanes<KWP>, 256, c->launch_sms, c->pin_bps[vec ? 1 : 0]);
+  if (vec) k_pincounts<KWP, true><<<g, 256, 0, c->stream>>>(c->eptr, c->pins, part, c->m, c->k, phi, c->mask, c->cnt);
+  else k_pincounts<KWP, false><<<g, 256, 0, c->stream>>>(c->eptr, c->pins, part, c->m, c->k, phi, c->mask, c->cnt);
+}
+
+// Resident blocks per SM of the pin-count kernels.
+template <int KWP>
+static cudaError_t prepare_pincounts_kwp(jet_ctx *c) {
+  cudaError_t e = resident_blocks(k_pincounts<KWP, false>, 256, 0, &c->pin_bps[0]);
+  if (e == cudaSuccess) e = resident_blocks(k_pincounts<KWP, true>, 256, 0, &c->pin_bps[1]);
+  return e;
+}
+
+cudaError_t prepare_state_kernels(jet_ctx *c) {
+  switch (c->kwp) {
+    case 1: return prepare_pincounts_kwp<1>(c);
+    case 2: return prepare_pincounts_kwp<2>(c);
+    case 4: return prepare_pincounts_kwp<4>(c);
+    default: return prepare_pincounts_kwp<8>(c);
+  }
+}
+
 cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int64_t *block_w) {
   cudaStream_t s = c->stream;
   cudaError_t e = cudaMemsetAsync(block_w, 0, sizeof(int64_t) * c->k, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->vcount, 0, sizeof(int32_t) * c->k, s);
   if (e != cudaSuccess) return e;
   if (c->m > 0 && phi) {
-    const int threads = 256;
-    size_t smem = (size_t)(threads / 32) * c->k * sizeof(int);
-    k_pincounts<<<grid_for((int64_t)c->m * 32, threads, c->launch_sms), threads, smem, s>>>(
-        c->eptr, c->pins, part, c->m, c->k, c->kwp, phi, c->mask, c->cnt);
+    const bool vec = c->k % 4 == 0 && ((uintptr_t)phi & 15) == 0;
+    switch (c->kwp) {
+      case 1: launch_pincounts_kwp<1>(c, part, phi, vec); break;
+      case 2: launch_pincounts_kwp<2>(c, part, phi, vec); break;
+      case 4: launch_pincounts_kwp<4>(c, part, phi, vec); break;
+      default: launch_pincounts_kwp<8>(c, part, phi, vec); break;
+    }
     ++c->kernel_launches;
+    if (c->n_seg > 0) {  // edges above kWarpEdge pins
+      k_pincounts_seg<<<grid_for(c->n_seg, 1, c->launch_sms), kMaxK, 0, s>>>(c->eptr, c->pins, part, c->ab_seg, c->n_seg,
+                                                                             c->k, c->kwp, phi, c->mask, c->cnt);
+      ++c->kernel_launches;
+    }
     if (c->n_slots > 0) {  // edges longer than one segment
-      k_pincounts_seg<<<grid_for(c->n_seg, 1, c->launch_sms), 256, 0, s>>>(c->eptr, c->pins, part, c->ab_seg,
-                                                                           c->n_seg, c->k, phi, c->cnt);
       k_masks_from_phi<<<grid_for((int64_t)c->n_slots * 32, 256, c->launch_sms), 256, 0, s>>>(
           phi, c->n_slots, c->k, c->kwp, c->mask, c->ab_slot_edge);
-      c->kernel_launches += 2;
+      ++c->kernel_launches;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (c->n > 0) {
-    k_block_weights<<<grid_for(c->n, 256, c->launch_sms, 2), 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w,
-                                                                        c->vcount, c->cnt);
+    const int g = grid_for(c->n, 1024, c->launch_sms, 4);
+    const long long share = ((c->n - 1ll) / (1024ll * g) + 1) * 1024;  // vertices of a block, at most
+    if (c->cmax <= 1)
+      k_block_weights<unsigned, true><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->vcount, c->cnt);
+    else if (share * c->cmax < (1ll << 32))
+      k_block_weights<unsigned, false><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->vcount, c->cnt);
+    else
+      k_block_weights<unsigned long long, false><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->vcount,
+                                                                   c->cnt);
     ++c->kernel_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -507,8 +663,23 @@ cudaError_t launch_masks_from_phi(jet_ctx *c, const int32_t *phi) {
 cudaError_t launch_connectivity_dense(jet_ctx *c, const int32_t *phi, int64_t *out) {
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(int64_t), c->stream);
   if (e != cudaSuccess || c->m == 0) return e;
-  k_connectivity_dense<<<grid_for((int64_t)c->m * 32, 256, c->launch_sms), 256, 0, c->stream>>>(
-      phi, c->ewgt, c->m, c->k, reinterpret_cast<long long *>(out));
+  const bool vec = c->k % 4 == 0 && ((uintptr_t)phi & 15) == 0;
+  const int lanes = vec ? (c->k + 3) / 4 : c->k;  // lanes that one load of a row needs
+  const int G = lanes > 16 ? 32 : lanes > 8 ? 16 : lanes > 4 ? 8 : lanes > 2 ? 4 : 2;
+  const int g = grid_for((int64_t)c->m * G, 256, c->launch_sms);
+  long long *o = reinterpret_cast<long long *>(out);
+  auto go = [&](auto lanes_c) {
+    constexpr int L = decltype(lanes_c)::value;
+    if (vec) k_connectivity_dense<L, true><<<g, 256, 0, c->stream>>>(phi, c->ewgt, c->m, c->k, o);
+    else k_connectivity_dense<L, false><<<g, 256, 0, c->stream>>>(phi, c->ewgt, c->m, c->k, o);
+  };
+  switch (G) {
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 4: go(std::integral_constant<int, 4>()); break;
+    case 8: go(std::integral_constant<int, 8>()); break;
+    case 16: go(std::integral_constant<int, 16>()); break;
+    default: go(std::integral_constant<int, 32>()); break;
+  }
   ++c->kernel_launches;
   return cudaGetLastError();
 }
