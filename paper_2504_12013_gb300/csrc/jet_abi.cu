@@ -227,7 +227,7 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     if ((e = launch_candidates(c, tn, td, part, phi, locked)) != cudaSuccess) return e;
     if (ev1 && (e = cudaEventRecordWithFlags(ev1, s_main, cudaEventRecordExternal)) != cudaSuccess) return e;
     if ((e = launch_afterburner(c, part, phi)) != cudaSuccess) return e;
-    if ((e = launch_approve(c, locked, nullptr, nullptr, true)) != cudaSuccess) return e;
+    if ((e = launch_approve(c, part, locked, nullptr, nullptr, true)) != cudaSuccess) return e;
     if ((e = launch_apply(c, part, phi, bw)) != cudaSuccess) return e;
     if ((e = launch_rb_check(c, bw, h, 1)) != cudaSuccess) return e;
     // WHILE node: rebalancing rounds
@@ -482,20 +482,22 @@ int jet_ctx_create(jet_ctx **out, const jet_hypergraph *hg, const jet_params *p,
     if ((e = dalloc(c, &c->v_light, c->n)) != cudaSuccess || (e = dalloc(c, &c->e_tiny, (size_t)c->m)) != cudaSuccess ||
         (e = dalloc(c, &c->mask, (size_t)c->m * 2 * c->kwp)) != cudaSuccess || (e = dalloc(c, &c->cand, c->n)) != cudaSuccess ||
         (e = dalloc(c, &c->rg, c->n)) != cudaSuccess || (e = dalloc(c, &c->mv_v, c->n)) != cudaSuccess ||
-        (e = dalloc(c, &c->mv_st, c->n)) != cudaSuccess || (e = dalloc(c, &c->vcount, c->k)) != cudaSuccess ||
-        (e = dalloc(c, &c->rbb, c->k)) != cudaSuccess || (e = dalloc(c, &c->rb_hi, c->n)) != cudaSuccess ||
-        (e = dalloc(c, &c->rb_v, c->n)) != cudaSuccess ||
+        (e = dalloc(c, &c->mv_st, c->n)) != cudaSuccess || (e = dalloc(c, &c->rbb, c->k)) != cudaSuccess ||
+        (e = dalloc(c, &c->rb_rec, c->n)) != cudaSuccess ||
+        (e = dalloc(c, &c->rb_cur, (size_t)c->k * kCurStride)) != cudaSuccess ||
         (e = dalloc(c, &c->rb_hist, (size_t)c->k << c->rb_digit)) != cudaSuccess ||
-        (e = dalloc(c, &c->rb_ct, c->n)) != cudaSuccess || (e = dalloc(c, &c->best_part, c->n)) != cudaSuccess ||
+        (e = dalloc(c, &c->best_part, c->n)) != cudaSuccess ||
         (e = dalloc(c, &c->locked_ws, c->n)) != cudaSuccess || (e = dalloc(c, &c->vheavy, c->n)) != cudaSuccess ||
         (e = dalloc(c, &c->stats_scratch, 1)) != cudaSuccess ||
         (e = cudaMallocHost(reinterpret_cast<void **>(&c->stats_host), sizeof(jet_round_stats))) != cudaSuccess) {
       rc = cuda_fail(c, e, "workspace allocation");
       break;
     }
+    c->rb_hi = reinterpret_cast<uint64_t *>(c->rb_rec);
+    c->rb_v = reinterpret_cast<int32_t *>(c->rb_hi + c->n);
+    c->rb_ct = c->rb_v + c->n;
     if ((e = cudaMemsetAsync(c->rg, 0, sizeof(int32_t) * (c->n > 0 ? c->n : 1), c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->cand, 0, sizeof(uint64_t) * (c->n > 0 ? c->n : 1), c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->vcount, 0, sizeof(int32_t) * c->k, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->rb_hist, 0, sizeof(unsigned long long) * ((size_t)c->k << c->rb_digit), c->stream)) !=
             cudaSuccess) {
       rc = cuda_fail(c, e, "workspace init");
@@ -520,8 +522,8 @@ int jet_ctx_create(jet_ctx **out, const jet_hypergraph *hg, const jet_params *p,
 void jet_ctx_destroy(jet_ctx *c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  void *dev[] = {c->cnt, c->v_light, c->e_tiny, c->mask, c->cand, c->rg, c->mv_v, c->mv_st, c->vcount, c->rbb,
-                 c->rb_hi, c->rb_v, c->rb_hist, c->rb_ct, c->best_part, c->locked_ws, c->vheavy, c->stats_scratch,
+  void *dev[] = {c->cnt, c->v_light, c->e_tiny, c->mask, c->cand, c->rg, c->mv_v, c->mv_st, c->rbb,
+                 c->rb_rec, c->rb_cur, c->rb_hist, c->best_part, c->locked_ws, c->vheavy, c->stats_scratch,
                  c->ab_seg, c->ab_slot_edge, c->ab_tab, c->ab_nm, c->sched_q, c->sched_counts, c->adj};
   for (void *p : dev) dfree(c, p);
   cudaStreamSynchronize(c->stream);
@@ -582,7 +584,7 @@ int jet_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi, int32_t
   CKP(F_PIN, ensure_masks(c, phi), "bitmasks");
   CK(reset_counters(c), "counters");
   CKP(F_AB, launch_afterburner(c, part, phi), "afterburner");
-  CKP(F_APPROVE, launch_approve(c, nullptr, rg, approved, false), "approve");
+  CKP(F_APPROVE, launch_approve(c, part, nullptr, rg, approved, false), "approve");
   return JET_OK;
 }
 
@@ -593,6 +595,7 @@ int jet_rebalance(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w, jet
     return fail(c, JET_ERR_INVALID_ARG, "part, phi or block_w is NULL");
   CKP(F_PIN, ensure_masks(c, phi), "bitmasks");
   CK(reset_counters(c), "counters");
+  CKP(F_RB_CTL, launch_count_blocks(c, part), "block counts");
   if ((rc = rebalance_loop(c, part, phi, block_w))) return rc;
   CKP(F_OBJ, launch_objective(c, part), "objective");
   CKP(F_OBJ, launch_stats(c, block_w, stats ? stats : c->stats_scratch, 1), "stats");
@@ -612,7 +615,7 @@ int jet_refine_round(jet_ctx *c, int32_t tau_num, int32_t tau_den, int32_t *part
   CK(reset_counters(c), "counters");
   CKP(F_CAND, launch_candidates(c, tau_num, tau_den, part, phi, locked), "candidates");
   CKP(F_AB, launch_afterburner(c, part, phi), "afterburner");
-  CKP(F_APPROVE, launch_approve(c, locked, nullptr, nullptr, true), "approve");
+  CKP(F_APPROVE, launch_approve(c, part, locked, nullptr, nullptr, true), "approve");
   CKP(F_APPLY, launch_apply(c, part, phi, block_w), "apply");
   if ((rc = rebalance_loop(c, part, phi, block_w))) return rc;
   CKP(F_OBJ, launch_objective(c, part), "objective");

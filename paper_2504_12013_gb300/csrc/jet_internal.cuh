@@ -11,7 +11,6 @@
 //     cand[n]        uint64 move-candidate record (0 = not in M), see below
 //     rg[n]          recomputed gain of Algorithm 2 (zeroed after use)
 //     mv_v/mv_st[n]  move list: vertex, (source | target << 16)
-//     vcount[k]      vertices per block (segment sizes for rebalancing)
 //     rb_*           rebalancing records and per-block state
 //     class lists    vertex / edge ids by size class (built once)
 #pragma once
@@ -49,6 +48,9 @@ __host__ __device__ inline uint64_t cand_key(uint64_t r, int32_t v) { return (r 
 
 // Device-side counters of one call (one cache line each group).
 struct Counters {
+  // |V_b|, recounted from the partition in every call that may rebalance (they size the blocks'
+  // segments of rebalancing records) and kept up by the apply kernels
+  int vcount[kMaxK];
   unsigned long long n_moves;     // entries in the move list
   unsigned long long n_cand;      // |M|
   unsigned long long approved;    // afterburner-approved moves
@@ -77,6 +79,7 @@ struct RbBlock {
   long long before;              // selection: weight of b's records below the fixed key prefix
   unsigned long long pre_hi;     // selection: fixed prefix of the threshold key (high word)
   unsigned long long pre_lo;     //   ... (low word)
+  int base, room;                // segmented records: first record of b, and |V_b| (their number at most)
   int over;                      // 1 if c(V_b) > L_max
   int all;                       // selection: every record of b moves
 };
@@ -92,6 +95,17 @@ struct RefineState {
 };
 
 constexpr int kRbMaxDigit = 11;  // widest radix-select digit (bins per block row <= 2048)
+
+// A rebalancing record in a block's segment: priority part of the key, vertex, c(v) << 16 | block << 8 | target.
+struct __align__(16) RbRec {
+  unsigned long long hi;
+  int32_t v, ct;
+};
+
+// Up to this many vertices per block on average, the records of a block are kept in a segment of their own and
+// selected by one thread block (k_rb_select, where the line is explained).
+constexpr int kSegVertices = 4096;
+constexpr int kCurStride = 32;  // ints between the blocks' record cursors (a line each)
 
 }  // namespace jet
 
@@ -147,10 +161,12 @@ struct jet_ctx {
   int32_t *rg = nullptr;
   int32_t *mv_v = nullptr;
   uint32_t *mv_st = nullptr;
-  int32_t *vcount = nullptr;
   jet::Counters *cnt = nullptr;
   jet::Counters *cnt_host = nullptr;  // pinned mirror
   jet::RbBlock *rbb = nullptr;
+  int rb_segments = 0;                // records in a segment per block
+  jet::RbRec *rb_rec = nullptr;       // segmented records; else the same memory holds the three arrays below
+  int32_t *rb_cur = nullptr;          // segmented: records of each block (kCurStride ints apart)
   uint64_t *rb_hi = nullptr;          // per record: priority part of the rebalancing key
   int32_t *rb_v = nullptr;            // per record: vertex
   int32_t *rb_ct = nullptr;           // per record: c(v) << 16 | block << 8 | target
@@ -249,11 +265,14 @@ cudaError_t launch_rebalance_candidates(jet_ctx *c, const int32_t *part, const i
 cudaError_t prepare_afterburner(jet_ctx *c);
 cudaError_t prepare_afterburner_kernels(jet_ctx *c);  // ab_bps
 cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi);
-cudaError_t launch_approve(jet_ctx *c, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out, bool build_moves);
+// part (with build_moves): the partition, whose blocks' vertices are counted
+cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
+                           bool build_moves);
 cudaError_t launch_export_candidates(jet_ctx *c, int32_t *target, int32_t *gain, uint8_t *in_m);
 // moves, rebalancing, loop control (k_moves.cu)
 cudaError_t prepare_move_kernels(jet_ctx *c);  // move_bps
 cudaError_t launch_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // applies the move list
+cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part);  // cnt->vcount (zeroed by reset_counters)
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                             int use_cond = 0);
 cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part);

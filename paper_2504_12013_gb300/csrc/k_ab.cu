@@ -479,7 +479,8 @@ __global__ void k_ab_slots_init(unsigned long long *tab, int32_t nslots, int32_t
 // Approval: v in M and recomputed gain > 0.  Resets rg, counts |M|; with
 // build_moves writes the move list and locked[v] := approved.
 struct ApArgs {
-  int32_t n;
+  int32_t n, k;
+  const int32_t *part;  // with build_moves
   const uint64_t *cand;
   int32_t *rg;
   uint8_t *locked;
@@ -499,6 +500,10 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   __shared__ unsigned s_wc[kWarps];
   __shared__ unsigned long long s_base;
   __shared__ unsigned long long s_cand[kWarps];
+  __shared__ int s_vc[kMaxK];  // vertices per block of the partition
+  if (a.build_moves)
+    for (int b = threadIdx.x; b < a.k; b += blockDim.x) s_vc[b] = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned long long ncand = 0;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += (int64_t)gridDim.x * blockDim.x) {
@@ -516,6 +521,10 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     }
     ncand += __popc(__ballot_sync(kFull, in));
     if (a.build_moves) {
+      if (valid) {
+        const int b = a.part[v];
+        if ((unsigned)b < (unsigned)a.k) atomicAdd(&s_vc[b], 1);
+      }
       const unsigned bap = __ballot_sync(kFull, ap);
       if (lane == 0) s_wc[wid] = __popc(bap);
       __syncthreads();
@@ -545,6 +554,9 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     for (int i = 0; i < kWarps; ++i) t += s_cand[i];
     if (t) atomicAdd(&a.cnt->n_cand, t);
   }
+  if (a.build_moves)
+    for (int b = threadIdx.x; b < a.k; b += blockDim.x)
+      if (s_vc[b]) atomicAdd(&a.cnt->vcount[b], s_vc[b]);
 }
 
 __global__ void k_export_cand(const uint64_t *cand, int32_t n, int32_t *target, int32_t *gain, uint8_t *in_m) {
@@ -778,10 +790,13 @@ cudaError_t prepare_afterburner(jet_ctx *c) {
   return cudaStreamSynchronize(c->stream);
 }
 
-cudaError_t launch_approve(jet_ctx *c, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out, bool build_moves) {
+cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
+                           bool build_moves) {
   if (c->n == 0) return cudaSuccess;
   ApArgs a{};
   a.n = c->n;
+  a.k = c->k;
+  a.part = part;
   a.cand = c->cand;
   a.rg = c->rg;
   a.locked = locked;

@@ -43,6 +43,8 @@ struct CandArgs {
   Counters *cnt;
   int rb_compact;
   long long rb_L, rb_Pmax;
+  RbRec *rb_rec;                // segmented records (NULL: one list, and the first-level histogram below)
+  int32_t *rb_cur;
   unsigned long long *rb_hist;  // first-level histogram of the rebalancing selection
   int rb_vbits, rb_tbits, rb_digit;
 };
@@ -181,6 +183,22 @@ __device__ __forceinline__ void rb_first_level(const CandArgs &a, bool rec, int 
     }
   }
   if (rec) atomicAdd(&a.rb_hist[((int64_t)s << a.rb_digit) + d], (unsigned long long)c);
+}
+
+// Appends the records to their blocks' segments: one atomic per (warp, block)
+// on the block's cursor (a line of its own), so that a pass over few
+// overloaded blocks does not serialise on their cursors, and one 16-byte store
+// per record.  Every vertex of a block has at most one record, so a segment
+// of |V_b| records holds them; the bound keeps a store inside the array.
+__device__ __forceinline__ void rb_append(const CandArgs &a, const int *s_base, bool mine, int s, uint64_t hi, int v,
+                                          int32_t ct) {
+  const int lane = threadIdx.x & 31;
+  const unsigned peers = match_bits<9>(mine ? (unsigned)s : 256u);
+  const int first = __ffs(peers) - 1;
+  int at = 0;
+  if (mine && lane == first) at = s_base[s] + atomicAdd(&a.rb_cur[s * kCurStride], __popc(peers));
+  at = __shfl_sync(kFull, at, first) + __popc(peers & ((1u << lane) - 1));
+  if (mine && at < a.n) a.rb_rec[at] = RbRec{hi, v, ct};
 }
 
 template <int KWP>
@@ -496,7 +514,7 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_cand_light(CandArgs 
 // Evaluates queue entries 0..cnt-1 for rebalancing and appends their records.
 template <int KWP, bool UNIT, int kTab>
 __device__ __forceinline__ void rb_batch(const CandArgs &a, uint8_t *stage, const WarpQueue *q, int cnt,
-                                         const long long *s_cap, const uint32_t (*s_elig)[KWP]) {
+                                         const long long *s_cap, const int *s_base, const uint32_t (*s_elig)[KWP]) {
   constexpr int NP = kLightPlanes;
   const int lane = threadIdx.x & 31;
   const bool mine = lane < cnt;
@@ -520,6 +538,10 @@ __device__ __forceinline__ void rb_batch(const CandArgs &a, uint8_t *stage, cons
     hi = rb_hi_of(a, conn - A, c);
     ct = (c << 16) | (s << 8) | t;
   }
+  if (a.rb_rec) {
+    rb_append(a, s_base, mine, s, hi, v, ct);
+    return;
+  }
   rb_first_level(a, mine, s, hi, v, c);
   const unsigned bal = __ballot_sync(kFull, mine);
   unsigned long long pos0 = 0;
@@ -537,7 +559,7 @@ template <int KWP, bool UNIT>
 __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArgs a) {
   constexpr int kTab = 32;  // eligibility words tabulated for c(v) <= 32
   __shared__ long long s_cap[kMaxK], s_bw[kMaxK];
-  __shared__ int s_over[kMaxK];
+  __shared__ int s_over[kMaxK], s_base[kMaxK];
   __shared__ uint32_t s_elig[kTab][KWP];
   __shared__ WarpQueue s_q[8];
   extern __shared__ __align__(16) uint8_t dyn_smem[];
@@ -548,6 +570,7 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
     s_cap[b] = a.rbb[b].cap;
     s_bw[b] = a.rbb[b].bw;
     s_over[b] = a.rbb[b].over;
+    s_base[b] = a.rbb[b].base;
   }
   __syncthreads();
   for (int x = threadIdx.x; x < kTab * KWP; x += blockDim.x) {
@@ -566,7 +589,7 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
   int64_t base = ((int64_t)blockIdx.x * warps + w) * 32;
   GroupRaw cur = fetch_group(a, base + lane, false);
   int qn = 0;
-  unsigned long long w_over = 0, w_eval = 0, w_pins = 0;
+  unsigned w_over = 0, w_eval = 0, w_pins = 0;  // one thread's share: light vertices have fewer than 64 incidences
   for (; base < a.n; base += stride) {
     const GroupRaw nxt = fetch_group(a, base + stride + lane, false);
     const int64_t v = base + lane;
@@ -600,12 +623,12 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
     }
     qn = enqueue(q, qn, act, (int)v, s, c, j0, deg);
     if (qn >= 32) {
-      rb_batch<KWP, UNIT, kTab>(a, stage, q, 32, s_cap, s_elig);
+      rb_batch<KWP, UNIT, kTab>(a, stage, q, 32, s_cap, s_base, s_elig);
       qn = dequeue32(q, qn);
     }
     cur = nxt;
   }
-  if (qn > 0) rb_batch<KWP, UNIT, kTab>(a, stage, q, qn, s_cap, s_elig);
+  if (qn > 0) rb_batch<KWP, UNIT, kTab>(a, stage, q, qn, s_cap, s_base, s_elig);
   count_work(a.cnt, w_over, w_eval, w_pins);
 }
 
@@ -653,6 +676,13 @@ __global__ void __launch_bounds__(256) k_rbcand_heavy(CandArgs a) {
     }
     warp_argmax(bc, bb);
     const uint64_t hi = rb_hi_of(a, bc - A, c);
+    if (a.rb_rec) {
+      if (lane == 0) {
+        const int at = a.rbb[s].base + atomicAdd(&a.rb_cur[s * kCurStride], 1);
+        if (at < a.n) a.rb_rec[at] = RbRec{hi, v, (c << 16) | (s << 8) | bb};
+      }
+      continue;
+    }
     rb_first_level(a, lane == 0, s, hi, v, c);
     if (lane == 0) {
       const unsigned long long pos = atomicAdd(&a.cnt->n_rec, 1ull);
@@ -729,6 +759,8 @@ CandArgs make_args(jet_ctx *c, const int32_t *part, const int32_t *phi) {
   a.rb_compact = c->rb_compact;
   a.rb_L = c->rb_L;
   a.rb_Pmax = c->rb_Pmax;
+  a.rb_rec = c->rb_segments ? c->rb_rec : nullptr;
+  a.rb_cur = c->rb_cur;
   a.rb_hist = c->rb_hist;
   a.rb_vbits = c->rb_vbits;
   a.rb_tbits = c->rb_hbits + c->rb_vbits;

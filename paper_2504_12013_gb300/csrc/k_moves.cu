@@ -20,7 +20,6 @@ struct MoveArgs {
   const int32_t *inc, *vwgt;
   int32_t *part, *phi;
   int64_t *bw;
-  int32_t *vcount;
   uint32_t *mask;
   const int32_t *mv_v;
   const uint32_t *mv_st;
@@ -124,7 +123,7 @@ __global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
   if (threadIdx.x == 0 && s_pins) atomicAdd(&a.cnt->w_apply_pins, s_pins);
   for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
     if (s_dw[b]) add_i64(reinterpret_cast<long long *>(&a.bw[b]), s_dw[b]);
-    if (s_dc[b]) atomicAdd(&a.vcount[b], s_dc[b]);
+    if (s_dc[b]) atomicAdd(&a.cnt->vcount[b], s_dc[b]);
   }
 }
 
@@ -148,6 +147,8 @@ constexpr int kPickThreads = 1024;
 struct RbArgs {
   const int64_t *bw;
   RbBlock *rbb;
+  const RbRec *rec;              // segmented records
+  int32_t *cur;                  // records of each block (kCurStride apart)
   const uint64_t *rb_hi;
   const int32_t *rb_v, *rb_ct;  // record: vertex; c << 16 | block << 8 | target
   unsigned long long *hist;
@@ -161,13 +162,33 @@ struct RbArgs {
   Counters *cnt;
 };
 
+// Exclusive prefix sum of x over the kMaxK threads of the block (every thread calls it).
+__device__ __forceinline__ int segment_base(int x) {
+  __shared__ int s_w[kMaxK / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int incl = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_w[wid] = incl;
+  __syncthreads();
+  int before = 0;
+#pragma unroll
+  for (int w = 0; w < kMaxK / 32; ++w) before += w < wid ? s_w[w] : 0;
+  return before + incl - x;
+}
+
 // Per-block state of the next round: overloaded flag, excess, target
 // capacity (deadzone and L_max), cleared selection state and counters.  One
 // block of kMaxK threads, thread b for block b.
 __device__ __forceinline__ void rb_prep_blocks(const RbArgs &a) {
   const int b = threadIdx.x;
+  const long long bwb = b < a.k ? a.bw[b] : 0;
+  const int room = bwb > a.Lmax ? a.cnt->vcount[b] : 0;
+  const int base = segment_base(room);
   if (b < a.k) {
-    const long long bwb = a.bw[b];
     RbBlock r;
     r.bw = bwb;
     r.over = bwb > a.Lmax ? 1 : 0;
@@ -177,7 +198,10 @@ __device__ __forceinline__ void rb_prep_blocks(const RbArgs &a) {
     r.pre_hi = 0;
     r.pre_lo = 0;
     r.all = 0;
+    r.room = room;
+    r.base = base;
     a.rbb[b] = r;
+    a.cur[b * kCurStride] = 0;
   }
   if (b == 0) {
     a.cnt->n_moves = 0;
@@ -298,6 +322,179 @@ __global__ void __launch_bounds__(kPickThreads) k_rb_pick(RbArgs a, int lo, int 
   for (int x = x0 + lane; x < x1; x += 32) row[x] = 0ull;
 }
 
+// Segmented form: one thread block per overloaded block of the partition does
+// the whole selection of a round in one launch.  The target kernels have put
+// the block's records into a segment of their own; each thread holds kSelHeld
+// of them in registers (any beyond are read again per level).  Per 8-bit
+// digit the block histograms its records in shared memory and every warp
+// picks the digit by itself, so a level has two barriers; after the last digit
+// the records up to the threshold go to the move list, which k_apply works
+// through.  Bound by the latency of the loads and levels.  A round's selection
+// was 2 x levels - 1 dependent launches whatever the number of records, and
+// the apply kernel looked at every record again: 1.03 -> 0.38 ms for the 26
+// rounds of 300k vertices at k = 200.  The line (kSegVertices, on average):
+// beyond a segment that fits the registers of one block, the grid-wide passes
+// are as fast.  Measured per round on 31k vertices per block: they take 34 us
+// at k = 128; clusters of 4 to 16 blocks per segment that sum their histograms
+// over distributed shared memory took 33 to 61, and the target kernels lose
+// more to the segments' cursors than that gives.
+constexpr int kSelThreads = 512;
+constexpr int kSelHeld = 8;  // records per thread held in registers
+constexpr int kSelBits = 8;
+constexpr int kSelBins = 1 << kSelBits;
+static_assert(kSelThreads * kSelHeld == kSegVertices, "a segment of average size fits the registers");
+
+template <class T>
+__device__ __forceinline__ T warp_incl(T x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(kFull, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// A record in registers; the priority part of a 64-bit key is compact (below 2^32).
+template <class KT>
+struct SelRec {
+  uint32_t hi = 0;
+  int32_t v = 0, ct = 0;
+  SelRec() = default;
+  __device__ __forceinline__ explicit SelRec(const RbRec &r) : hi((uint32_t)r.hi), v(r.v), ct(r.ct) {}
+};
+template <>
+struct SelRec<u128> {
+  unsigned long long hi = 0;
+  int32_t v = 0, ct = 0;
+  SelRec() = default;
+  __device__ __forceinline__ explicit SelRec(const RbRec &r) : hi(r.hi), v(r.v), ct(r.ct) {}
+};
+
+// WT: unsigned when c(V) < 2^32 (no sum of weights leaves it), else unsigned long long.
+template <class KT, class WT>
+__global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a) {
+  typedef SelRec<KT> Rec;
+  constexpr int kPer = kSelBins / 32;  // bins per lane
+  __shared__ __align__(16) WT s_hist[2][kSelBins];
+  const int t = threadIdx.x, lane = t & 31, b = blockIdx.x;
+  const RbBlock &blk = a.rbb[b];
+  const int over = blk.over, room = blk.room, count = a.cur[b * kCurStride];
+  const WT excess = (WT)blk.excess;
+  const RbRec *rec = a.rec + blk.base;
+  if (!over) return;
+  const int cnt = min(count, room);
+  Rec held[kSelHeld];  // weight 0: no record
+#pragma unroll
+  for (int q = 0; q < kSelHeld; ++q)
+    held[q] = t + q * kSelThreads < cnt ? Rec(rec[t + q * kSelThreads]) : Rec();
+  if (t < kSelBins) s_hist[0][t] = s_hist[1][t] = 0;
+  __syncthreads();
+  KT pre = 0;  // the fixed digits of the threshold key
+  WT before = 0;
+  bool all = false;
+  int buf = 0;
+  for (int up = a.tbits; up > 0; buf ^= 1) {
+    const int lo = up > kSelBits ? up - kSelBits : 0;
+    const unsigned dmask = (1u << (up - lo)) - 1;
+    auto add = [&](const Rec &r) {
+      const KT K = rb_full_key<KT>(r.hi, r.v, a.vbits);
+      const WT c = (WT)(unsigned)(r.ct >> 16);
+      if (c && (up >= a.tbits || (K >> up) == (pre >> up))) atomicAdd(&s_hist[buf][(unsigned)(K >> lo) & dmask], c);
+    };
+#pragma unroll
+    for (int q = 0; q < kSelHeld; ++q)
+      if (q * kSelThreads < cnt) add(held[q]);
+    for (int i = t + kSelHeld * kSelThreads; i < cnt; i += 4 * kSelThreads) {
+      Rec r[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = i + q * kSelThreads < cnt ? Rec(rec[i + q * kSelThreads]) : Rec();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) add(r[q]);
+    }
+    __syncthreads();
+    if (t < kSelBins) s_hist[buf ^ 1][t] = 0;  // read a level ago
+    const WT *sum = s_hist[buf] + lane * kPer;
+    WT w[kPer], mine = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      w[q] = sum[q];
+      mine += w[q];
+    }
+    const WT incl = warp_incl(mine);
+    if (up >= a.tbits && __shfl_sync(kFull, incl, 31) < excess) {  // every record moves
+      all = true;
+      break;
+    }
+    // the lane whose bins reach the excess, and the bin
+    WT run = before + incl - mine;
+    const unsigned hit = __ballot_sync(kFull, run < excess && run + mine >= excess);
+    int digit = lane * kPer;
+    bool more = true;
+#pragma unroll
+    for (int q = 0; q < kPer - 1; ++q) {
+      more = more && run + w[q] < excess;
+      if (more) {
+        run += w[q];
+        ++digit;
+      }
+    }
+    const int src = hit ? __ffs(hit) - 1 : 0;
+    before = __shfl_sync(kFull, run, src);
+    pre |= (KT)(unsigned)__shfl_sync(kFull, digit, src) << lo;
+    up = lo;
+    if (up > 0) __syncthreads();  // the cleared buffer is added to next
+  }
+  // the records up to the threshold: one atomic per warp (and batch) on the move list
+  auto emit = [&](const Rec *r, int n) {
+    unsigned bal[kSelHeld], tot = 0;
+#pragma unroll
+    for (int q = 0; q < kSelHeld; ++q) {
+      bal[q] = 0;
+      if (q < n) {
+        const bool sel = (r[q].ct >> 16) && (all || rb_full_key<KT>(r[q].hi, r[q].v, a.vbits) <= pre);
+        bal[q] = __ballot_sync(kFull, sel);
+        tot += __popc(bal[q]);
+      }
+    }
+    if (!tot) return;
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(&a.cnt->n_moves, (unsigned long long)tot);
+    at = __shfl_sync(kFull, at, 0);
+#pragma unroll
+    for (int q = 0; q < kSelHeld; ++q) {
+      if (q < n) {
+        if ((bal[q] >> lane) & 1u) {
+          const unsigned long long x = at + __popc(bal[q] & ((1u << lane) - 1));
+          a.mv_v[x] = r[q].v;
+          a.mv_st[x] = (uint32_t)b | ((uint32_t)(r[q].ct & 255) << 16);
+        }
+        at += __popc(bal[q]);
+      }
+    }
+  };
+  emit(held, kSelHeld);
+  // the warp's lanes go together, from its first record
+  for (int i = t + kSelHeld * kSelThreads, iw = i - lane; iw < cnt; i += 4 * kSelThreads, iw += 4 * kSelThreads) {
+    Rec r[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) r[q] = i + q * kSelThreads < cnt ? Rec(rec[i + q * kSelThreads]) : Rec();
+    emit(r, 4);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_count_blocks(const int32_t *part, int32_t n, int32_t k, Counters *cnt) {
+  __shared__ int s_c[kMaxK];
+  s_c[threadIdx.x] = 0;  // kMaxK = blockDim.x
+  __syncthreads();
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int b = part[v];
+    if ((unsigned)b < (unsigned)k) atomicAdd(&s_c[b], 1);
+  }
+  __syncthreads();
+  if (s_c[threadIdx.x]) atomicAdd(&cnt->vcount[threadIdx.x], s_c[threadIdx.x]);
+}
+
 // Apply the selection: every record with K(v) <= its block's threshold (or of
 // an `all` block) moves v to its target.  A warp tests 32 records (one per
 // lane) and then applies the selected ones four at a time, kMoveLanes lanes
@@ -372,7 +569,7 @@ __global__ void __launch_bounds__(256) k_rb_apply(RbArgs r, MoveArgs a) {
   }
   for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
     if (s_dw[b]) add_i64(reinterpret_cast<long long *>(&a.bw[b]), s_dw[b]);
-    if (s_dc[b]) atomicAdd(&a.vcount[b], s_dc[b]);
+    if (s_dc[b]) atomicAdd(&a.cnt->vcount[b], s_dc[b]);
   }
 }
 
@@ -453,7 +650,6 @@ MoveArgs move_args(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   a.part = part;
   a.phi = phi;
   a.bw = block_w;
-  a.vcount = c->vcount;
   a.mask = c->mask;
   a.graph = c->graph_path;
   a.mv_v = c->mv_v;
@@ -468,6 +664,8 @@ RbArgs rb_args(jet_ctx *c, const int64_t *block_w, const int32_t *part) {
   RbArgs a{};
   a.bw = block_w;
   a.rbb = c->rbb;
+  a.rec = c->rb_rec;
+  a.cur = c->rb_cur;
   a.rb_hi = c->rb_hi;
   a.rb_v = c->rb_v;
   a.rb_ct = c->rb_ct;
@@ -491,6 +689,7 @@ RbArgs rb_args(jet_ctx *c, const int64_t *block_w, const int32_t *part) {
 }  // namespace
 
 cudaError_t prepare_move_kernels(jet_ctx *c) {
+  c->rb_segments = c->n / c->k <= kSegVertices ? 1 : 0;
   cudaError_t e = resident_blocks(k_apply, 256, 0, &c->move_bps[0]);
   if (e == cudaSuccess) e = resident_blocks(k_rb_apply<unsigned long long>, 256, 0, &c->move_bps[1]);
   if (e == cudaSuccess) e = resident_blocks(k_rb_apply<u128>, 256, 0, &c->move_bps[2]);
@@ -528,9 +727,26 @@ void rb_select_levels(jet_ctx *c, const RbArgs &a) {
   }
 }
 
+template <class KT>
+cudaError_t select_segments(jet_ctx *c, const RbArgs &a) {
+  if (c->W < (1ll << 32)) k_rb_select<KT, unsigned><<<c->k, kSelThreads, 0, c->stream>>>(a);
+  else k_rb_select<KT, unsigned long long><<<c->k, kSelThreads, 0, c->stream>>>(a);
+  ++c->kernel_launches;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
+  if (c->n == 0) return cudaSuccess;
+  k_count_blocks<<<grid_for(c->n, 1024, c->launch_sms, 4), kMaxK, 0, c->stream>>>(part, c->n, c->k, c->cnt);
+  ++c->kernel_launches;
+  return cudaGetLastError();
+}
+
 cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part) {
   if (c->n == 0) return cudaSuccess;
   const RbArgs a = rb_args(c, nullptr, part);
+  if (c->rb_segments)
+    return a.tbits <= 64 ? select_segments<unsigned long long>(c, a) : select_segments<u128>(c, a);
   if (a.tbits <= 64) rb_select_levels<unsigned long long>(c, a);
   else rb_select_levels<u128>(c, a);
   return cudaGetLastError();
@@ -538,6 +754,7 @@ cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part) {
 
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   if (c->n == 0) return cudaSuccess;
+  if (c->rb_segments) return launch_apply(c, part, phi, block_w);  // the selection is a move list
   const RbArgs r = rb_args(c, block_w, part);
   const MoveArgs a = move_args(c, part, phi, block_w);
   if (r.tbits <= 64)

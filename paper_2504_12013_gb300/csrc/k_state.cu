@@ -307,17 +307,15 @@ __global__ void __launch_bounds__(256) k_pincounts_seg(const int64_t *eptr, cons
   if (err) atomicOr(&cnt->err, err);
 }
 
-// c(V_i) and |V_i|, aggregated per thread block in shared memory.  Bound by
-// the shared-memory atomics on k addresses, so their number and width count:
-// W = uint32_t when a block's share of the weights cannot leave 32 bits (the
-// launcher checks it against max c(v)), and no weight atomics at all when
-// every c(v) is 1.  Four vertices in flight per thread.
-template <class W, bool UNIT>
+// c(V_i), aggregated per thread block in shared memory.  Bound by the
+// shared-memory atomics on k addresses, so their width counts: W = unsigned
+// when a block's share of the weights cannot leave 32 bits (the launcher
+// checks it against max c(v)).  Four vertices in flight per thread.
+template <class W>
 __global__ void __launch_bounds__(256) k_block_weights(const int32_t *part, const int32_t *vwgt, int32_t n, int32_t k,
-                                                       int64_t *bw, int32_t *vcount, Counters *cnt) {
+                                                       int64_t *bw, Counters *cnt) {
   __shared__ W s_bw[kMaxK];
-  __shared__ int s_cnt[kMaxK];
-  for (int b = threadIdx.x; b < k; b += blockDim.x) { s_bw[b] = 0; s_cnt[b] = 0; }
+  for (int b = threadIdx.x; b < k; b += blockDim.x) s_bw[b] = 0;
   __syncthreads();
   int err = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -327,24 +325,17 @@ __global__ void __launch_bounds__(256) k_block_weights(const int32_t *part, cons
     for (int q = 0; q < 4; ++q) {
       const int64_t v = v0 + q * stride;
       b[q] = v < n ? part[v] : -2;
-      c[q] = !UNIT && v < n ? vwgt[v] : 1;
+      c[q] = v < n ? vwgt[v] : 0;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      if ((unsigned)b[q] < (unsigned)k) {
-        if constexpr (!UNIT) atomicAdd(&s_bw[b[q]], (W)c[q]);
-        atomicAdd(&s_cnt[b[q]], 1);
-      } else if (v0 + q * stride < n) {
-        err |= kErrPartRange;
-      }
+      if ((unsigned)b[q] < (unsigned)k) atomicAdd(&s_bw[b[q]], (W)c[q]);
+      else if (v0 + q * stride < n) err |= kErrPartRange;
     }
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < k; b += blockDim.x) {
-    if (!s_cnt[b]) continue;
-    add_i64(reinterpret_cast<long long *>(&bw[b]), UNIT ? (long long)s_cnt[b] : (long long)s_bw[b]);
-    atomicAdd(&vcount[b], s_cnt[b]);
-  }
+  for (int b = threadIdx.x; b < k; b += blockDim.x)
+    if (s_bw[b]) add_i64(reinterpret_cast<long long *>(&bw[b]), (long long)s_bw[b]);
   if (err) atomicOr(&cnt->err, err);
 }
 
@@ -608,7 +599,6 @@ cudaError_t prepare_state_kernels(jet_ctx *c) {
 cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int64_t *block_w) {
   cudaStream_t s = c->stream;
   cudaError_t e = cudaMemsetAsync(block_w, 0, sizeof(int64_t) * c->k, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->vcount, 0, sizeof(int32_t) * c->k, s);
   if (e != cudaSuccess) return e;
   if (c->m > 0 && phi) {
     const bool vec = c->k % 4 == 0 && ((uintptr_t)phi & 15) == 0;
@@ -634,13 +624,10 @@ cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int6
   if (c->n > 0) {
     const int g = grid_for(c->n, 1024, c->launch_sms, 4);
     const long long share = ((c->n - 1ll) / (1024ll * g) + 1) * 1024;  // vertices of a block, at most
-    if (c->cmax <= 1)
-      k_block_weights<unsigned, true><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->vcount, c->cnt);
-    else if (share * c->cmax < (1ll << 32))
-      k_block_weights<unsigned, false><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->vcount, c->cnt);
+    if (share * c->cmax < (1ll << 32))
+      k_block_weights<unsigned><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->cnt);
     else
-      k_block_weights<unsigned long long, false><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->vcount,
-                                                                   c->cnt);
+      k_block_weights<unsigned long long><<<g, 256, 0, s>>>(part, c->vwgt, c->n, c->k, block_w, c->cnt);
     ++c->kernel_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
