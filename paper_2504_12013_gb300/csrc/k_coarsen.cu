@@ -16,16 +16,17 @@
 // vertices move together.
 //
 //   k_cl_serial   the leading one-vertex sub-rounds, one block, in order
-//   k_cl_rate     hash table of the neighbour clusters per vertex, a warp
-//                 per vertex (table in shared memory, else a slice of a
-//                 global pool sized per sub-round)
-//   k_cl_rate_heavy  a 16-warp block per vertex whose table exceeds 2048
-//                 entries: the warps take its edges from a shared counter
-//                 (edges above 64 pins first), each edge's clusters
-//                 deduplicated in a per-warp set, the sums integer atomics
-//   k_cl_swap     swap prevention, group lists of the proposals
-//   k_cl_approve  weight-ordered prefix per target (fast path: all fit)
-//   k_cl_apply    moves, resets the per-sub-round state
+//   k_cl_rate     the rating of vertices with few rated pins, a warp each;
+//   k_cl_rate_block  of those with more, a thread block each (two sizes): the
+//                 (edge, pin) pairs are spread evenly over the threads, a
+//                 hash set of (edge, cluster) pairs counts a cluster once per
+//                 edge and a hash table of clusters sums, both in shared memory
+//   k_cl_rate_pool   vertices whose tables exceed shared memory: edges are
+//                 deduplicated one at a time, the sums in a global pool
+//   k_cl_settle   swap prevention and group lists of the proposals, the
+//                 weight-ordered prefix per target (fast path: all fit), the
+//                 moves, in one cluster (k_cl_swap, k_cl_approve, k_cl_apply
+//                 for large sub-rounds)
 //
 // Contraction.  Non-empty label classes become coarse vertices in label
 // order; each edge keeps its distinct coarse pins (ascending), is dropped
@@ -42,14 +43,22 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kTile = 2048;        // scan / radix tile: 256 threads x 8 items
-constexpr int kSmemTab = 128;      // hash-table entries per warp held in shared memory
-constexpr int kWarpTab = 2048;     // larger tables: the whole block rates the vertex (heavy vertices)
-constexpr int kBlockTab = 4096;    // a heavy vertex's table in shared memory up to this size
-constexpr int kHeavyWarps = 16;    // warps of a block that rates one heavy vertex
+// Classes of vertices by table size (entries, at least twice the rated pins): a warp, a small and a large block,
+// the pool.
+constexpr int kWarpTab = 128, kMidTab = 2048, kBlockTab = 8192;
+constexpr int kMidThreads = 256, kBigThreads = 512;
+constexpr int kSettleSize = 16384;  // sub-rounds up to this size are settled by one cluster
+constexpr int kSettleBlocks = 8, kSettleThreads = 1024;
+constexpr int kHeavyWarps = 16;    // warps of a block that rates one vertex with a table in the pool
 constexpr int kFirstEdge = 64;     // a heavy vertex's edges above this size are rated first
 constexpr int kSetCap = 2048;      // per-warp set of the distinct clusters of one edge (heavy vertices)
 constexpr int kSetEdge = kSetCap / 2;  // edges up to this size are deduplicated in that set
-constexpr size_t kHeavySmem = sizeof(int32_t) * kHeavyWarps * kSetCap + 16 * kBlockTab;
+constexpr size_t kHeavySmem = sizeof(int32_t) * kHeavyWarps * kSetCap;
+
+// Shared memory of a block that rates one vertex: pair set, sums, labels, and the edges of a chunk.
+constexpr size_t rate_smem(int tab, int threads) { return (size_t)tab * 20 + (size_t)threads * 20; }
+constexpr size_t kSerialSmem =
+    rate_smem(kBlockTab, kBigThreads) > kHeavySmem ? rate_smem(kBlockTab, kBigThreads) : kHeavySmem;
 constexpr int64_t kMaxTab = 1 << 28;
 
 struct Tab {
@@ -338,26 +347,32 @@ __device__ __forceinline__ int round_of(const int32_t *bounds, int32_t rounds, i
   return lo;
 }
 
-// Per sub-round: heavy vertices (tables beyond kWarpTab) and the global-pool entries of the tables that
-// fit neither a warp's shared slice nor a block's shared memory.
+// Class of a vertex by its table: 0 a warp, 1 a small block, 2 a large block, 3 the pool.
+__device__ __forceinline__ int rate_class(int32_t cap) {
+  return cap <= kWarpTab ? 0 : cap <= kMidTab ? 1 : cap <= kBlockTab ? 2 : 3;
+}
+
+// Per sub-round: vertices of classes 1..3 (counts[(class - 1) * rounds + r]) and the pool entries of class 3.
 __global__ void k_cl_need(const int32_t *order, int32_t n, const int32_t *bounds, int32_t rounds, const int32_t *cap,
-                          unsigned long long *need, unsigned long long *heavy) {
+                          unsigned long long *need, unsigned long long *counts) {
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
     const int32_t c = cap[order[x]];
-    if (c <= kSmemTab) continue;
+    const int cl = rate_class(c);
+    if (cl == 0) continue;
     const int r = round_of(bounds, rounds, x);
-    if (c > kWarpTab) atomicAdd(&heavy[r], 1ull);
-    if (c <= kWarpTab || c > kBlockTab) atomicAdd(&need[r], (unsigned long long)c);
+    atomicAdd(&counts[(int64_t)(cl - 1) * rounds + r], 1ull);
+    if (cl == 3) atomicAdd(&need[r], (unsigned long long)c);
   }
 }
 
-// The heavy positions of every sub-round, at hoff[r] onwards (any order within a sub-round).
-__global__ void k_cl_heavy_list(const int32_t *order, int32_t n, const int32_t *bounds, int32_t rounds,
-                                const int32_t *cap, const int64_t *hoff, unsigned long long *hcur, int32_t *hpos) {
+// The positions of classes 1..3 of every sub-round, at off[(class - 1) * rounds + r] onwards (any order within).
+__global__ void k_cl_class_list(const int32_t *order, int32_t n, const int32_t *bounds, int32_t rounds,
+                                const int32_t *cap, const int64_t *off, unsigned long long *cur, int32_t *pos) {
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-    if (cap[order[x]] <= kWarpTab) continue;
-    const int r = round_of(bounds, rounds, x);
-    hpos[hoff[r] + (int64_t)atomicAdd(&hcur[r], 1ull)] = (int32_t)x;
+    const int cl = rate_class(cap[order[x]]);
+    if (cl == 0) continue;
+    const int64_t i = (int64_t)(cl - 1) * rounds + round_of(bounds, rounds, x);
+    pos[off[i] + (int64_t)atomicAdd(&cur[i], 1ull)] = (int32_t)x;
   }
 }
 
@@ -376,69 +391,229 @@ __device__ __forceinline__ uint32_t tab_slot(Tab *tab, int32_t cap, int32_t C) {
 }
 
 
-// The rating of u over the clusters of its neighbours, accumulated in tab (cap entries, a power of
-// two above twice the rated pins), and the best cluster within the weight bound (-1 if none).
-// Called by a whole warp.
-__device__ int32_t rate_vertex(const jet_hypergraph &g, int32_t u, const int32_t *label, const long long *cw,
-                               long long cmax, int32_t rmax, Tab *tab, int32_t cap, int lane) {
-  for (int i = lane; i < cap; i += 32) {
-    tab[i].key = -1;
-    tab[i].last = -1;
-    tab[i].val = 0;
-  }
-  __syncwarp();
-  const int64_t i1 = g.vptr[u + 1];
-  for (int64_t i = g.vptr[u]; i < i1; ++i) {
-    const int32_t e = g.inc[i];
-    const int64_t p0 = g.eptr[e], p1 = g.eptr[e + 1];
-    const int64_t size = p1 - p0;
-    if (size < 2 || size > rmax) continue;
-    const unsigned long long term = ((unsigned long long)(uint32_t)g.ewgt[e] << 32) / (unsigned long long)(size - 1);
-    for (int64_t p = p0; p < p1; p += 128) {  // four chunks of 32 pins in flight, applied in order
-      int32_t C[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int64_t pp = p + q * 32 + lane;
-        C[q] = pp < p1 ? g.pins[pp] : u;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) C[q] = C[q] != u ? label[C[q]] : -1;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const unsigned peers = __match_any_sync(kFull, C[q]);
-        if (C[q] >= 0 && C[q] != u && lane == __ffs(peers) - 1) {  // one lane per distinct cluster of this chunk
-          const uint32_t h = tab_slot(tab, cap, C[q]);
-          if (tab[h].last != e) {  // once per edge and cluster
-            tab[h].last = e;
-            tab[h].val += term;
-          }
-        }
-        __syncwarp();
-      }
+// A vertex's rating in shared memory.  Every rated pin is one (edge, pin)
+// item; an item adds omega(e)/(|e|-1) to its cluster if it is the first of its
+// (edge, cluster) pair, so the items can go in any order and all threads work
+// on them at once, four loads in flight each.  The rating was edge after edge
+// (four dependent loads, and a look at the entry's last edge, per 32 pins,
+// mostly in a global table), and a sub-round waited for its slowest vertex:
+// 215 us for the warps plus 114 us for the heavy vertices after them, on 5,000
+// vertices of the VLSI workload.
+struct RateTab {
+  unsigned long long *pairs;  // edge (index in I(u)) << 32 | cluster; ~0 = empty
+  unsigned long long *vals;
+  int32_t *keys;              // cluster label; -1 = empty
+  uint32_t mask;              // entries - 1; entries >= 2 x rated pins, so neither table fills up
+};
+
+__device__ __forceinline__ void rate_item(const RateTab &tb, uint32_t edge, int32_t C, unsigned long long term) {
+  const unsigned long long key = ((unsigned long long)edge << 32) | (uint32_t)C;
+  uint32_t h = mix32((uint32_t)C + edge * 0x9e3779b9u) & tb.mask;
+  for (;;) {
+    unsigned long long k = *(volatile unsigned long long *)&tb.pairs[h];
+    if (k == ~0ull) {
+      k = atomicCAS(&tb.pairs[h], ~0ull, key);
+      if (k == ~0ull) break;
     }
+    if (k == key) return;  // counted
+    h = (h + 1) & tb.mask;
   }
-  const long long cu = g.vwgt[u];
-  unsigned long long bv = 0;
-  int32_t bk = -1;
-  for (int i = lane; i < cap; i += 32) {
-    const int32_t k = tab[i].key;
-    if (k < 0 || cw[k] + cu > cmax) continue;
-    const unsigned long long v = tab[i].val;
-    if (bk < 0 || v > bv || (v == bv && k < bk)) {
-      bv = v;
-      bk = k;
+  h = mix32((uint32_t)C) & tb.mask;
+  for (;;) {
+    int32_t k = *(volatile int32_t *)&tb.keys[h];
+    if (k == -1) {
+      k = atomicCAS(&tb.keys[h], -1, C);
+      if (k == -1) k = C;
     }
+    if (k == C) break;
+    h = (h + 1) & tb.mask;
+  }
+  atomicAdd(&tb.vals[h], term);
+}
+
+__device__ __forceinline__ void better(unsigned long long &bv, int32_t &bk, unsigned long long v, int32_t k) {
+  if (k >= 0 && (bk < 0 || v > bv || (v == bv && k < bk))) {
+    bv = v;
+    bk = k;
+  }
+}
+
+// The best cluster of entries i0, i0 + step, ... of the table within the weight bound, reduced over the warp.
+__device__ __forceinline__ void rate_best(const RateTab &tb, int i0, int step, const long long *cw, long long room,
+                                          unsigned long long &bv, int32_t &bk) {
+  bv = 0;
+  bk = -1;
+  for (uint32_t i = i0; i <= tb.mask; i += 4 * step) {
+    int32_t k[4];
+    long long w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      k[q] = i + q * step <= tb.mask ? tb.keys[i + q * step] : -1;
+      w[q] = k[q] >= 0 ? cw[k[q]] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (k[q] >= 0 && w[q] <= room) better(bv, bk, tb.vals[i + q * step], k[q]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long ov = __shfl_xor_sync(kFull, bv, o);
     const int32_t ok = __shfl_xor_sync(kFull, bk, o);
-    if (ok >= 0 && (bk < 0 || ov > bv || (ov == bv && ok < bk))) {
-      bv = ov;
-      bk = ok;
+    better(bv, bk, ov, ok);
+  }
+}
+
+// The rated edge i of u: first pin, pins (0 if it adds nothing) and the term of its clusters.
+__device__ __forceinline__ int rated_edge(const jet_hypergraph &g, int64_t i, int32_t rmax, int64_t &p0,
+                                          unsigned long long &term) {
+  const int32_t e = g.inc[i];
+  const uint32_t w = (uint32_t)g.ewgt[e];
+  p0 = g.eptr[e];
+  const int64_t size = g.eptr[e + 1] - p0;
+  if (size < 2 || size > rmax) return 0;
+  term = ((unsigned long long)w << 32) / (unsigned long long)(size - 1);
+  return (int)size;
+}
+
+// By one warp: the edges go 32 at a time, one per lane; the lanes share out their pins.
+__device__ __forceinline__ int32_t rate_warp(const jet_hypergraph &g, int32_t u, const int32_t *label,
+                                             const long long *cw, long long cmax, int32_t rmax, const RateTab &tb,
+                                             int lane) {
+  for (uint32_t i = lane; i <= tb.mask; i += 32) {
+    tb.pairs[i] = ~0ull;
+    tb.vals[i] = 0;
+    tb.keys[i] = -1;
+  }
+  __syncwarp();
+  const int64_t i0 = g.vptr[u], i1 = g.vptr[u + 1];
+  const long long room = cmax - g.vwgt[u];
+  for (int64_t c = i0; c < i1; c += 32) {
+    int64_t p0 = 0;
+    unsigned long long term = 0;
+    const int size = c + lane < i1 ? rated_edge(g, c + lane, rmax, p0, term) : 0;
+    int off = size;  // exclusive prefix of the sizes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, off, o);
+      if (lane >= o) off += y;
+    }
+    const int total = __shfl_sync(kFull, off, 31);
+    off -= size;
+    for (int x0 = 0; x0 < total; x0 += 128) {
+      int src[4];
+      int32_t C[4];
+      unsigned long long tm[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int x = x0 + q * 32 + lane;
+        int j = 0;  // the last lane whose offset is <= x (of equal ones, that with pins)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const int y = __shfl_sync(kFull, off, j + o);
+          if (y <= x) j += o;
+        }
+        src[q] = j;
+        const int64_t p = __shfl_sync(kFull, p0, j);
+        const int of = __shfl_sync(kFull, off, j);
+        tm[q] = __shfl_sync(kFull, term, j);
+        C[q] = x < total ? g.pins[p + (x - of)] : u;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) C[q] = C[q] != u ? label[C[q]] : -1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (C[q] >= 0 && C[q] != u) rate_item(tb, (uint32_t)(c - i0) + src[q], C[q], tm[q]);
     }
   }
   __syncwarp();
+  unsigned long long bv;
+  int32_t bk;
+  rate_best(tb, lane, 32, cw, room, bv, bk);
+  __syncwarp();
+  return bk;
+}
+
+// By a block of T threads: the edges go T at a time.  smem: rate_smem(table entries, T).
+template <int T>
+__device__ __forceinline__ int32_t rate_block(const jet_hypergraph &g, int32_t u, const int32_t *label,
+                                              const long long *cw, long long cmax, int32_t rmax, int32_t cap,
+                                              unsigned long long *smem) {
+  __shared__ int s_scan[T / 32 + 1];
+  __shared__ unsigned long long s_bv[T / 32];
+  __shared__ int32_t s_bk[T / 32];
+  RateTab tb;
+  tb.mask = (uint32_t)cap - 1;
+  unsigned long long *s_term = smem;
+  long long *s_p0 = reinterpret_cast<long long *>(s_term + T);
+  int *s_off = reinterpret_cast<int *>(s_p0 + T);
+  tb.pairs = reinterpret_cast<unsigned long long *>(s_off + T);
+  tb.vals = tb.pairs + cap;
+  tb.keys = reinterpret_cast<int32_t *>(tb.vals + cap);
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  for (int i = t; i < cap; i += T) {
+    tb.pairs[i] = ~0ull;
+    tb.vals[i] = 0;
+    tb.keys[i] = -1;
+  }
+  const int64_t i0 = g.vptr[u], i1 = g.vptr[u + 1];
+  const long long room = cmax - g.vwgt[u];
+  for (int64_t c = i0; c < i1; c += T) {
+    int64_t p0 = 0;
+    unsigned long long term = 0;
+    const int size = c + t < i1 ? rated_edge(g, c + t, rmax, p0, term) : 0;
+    int off = size;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, off, o);
+      if (lane >= o) off += y;
+    }
+    __syncthreads();  // the chunk before has been used (and, at first, the tables are clear)
+    if (lane == 31) s_scan[wid] = off;
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) {
+      before += w < wid ? s_scan[w] : 0;
+      total += s_scan[w];
+    }
+    s_off[t] = before + off - size;
+    s_p0[t] = p0;
+    s_term[t] = term;
+    __syncthreads();
+    for (int x0 = t; x0 < total; x0 += 4 * T) {
+      int src[4];
+      int32_t C[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int x = x0 + q * T;
+        int j = 0;  // the last edge whose offset is <= x
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1)
+          if (s_off[j + o] <= x) j += o;
+        src[q] = j;
+        C[q] = x < total ? g.pins[s_p0[j] + (x - s_off[j])] : u;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) C[q] = C[q] != u ? label[C[q]] : -1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (C[q] >= 0 && C[q] != u) rate_item(tb, (uint32_t)(c - i0) + src[q], C[q], s_term[src[q]]);
+    }
+  }
+  __syncthreads();
+  unsigned long long bv;
+  int32_t bk;
+  rate_best(tb, t, T, cw, room, bv, bk);
+  if (lane == 0) {
+    s_bv[wid] = bv;
+    s_bk[wid] = bk;
+  }
+  __syncthreads();
+  bk = -1;
+  bv = 0;
+#pragma unroll
+  for (int w = 0; w < T / 32; ++w) better(bv, bk, s_bv[w], s_bk[w]);
+  __syncthreads();
   return bk;
 }
 
@@ -457,15 +632,15 @@ __device__ __forceinline__ bool set_insert(int32_t *set, int32_t scap, int32_t C
   }
 }
 
-// The rating of a heavy vertex by the whole block (same result as rate_vertex).  Its edges are spread
+// The rating of a vertex with its table in the pool, by the whole block (same result).  Its edges are spread
 // over the warps and the sums are atomic (integer, order-free); a cluster counts once per edge through
 // match_any within a chunk and, for edges of 33 to kSetEdge pins, the warp's set of the edge's
 // clusters.  Larger edges follow, by warp 0 alone, counted once per edge and cluster through the
 // entry's last edge.  s_set: kHeavyWarps x kSetCap words; s_bk/s_bv: per-warp reduction scratch;
 // s_next: the shared edge counters of the two passes.
 // Chunks of an edge are taken four at a time, so that their loads overlap.
-__device__ int32_t rate_block(const jet_hypergraph &g, int32_t u, const int32_t *label, const long long *cw,
-                              long long cmax, int32_t rmax, Tab *tab, int32_t cap, int32_t *s_set,
+__device__ int32_t rate_pool(const jet_hypergraph &g, int32_t u, const int32_t *label, const long long *cw,
+                             long long cmax, int32_t rmax, Tab *tab, int32_t cap, int32_t *s_set,
                               int32_t *s_bk, unsigned long long *s_bv, int *s_next) {
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
   for (int i = t; i < cap; i += blockDim.x) {
@@ -597,21 +772,25 @@ __device__ int32_t rate_block(const jet_hypergraph &g, int32_t u, const int32_t 
 }
 
 // One-vertex sub-rounds x0..x1 in order, by one block: no swaps, and a proposal always fits (it was
-// rated only if c(C) + c(u) <= cmax), so the vertex moves at once.  Dynamic shared memory: kHeavySmem.
-__global__ void __launch_bounds__(kHeavyWarps * 32) k_cl_serial(jet_hypergraph g, const int32_t *order, int32_t x0, int32_t x1,
-                                                   long long cmax, int32_t rmax, Cl cl, Tab *pool) {
+// rated only if c(C) + c(u) <= cmax), so the vertex moves at once.  Dynamic shared memory: kSerialSmem.
+__global__ void __launch_bounds__(kBigThreads) k_cl_serial(jet_hypergraph g, const int32_t *order, int32_t x0,
+                                                           int32_t x1, long long cmax, int32_t rmax, Cl cl,
+                                                           Tab *pool) {
   extern __shared__ unsigned long long s_dyn[];
   __shared__ int32_t s_bk[kHeavyWarps];
   __shared__ unsigned long long s_bv[kHeavyWarps];
   __shared__ int s_next[2];
-  Tab *s_tab = reinterpret_cast<Tab *>(s_dyn);
-  int32_t *s_set = reinterpret_cast<int32_t *>(s_tab + kBlockTab);
   for (int32_t x = x0; x < x1; ++x) {
     const int32_t u = order[x];
     if (cl.csize[u] != 1 || cl.label[u] != u) continue;
     const int32_t cap = cl.cap[u];
-    const int32_t j = rate_block(g, u, cl.label, cl.cw, cmax, rmax, cap <= kBlockTab ? s_tab : pool, cap, s_set,
-                                 s_bk, s_bv, s_next);
+    if (cap == 0) continue;  // no rated edge
+    int32_t j;
+    if (cap <= kBlockTab)
+      j = rate_block<kBigThreads>(g, u, cl.label, cl.cw, cmax, rmax, cap, s_dyn);
+    else
+      j = rate_pool(g, u, cl.label, cl.cw, cmax, rmax, pool, cap, reinterpret_cast<int32_t *>(s_dyn), s_bk, s_bv,
+                    s_next);
     if (j >= 0 && threadIdx.x == 0) {
       const long long c = g.vwgt[u];
       cl.label[u] = j;
@@ -624,61 +803,60 @@ __global__ void __launch_bounds__(kHeavyWarps * 32) k_cl_serial(jet_hypergraph g
   }
 }
 
-// Warp per position of the sub-round: the vertices of tables up to kWarpTab entries (in the warp's
-// shared slice, else a slice of the global pool).
+__device__ __forceinline__ void propose(const jet_hypergraph &g, const Cl &cl, int32_t u, int32_t j) {
+  cl.T[u] = j;
+  atomicAdd(reinterpret_cast<unsigned long long *>(&cl.pw[j]), (unsigned long long)g.vwgt[u]);
+}
+
+// Warp per position of the sub-round: the vertices of class 0.
 __global__ void __launch_bounds__(256) k_cl_rate(jet_hypergraph g, const int32_t *order, int32_t a, int32_t b,
-                                                 long long cmax, int32_t rmax, Cl cl, Tab *pool,
-                                                 unsigned long long *ctr) {
-  __shared__ Tab s_tab[8][kSmemTab];
+                                                 long long cmax, int32_t rmax, Cl cl) {
+  __shared__ unsigned long long s_pairs[8][kWarpTab], s_vals[8][kWarpTab];
+  __shared__ int32_t s_keys[8][kWarpTab];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t x = a + blockIdx.x * 8ll + wid;
   if (x >= b) return;
   const int32_t u = order[x];
   const int32_t cap = cl.cap[u];
-  if (cap > kWarpTab || cl.csize[u] != 1 || cl.label[u] != u) return;
-  Tab *tab = s_tab[wid];
-  if (cap > kSmemTab) {
-    unsigned long long off = 0;
-    if (lane == 0) off = atomicAdd(ctr, (unsigned long long)cap);
-    tab = pool + __shfl_sync(kFull, off, 0);
-  }
-  const int32_t j = rate_vertex(g, u, cl.label, cl.cw, cmax, rmax, tab, cap, lane);
-  if (lane == 0 && j >= 0) {
-    cl.T[u] = j;
-    atomicAdd(reinterpret_cast<unsigned long long *>(&cl.pw[j]), (unsigned long long)g.vwgt[u]);
-  }
+  if (cap == 0 || cap > kWarpTab || cl.csize[u] != 1 || cl.label[u] != u) return;
+  const RateTab tb{s_pairs[wid], s_vals[wid], s_keys[wid], (uint32_t)cap - 1};
+  const int32_t j = rate_warp(g, u, cl.label, cl.cw, cmax, rmax, tb, lane);
+  if (lane == 0 && j >= 0) propose(g, cl, u, j);
 }
 
-// Block per heavy position of the sub-round (hpos).  Dynamic shared memory: kHeavySmem.
-__global__ void __launch_bounds__(kHeavyWarps * 32) k_cl_rate_heavy(jet_hypergraph g, const int32_t *order, const int32_t *hpos,
-                                                       long long cmax, int32_t rmax, Cl cl, Tab *pool,
-                                                       unsigned long long *ctr) {
+// Block of T threads per listed position.  Dynamic shared memory: rate_smem(largest table of the class, T).
+template <int T>
+__global__ void __launch_bounds__(T) k_cl_rate_block(jet_hypergraph g, const int32_t *order, const int32_t *pos,
+                                                     long long cmax, int32_t rmax, Cl cl) {
+  extern __shared__ unsigned long long s_dyn[];
+  const int32_t u = order[pos[blockIdx.x]];
+  if (cl.csize[u] != 1 || cl.label[u] != u) return;
+  const int32_t j = rate_block<T>(g, u, cl.label, cl.cw, cmax, rmax, cl.cap[u], s_dyn);
+  if (threadIdx.x == 0 && j >= 0) propose(g, cl, u, j);
+}
+
+// Block per position of class 3.  Dynamic shared memory: kHeavySmem.
+__global__ void __launch_bounds__(kHeavyWarps * 32) k_cl_rate_pool(jet_hypergraph g, const int32_t *order,
+                                                                   const int32_t *pos, long long cmax, int32_t rmax,
+                                                                   Cl cl, Tab *pool, unsigned long long *ctr) {
   extern __shared__ unsigned long long s_dyn[];
   __shared__ int32_t s_bk[kHeavyWarps];
   __shared__ unsigned long long s_bv[kHeavyWarps];
   __shared__ unsigned long long s_off;
   __shared__ int s_next[2];
-  const int32_t u = order[hpos[blockIdx.x]];
+  const int32_t u = order[pos[blockIdx.x]];
   if (cl.csize[u] != 1 || cl.label[u] != u) return;
   const int32_t cap = cl.cap[u];
-  Tab *tab = reinterpret_cast<Tab *>(s_dyn);
-  int32_t *s_set = reinterpret_cast<int32_t *>(tab + kBlockTab);
-  if (cap > kBlockTab) {
-    if (threadIdx.x == 0) s_off = atomicAdd(ctr, (unsigned long long)cap);
-    __syncthreads();
-    tab = pool + s_off;
-  }
-  const int32_t j = rate_block(g, u, cl.label, cl.cw, cmax, rmax, tab, cap, s_set, s_bk, s_bv, s_next);
-  if (threadIdx.x == 0 && j >= 0) {
-    cl.T[u] = j;
-    atomicAdd(reinterpret_cast<unsigned long long *>(&cl.pw[j]), (unsigned long long)g.vwgt[u]);
-  }
+  if (threadIdx.x == 0) s_off = atomicAdd(ctr, (unsigned long long)cap);
+  __syncthreads();
+  const int32_t j = rate_pool(g, u, cl.label, cl.cw, cmax, rmax, pool + s_off, cap, reinterpret_cast<int32_t *>(s_dyn),
+                              s_bk, s_bv, s_next);
+  if (threadIdx.x == 0 && j >= 0) propose(g, cl, u, j);
 }
 
-__global__ void k_cl_swap(const int32_t *vwgt, const int32_t *order, int32_t a, int32_t b, Cl cl) {
-  const int64_t x = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (x >= b) return;
-  const int32_t u = order[x];
+// The three steps after the rating.  Values that another thread wrote in the
+// step before are read past L1 (another block of the cluster may have).
+__device__ __forceinline__ void settle_swap(const int32_t *vwgt, int32_t u, const Cl &cl) {
   const int32_t v = cl.T[u];
   int32_t t2 = v;
   if (v >= 0 && cl.T[v] == u) {
@@ -693,32 +871,23 @@ __global__ void k_cl_swap(const int32_t *vwgt, const int32_t *order, int32_t a, 
   }
 }
 
-__global__ void k_cl_approve(const int32_t *vwgt, const int32_t *order, int32_t a, int32_t b, long long cmax, Cl cl) {
-  const int64_t x = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (x >= b) return;
-  const int32_t u = order[x];
-  const int32_t j = cl.T2[u];
-  if (j < 0) return;
+__device__ __forceinline__ bool settle_approve(const int32_t *vwgt, int32_t u, int32_t j, long long cmax,
+                                               const Cl &cl) {
   const long long room = cmax - cl.cw[j];
-  bool ok = cl.pw2[j] <= room;
-  if (!ok) {  // the proposers before u in (weight, id) order, and u itself, must fit
-    const int32_t cu = vwgt[u];
-    long long s = cu;
-    for (int32_t w = cl.head[j]; w >= 0 && s <= room; w = cl.next[w]) {
-      const int32_t c = vwgt[w];
-      if (c < cu || (c == cu && w < u)) s += c;
-    }
-    ok = s <= room;
+  if (__ldcg(&cl.pw2[j]) <= room) return true;
+  // the proposers before u in (weight, id) order, and u itself, must fit
+  const int32_t cu = vwgt[u];
+  long long s = cu;
+  for (int32_t w = __ldcg(&cl.head[j]); w >= 0 && s <= room; w = __ldcg(&cl.next[w])) {
+    const int32_t c = vwgt[w];
+    if (c < cu || (c == cu && w < u)) s += c;
   }
-  cl.acc[u] = ok ? 1 : 0;
+  return s <= room;
 }
 
-__global__ void k_cl_apply(const int32_t *vwgt, const int32_t *order, int32_t a, int32_t b, Cl cl) {
-  const int64_t x = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (x >= b) return;
-  const int32_t u = order[x];
-  const int32_t t = cl.T[u], j = cl.T2[u];
-  if (j >= 0 && cl.acc[u]) {
+__device__ __forceinline__ void settle_apply(const int32_t *vwgt, int32_t u, int32_t t, int32_t j, bool accepted,
+                                             const Cl &cl) {
+  if (j >= 0 && accepted) {
     const long long c = vwgt[u];
     cl.label[u] = j;
     atomicAdd(reinterpret_cast<unsigned long long *>(&cl.cw[j]), (unsigned long long)c);
@@ -732,6 +901,58 @@ __global__ void k_cl_apply(const int32_t *vwgt, const int32_t *order, int32_t a,
     cl.head[j] = -1;
   }
   cl.T[u] = cl.T2[u] = -1;
+}
+
+// All three steps of a sub-round of at most kSettleSize vertices by one
+// cluster, its barrier between the steps: one launch instead of three of a few
+// microseconds each for 5,000 vertices.
+__global__ void __launch_bounds__(kSettleThreads) k_cl_settle(const int32_t *vwgt, const int32_t *order, int32_t a,
+                                                              int32_t b, long long cmax, Cl cl) {
+  constexpr int kPer = kSettleSize / (kSettleBlocks * kSettleThreads);
+  const int i0 = a + blockIdx.x * kSettleThreads + threadIdx.x;
+  auto barrier = [] {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  };
+  int32_t u[kPer], t[kPer], j[kPer];
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const int x = i0 + q * kSettleBlocks * kSettleThreads;
+    u[q] = x < b ? order[x] : -1;
+    if (u[q] >= 0) settle_swap(vwgt, u[q], cl);
+  }
+  barrier();
+  bool ok[kPer];
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    t[q] = u[q] >= 0 ? cl.T[u[q]] : -1;
+    j[q] = u[q] >= 0 ? cl.T2[u[q]] : -1;  // this thread's own
+    ok[q] = j[q] >= 0 && settle_approve(vwgt, u[q], j[q], cmax, cl);
+  }
+  barrier();
+#pragma unroll
+  for (int q = 0; q < kPer; ++q)
+    if (u[q] >= 0) settle_apply(vwgt, u[q], t[q], j[q], ok[q], cl);
+}
+
+__global__ void k_cl_swap(const int32_t *vwgt, const int32_t *order, int32_t a, int32_t b, Cl cl) {
+  const int64_t x = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (x < b) settle_swap(vwgt, order[x], cl);
+}
+
+__global__ void k_cl_approve(const int32_t *vwgt, const int32_t *order, int32_t a, int32_t b, long long cmax, Cl cl) {
+  const int64_t x = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (x >= b) return;
+  const int32_t u = order[x];
+  const int32_t j = cl.T2[u];
+  cl.acc[u] = j >= 0 && settle_approve(vwgt, u, j, cmax, cl) ? 1 : 0;
+}
+
+__global__ void k_cl_apply(const int32_t *vwgt, const int32_t *order, int32_t a, int32_t b, Cl cl) {
+  const int64_t x = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (x >= b) return;
+  const int32_t u = order[x];
+  settle_apply(vwgt, u, cl.T[u], cl.T2[u], cl.acc[u] != 0, cl);
   cl.acc[u] = 0;
 }
 
@@ -942,6 +1163,46 @@ struct Scratch {
   }
 };
 
+// Two streams beside a call's own, for launches that may overlap with its next one.
+struct Side {
+  cudaStream_t main, s[2] = {nullptr, nullptr};
+  cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+  explicit Side(cudaStream_t m) : main(m) {}
+  cudaError_t open() {
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking);
+    for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+    return e;
+  }
+  // what follows on the used side streams comes after everything on the main stream so far
+  cudaError_t fork(bool use0, bool use1) {
+    cudaError_t e = cudaEventRecord(ev[2], main);
+    if (e == cudaSuccess && use0) e = cudaStreamWaitEvent(s[0], ev[2], 0);
+    if (e == cudaSuccess && use1) e = cudaStreamWaitEvent(s[1], ev[2], 0);
+    return e;
+  }
+  cudaError_t join(bool use0, bool use1) {
+    const bool use[2] = {use0, use1};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+      if (!use[i]) continue;
+      e = cudaEventRecord(ev[i], s[i]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(main, ev[i], 0);
+    }
+    return e;
+  }
+  // waits for its own work first: after an error a launch on a side stream may not have been joined
+  ~Side() {
+    for (int i = 0; i < 2; ++i)
+      if (s[i]) {
+        cudaStreamSynchronize(s[i]);
+        cudaStreamDestroy(s[i]);
+      }
+    for (int i = 0; i < 3; ++i)
+      if (ev[i]) cudaEventDestroy(ev[i]);
+  }
+};
+
 int gfail(int code, const char *fmt, const char *what) {
   set_global_error(fmt, what);
   return code;
@@ -1026,34 +1287,42 @@ int jet_cluster(const jet_hypergraph *hg, const jet_coarsen_params *p, const int
   const std::vector<int32_t> bounds = subround_bounds(n, p->single_subrounds, p->subround_cap_div);
   const int32_t rounds = (int32_t)bounds.size() - 1;
   int32_t *d_bounds = sc.get<int32_t>((int64_t)bounds.size());
-  // per sub-round: pool entries, pool cursor, heavy count, heavy cursor
-  unsigned long long *d_need = sc.get<unsigned long long>(4 * (int64_t)rounds);
-  int64_t *d_hoff = sc.get<int64_t>(rounds);
+  // per sub-round: pool entries, pool cursor; then the sizes and the list cursors of classes 1..3
+  const int64_t R = rounds;
+  unsigned long long *d_need = sc.get<unsigned long long>(8 * R);
+  int64_t *d_off = sc.get<int64_t>(3 * R);
   if (sc.err != cudaSuccess) return cuda_error(sc.err, "jet_cluster: workspace");
-  unsigned long long *d_ctr = d_need + rounds, *d_heavy = d_need + 2 * rounds, *d_hcur = d_need + 3 * rounds;
+  unsigned long long *d_ctr = d_need + R, *d_counts = d_need + 2 * R, *d_cur = d_need + 5 * R;
   cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_need, 0, sizeof(unsigned long long) * 4 * (size_t)rounds, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_need, 0, sizeof(unsigned long long) * 8 * (size_t)rounds, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_bounds, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(cl.T, 0, sizeof(int32_t) * (size_t)n, s);  // "seen" of the order check
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cl_serial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeavySmem);
+    e = cudaFuncSetAttribute(k_cl_serial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSerialSmem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cl_rate_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeavySmem);
+    e = cudaFuncSetAttribute(k_cl_rate_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeavySmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_cl_rate_block<kMidThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)rate_smem(kMidTab, kMidThreads));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_cl_rate_block<kBigThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)rate_smem(kBlockTab, kBigThreads));
   if (e != cudaSuccess) return cuda_error(e, "jet_cluster");
   rc = validate_hg(hg, d_err, s, sms);
   if (rc != JET_OK) return rc;
   const int g = grid_for(n, 256, sms, 4);
   k_check_order<<<g, 256, 0, s>>>(order, n, cl.T, d_err);
   k_cl_setup<<<g, 256, 0, s>>>(*hg, p->rating_max_edge, cl, d_err);
-  k_cl_need<<<g, 256, 0, s>>>(order, n, d_bounds, rounds, cl.cap, d_need, d_heavy);
+  k_cl_need<<<g, 256, 0, s>>>(order, n, d_bounds, rounds, cl.cap, d_need, d_counts);
   int h_err = 0;
-  std::vector<unsigned long long> need(rounds), heavy(rounds);
+  std::vector<unsigned long long> need(rounds), counts(3 * R);
   e = cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(need.data(), d_need, sizeof(unsigned long long) * (size_t)rounds, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(heavy.data(), d_heavy, sizeof(unsigned long long) * (size_t)rounds, cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(counts.data(), d_counts, sizeof(unsigned long long) * 3 * (size_t)rounds,
+                        cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_error(e, "jet_cluster: set-up");
   if (h_err & 2) return gfail(JET_ERR_DATA, "%s", "order is not a permutation of the vertices");
@@ -1061,34 +1330,64 @@ int jet_cluster(const jet_hypergraph *hg, const jet_coarsen_params *p, const int
   if (h_err & 8) return gfail(JET_ERR_OVERFLOW, "%s", "a vertex's rated neighbourhood exceeds 2^27 pins");
   unsigned long long pool_entries = 1;
   for (unsigned long long x : need) pool_entries = std::max(pool_entries, x);
-  std::vector<int64_t> hoff(rounds);
-  int64_t n_heavy = 0;
-  for (int32_t q = 0; q < rounds; ++q) {
-    hoff[q] = n_heavy;
-    n_heavy += (int64_t)heavy[q];
+  std::vector<int64_t> off(3 * R);
+  int64_t listed = 0;
+  for (int64_t i = 0; i < 3 * R; ++i) {
+    off[i] = listed;
+    listed += (int64_t)counts[i];
   }
   Tab *pool = sc.get<Tab>((int64_t)pool_entries);
-  int32_t *hpos = sc.get<int32_t>(n_heavy);
+  int32_t *pos = sc.get<int32_t>(listed);
   if (sc.err != cudaSuccess) return cuda_error(sc.err, "jet_cluster: rating tables");
-  e = cudaMemcpyAsync(d_hoff, hoff.data(), sizeof(int64_t) * (size_t)rounds, cudaMemcpyHostToDevice, s);
+  e = cudaMemcpyAsync(d_off, off.data(), sizeof(int64_t) * 3 * (size_t)rounds, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return cuda_error(e, "jet_cluster");
-  if (n_heavy > 0) k_cl_heavy_list<<<g, 256, 0, s>>>(order, n, d_bounds, rounds, cl.cap, d_hoff, d_hcur, hpos);
+  if (listed > 0) k_cl_class_list<<<g, 256, 0, s>>>(order, n, d_bounds, rounds, cl.cap, d_off, d_cur, pos);
   // leading one-vertex sub-rounds: one block, in order
+  const long long cmax = p->max_cluster_weight;
+  const int32_t rmax = p->rating_max_edge;
   int32_t r = 0;
   while (r < rounds && bounds[r + 1] - bounds[r] == 1) ++r;
-  if (r > 0) k_cl_serial<<<1, kHeavyWarps * 32, kHeavySmem, s>>>(*hg, order, bounds[0], bounds[r], p->max_cluster_weight,
-                                                    p->rating_max_edge, cl, pool);
-  for (; r < rounds; ++r) {
+  if (r > 0)
+    k_cl_serial<<<1, kBigThreads, kSerialSmem, s>>>(*hg, order, bounds[0], bounds[r], cmax, rmax, cl, pool);
+  // the classes of a sub-round rate different vertices from the same state: side by side
+  Side side(s);
+  if (r < rounds && listed > 0 && (e = side.open()) != cudaSuccess) return cuda_error(e, "jet_cluster: streams");
+  for (; r < rounds && e == cudaSuccess; ++r) {
     const int32_t a = bounds[r], b = bounds[r + 1];
-    const unsigned gw = (unsigned)((b - a + 7) / 8), gt = (unsigned)((b - a + 255) / 256);
-    k_cl_rate<<<gw, 256, 0, s>>>(*hg, order, a, b, p->max_cluster_weight, p->rating_max_edge, cl, pool, d_ctr + r);
-    if (heavy[r] > 0)
-      k_cl_rate_heavy<<<(unsigned)heavy[r], kHeavyWarps * 32, kHeavySmem, s>>>(*hg, order, hpos + hoff[r], p->max_cluster_weight,
-                                                                  p->rating_max_edge, cl, pool, d_ctr + r);
-    k_cl_swap<<<gt, 256, 0, s>>>(hg->vwgt, order, a, b, cl);
-    k_cl_approve<<<gt, 256, 0, s>>>(hg->vwgt, order, a, b, p->max_cluster_weight, cl);
-    k_cl_apply<<<gt, 256, 0, s>>>(hg->vwgt, order, a, b, cl);
+    const unsigned n1 = (unsigned)counts[r], n2 = (unsigned)counts[R + r], n3 = (unsigned)counts[2 * R + r];
+    if (n1 || n2 || n3) e = side.fork(n1 > 0, n2 || n3);
+    if (n3 > 0)
+      k_cl_rate_pool<<<n3, kHeavyWarps * 32, kHeavySmem, side.s[1]>>>(*hg, order, pos + off[2 * R + r], cmax, rmax, cl,
+                                                                      pool, d_ctr + r);
+    if (n2 > 0)
+      k_cl_rate_block<kBigThreads><<<n2, kBigThreads, rate_smem(kBlockTab, kBigThreads), side.s[1]>>>(
+          *hg, order, pos + off[R + r], cmax, rmax, cl);
+    if (n1 > 0)
+      k_cl_rate_block<kMidThreads><<<n1, kMidThreads, rate_smem(kMidTab, kMidThreads), side.s[0]>>>(
+          *hg, order, pos + off[r], cmax, rmax, cl);
+    k_cl_rate<<<(unsigned)((b - a + 7) / 8), 256, 0, s>>>(*hg, order, a, b, cmax, rmax, cl);
+    if (e == cudaSuccess && (n1 || n2 || n3)) e = side.join(n1 > 0, n2 || n3);
+    if (b - a <= kSettleSize) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(kSettleBlocks);
+      cfg.blockDim = dim3(kSettleThreads);
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = kSettleBlocks;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_cl_settle, hg->vwgt, order, a, b, cmax, cl);
+    } else {
+      const unsigned gt = (unsigned)((b - a + 255) / 256);
+      k_cl_swap<<<gt, 256, 0, s>>>(hg->vwgt, order, a, b, cl);
+      k_cl_approve<<<gt, 256, 0, s>>>(hg->vwgt, order, a, b, cmax, cl);
+      k_cl_apply<<<gt, 256, 0, s>>>(hg->vwgt, order, a, b, cl);
+    }
   }
+  if (e != cudaSuccess) return cuda_error(e, "jet_cluster");
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_error(e, "jet_cluster");
