@@ -47,23 +47,39 @@ __global__ void __launch_bounds__(256) k_quotient(const uint32_t *mask, int32_t 
   __shared__ __align__(16) uint32_t s_q[kMaxK * KWP];
   for (int x = threadIdx.x; x < k * KWP; x += blockDim.x) s_q[x] = 0u;
   __syncthreads();
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  auto add_row = [&](int i, const uint32_t (&L)[KWP]) {  // row i |= L
+    uint32_t *row = s_q + i * KWP;
+    uint32_t R[KWP];
+    lds_row<KWP>(row, R);
+#pragma unroll
+    for (int u = 0; u < KWP; ++u)
+      if (L[u] & ~R[u]) atomicOr(&row[u], L[u]);
+  };
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); e0 < m;
+       e0 += (int64_t)gridDim.x * blockDim.x) {  // a warp's lanes go together
+    const int64_t e = e0 + lane;
     uint32_t L[KWP], L2[KWP];
-    load_rows<KWP>(mask + e * 2 * KWP, L, L2);
+#pragma unroll
+    for (int w = 0; w < KWP; ++w) L[w] = 0;
+    if (e < m) load_rows<KWP>(mask + e * 2 * KWP, L, L2);
     int bits = 0;
 #pragma unroll
     for (int w = 0; w < KWP; ++w) bits += __popc(L[w]);
-    if (bits < 2) continue;  // a hyperedge inside one block links no pair
+    // a hyperedge inside one block links no pair; rows of many blocks (hubs) are left to the whole warp
+    const bool wide = bits > 8;
+    if (bits >= 2 && !wide) {
 #pragma unroll
-    for (int w = 0; w < KWP; ++w) {
-      for (uint32_t x = L[w]; x; x &= x - 1) {
-        uint32_t *row = s_q + (w * 32 + __ffs(x) - 1) * KWP;
-        uint32_t R[KWP];
-        lds_row<KWP>(row, R);
+      for (int w = 0; w < KWP; ++w)
+        for (uint32_t x = L[w]; x; x &= x - 1) add_row(w * 32 + __ffs(x) - 1, L);
+    }
+    for (unsigned bal = __ballot_sync(kFull, wide); bal; bal &= bal - 1) {
+      uint32_t W[KWP];
 #pragma unroll
-        for (int u = 0; u < KWP; ++u)
-          if (L[u] & ~R[u]) atomicOr(&row[u], L[u]);
-      }
+      for (int w = 0; w < KWP; ++w) W[w] = __shfl_sync(kFull, L[w], __ffs(bal) - 1);
+#pragma unroll
+      for (int w = 0; w < KWP; ++w)
+        if ((W[w] >> lane) & 1u) add_row(w * 32 + lane, W);
     }
   }
   __syncthreads();
@@ -81,17 +97,17 @@ __global__ void __launch_bounds__(256) k_quotient(const uint32_t *mask, int32_t 
 //      neighbour of largest degree, smallest id" is the lowest set bit of
 //      row & unmatched;
 //   3. the turns, by one warp, in registers: rows do not depend on the turns,
-//      so their loads run ahead, and a turn is a dozen dependent integer
+//      so their loads run ahead, and a turn is some eight dependent integer
 //      instructions with no memory access, vote or branch on its path (the
 //      partner leaves the unmatched set by its one-bit word; its index is
 //      found beside the chain);
 //   4. the matched pairs, in turn order, by all threads.
 constexpr int kSchedThreads = 512;
-constexpr int kRankLanes = 2;  // kSchedThreads / kMaxK
 
 template <int KWP>
 __global__ void __launch_bounds__(kSchedThreads) k_schedule(const uint32_t *q, int32_t k, int32_t *pairs,
                                                             int32_t *round_of, int32_t *out_counts) {
+  constexpr int kRankLanes = kSchedThreads / (32 * KWP) < 16 ? kSchedThreads / (32 * KWP) : 16;  // lanes per block
   constexpr int K = 32 * KWP;  // ranks; those of k.. and of blocks with no edge left have empty rows
   __shared__ __align__(16) uint32_t s_rem[K * KWP];
   __shared__ __align__(16) uint32_t s_perm[K * KWP];
@@ -158,22 +174,27 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const uint32_t *q, i
             const int x = w0 * 32 + i;
             uint32_t R[KWP];
             lds_row<KWP>(s_perm + x * KWP, R);  // rows from `live` on are stale: masked below
-            const bool turn = ((U[w0] >> i) & 1u) && x < live;
-            uint32_t first = 0, at = 0;  // the lowest nonzero word of row & unmatched
+            // the lowest set bit of row & unmatched, word by word: its own word's lowest bit, if the words below
+            // have none
+            const uint32_t turn = x < live ? 0u - ((U[w0] >> i) & 1u) : 0u;
+            uint32_t take[KWP], low = 0;
 #pragma unroll
-            for (int w = KWP - 1; w >= 0; --w) {
+            for (int w = 0; w < KWP; ++w) {
               const uint32_t c = R[w] & U[w];
-              if (c) {
-                first = c;
-                at = w;
-              }
+              take[w] = low == 0 ? c & (0u - c) : 0u;
+              low |= c;
             }
-            if (!turn) first = 0;
-            const uint32_t bit = first & (0u - first);
 #pragma unroll
-            for (int w = 0; w < KWP; ++w) U[w] &= ~(at == w ? bit : 0u);
-            U[w0] &= ~((bit ? 1u : 0u) << i);
-            if (lane == 0) s_pick[x] = bit ? (int)(at * 32 + __ffs(bit) - 1) : -1;
+            for (int w = 0; w < KWP; ++w) {
+              take[w] &= turn;
+              U[w] ^= take[w];
+            }
+            U[w0] &= ~(1u << i);  // no later turn finds it: a neighbour still unmatched would have been taken
+            int pick = -1;
+#pragma unroll
+            for (int w = 0; w < KWP; ++w)
+              if (take[w]) pick = w * 32 + 31 - __clz(take[w]);
+            if (lane == 0) s_pick[x] = pick;
           }
         } else {
           s_pick[w0 * 32 + lane] = -1;
