@@ -162,9 +162,8 @@ int check_ctx(jet_ctx *c) {
   return JET_OK;
 }
 
-// Rebalancing rounds (Section 4.3) until balanced, nothing moved or the cap.
-int rebalance_loop(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
-  CKP(F_RB_CTL, launch_rb_check(c, block_w), "rebalance check");  // eager form; the graph form is below
+// Rebalancing rounds (Section 4.3) until balanced, nothing moved or the cap; the check has been launched.
+int rebalance_loop(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {  // eager form; the graph form is below
   int rc = sync_counters(c);
   if (rc) return rc;
   if (!c->cnt_host->rb_any || c->params.max_rebalance_rounds <= 0) return JET_OK;
@@ -191,6 +190,10 @@ cudaError_t ensure_capture_streams(jet_ctx *c) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 3 && e == cudaSuccess; ++i)
     if (!c->cap_stream[i]) e = cudaStreamCreateWithFlags(&c->cap_stream[i], cudaStreamNonBlocking);
+  for (int i = 0; i < 3 && e == cudaSuccess; ++i)
+    if (!c->side_stream[i]) e = cudaStreamCreateWithFlags(&c->side_stream[i], cudaStreamNonBlocking);
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+    if (!c->side_ev[i]) e = cudaEventCreateWithFlags(&c->side_ev[i], cudaEventDisableTiming);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i)
     if (!c->graph_ev[i]) e = cudaEventCreate(&c->graph_ev[i]);
   return e;
@@ -208,9 +211,12 @@ cudaError_t ensure_capture_streams(jet_ctx *c) {
 // enclosing conditional node); the rebalancing body is captured on s_body.
 cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_body, int32_t tn, int32_t td,
                               int32_t *part, int32_t *phi, int64_t *bw, uint8_t *locked, jet_round_stats *stats,
-                              cudaEvent_t ev0, cudaEvent_t ev1) {
+                              cudaEvent_t ev0, cudaEvent_t ev1, RefineState *rs, int32_t limit,
+                              cudaGraphConditionalHandle loop) {
   cudaStream_t saved = c->stream;
   c->stream = s_main;
+  c->side_first = 0;
+  c->side_count = 2;
   cudaError_t e = [&]() -> cudaError_t {
     cudaError_t e;
     cudaStreamCaptureStatus st;
@@ -221,13 +227,14 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     if ((e = cudaStreamGetCaptureInfo(s_main, &st, nullptr, &cg, &deps, &ed, &nd)) != cudaSuccess) return e;
     cudaGraphConditionalHandle h;
     if ((e = cudaGraphConditionalHandleCreate(&h, cg, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
-    if ((e = reset_counters(c)) != cudaSuccess) return e;
+    // in Algorithm 1's loop the end of the iteration before has reset them
+    if (!rs && (e = reset_counters(c)) != cudaSuccess) return e;
     // external records become event-record nodes (a plain record in capture only orders streams)
     if (ev0 && (e = cudaEventRecordWithFlags(ev0, s_main, cudaEventRecordExternal)) != cudaSuccess) return e;
     if ((e = launch_candidates(c, tn, td, part, phi, locked)) != cudaSuccess) return e;
     if (ev1 && (e = cudaEventRecordWithFlags(ev1, s_main, cudaEventRecordExternal)) != cudaSuccess) return e;
     if ((e = launch_afterburner(c, part, phi)) != cudaSuccess) return e;
-    if ((e = launch_approve(c, part, locked, nullptr, nullptr, true)) != cudaSuccess) return e;
+    if ((e = launch_approve(c, part, locked, nullptr, nullptr, true, rs)) != cudaSuccess) return e;
     if ((e = launch_apply(c, part, phi, bw)) != cudaSuccess) return e;
     if ((e = launch_rb_check(c, bw, h, 1)) != cudaSuccess) return e;
     // WHILE node: rebalancing rounds
@@ -247,6 +254,8 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
         cudaSuccess)
       return e;
     c->stream = s_body;
+    c->side_first = 2;
+    c->side_count = 1;
     cudaError_t eb = launch_rebalance_candidates(c, part, phi);
     if (eb == cudaSuccess) eb = launch_rb_select(c, part);
     if (eb == cudaSuccess) eb = launch_rb_apply(c, part, phi, bw);
@@ -254,12 +263,13 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     cudaGraph_t tmp = nullptr;
     e = cudaStreamEndCapture(s_body, &tmp);
     c->stream = s_main;
+    c->side_count = 0;
     if (eb != cudaSuccess) return eb;
     if (e != cudaSuccess) return e;
-    if ((e = launch_objective(c, part)) != cudaSuccess) return e;
-    return launch_stats(c, bw, stats, 0);
+    return launch_objective(c, part, bw, stats, 0, rs, limit, loop);
   }();
   c->stream = saved;
+  c->side_count = 0;
   return e;
 }
 
@@ -533,6 +543,10 @@ void jet_ctx_destroy(jet_ctx *c) {
   }
   for (int i = 0; i < 3; ++i)
     if (c->cap_stream[i]) cudaStreamDestroy(c->cap_stream[i]);
+  for (int i = 0; i < 3; ++i)
+    if (c->side_stream[i]) cudaStreamDestroy(c->side_stream[i]);
+  for (int i = 0; i < 4; ++i)
+    if (c->side_ev[i]) cudaEventDestroy(c->side_ev[i]);
   for (int i = 0; i < 2; ++i)
     if (c->graph_ev[i]) cudaEventDestroy(c->graph_ev[i]);
   destroy_refine_graph(c);
@@ -596,9 +610,9 @@ int jet_rebalance(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w, jet
   CKP(F_PIN, ensure_masks(c, phi), "bitmasks");
   CK(reset_counters(c), "counters");
   CKP(F_RB_CTL, launch_count_blocks(c, part), "block counts");
+  CKP(F_RB_CTL, launch_rb_check(c, block_w), "rebalance check");
   if ((rc = rebalance_loop(c, part, phi, block_w))) return rc;
-  CKP(F_OBJ, launch_objective(c, part), "objective");
-  CKP(F_OBJ, launch_stats(c, block_w, stats ? stats : c->stats_scratch, 1), "stats");
+  CKP(F_OBJ, launch_objective(c, part, block_w, stats ? stats : c->stats_scratch, 1), "objective");
   return JET_OK;
 }
 
@@ -617,9 +631,9 @@ int jet_refine_round(jet_ctx *c, int32_t tau_num, int32_t tau_den, int32_t *part
   CKP(F_AB, launch_afterburner(c, part, phi), "afterburner");
   CKP(F_APPROVE, launch_approve(c, part, locked, nullptr, nullptr, true), "approve");
   CKP(F_APPLY, launch_apply(c, part, phi, block_w), "apply");
+  CKP(F_RB_CTL, launch_rb_check(c, block_w), "rebalance check");
   if ((rc = rebalance_loop(c, part, phi, block_w))) return rc;
-  CKP(F_OBJ, launch_objective(c, part), "objective");
-  CKP(F_OBJ, launch_stats(c, block_w, stats, 0), "stats");
+  CKP(F_OBJ, launch_objective(c, part, block_w, stats, 0), "objective");
   return JET_OK;
 }
 
@@ -681,8 +695,7 @@ int jet_refine(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, int32_t limi
   };
   CKP(F_PIN, launch_pincounts(c, part, phi, block_w), "pin counts");
   CK(reset_counters(c), "counters");
-  CKP(F_OBJ, launch_objective(c, part), "objective");
-  CKP(F_OBJ, launch_stats(c, block_w, c->stats_scratch, 1), "stats");
+  CKP(F_OBJ, launch_objective(c, part, block_w, c->stats_scratch, 1), "objective");
   if ((rc = read_stats())) return rc;
   result->initial_objective = st->objective;
   bool have_best = !st->imbalanced;
@@ -718,8 +731,7 @@ int jet_refine(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, int32_t limi
   }
   if (c->graph_path && phi) CKP(F_PIN, launch_pincounts(c, part, phi, block_w), "final pin counts");
   CK(reset_counters(c), "counters");
-  CKP(F_OBJ, launch_objective(c, part), "objective");
-  CKP(F_OBJ, launch_stats(c, block_w, c->stats_scratch, 1), "stats");
+  CKP(F_OBJ, launch_objective(c, part, block_w, c->stats_scratch, 1), "objective");
   if ((rc = read_stats())) return rc;
   result->objective = st->objective;
   result->balanced = !st->imbalanced;

@@ -4,11 +4,11 @@
 //
 // Per temperature phase the graph holds a WHILE node over Jet iterations.
 // Its body is one iteration (the same nodes as jet_refine_round, including
-// the nested WHILE node of the rebalancing rounds) followed by a control
-// kernel that applies Algorithm 1's rule: a balanced iteration with a
-// strictly smaller (lambda-1) than the best so far resets the counter and
-// snapshots the partition; the loop runs while the counter is below the
-// limit.  After the phase the partition is rolled back to the snapshot by
+// the nested WHILE node of the rebalancing rounds), whose objective kernel
+// ends with Algorithm 1's rule: a balanced iteration with a strictly smaller
+// (lambda-1) than the best so far resets the counter and asks for a snapshot
+// (there is then a next iteration, whose approval takes it before it moves
+// anything); the loop runs while the counter is below the limit.  After the phase the partition is rolled back to the snapshot by
 // moves.  Nothing is read on the host until the graph has finished.
 #include <cstdio>
 #include <cstring>
@@ -49,23 +49,6 @@ __global__ void k_phase_begin(RefineState *rs, int32_t limit, cudaGraphCondition
   rs->in_phase = 0;
   rs->snap = 0;
   cudaGraphSetConditional(h, limit > 0 ? 1u : 0u);
-}
-
-// Algorithm 1's loop control after one iteration.
-__global__ void k_iteration_end(const jet_round_stats *st, RefineState *rs, int32_t limit,
-                                cudaGraphConditionalHandle h) {
-  rs->res.iterations += 1;
-  rs->in_phase += 1;
-  rs->it += 1;
-  int snap = 0;
-  if (!st->imbalanced && (!rs->have_best || st->objective < rs->best)) {
-    rs->have_best = 1;
-    rs->best = st->objective;
-    rs->it = 0;
-    snap = 1;
-  }
-  rs->snap = snap;
-  cudaGraphSetConditional(h, rs->it < limit ? 1u : 0u);
 }
 
 __global__ void k_phase_end(RefineState *rs, int32_t phase) {
@@ -117,13 +100,13 @@ cudaError_t capture_refine(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, 
     cudaError_t e;
     if ((e = launch_pincounts(c, part, phi, block_w)) != cudaSuccess) return e;
     if ((e = reset_counters(c)) != cudaSuccess) return e;
-    if ((e = launch_objective(c, part)) != cudaSuccess) return e;
-    if ((e = launch_stats(c, block_w, c->stats_scratch, 1)) != cudaSuccess) return e;
+    if ((e = launch_objective(c, part, block_w, c->stats_scratch, 1)) != cudaSuccess) return e;
     k_refine_begin<<<1, 1, 0, s0>>>(c->stats_scratch, rs);
     k_snapshot<<<gn, 256, 0, s0>>>(c->best_part, part, c->n, rs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int ti = 0; ti < n_tau; ++ti) {
       if (c->n > 0 && (e = cudaMemsetAsync(c->locked_ws, 0, c->n, s0)) != cudaSuccess) return e;
+      if ((e = reset_counters(c)) != cudaSuccess) return e;
       cudaStreamCaptureStatus st;
       cudaGraph_t cg = nullptr;
       const cudaGraphNode_t *deps = nullptr;
@@ -149,12 +132,7 @@ cudaError_t capture_refine(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, 
                                              cudaStreamCaptureModeRelaxed)) != cudaSuccess)
         return e;
       cudaError_t eb = capture_iteration(c, s1, s2, tau_pairs[2 * ti], tau_pairs[2 * ti + 1], part, phi, block_w,
-                                         c->locked_ws, c->stats_scratch, nullptr, nullptr);
-      if (eb == cudaSuccess) {
-        k_iteration_end<<<1, 1, 0, s1>>>(c->stats_scratch, rs, limit, h);
-        k_snapshot<<<gn, 256, 0, s1>>>(c->best_part, part, c->n, rs);
-        eb = cudaGetLastError();
-      }
+                                         c->locked_ws, c->stats_scratch, nullptr, nullptr, rs, limit, h);
       cudaGraph_t tmp = nullptr;
       e = cudaStreamEndCapture(s1, &tmp);
       if (eb != cudaSuccess) return eb;
@@ -167,8 +145,7 @@ cudaError_t capture_refine(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, 
     }
     if (c->graph_path && phi && (e = launch_pincounts(c, part, phi, block_w)) != cudaSuccess) return e;  // final phi
     if ((e = reset_counters(c)) != cudaSuccess) return e;
-    if ((e = launch_objective(c, part)) != cudaSuccess) return e;
-    if ((e = launch_stats(c, block_w, c->stats_scratch, 1)) != cudaSuccess) return e;
+    if ((e = launch_objective(c, part, block_w, c->stats_scratch, 1)) != cudaSuccess) return e;
     k_refine_end<<<1, 1, 0, s0>>>(c->stats_scratch, rs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return cudaMemcpyAsync(result_dst, &rs->res, sizeof(jet_refine_result), cudaMemcpyDefault, s0);

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "jet.h"
@@ -62,6 +63,8 @@ struct Counters {
   // rebalancing target passes, vertices they evaluated, the incidences of those, incidences moved
   unsigned long long w_over, w_eval, w_eval_pins, w_apply_pins;
   unsigned long long n_rec;       // rebalancing records of the current round
+  unsigned ob_done;               // blocks of the objective kernel that have finished
+  unsigned unused1;
   int rb_done;                    // rebalancing loop may stop
   int rb_any;                     // an overloaded block exists
   int err;                        // bit flags of data errors found on the device
@@ -199,6 +202,11 @@ struct jet_ctx {
   int32_t *adj = nullptr;
   int capturing = 0;
   cudaStream_t cap_stream[3] = {nullptr, nullptr, nullptr};
+  // side streams of a capture: two for an iteration, one for the rebalancing body nested in it (a stream stays with
+  // the capture it was forked into), and the events that fork and join them
+  cudaStream_t side_stream[3] = {nullptr, nullptr, nullptr};
+  cudaEvent_t side_ev[4] = {nullptr, nullptr, nullptr, nullptr};
+  int side_first = 0, side_count = 0;  // the side streams that the current capture may use
   cudaEvent_t graph_ev[2] = {nullptr, nullptr};  // idle targets of the graphs' event-record nodes
 
   // CUDA graph of jet_refine (Algorithm 1 on the device), one cached argument set
@@ -238,13 +246,41 @@ int check_tau(jet_ctx *c, int32_t tau_num, int32_t tau_den);
 cudaError_t ensure_capture_streams(jet_ctx *c);
 cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_body, int32_t tn, int32_t td,
                               int32_t *part, int32_t *phi, int64_t *bw, uint8_t *locked, jet_round_stats *stats,
-                              cudaEvent_t ev0, cudaEvent_t ev1);
+                              cudaEvent_t ev0, cudaEvent_t ev1, RefineState *rs = nullptr, int32_t limit = 0,
+                              cudaGraphConditionalHandle loop = 0);
 // ---- device-side Algorithm 1 and batches (jet_graph.cu) ----
 int refine_graph(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, int32_t limit, int32_t *part, int32_t *phi,
                  int64_t *block_w, jet_refine_result *result);
 cudaError_t capture_refine(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, int32_t limit, int32_t *part,
                            int32_t *phi, int64_t *block_w, jet_refine_result *result_dst);
 void destroy_refine_graph(jet_ctx *c);
+
+// Launches that do not depend on each other, as parallel branches of the graph being captured: stream(i) takes the
+// i-th of them (the context's own stream when nothing is captured, so they run in order), join() ends the fork.
+class Fork {
+ public:
+  Fork(jet_ctx *c, int branches) : c_(c), main_(c->stream) {
+    n_ = c->capturing ? std::min(branches - 1, c->side_count) : 0;
+    if (n_ <= 0) { n_ = 0; return; }
+    err_ = cudaEventRecord(c->side_ev[3], main_);
+    for (int i = 0; i < n_ && err_ == cudaSuccess; ++i) err_ = cudaStreamWaitEvent(side(i), c->side_ev[3], 0);
+  }
+  cudaStream_t stream(int i) const { return n_ == 0 || i % (n_ + 1) == 0 ? main_ : side(i % (n_ + 1) - 1); }
+  cudaError_t join() {
+    for (int i = 0; i < n_ && err_ == cudaSuccess; ++i) {
+      err_ = cudaEventRecord(c_->side_ev[c_->side_first + i], side(i));
+      if (err_ == cudaSuccess) err_ = cudaStreamWaitEvent(main_, c_->side_ev[c_->side_first + i], 0);
+    }
+    return err_ == cudaSuccess ? cudaGetLastError() : err_;
+  }
+
+ private:
+  cudaStream_t side(int i) const { return c_->side_stream[c_->side_first + i]; }
+  jet_ctx *c_;
+  cudaStream_t main_;
+  int n_ = 0;
+  cudaError_t err_ = cudaSuccess;
+};
 
 // ---- launchers (one per kernel family); all enqueue on ctx->stream ----
 // state kernels (k_state.cu)
@@ -254,7 +290,11 @@ cudaError_t prepare_state_kernels(jet_ctx *c);  // pin_bps
 cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int64_t *block_w);
 cudaError_t launch_masks_from_phi(jet_ctx *c, const int32_t *phi);
 cudaError_t launch_connectivity_dense(jet_ctx *c, const int32_t *phi, int64_t *out);
-cudaError_t launch_objective(jet_ctx *c, const int32_t *part);  // (lambda-1) into cnt->objective
+// (lambda-1) of the state and its statistics into *stats; cnt->objective must be zero (reset_counters).  With rs:
+// one iteration of Algorithm 1 has ended: its loop control on rs and the condition h, and the counters are reset.
+cudaError_t launch_objective(jet_ctx *c, const int32_t *part, const int64_t *block_w, jet_round_stats *stats,
+                             int rebalance_only, RefineState *rs = nullptr, int32_t limit = 0,
+                             cudaGraphConditionalHandle h = 0);
 cudaError_t launch_build_adj(jet_ctx *c, int32_t *bad_edges);       // graph path set-up
 // candidates (k_cand.cu)
 cudaError_t prepare_candidate_kernels(jet_ctx *c);
@@ -265,9 +305,10 @@ cudaError_t launch_rebalance_candidates(jet_ctx *c, const int32_t *part, const i
 cudaError_t prepare_afterburner(jet_ctx *c);
 cudaError_t prepare_afterburner_kernels(jet_ctx *c);  // ab_bps
 cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi);
-// part (with build_moves): the partition, whose blocks' vertices are counted
+// part (with build_moves): the partition, whose blocks' vertices are counted.  rs (may be NULL): if the last
+// iteration improved (rs->snap), the partition is also copied to c->best_part.
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
-                           bool build_moves);
+                           bool build_moves, const RefineState *rs = nullptr);
 cudaError_t launch_export_candidates(jet_ctx *c, int32_t *target, int32_t *gain, uint8_t *in_m);
 // moves, rebalancing, loop control (k_moves.cu)
 cudaError_t prepare_move_kernels(jet_ctx *c);  // move_bps
@@ -279,7 +320,6 @@ cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part);
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // applies the selection
 cudaError_t launch_rb_post(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                            int use_cond = 0);
-cudaError_t launch_stats(jet_ctx *c, const int64_t *block_w, jet_round_stats *stats, int rebalance_only);
 cudaError_t launch_rollback_moves(jet_ctx *c, const int32_t *part, const int32_t *best, const int *enable = nullptr);
 // matching schedule of k-way refinement (k_sched.cu)
 cudaError_t launch_quotient_schedule(jet_ctx *c, uint32_t *qbits, int32_t *pairs, int32_t *round_of, int32_t *counts);

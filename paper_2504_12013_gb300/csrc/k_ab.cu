@@ -28,6 +28,7 @@
 // with a per-block max / min table and a non-candidate bitmask in shared
 // memory.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "jet_internal.cuh"
@@ -108,32 +109,44 @@ __global__ void __launch_bounds__(256) k_ab_tiny(AbArgs a) {
     for (int q = 0; q < kTinyEdge; ++q)
       if (st[q] & 0x20000u) st[q] |= (uint32_t)(a.part[vid[q]] & 255);  // block of a non-candidate pin
     const int w = a.ewgt[e];
+    // Every pair of pins is compared, so the comparisons are made for the edge's size: the list is ordered by
+    // size, so a warp's edges mostly take one of these branches together (comparing eight slots for every edge
+    // bound the kernel by its instructions: 76 us for 2 M edges of 3 pins on average).
+    auto decide = [&](auto size) {
+      constexpr int N = decltype(size)::value;
 #pragma unroll
-    for (int q = 0; q < kTinyEdge; ++q) {
-      if (!(st[q] & 0x10000u)) continue;
-      const int s = st[q] & 255, t = (st[q] >> 8) & 255;
-      const uint64_t K = key[q];
-      bool last_dep = true, no_arr_before = true, first_arr = true, no_dep_after = true, nm_s = false, nm_t = false;
+      for (int q = 0; q < N; ++q) {
+        if (!(st[q] & 0x10000u)) continue;
+        const int s = st[q] & 255, t = (st[q] >> 8) & 255;
+        const uint64_t K = key[q];
+        bool last_dep = true, no_arr_before = true, first_arr = true, no_dep_after = true, nm_s = false, nm_t = false;
 #pragma unroll
-      for (int r = 0; r < kTinyEdge; ++r) {
-        if (st[r] & 0x20000u) {
-          const int br = st[r] & 255;
-          nm_s |= br == s;
-          nm_t |= br == t;
+        for (int r = 0; r < N; ++r) {
+          if (r == q) continue;
+          if (st[r] & 0x20000u) {
+            const int br = st[r] & 255;
+            nm_s |= br == s;
+            nm_t |= br == t;
+          }
+          if (!(st[r] & 0x10000u)) continue;
+          const int sr = st[r] & 255, tr = (st[r] >> 8) & 255;
+          const uint64_t Kr = key[r];
+          if (sr == s && Kr > K) last_dep = false;
+          if (tr == s && Kr < K) no_arr_before = false;
+          if (tr == t && Kr < K) first_arr = false;
+          if (sr == t && Kr > K) no_dep_after = false;
         }
-        if (!(st[r] & 0x10000u)) continue;
-        const int sr = st[r] & 255, tr = (st[r] >> 8) & 255;
-        const uint64_t Kr = key[r];
-        if (sr == s && Kr > K) last_dep = false;
-        if (tr == s && Kr < K) no_arr_before = false;
-        if (tr == t && Kr < K) first_arr = false;
-        if (sr == t && Kr > K) no_dep_after = false;
+        int delta = 0;
+        if (last_dep && no_arr_before && !nm_s) delta += w;
+        if (first_arr && no_dep_after && !nm_t) delta -= w;
+        if (delta) atomicAdd(&a.rg[(int)(K & 0xffffffffu)], delta);
       }
-      int delta = 0;
-      if (last_dep && no_arr_before && !nm_s) delta += w;
-      if (first_arr && no_dep_after && !nm_t) delta -= w;
-      if (delta) atomicAdd(&a.rg[(int)(K & 0xffffffffu)], delta);
-    }
+    };
+    if (sz <= 2) decide(std::integral_constant<int, 2>());
+    else if (sz == 3) decide(std::integral_constant<int, 3>());
+    else if (sz == 4) decide(std::integral_constant<int, 4>());
+    else if (sz <= 6) decide(std::integral_constant<int, 6>());
+    else decide(std::integral_constant<int, kTinyEdge>());
   }
 }
 
@@ -481,6 +494,8 @@ __global__ void k_ab_slots_init(unsigned long long *tab, int32_t nslots, int32_t
 struct ApArgs {
   int32_t n, k;
   const int32_t *part;  // with build_moves
+  const RefineState *rs;  // may be NULL
+  int32_t *best;
   const uint64_t *cand;
   int32_t *rg;
   uint8_t *locked;
@@ -505,6 +520,8 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     for (int b = threadIdx.x; b < a.k; b += blockDim.x) s_vc[b] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // the snapshot of an improved partition, taken here, before the next moves, and not by a launch of its own
+  const bool snap = a.rs && a.rs->snap;
   unsigned long long ncand = 0;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = base + threadIdx.x;
@@ -524,6 +541,7 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
       if (valid) {
         const int b = a.part[v];
         if ((unsigned)b < (unsigned)a.k) atomicAdd(&s_vc[b], 1);
+        if (snap) a.best[v] = b;
       }
       const unsigned bap = __ballot_sync(kFull, ap);
       if (lane == 0) s_wc[wid] = __popc(bap);
@@ -655,10 +673,17 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
   a.rg = c->rg;
   a.k = c->k;
   a.cnt = c->cnt;
+  // The size classes add to rg by atomics in any order: side by side, so that one class fills what the end of another
+  // leaves idle (with the light and heavy vertices' kernels side by side too: vlsi_2m 8.06 -> 7.95 ms for 8
+  // iterations, 300k at k = 200 2.76 -> 2.58 for 4, refine 100k 40.2 -> 38.6).
+  Fork fork(c, (c->n_tiny > 0) + (c->n_mid_half > 0) + (c->n_mid_small > 0) + (c->n_mid_hi > 0) +
+                   (c->n_mid > c->n_mid_hi) + (c->n_seg > 0));
+  int branch = 0;
   if (c->n_tiny > 0) {
     a.elist = c->e_tiny;
     a.nlist = c->n_tiny;
-    k_ab_tiny<<<grid_for(c->n_tiny, 256, c->launch_sms, c->ab_bps[0]), 256, 0, c->stream>>>(a);
+    k_ab_tiny<<<grid_for(c->n_tiny, 256, c->launch_sms, c->ab_bps[0]), 256, 0,
+                fork.stream(branch++)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_mid_half > 0) {
@@ -666,7 +691,7 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
     a.nlist = c->n_mid_half;
     const size_t smem = (size_t)kAbWarps * 2 * 2 * c->k * sizeof(unsigned long long);
     k_ab_warp_small<16><<<grid_for((int64_t)c->n_mid_half * 16, kAbWarps * 32, c->launch_sms, c->ab_bps[1]),
-                          kAbWarps * 32, smem, c->stream>>>(a);
+                          kAbWarps * 32, smem, fork.stream(branch++)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_mid_small > 0) {
@@ -674,7 +699,7 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
     a.nlist = c->n_mid_small;
     const size_t smem = (size_t)kAbWarps * 2 * c->k * sizeof(unsigned long long);
     k_ab_warp_small<32><<<grid_for((int64_t)c->n_mid_small * 32, kAbWarps * 32, c->launch_sms, c->ab_bps[2]),
-                          kAbWarps * 32, smem, c->stream>>>(a);
+                          kAbWarps * 32, smem, fork.stream(branch++)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_mid > 0) {  // 65..128 pins first, then 33..64
@@ -683,14 +708,14 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
       a.elist = c->e_mid;
       a.nlist = c->n_mid_hi;
       k_ab_warp<4><<<grid_for((int64_t)c->n_mid_hi * 32, kAbWarps * 32, c->launch_sms, c->ab_bps[3]), kAbWarps * 32,
-                     smem, c->stream>>>(a);
+                     smem, fork.stream(branch++)>>>(a);
       ++c->kernel_launches;
     }
     if (c->n_mid > c->n_mid_hi) {
       a.elist = c->e_mid + c->n_mid_hi;
       a.nlist = c->n_mid - c->n_mid_hi;
       k_ab_warp<2><<<grid_for((int64_t)a.nlist * 32, kAbWarps * 32, c->launch_sms, c->ab_bps[5]), kAbWarps * 32, smem,
-                     c->stream>>>(a);
+                     fork.stream(branch++)>>>(a);
       ++c->kernel_launches;
     }
   }
@@ -704,16 +729,17 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
     sa.nmw = c->ab_nm;
     sa.nslots = c->n_slots;
     const size_t smem = (size_t)c->k * 2 * sizeof(unsigned long long);
-    k_ab_block<<<grid_for(c->n_seg, 1, c->launch_sms, c->ab_bps[4]), kSegThreads, smem, c->stream>>>(sa);
+    const cudaStream_t st = fork.stream(branch++);
+    k_ab_block<<<grid_for(c->n_seg, 1, c->launch_sms, c->ab_bps[4]), kSegThreads, smem, st>>>(sa);
     ++c->kernel_launches;
     if (c->n_slots > 0) {
-      k_ab_slots<<<grid_for((int64_t)c->n_slots * c->k, 256, c->launch_sms), 256, 0, c->stream>>>(sa);
-      k_ab_slots_clear_nm<<<grid_for((int64_t)c->n_slots * 8, 256, c->launch_sms), 256, 0, c->stream>>>(
+      k_ab_slots<<<grid_for((int64_t)c->n_slots * c->k, 256, c->launch_sms), 256, 0, st>>>(sa);
+      k_ab_slots_clear_nm<<<grid_for((int64_t)c->n_slots * 8, 256, c->launch_sms), 256, 0, st>>>(
           c->ab_nm, c->n_slots * 8);
       c->kernel_launches += 2;
     }
   }
-  return cudaGetLastError();
+  return fork.join();
 }
 
 // Resident blocks per SM of the afterburner kernels at this context's k.
@@ -791,9 +817,11 @@ cudaError_t prepare_afterburner(jet_ctx *c) {
 }
 
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
-                           bool build_moves) {
+                           bool build_moves, const RefineState *rs) {
   if (c->n == 0) return cudaSuccess;
   ApArgs a{};
+  a.rs = rs;
+  a.best = c->best_part;
   a.n = c->n;
   a.k = c->k;
   a.part = part;

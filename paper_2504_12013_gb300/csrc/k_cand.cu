@@ -217,9 +217,9 @@ __device__ __forceinline__ void eligible_words(const long long *s_cap, int k, in
 // ------------------------------------------------------------ light vertices
 // A warp takes 32 consecutive vertex ids; each lane evaluates one light
 // vertex.  Its incidences I(v) are processed in batches of kBatch: the mask
-// rows of a batch are copied into the lane's slots of a double-buffered
-// shared-memory stage with cp.async, so batch b+1's gathers (and batch b+2's
-// incidence loads) are in flight while batch b is added into the bit planes.
+// rows of a batch are copied into the lane's slots of a double-buffered shared-memory stage with cp.async, so batch b+1's gathers (and
+// batch b+2's incidence loads) are in flight while batch b is added into the
+// bit planes.
 // Slot t of lane l is row t*32 + l of a buffer, so the lanes' reads of the
 // stage are bank-conflict free.  Lanes never read each other's slots.
 
@@ -234,10 +234,14 @@ template <int KWP>
 struct Stage {
   static constexpr int kRow = 2 * KWP;                          // words of one mask row
   static constexpr int kBatch = KWP <= 2 ? 4 : 2;  // rows per lane per batch
-  // per-warp stage: 2 buffers x kBatch x 32 rows | the same for omega (weighted only)
+  // buffers of the stage: one batch in flight beside the one that is added.  (A third at k <= 128, with more shared
+  // memory and less L1: the targets of the row-net's rounds took 11.2 against 10.5 ms, its candidates 4.47 against
+  // 4.59.)
+  static constexpr int kBufs = 2;
+  // per-warp stage: kBufs buffers x kBatch x 32 rows | the same for omega (weighted only)
   template <bool UNIT>
   static constexpr int bytes() {
-    return 2 * kBatch * 32 * (kRow + (UNIT ? 0 : 1)) * 4;
+    return kBufs * kBatch * 32 * (kRow + (UNIT ? 0 : 1)) * 4;
   }
 };
 
@@ -254,9 +258,9 @@ __device__ __forceinline__ void cp_async_4(int32_t *dst, const int32_t *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// every committed group but the most recent one has completed
-__device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+// every committed group but the N most recent ones has completed
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 template <int KWP>
 __device__ __forceinline__ void smem_row(const uint32_t *r, uint32_t (&M)[KWP]) {
@@ -282,10 +286,10 @@ template <int KWP, int NP, bool UNIT>
 __device__ __forceinline__ int32_t stage_accumulate(const CandArgs &a, uint8_t *stage, int64_t j0, int deg, int s,
                                                     uint32_t (&pl)[NP][KWP], uint32_t (&any)[KWP]) {
   using S = Stage<KWP>;
-  constexpr int R = S::kBatch;
+  constexpr int R = S::kBatch, B = S::kBufs;
   const int lane = threadIdx.x & 31;
   uint32_t *rows = reinterpret_cast<uint32_t *>(stage);
-  int32_t *wts = reinterpret_cast<int32_t *>(rows + 2 * R * 32 * S::kRow);
+  int32_t *wts = reinterpret_cast<int32_t *>(rows + B * R * 32 * S::kRow);
 #pragma unroll
   for (int q = 0; q < KWP; ++q) {
     any[q] = 0;
@@ -293,18 +297,21 @@ __device__ __forceinline__ int32_t stage_accumulate(const CandArgs &a, uint8_t *
     for (int p = 0; p < NP; ++p) pl[p][q] = 0;
   }
   int32_t A = 0;
-  if (a.adj) {  // graph path: e = {v, u} gives Lambda(e) = {s, Pi(u)}; four neighbours in flight
-    for (int j = 0; j < deg; j += 4) {
-      int pu[4], w[4];
+  if (a.adj) {  // graph path: e = {v, u} gives Lambda(e) = {s, Pi(u)}
+    constexpr int F = 8;  // neighbours in flight (most vertices of a graph have no more)
+    for (int j = 0; j < deg; j += F) {
+      int pu[F], w[F];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) pu[t] = j + t < deg ? a.adj[j0 + j + t] : -1;
+      for (int t = 0; t < F; ++t) pu[t] = j + t < deg ? a.adj[j0 + j + t] : -1;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        w[t] = UNIT || pu[t] < 0 ? 1 : a.ewgt[a.inc[j0 + j + t]];
+      for (int t = 0; t < F; ++t) w[t] = UNIT || pu[t] < 0 ? 1 : a.inc[j0 + j + t];
+#pragma unroll
+      for (int t = 0; t < F; ++t) {
+        if (!UNIT && pu[t] >= 0) w[t] = a.ewgt[w[t]];
         pu[t] = pu[t] >= 0 ? a.part[pu[t]] : -1;
       }
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
+      for (int t = 0; t < F; ++t) {
         if (pu[t] < 0) continue;
         uint32_t M[KWP];
 #pragma unroll
@@ -328,8 +335,7 @@ __device__ __forceinline__ int32_t stage_accumulate(const CandArgs &a, uint8_t *
       e[t] = j < deg ? a.inc[j0 + j] : -1;
     }
   };
-  auto issue_rows = [&](int b) {
-    const int q = b & 1;
+  auto issue_rows = [&](int q) {  // into buffer q
 #pragma unroll
     for (int t = 0; t < R; ++t) {
       if (e[t] >= 0) {
@@ -347,20 +353,19 @@ __device__ __forceinline__ int32_t stage_accumulate(const CandArgs &a, uint8_t *
     }
     cp_async_commit();
   };
-  if (nb > 0) {
-    load_inc(0);
-    issue_rows(0);
-    if (nb > 1) load_inc(1);
+  // batches 0 .. B-2 on their way, the incidences of batch B-1 loaded; a group is committed per batch, empty past
+  // the last, so that the wait below counts the same
+#pragma unroll
+  for (int b = 0; b < B - 1; ++b) {
+    load_inc(b);
+    issue_rows(b);
   }
+  load_inc(B - 1);
+  int q = 0, qn = B - 1;  // buffers of batch b and of the batch issued beside it
   for (int b = 0; b < nb; ++b) {
-    if (b + 1 < nb) {
-      issue_rows(b + 1);
-      if (b + 2 < nb) load_inc(b + 2);
-      cp_async_wait_prior();  // batch b has landed, batch b+1 may be in flight
-    } else {
-      cp_async_wait_all();
-    }
-    const int q = b & 1;
+    issue_rows(qn);
+    load_inc(b + B);
+    cp_async_wait<B - 1>();  // batch b has landed
 #pragma unroll
     for (int t = 0; t < R; ++t) {
       if (b * R + t < deg) {
@@ -376,6 +381,8 @@ __device__ __forceinline__ int32_t stage_accumulate(const CandArgs &a, uint8_t *
         else add_weighted<KWP, NP>(pl, M, (uint32_t)w);
       }
     }
+    q = q + 1 < B ? q + 1 : 0;
+    qn = qn + 1 < B ? qn + 1 : 0;
   }
   return A;
 }
@@ -566,6 +573,11 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
   const int w = threadIdx.x >> 5;
   uint8_t *stage = dyn_smem + w * Stage<KWP>::template bytes<UNIT>();
   WarpQueue *q = &s_q[w];
+  const int lane = threadIdx.x & 31;
+  const int warps = blockDim.x >> 5;
+  const int64_t stride = (int64_t)gridDim.x * warps * 32;
+  int64_t base = ((int64_t)blockIdx.x * warps + w) * 32;
+  GroupRaw cur = fetch_group(a, base + lane, false);  // on its way while the tables are made
   for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
     s_cap[b] = a.rbb[b].cap;
     s_bw[b] = a.rbb[b].bw;
@@ -583,11 +595,6 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
     s_elig[c - 1][qq] = wd;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int warps = blockDim.x >> 5;
-  const int64_t stride = (int64_t)gridDim.x * warps * 32;
-  int64_t base = ((int64_t)blockIdx.x * warps + w) * 32;
-  GroupRaw cur = fetch_group(a, base + lane, false);
   int qn = 0;
   unsigned w_over = 0, w_eval = 0, w_pins = 0;  // one thread's share: light vertices have fewer than 64 incidences
   for (; base < a.n; base += stride) {
@@ -601,6 +608,8 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
     if (v < a.n && !cur.hv && (unsigned)s < (unsigned)a.k && s_over[s]) {
       ++w_over;
       c = a.vwgt[v];
+      j0 = a.vptr[v];  // loaded together
+      deg = (int)(a.vptr[v + 1] - j0);
       if (2ll * c <= 3ll * (s_bw[s] - a.A)) {  // heavy vertices (Section 4.3) are never moved
         uint32_t nz = 0;
         if (c <= kTab) {
@@ -614,8 +623,6 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
         }
         if (nz) {
           act = true;
-          j0 = a.vptr[v];
-          deg = (int)(a.vptr[v + 1] - j0);
           ++w_eval;
           w_pins += deg;
         }
@@ -697,43 +704,45 @@ __global__ void __launch_bounds__(256) k_rbcand_heavy(CandArgs a) {
 template <int KWP>
 cudaError_t launch_cand_kwp(jet_ctx *c, const CandArgs &base) {
   CandArgs a = base;
+  Fork fork(c, (c->n_light > 0) + (c->n_heavy > 0));  // light and heavy vertices side by side
   if (c->n_light > 0) {
     a.vlist = c->v_light;
     a.nlist = c->n_light;
     const int g = grid_for(c->n, 256, c->launch_sms, c->stage_bps[0]);
-    if (c->unit_ewgt) k_cand_light<KWP, true><<<g, 256, 8 * Stage<KWP>::template bytes<true>(), c->stream>>>(a);
-    else k_cand_light<KWP, false><<<g, 256, 8 * Stage<KWP>::template bytes<false>(), c->stream>>>(a);
+    if (c->unit_ewgt) k_cand_light<KWP, true><<<g, 256, 8 * Stage<KWP>::template bytes<true>(), fork.stream(0)>>>(a);
+    else k_cand_light<KWP, false><<<g, 256, 8 * Stage<KWP>::template bytes<false>(), fork.stream(0)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_heavy > 0) {
     a.vlist = c->v_heavy;
     a.nlist = c->n_heavy;
     k_cand_heavy<KWP><<<grid_for((int64_t)c->n_heavy * 32, 256, c->launch_sms, c->heavy_bps[0]), 256, 0,
-                            c->stream>>>(a);
+                            fork.stream(1)>>>(a);
     ++c->kernel_launches;
   }
-  return cudaGetLastError();
+  return fork.join();
 }
 
 template <int KWP>
 cudaError_t launch_rbcand_kwp(jet_ctx *c, const CandArgs &base) {
   CandArgs a = base;
+  Fork fork(c, (c->n_light > 0) + (c->n_heavy > 0));  // light and heavy vertices side by side
   if (c->n_light > 0) {
     a.vlist = c->v_light;
     a.nlist = c->n_light;
     const int g = grid_for(c->n, 256, c->launch_sms, c->stage_bps[1]);
-    if (c->unit_ewgt) k_rbcand_light<KWP, true><<<g, 256, 8 * Stage<KWP>::template bytes<true>(), c->stream>>>(a);
-    else k_rbcand_light<KWP, false><<<g, 256, 8 * Stage<KWP>::template bytes<false>(), c->stream>>>(a);
+    if (c->unit_ewgt) k_rbcand_light<KWP, true><<<g, 256, 8 * Stage<KWP>::template bytes<true>(), fork.stream(0)>>>(a);
+    else k_rbcand_light<KWP, false><<<g, 256, 8 * Stage<KWP>::template bytes<false>(), fork.stream(0)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_heavy > 0) {
     a.vlist = c->v_heavy;
     a.nlist = c->n_heavy;
     k_rbcand_heavy<KWP><<<grid_for((int64_t)c->n_heavy * 32, 256, c->launch_sms, c->heavy_bps[1]), 256, 0,
-                              c->stream>>>(a);
+                              fork.stream(1)>>>(a);
     ++c->kernel_launches;
   }
-  return cudaGetLastError();
+  return fork.join();
 }
 
 CandArgs make_args(jet_ctx *c, const int32_t *part, const int32_t *phi) {

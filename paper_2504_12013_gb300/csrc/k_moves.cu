@@ -78,55 +78,6 @@ __device__ __forceinline__ void move_incidences(const MoveArgs &a, int64_t j, in
   }
 }
 
-// Pi(v) <- t and phi_e[s]--, phi_e[t]++ for every e in I(v); c(V_s), c(V_t)
-// and |V_s|, |V_t| through shared-memory partial sums; and both bitmasks of
-// every touched edge, exactly, without a second pass: the atomic updates of
-// one phi entry are serialized in some order, so its 0 <-> 1 crossings (and
-// 1 <-> 2 crossings) alternate, and the final bit is the initial bit XOR the
-// parity of the crossings.  Each thread whose own atomic crosses toggles the
-// bit with atomicXor; XOR commutes, so the order of the toggles is irrelevant.
-__global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
-  __shared__ long long s_dw[kMaxK];
-  __shared__ int s_dc[kMaxK];
-  const long long nm = (long long)a.cnt->n_moves;
-  if ((long long)blockIdx.x * (blockDim.x / kMoveLanes) >= nm) return;  // no move for this block
-  for (int b = threadIdx.x; b < a.k; b += blockDim.x) { s_dw[b] = 0; s_dc[b] = 0; }
-  __syncthreads();
-  unsigned long long pins = 0;  // incidences moved by this thread's moves (work count)
-  const int sub = threadIdx.x % kMoveLanes;
-  const long long g0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kMoveLanes;
-  const long long ng = ((long long)gridDim.x * blockDim.x) / kMoveLanes;
-  for (long long i = g0; i < nm; i += ng) {
-    const int v = a.mv_v[i];
-    const uint32_t st = a.mv_st[i];
-    const int s = st & 0xffff, t = st >> 16;
-    if (sub == 0) {
-      a.part[v] = t;
-      const int c = a.vwgt[v];
-      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[s]), (unsigned long long)(-(long long)c));
-      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c);
-      atomicSub(&s_dc[s], 1);
-      atomicAdd(&s_dc[t], 1);
-    }
-    const int64_t j1 = a.vptr[v + 1];
-    if (sub == 0) pins += (unsigned long long)(j1 - a.vptr[v]);
-    if (a.graph) continue;
-    move_incidences(a, a.vptr[v] + sub, j1, s, t);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) pins += __shfl_xor_sync(kFull, pins, o);
-  __shared__ unsigned long long s_pins;
-  if (threadIdx.x == 0) s_pins = 0;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0 && pins) atomicAdd(&s_pins, pins);
-  __syncthreads();
-  if (threadIdx.x == 0 && s_pins) atomicAdd(&a.cnt->w_apply_pins, s_pins);
-  for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
-    if (s_dw[b]) add_i64(reinterpret_cast<long long *>(&a.bw[b]), s_dw[b]);
-    if (s_dc[b]) atomicAdd(&a.cnt->vcount[b], s_dc[b]);
-  }
-}
-
 // ---------------------------------------------------------------- rebalancing
 // Selection of the minimal prefix per overloaded block (Section 4.3) as a
 // radix select over all records at once.  Every vertex v of an overloaded
@@ -185,8 +136,8 @@ __device__ __forceinline__ int segment_base(int x) {
 // block of kMaxK threads, thread b for block b.
 __device__ __forceinline__ void rb_prep_blocks(const RbArgs &a) {
   const int b = threadIdx.x;
-  const long long bwb = b < a.k ? a.bw[b] : 0;
-  const int room = bwb > a.Lmax ? a.cnt->vcount[b] : 0;
+  const long long bwb = b < a.k ? __ldcg(&a.bw[b]) : 0;
+  const int room = bwb > a.Lmax ? __ldcg(&a.cnt->vcount[b]) : 0;
   const int base = segment_base(room);
   if (b < a.k) {
     RbBlock r;
@@ -211,9 +162,9 @@ __device__ __forceinline__ void rb_prep_blocks(const RbArgs &a) {
 
 // Any block above L_max?  If so, the state of the first round.  In a CUDA
 // graph (use_cond) it also sets the condition of the rebalancing WHILE node.
-__global__ void k_rb_check(RbArgs a, cudaGraphConditionalHandle cond, int use_cond) {
+__device__ __forceinline__ void rb_check(const RbArgs &a, cudaGraphConditionalHandle cond, int use_cond) {
   const int b = threadIdx.x;
-  const bool over = b < a.k && a.bw[b] > a.Lmax;
+  const bool over = b < a.k && __ldcg(&a.bw[b]) > a.Lmax;
   const int any = __syncthreads_or(over);
   if (b == 0) {
     a.cnt->rb_any = any;
@@ -221,6 +172,80 @@ __global__ void k_rb_check(RbArgs a, cudaGraphConditionalHandle cond, int use_co
     if (use_cond) cudaGraphSetConditional(cond, (any && a.max_rounds > 0) ? 1u : 0u);
   }
   if (any) rb_prep_blocks(a);
+}
+
+__global__ void k_rb_check(RbArgs a, cudaGraphConditionalHandle cond, int use_cond) { rb_check(a, cond, use_cond); }
+
+// End of a round: count it, and stop if nothing moved, nothing is overloaded
+// any more, or the round cap is reached; otherwise the state of the next round.
+__device__ __forceinline__ void rb_post(const RbArgs &a, cudaGraphConditionalHandle cond, int use_cond) {
+  __shared__ int s_done;
+  const int b = threadIdx.x;
+  const bool over = b < a.k && __ldcg(&a.bw[b]) > a.Lmax;
+  const int any = __syncthreads_or(over);
+  if (b == 0) {
+    const long long moved = (long long)__ldcg(&a.cnt->n_moves);
+    a.cnt->rb_rounds += 1;
+    a.cnt->rb_moves += moved;
+    a.cnt->rb_any = any;
+    const int done = (moved == 0) || !any || (a.cnt->rb_rounds >= a.max_rounds);
+    a.cnt->rb_done = done;
+    s_done = done;
+    if (use_cond) cudaGraphSetConditional(cond, done ? 0u : 1u);
+  }
+  __syncthreads();
+  if (!s_done) rb_prep_blocks(a);
+}
+
+__global__ void k_rb_post(RbArgs a, cudaGraphConditionalHandle cond, int use_cond) { rb_post(a, cond, use_cond); }
+
+// Pi(v) <- t and phi_e[s]--, phi_e[t]++ for every e in I(v); c(V_s), c(V_t)
+// and |V_s|, |V_t| through shared-memory partial sums; and both bitmasks of
+// every touched edge, exactly, without a second pass: the atomic updates of
+// one phi entry are serialized in some order, so its 0 <-> 1 crossings (and
+// 1 <-> 2 crossings) alternate, and the final bit is the initial bit XOR the
+// parity of the crossings.  Each thread whose own atomic crosses toggles the
+// bit with atomicXor; XOR commutes, so the order of the toggles is irrelevant.
+__global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
+  __shared__ long long s_dw[kMaxK];
+  __shared__ int s_dc[kMaxK];
+  const long long nm = (long long)a.cnt->n_moves;
+  if ((long long)blockIdx.x * (blockDim.x / kMoveLanes) >= nm) return;  // no move for this block
+  for (int b = threadIdx.x; b < a.k; b += blockDim.x) { s_dw[b] = 0; s_dc[b] = 0; }
+  __syncthreads();
+  unsigned long long pins = 0;  // incidences moved by this thread's moves (work count)
+  const int sub = threadIdx.x % kMoveLanes;
+  const long long g0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kMoveLanes;
+  const long long ng = ((long long)gridDim.x * blockDim.x) / kMoveLanes;
+  for (long long i = g0; i < nm; i += ng) {
+    const int v = a.mv_v[i];
+    const uint32_t st = a.mv_st[i];
+    const int s = st & 0xffff, t = st >> 16;
+    if (sub == 0) {
+      a.part[v] = t;
+      const int c = a.vwgt[v];
+      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[s]), (unsigned long long)(-(long long)c));
+      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c);
+      atomicSub(&s_dc[s], 1);
+      atomicAdd(&s_dc[t], 1);
+    }
+    const int64_t j1 = a.vptr[v + 1];
+    if (sub == 0) pins += (unsigned long long)(j1 - a.vptr[v]);
+    if (a.graph) continue;
+    move_incidences(a, a.vptr[v] + sub, j1, s, t);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) pins += __shfl_xor_sync(kFull, pins, o);
+  __shared__ unsigned long long s_pins;
+  if (threadIdx.x == 0) s_pins = 0;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && pins) atomicAdd(&s_pins, pins);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_pins) atomicAdd(&a.cnt->w_apply_pins, s_pins);
+  for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
+    if (s_dw[b]) add_i64(reinterpret_cast<long long *>(&a.bw[b]), s_dw[b]);
+    if (s_dc[b]) atomicAdd(&a.cnt->vcount[b], s_dc[b]);
+  }
 }
 
 template <class KT>
@@ -331,8 +356,10 @@ __global__ void __launch_bounds__(kPickThreads) k_rb_pick(RbArgs a, int lo, int 
 // the records up to the threshold go to the move list, which k_apply works
 // through.  Bound by the latency of the loads and levels.  A round's selection
 // was 2 x levels - 1 dependent launches whatever the number of records, and
-// the apply kernel looked at every record again: 1.03 -> 0.38 ms for the 26
-// rounds of 300k vertices at k = 200.  The line (kSegVertices, on average):
+// the apply kernel looked at every record again: 1.03 -> 0.31 ms for the 26
+// rounds of 300k vertices at k = 200.  (Moving the selected records here, and
+// not through the list, saves a launch and leaves most of the GPU idle: the
+// four iterations of that case took 3.08 against 2.58 ms.)  The line (kSegVertices, on average):
 // beyond a segment that fits the registers of one block, the grid-wide passes
 // are as fast.  Measured per round on 31k vertices per block: they take 34 us
 // at k = 128; clusters of 4 to 16 blocks per segment that sum their histograms
@@ -573,51 +600,6 @@ __global__ void __launch_bounds__(256) k_rb_apply(RbArgs r, MoveArgs a) {
   }
 }
 
-// End of a round: count it, and stop if nothing moved, nothing is overloaded
-// any more, or the round cap is reached; otherwise the state of the next round.
-__global__ void k_rb_post(RbArgs a, cudaGraphConditionalHandle cond, int use_cond) {
-  __shared__ int s_done;
-  const int b = threadIdx.x;
-  const bool over = b < a.k && a.bw[b] > a.Lmax;
-  const int any = __syncthreads_or(over);
-  if (b == 0) {
-    const long long moved = (long long)a.cnt->n_moves;
-    a.cnt->rb_rounds += 1;
-    a.cnt->rb_moves += moved;
-    a.cnt->rb_any = any;
-    const int done = (moved == 0) || !any || (a.cnt->rb_rounds >= a.max_rounds);
-    a.cnt->rb_done = done;
-    s_done = done;
-    if (use_cond) cudaGraphSetConditional(cond, done ? 0u : 1u);
-  }
-  __syncthreads();
-  if (!s_done) rb_prep_blocks(a);
-}
-
-__global__ void k_stats(const int64_t *bw, int32_t k, long long Lmax, const Counters *cnt, jet_round_stats *out,
-                        int rebalance_only) {
-  __shared__ long long s_mx[256];
-  const int b = threadIdx.x;
-  s_mx[b] = b < k ? bw[b] : 0;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (b < o && s_mx[b + o] > s_mx[b]) s_mx[b] = s_mx[b + o];
-    __syncthreads();
-  }
-  if (b == 0) {
-    jet_round_stats st;
-    st.candidates = rebalance_only ? 0 : (long long)cnt->n_cand;
-    st.approved = rebalance_only ? 0 : (long long)cnt->approved;
-    st.rebalance_rounds = cnt->rb_rounds;
-    st.rebalance_moves = cnt->rb_moves;
-    st.objective = cnt->objective;
-    st.max_block_weight = s_mx[0];
-    st.imbalanced = s_mx[0] > Lmax ? 1 : 0;
-    st.reserved = 0;
-    *out = st;
-  }
-}
-
 // Moves that take part back to best (rollback at the end of a phase).
 __global__ void __launch_bounds__(256) k_rollback_moves(const int32_t *part, const int32_t *best, int32_t n,
                                                         int32_t *mv_v, uint32_t *mv_st, Counters *cnt,
@@ -745,8 +727,7 @@ cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
 cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part) {
   if (c->n == 0) return cudaSuccess;
   const RbArgs a = rb_args(c, nullptr, part);
-  if (c->rb_segments)
-    return a.tbits <= 64 ? select_segments<unsigned long long>(c, a) : select_segments<u128>(c, a);
+  if (c->rb_segments) return a.tbits <= 64 ? select_segments<unsigned long long>(c, a) : select_segments<u128>(c, a);
   if (a.tbits <= 64) rb_select_levels<unsigned long long>(c, a);
   else rb_select_levels<u128>(c, a);
   return cudaGetLastError();
@@ -768,12 +749,6 @@ cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *bl
 
 cudaError_t launch_rb_post(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond, int use_cond) {
   k_rb_post<<<1, kMaxK, 0, c->stream>>>(rb_args(c, block_w, nullptr), cond, use_cond);
-  ++c->kernel_launches;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stats(jet_ctx *c, const int64_t *block_w, jet_round_stats *stats, int rebalance_only) {
-  k_stats<<<1, 256, 0, c->stream>>>(block_w, c->k, c->Lmax, c->cnt, stats, rebalance_only);
   ++c->kernel_launches;
   return cudaGetLastError();
 }

@@ -1,6 +1,7 @@
 // State kernels: input validation, size classes, pin counts phi_e[i] with
 // their connectivity bitmasks, block weights, and the connectivity metric
 // (lambda-1) of Section 2.
+#include <cstddef>
 #include <type_traits>
 #include <vector>
 
@@ -183,13 +184,14 @@ __global__ void k_edge_codes(const int64_t *eptr, int32_t m, uint8_t *code) {
 // in one step, and most edges are that short.  Longer edges are counted by
 // k_pincounts_seg; the rows of those longer than one segment are cleared here.
 template <int KWP>
-constexpr int kPinLanes = KWP == 1 ? 8 : KWP == 2 ? 16 : 32;
+constexpr int kPinLanes = KWP <= 2 ? 8 : 16;
+constexpr int kPinRegs = 2;  // pins per lane in flight
 
 template <int KWP, bool VEC>  // VEC: rows are 16-byte aligned (k a multiple of 4, phi aligned)
 __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const int32_t *pins, const int32_t *part,
                                                    int32_t m, int32_t k, int32_t *phi, uint32_t *mask,
                                                    Counters *cnt) {
-  constexpr int G = kPinLanes<KWP>, K = 32 * KWP, Q = K / (4 * G);
+  constexpr int G = kPinLanes<KWP>, K = 32 * KWP, Q = K / (4 * G), R = kPinRegs;
   __shared__ __align__(16) int s_h[256 / G][K];
   const int li = threadIdx.x % G;
   int *h = s_h[threadIdx.x / G];
@@ -207,26 +209,36 @@ __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const in
     p = e < m ? eptr[e] : 0;
     sz = e < m ? (int)min(eptr[e + 1] - p, (int64_t)kSegPins + 1) : 0;
   };
-  auto pin_of = [&](int64_t p, int sz) { return li < sz && sz <= kWarpEdge ? pins[p + li] : -1; };
+  auto load_pins = [&](int64_t p, int sz, int (&v)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = li + r * G < sz && sz <= kWarpEdge ? pins[p + li + r * G] : -1;
+  };
+  auto load_blocks = [&](const int (&v)[R], int (&b)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) b[r] = v[r] >= 0 ? part[v[r]] : 0;
+  };
   int64_t p0, p1, p2, p3;
-  int sz0, sz1, sz2, sz3;
+  int sz0, sz1, sz2, sz3, v0[R], v1[R], v2[R], b0[R], b1[R];
   offsets(i, p0, sz0);
   offsets(i + nw, p1, sz1);
   offsets(i + 2 * nw, p2, sz2);
-  int v0 = pin_of(p0, sz0), v1 = pin_of(p1, sz1);
-  int b0 = v0 >= 0 ? part[v0] : 0;
+  load_pins(p0, sz0, v0);
+  load_pins(p1, sz1, v1);
+  load_blocks(v0, b0);
   for (; iw < m; i += nw, iw += nw) {
     offsets(i + 3 * nw, p3, sz3);
-    const int v2 = pin_of(p2, sz2);
-    const int b1 = v1 >= 0 ? part[v1] : 0;
+    load_pins(p2, sz2, v2);
+    load_blocks(v1, b1);
     const bool store = i < m && sz0 <= kWarpEdge;
-    if (v0 >= 0) {
-      if ((unsigned)b0 < (unsigned)k) atomicAdd(&h[b0], 1);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (v0[r] < 0) continue;
+      if ((unsigned)b0[r] < (unsigned)k) atomicAdd(&h[b0[r]], 1);
       else err |= kErrPartRange;
     }
     if (store) {
 #pragma unroll 4
-      for (int j = G + li; j < sz0; j += G) {
+      for (int j = R * G + li; j < sz0; j += G) {
         const int b = part[pins[p0 + j]];
         if ((unsigned)b < (unsigned)k) atomicAdd(&h[b], 1);
         else err |= kErrPartRange;
@@ -260,9 +272,15 @@ __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const in
 #pragma unroll
     for (int q = 0; q < Q; ++q) h4[li + q * G] = make_int4(0, 0, 0, 0);
     __syncwarp();
-    p0 = p1; sz0 = sz1; v0 = v1; b0 = b1;
-    p1 = p2; sz1 = sz2; v1 = v2;
+    p0 = p1; sz0 = sz1;
+    p1 = p2; sz1 = sz2;
     p2 = p3; sz2 = sz3;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      v0[r] = v1[r];
+      b0[r] = b1[r];
+      v1[r] = v2[r];
+    }
   }
   if (err) atomicOr(&cnt->err, err);
 }
@@ -362,7 +380,7 @@ __global__ void __launch_bounds__(256) k_masks_from_phi(const int32_t *phi, int3
 }
 
 // (lambda-1) from a dense phi, read once: a group of G lanes per row (four
-// entries per lane and load), four rows in flight per group.  A lane adds
+// entries per lane and load), eight rows in flight per group.  A lane adds
 // omega(e) per nonzero entry it sees and the group's first lane takes one
 // omega(e) off if the row has any, so no sum crosses lanes until the end.
 // Bound by the read of phi (a warp per row, one load at a time: 300 us for
@@ -370,7 +388,7 @@ __global__ void __launch_bounds__(256) k_masks_from_phi(const int32_t *phi, int3
 template <int G, bool VEC>
 __global__ void __launch_bounds__(256) k_connectivity_dense(const int32_t *phi, const int32_t *ewgt, int32_t m,
                                                             int32_t k, long long *out) {
-  constexpr int kRows = 4;
+  constexpr int kRows = 8;
   const int lane = threadIdx.x & 31, li = lane % G;
   const unsigned group = (G == 32 ? kFull : ((1u << (G % 32)) - 1) << (lane - li));
   const int64_t ng = (int64_t)gridDim.x * blockDim.x / G;
@@ -410,31 +428,144 @@ __global__ void __launch_bounds__(256) k_connectivity_dense(const int32_t *phi, 
   if (threadIdx.x == 0 && tot) add_i64(out, tot);
 }
 
-// (lambda-1) from the bitmasks: thread per edge.
-__global__ void __launch_bounds__(256) k_objective_masks(const uint32_t *mask, const int32_t *ewgt, int32_t m,
-                                                         int32_t kwp, Counters *cnt) {
-  long long acc = 0;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    int lam = 0;
-    for (int q = 0; q < kwp; ++q) lam += __popc(mask[e * 2 * kwp + q]);
-    if (lam > 0) acc += (long long)(lam - 1) * ewgt[e];
+// What follows the objective, done by the last of its blocks (a launch each
+// took 1.3 to 2 us of an iteration of some 30 launches): the statistics and,
+// in Algorithm 1's loop (rs), its control: a balanced, strictly smaller
+// (lambda-1) resets the iteration counter and asks for a snapshot; the next
+// iteration starts from cleared counters.
+struct ObjEnd {
+  const int64_t *bw;
+  int32_t k;
+  long long Lmax;
+  jet_round_stats *out;
+  int rebalance_only;
+  RefineState *rs;
+  int32_t limit;
+  cudaGraphConditionalHandle loop;
+};
+
+__device__ void iteration_end(const ObjEnd &o, Counters *cnt, long long objective) {
+  __shared__ long long s_mx[kMaxK / 32];
+  const int t = threadIdx.x;  // kMaxK threads
+  long long mx = t < o.k ? __ldcg(&o.bw[t]) : 0;
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, q));
+  if ((t & 31) == 0) s_mx[t >> 5] = mx;
+  __syncthreads();
+  if (t == 0) {
+    for (int w = 0; w < kMaxK / 32; ++w) mx = max(mx, s_mx[w]);
+    jet_round_stats st;
+    st.candidates = o.rebalance_only ? 0 : (long long)cnt->n_cand;
+    st.approved = o.rebalance_only ? 0 : (long long)cnt->approved;
+    st.rebalance_rounds = cnt->rb_rounds;
+    st.rebalance_moves = cnt->rb_moves;
+    st.objective = objective;
+    st.max_block_weight = mx;
+    st.imbalanced = mx > o.Lmax ? 1 : 0;
+    st.reserved = 0;
+    *o.out = st;
+    if (o.rs) {
+      RefineState *rs = o.rs;
+      rs->res.iterations += 1;
+      rs->in_phase += 1;
+      rs->it += 1;
+      int snap = 0;
+      if (!st.imbalanced && (!rs->have_best || st.objective < rs->best)) {
+        rs->have_best = 1;
+        rs->best = st.objective;
+        rs->it = 0;
+        snap = 1;
+      }
+      rs->snap = snap;
+      cudaGraphSetConditional(o.loop, rs->it < o.limit ? 1u : 0u);
+    }
   }
-  long long tot = block_sum_ll(acc);
-  if (threadIdx.x == 0 && tot) add_i64(&cnt->objective, tot);
+  if (o.rs) {
+    __syncthreads();  // the counters have been read
+    for (int x = t; x < (int)(offsetof(Counters, err) / 4); x += blockDim.x) reinterpret_cast<int *>(cnt)[x] = 0;
+  }
+}
+
+// Adds the block's share of the objective; the last block to do so ends the call.
+__device__ __forceinline__ void objective_add(long long acc, const ObjEnd &o, Counters *cnt) {
+  __shared__ int s_last;
+  const long long tot = block_sum_ll(acc);
+  if (threadIdx.x == 0) {
+    if (tot) add_i64(&cnt->objective, tot);
+    __threadfence();
+    s_last = atomicAdd(&cnt->ob_done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_last) iteration_end(o, cnt, __ldcg(&cnt->objective));  // every block has added before it counted itself
+}
+
+// (lambda-1) from the bitmasks: thread per edge, four rows in flight.
+template <int KWP>
+__global__ void __launch_bounds__(256) k_objective_masks(const uint32_t *mask, const int32_t *ewgt, int32_t m,
+                                                         Counters *cnt, ObjEnd o) {
+  long long acc = 0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e0 < m; e0 += 4 * stride) {
+    int lam[4], w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int64_t e = e0 + r * stride;
+      lam[r] = 0;
+      w[r] = 0;
+      if (e < m) {
+        const uint32_t *row = mask + e * 2 * KWP;
+        w[r] = ewgt[e];
+        if constexpr (KWP == 1) {
+          lam[r] = __popc(row[0]);
+        } else if constexpr (KWP == 2) {
+          const uint2 x = *reinterpret_cast<const uint2 *>(row);
+          lam[r] = __popc(x.x) + __popc(x.y);
+        } else {
+#pragma unroll
+          for (int h = 0; h < KWP / 4; ++h) {
+            const uint4 x = reinterpret_cast<const uint4 *>(row)[h];
+            lam[r] += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (lam[r] > 0) acc += (long long)(lam[r] - 1) * w[r];
+  }
+  objective_add(acc, o, cnt);
 }
 
 // (lambda-1) of a graph (every edge two pins, so edge e's pins are pins[2e], pins[2e+1]): the weighted
 // edge cut.  `pairs` is pins read as 8-byte pairs (NULL when pins is not 8-byte aligned); unit: all omega = 1.
+// Bound by the gathers of the blocks: four edges in flight.
 __global__ void __launch_bounds__(256) k_objective_cut(const int32_t *pins, const int2 *pairs, const int32_t *part,
-                                                       const int32_t *ewgt, int32_t m, int unit, Counters *cnt) {
+                                                       const int32_t *ewgt, int32_t m, int unit, Counters *cnt,
+                                                       ObjEnd o) {
   long long acc = 0;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    const int2 p = pairs ? pairs[e] : make_int2(pins[2 * e], pins[2 * e + 1]);
-    if (part[p.x] != part[p.y]) acc += unit ? 1 : ewgt[e];
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e0 < m; e0 += 4 * stride) {
+    int2 p[4];
+    int a[4], b[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int64_t e = e0 + r * stride;
+      p[r] = e >= m ? make_int2(-1, -1) : pairs ? __ldcs(pairs + e) : make_int2(pins[2 * e], pins[2 * e + 1]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      a[r] = p[r].x >= 0 ? part[p[r].x] : 0;
+      b[r] = p[r].x >= 0 ? part[p[r].y] : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (a[r] != b[r]) acc += unit ? 1 : ewgt[e0 + r * stride];
   }
-  long long tot = block_sum_ll(acc);
-  if (threadIdx.x == 0 && tot) add_i64(&cnt->objective, tot);
+  objective_add(acc, o, cnt);
 }
+
+// The end of a call on a hypergraph without edges.
+__global__ void __launch_bounds__(kMaxK) k_objective_none(Counters *cnt, ObjEnd o) { iteration_end(o, cnt, 0); }
 
 // Edges that are not two distinct pins (the graph path needs none).
 __global__ void k_count_non_pairs(const int64_t *eptr, const int32_t *pins, int32_t m, int32_t *bad) {
@@ -671,17 +802,23 @@ cudaError_t launch_connectivity_dense(jet_ctx *c, const int32_t *phi, int64_t *o
   return cudaGetLastError();
 }
 
-cudaError_t launch_objective(jet_ctx *c, const int32_t *part) {
-  cudaError_t e = cudaMemsetAsync(&c->cnt->objective, 0, sizeof(long long), c->stream);
-  if (e != cudaSuccess || c->m == 0) return e;
-  if (c->graph_path) {
+cudaError_t launch_objective(jet_ctx *c, const int32_t *part, const int64_t *block_w, jet_round_stats *stats,
+                             int rebalance_only, RefineState *rs, int32_t limit, cudaGraphConditionalHandle h) {
+  const ObjEnd o{block_w, c->k, c->Lmax, stats, rebalance_only, rs, limit, h};
+  const int g = grid_for(c->m, 1024, c->launch_sms);
+  if (c->m == 0) {
+    k_objective_none<<<1, kMaxK, 0, c->stream>>>(c->cnt, o);
+  } else if (c->graph_path) {
     const int2 *pairs = ((uintptr_t)c->pins & 7) ? nullptr : reinterpret_cast<const int2 *>(c->pins);
-    k_objective_cut<<<grid_for(c->m, 256, c->launch_sms), 256, 0, c->stream>>>(c->pins, pairs, part, c->ewgt, c->m,
-                                                                             c->unit_ewgt, c->cnt);
+    k_objective_cut<<<g, 256, 0, c->stream>>>(c->pins, pairs, part, c->ewgt, c->m, c->unit_ewgt, c->cnt, o);
+  } else {
+    switch (c->kwp) {
+      case 1: k_objective_masks<1><<<g, 256, 0, c->stream>>>(c->mask, c->ewgt, c->m, c->cnt, o); break;
+      case 2: k_objective_masks<2><<<g, 256, 0, c->stream>>>(c->mask, c->ewgt, c->m, c->cnt, o); break;
+      case 4: k_objective_masks<4><<<g, 256, 0, c->stream>>>(c->mask, c->ewgt, c->m, c->cnt, o); break;
+      default: k_objective_masks<8><<<g, 256, 0, c->stream>>>(c->mask, c->ewgt, c->m, c->cnt, o); break;
+    }
   }
-  else
-    k_objective_masks<<<grid_for(c->m, 256, c->launch_sms), 256, 0, c->stream>>>(c->mask, c->ewgt, c->m, c->kwp,
-                                                                               c->cnt);
   ++c->kernel_launches;
   return cudaGetLastError();
 }
