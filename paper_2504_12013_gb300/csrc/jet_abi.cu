@@ -235,7 +235,7 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     if (ev1 && (e = cudaEventRecordWithFlags(ev1, s_main, cudaEventRecordExternal)) != cudaSuccess) return e;
     if ((e = launch_afterburner(c, part, phi)) != cudaSuccess) return e;
     if ((e = launch_approve(c, part, locked, nullptr, nullptr, true, rs)) != cudaSuccess) return e;
-    if ((e = launch_apply(c, part, phi, bw)) != cudaSuccess) return e;
+    if ((e = launch_apply_jet(c, part, phi, bw)) != cudaSuccess) return e;
     if ((e = launch_rb_check(c, bw, h, 1)) != cudaSuccess) return e;
     // WHILE node: rebalancing rounds
     if ((e = cudaStreamGetCaptureInfo(s_main, &st, nullptr, &cg, &deps, &ed, &nd)) != cudaSuccess) return e;
@@ -630,7 +630,7 @@ int jet_refine_round(jet_ctx *c, int32_t tau_num, int32_t tau_den, int32_t *part
   CKP(F_CAND, launch_candidates(c, tau_num, tau_den, part, phi, locked), "candidates");
   CKP(F_AB, launch_afterburner(c, part, phi), "afterburner");
   CKP(F_APPROVE, launch_approve(c, part, locked, nullptr, nullptr, true), "approve");
-  CKP(F_APPLY, launch_apply(c, part, phi, block_w), "apply");
+  CKP(F_APPLY, launch_apply_jet(c, part, phi, block_w), "apply");
   CKP(F_RB_CTL, launch_rb_check(c, block_w), "rebalance check");
   if ((rc = rebalance_loop(c, part, phi, block_w))) return rc;
   CKP(F_OBJ, launch_objective(c, part, block_w, stats, 0), "objective");

@@ -288,6 +288,9 @@ cudaError_t launch_validate(jet_ctx *c, int64_t *wdeg_tmp, int32_t *degcount_tmp
 cudaError_t launch_classify(jet_ctx *c, const int64_t *wdeg);
 cudaError_t prepare_state_kernels(jet_ctx *c);  // pin_bps
 cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int64_t *block_w);
+// phi and the bitmasks anew from part, if *value (device) >= min
+cudaError_t launch_recount(jet_ctx *c, const int32_t *part, int32_t *phi, const unsigned long long *value,
+                           unsigned long long min);
 cudaError_t launch_masks_from_phi(jet_ctx *c, const int32_t *phi);
 cudaError_t launch_connectivity_dense(jet_ctx *c, const int32_t *phi, int64_t *out);
 // (lambda-1) of the state and its statistics into *stats; cnt->objective must be zero (reset_counters).  With rs:
@@ -313,6 +316,7 @@ cudaError_t launch_export_candidates(jet_ctx *c, int32_t *target, int32_t *gain,
 // moves, rebalancing, loop control (k_moves.cu)
 cudaError_t prepare_move_kernels(jet_ctx *c);  // move_bps
 cudaError_t launch_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // applies the move list
+cudaError_t launch_apply_jet(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // ... of a Jet iteration
 cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part);  // cnt->vcount (zeroed by reset_counters)
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                             int use_cond = 0);

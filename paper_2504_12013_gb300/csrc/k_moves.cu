@@ -4,6 +4,8 @@
 // All updates are integer atomics whose final values do not depend on their
 // order: phi row entries +-1, block weights and counts aggregated per thread
 // block, and XOR toggles of the edge bitmasks at the phi crossings.
+#include <algorithm>
+
 #include "jet_internal.cuh"
 
 namespace jet {
@@ -25,6 +27,7 @@ struct MoveArgs {
   const uint32_t *mv_st;
   int32_t k, kwp;
   int graph;  // graph path: phi and the bitmasks are not kept, a move changes Pi and c(V_i) only
+  unsigned long long rebuild_min;  // from this many moves on, phi is counted anew (launch_apply_jet)
   Counters *cnt;
 };
 
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
   __shared__ int s_dc[kMaxK];
   const long long nm = (long long)a.cnt->n_moves;
   if ((long long)blockIdx.x * (blockDim.x / kMoveLanes) >= nm) return;  // no move for this block
+  if ((unsigned long long)nm >= a.rebuild_min) return;                  // k_apply_part's
   for (int b = threadIdx.x; b < a.k; b += blockDim.x) { s_dw[b] = 0; s_dc[b] = 0; }
   __syncthreads();
   unsigned long long pins = 0;  // incidences moved by this thread's moves (work count)
@@ -231,7 +235,6 @@ __global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
     }
     const int64_t j1 = a.vptr[v + 1];
     if (sub == 0) pins += (unsigned long long)(j1 - a.vptr[v]);
-    if (a.graph) continue;
     move_incidences(a, a.vptr[v] + sub, j1, s, t);
   }
 #pragma unroll
@@ -239,6 +242,58 @@ __global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
   __shared__ unsigned long long s_pins;
   if (threadIdx.x == 0) s_pins = 0;
   __syncthreads();
+  if ((threadIdx.x & 31) == 0 && pins) atomicAdd(&s_pins, pins);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_pins) atomicAdd(&a.cnt->w_apply_pins, s_pins);
+  for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
+    if (s_dw[b]) add_i64(reinterpret_cast<long long *>(&a.bw[b]), s_dw[b]);
+    if (s_dc[b]) atomicAdd(&a.cnt->vcount[b], s_dc[b]);
+  }
+}
+
+// The moves' share of the partition and the block weights only, a thread per
+// move: on the graph path, and where phi is counted anew afterwards
+// (rebuild_min moves or more).  k_apply's eight lanes per move left seven idle
+// here: 119 us for the 1.7 M moves of a graph's first iteration.
+__global__ void __launch_bounds__(256) k_apply_part(MoveArgs a) {
+  __shared__ long long s_dw[kMaxK];
+  __shared__ int s_dc[kMaxK];
+  __shared__ unsigned long long s_pins;
+  const long long nm = (long long)a.cnt->n_moves;
+  if ((long long)blockIdx.x * blockDim.x >= nm || (unsigned long long)nm < a.rebuild_min) return;
+  for (int b = threadIdx.x; b < a.k; b += blockDim.x) { s_dw[b] = 0; s_dc[b] = 0; }
+  if (threadIdx.x == 0) s_pins = 0;
+  __syncthreads();
+  unsigned long long pins = 0;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; i0 < nm; i0 += 2 * stride) {
+    int v[2], c[2];
+    uint32_t st[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      v[q] = i0 + q * stride < nm ? a.mv_v[i0 + q * stride] : -1;
+      st[q] = i0 + q * stride < nm ? a.mv_st[i0 + q * stride] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      c[q] = 0;
+      if (v[q] < 0) continue;
+      c[q] = a.vwgt[v[q]];
+      pins += (unsigned long long)(a.vptr[v[q] + 1] - a.vptr[v[q]]);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (v[q] < 0) continue;
+      const int s = st[q] & 0xffff, t = st[q] >> 16;
+      a.part[v[q]] = t;
+      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[s]), (unsigned long long)(-(long long)c[q]));
+      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c[q]);
+      atomicSub(&s_dc[s], 1);
+      atomicAdd(&s_dc[t], 1);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) pins += __shfl_xor_sync(kFull, pins, o);
   if ((threadIdx.x & 31) == 0 && pins) atomicAdd(&s_pins, pins);
   __syncthreads();
   if (threadIdx.x == 0 && s_pins) atomicAdd(&a.cnt->w_apply_pins, s_pins);
@@ -634,6 +689,7 @@ MoveArgs move_args(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   a.bw = block_w;
   a.mask = c->mask;
   a.graph = c->graph_path;
+  a.rebuild_min = c->graph_path ? 0 : ~0ull;
   a.mv_v = c->mv_v;
   a.mv_st = c->mv_st;
   a.k = c->k;
@@ -678,13 +734,42 @@ cudaError_t prepare_move_kernels(jet_ctx *c) {
   return e;
 }
 
-cudaError_t launch_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
-  if (c->n == 0) return cudaSuccess;
-  const MoveArgs a = move_args(c, part, phi, block_w);
+static cudaError_t apply_phi(jet_ctx *c, const MoveArgs &a) {
   k_apply<<<grid_for((int64_t)c->n * kMoveLanes, 256, c->launch_sms, kMoveWaves * c->move_bps[0]), 256, 0,
             c->stream>>>(a);
   ++c->kernel_launches;
   return cudaGetLastError();
+}
+
+static cudaError_t apply_part(jet_ctx *c, const MoveArgs &a) {
+  k_apply_part<<<grid_for(c->n, 512, c->launch_sms), 256, 0, c->stream>>>(a);
+  ++c->kernel_launches;
+  return cudaGetLastError();
+}
+
+// The Jet moves of an iteration.  An apply pays two atomics with return on random sectors of phi per moved incidence
+// (0.06 to 0.09 ns each on tables beyond L2, whatever their number), a count of phi from the partition streams the
+// table once (at 4.2 TB/s or so: 0.65 ms for the 2 GB of the row-net workload).  So from
+// rebuild_min = bytes / (4.2 TB/s * 0.075 ns * P/n) moves on, only the partition and the block weights move and phi
+// and the bitmasks are counted anew.  Both forms are launched and the move count decides on the device; below 256 MB
+// of phi, where the atomics stay in L2, only the first.  The first iterations of a refinement are of the second kind:
+// eight iterations of rownet_4m took 42.6 ms with the apply alone and 39.1 so (vlsi_2m 7.99 and 7.94).
+cudaError_t launch_apply_jet(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
+  const double phi_bytes = 4.0 * c->m * c->k;
+  if (c->n == 0 || c->graph_path || phi_bytes < 256e6) return launch_apply(c, part, phi, block_w);
+  const double bytes = phi_bytes + 8.0 * c->m * c->kwp + 8.0 * c->m + 8.0 * c->P;
+  MoveArgs a = move_args(c, part, phi, block_w);
+  a.rebuild_min = (unsigned long long)(bytes / (4.2e3 * 0.075) * c->n / std::max<int64_t>(c->P, 1)) + 1;
+  cudaError_t e = apply_phi(c, a);
+  if (e == cudaSuccess) e = apply_part(c, a);
+  if (e == cudaSuccess) e = launch_recount(c, part, phi, &c->cnt->n_moves, a.rebuild_min);
+  return e;
+}
+
+cudaError_t launch_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
+  if (c->n == 0) return cudaSuccess;
+  const MoveArgs a = move_args(c, part, phi, block_w);
+  return c->graph_path ? apply_part(c, a) : apply_phi(c, a);
 }
 
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond, int use_cond) {

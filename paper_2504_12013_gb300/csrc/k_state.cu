@@ -173,6 +173,13 @@ __global__ void k_edge_codes(const int64_t *eptr, int32_t m, uint8_t *code) {
 }
 
 // ---------------------------------------------------------------- pin counts
+// A count that the device may call off: it runs if *value >= min (always without a value).
+struct Gate {
+  const unsigned long long *value;
+  unsigned long long min;
+  __device__ __forceinline__ bool closed() const { return value && *value < min; }
+};
+
 // A group of G lanes per edge of at most kWarpEdge pins: the pins' blocks are
 // counted in the group's row in shared memory, which then goes out whole,
 // four counts per lane, with its two mask words.  Bound by the writes of phi
@@ -190,7 +197,8 @@ constexpr int kPinRegs = 2;  // pins per lane in flight
 template <int KWP, bool VEC>  // VEC: rows are 16-byte aligned (k a multiple of 4, phi aligned)
 __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const int32_t *pins, const int32_t *part,
                                                    int32_t m, int32_t k, int32_t *phi, uint32_t *mask,
-                                                   Counters *cnt) {
+                                                   Counters *cnt, Gate gate) {
+  if (gate.closed()) return;
   constexpr int G = kPinLanes<KWP>, K = 32 * KWP, Q = K / (4 * G), R = kPinRegs;
   __shared__ __align__(16) int s_h[256 / G][K];
   const int li = threadIdx.x % G;
@@ -293,7 +301,8 @@ __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const in
 // segment touches), and k_masks_from_phi completes it.
 __global__ void __launch_bounds__(256) k_pincounts_seg(const int64_t *eptr, const int32_t *pins, const int32_t *part,
                                                        const int4 *seg, int32_t nseg, int32_t k, int32_t kwp,
-                                                       int32_t *phi, uint32_t *mask, Counters *cnt) {
+                                                       int32_t *phi, uint32_t *mask, Counters *cnt, Gate gate) {
+  if (gate.closed()) return;
   __shared__ int s_h[kMaxK];
   int err = 0;
   for (int i = blockIdx.x; i < nseg; i += gridDim.x) {
@@ -360,7 +369,8 @@ __global__ void __launch_bounds__(256) k_block_weights(const int32_t *part, cons
 // Bitmasks of Lambda(e) and of the blocks with >= 2 pins from a dense phi
 // (warp per edge): of every edge, or of the m edges listed in `list`.
 __global__ void __launch_bounds__(256) k_masks_from_phi(const int32_t *phi, int32_t m, int32_t k, int32_t kwp,
-                                                        uint32_t *mask, const int32_t *list) {
+                                                        uint32_t *mask, const int32_t *list, Gate gate) {
+  if (gate.closed()) return;
   const int lane = threadIdx.x & 31;
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -704,10 +714,10 @@ cudaError_t launch_classify(jet_ctx *c, const int64_t *wdeg) {
 }
 
 template <int KWP>
-static void launch_pincounts_kwp(jet_ctx *c, const int32_t *part, int32_t *phi, bool vec) {
+static void launch_pincounts_kwp(jet_ctx *c, const int32_t *part, int32_t *phi, bool vec, Gate gate) {
   const int g = grid_for((int64_t)c->m * kPinLanes<KWP>, 256, c->launch_sms, c->pin_bps[vec ? 1 : 0]);
-  if (vec) k_pincounts<KWP, true><<<g, 256, 0, c->stream>>>(c->eptr, c->pins, part, c->m, c->k, phi, c->mask, c->cnt);
-  else k_pincounts<KWP, false><<<g, 256, 0, c->stream>>>(c->eptr, c->pins, part, c->m, c->k, phi, c->mask, c->cnt);
+  if (vec) k_pincounts<KWP, true><<<g, 256, 0, c->stream>>>(c->eptr, c->pins, part, c->m, c->k, phi, c->mask, c->cnt, gate);
+  else k_pincounts<KWP, false><<<g, 256, 0, c->stream>>>(c->eptr, c->pins, part, c->m, c->k, phi, c->mask, c->cnt, gate);
 }
 
 // Resident blocks per SM of the pin-count kernels.
@@ -727,31 +737,41 @@ cudaError_t prepare_state_kernels(jet_ctx *c) {
   }
 }
 
+// phi and both bitmasks of every edge from part.
+static cudaError_t launch_count_phi(jet_ctx *c, const int32_t *part, int32_t *phi, Gate gate) {
+  cudaStream_t s = c->stream;
+  const bool vec = c->k % 4 == 0 && ((uintptr_t)phi & 15) == 0;
+  switch (c->kwp) {
+    case 1: launch_pincounts_kwp<1>(c, part, phi, vec, gate); break;
+    case 2: launch_pincounts_kwp<2>(c, part, phi, vec, gate); break;
+    case 4: launch_pincounts_kwp<4>(c, part, phi, vec, gate); break;
+    default: launch_pincounts_kwp<8>(c, part, phi, vec, gate); break;
+  }
+  ++c->kernel_launches;
+  if (c->n_seg > 0) {  // edges above kWarpEdge pins
+    k_pincounts_seg<<<grid_for(c->n_seg, 1, c->launch_sms), kMaxK, 0, s>>>(c->eptr, c->pins, part, c->ab_seg, c->n_seg,
+                                                                           c->k, c->kwp, phi, c->mask, c->cnt, gate);
+    ++c->kernel_launches;
+  }
+  if (c->n_slots > 0) {  // edges longer than one segment
+    k_masks_from_phi<<<grid_for((int64_t)c->n_slots * 32, 256, c->launch_sms), 256, 0, s>>>(
+        phi, c->n_slots, c->k, c->kwp, c->mask, c->ab_slot_edge, gate);
+    ++c->kernel_launches;
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_recount(jet_ctx *c, const int32_t *part, int32_t *phi, const unsigned long long *value,
+                           unsigned long long min) {
+  if (c->m == 0) return cudaSuccess;
+  return launch_count_phi(c, part, phi, Gate{value, min});
+}
+
 cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int64_t *block_w) {
   cudaStream_t s = c->stream;
   cudaError_t e = cudaMemsetAsync(block_w, 0, sizeof(int64_t) * c->k, s);
   if (e != cudaSuccess) return e;
-  if (c->m > 0 && phi) {
-    const bool vec = c->k % 4 == 0 && ((uintptr_t)phi & 15) == 0;
-    switch (c->kwp) {
-      case 1: launch_pincounts_kwp<1>(c, part, phi, vec); break;
-      case 2: launch_pincounts_kwp<2>(c, part, phi, vec); break;
-      case 4: launch_pincounts_kwp<4>(c, part, phi, vec); break;
-      default: launch_pincounts_kwp<8>(c, part, phi, vec); break;
-    }
-    ++c->kernel_launches;
-    if (c->n_seg > 0) {  // edges above kWarpEdge pins
-      k_pincounts_seg<<<grid_for(c->n_seg, 1, c->launch_sms), kMaxK, 0, s>>>(c->eptr, c->pins, part, c->ab_seg, c->n_seg,
-                                                                             c->k, c->kwp, phi, c->mask, c->cnt);
-      ++c->kernel_launches;
-    }
-    if (c->n_slots > 0) {  // edges longer than one segment
-      k_masks_from_phi<<<grid_for((int64_t)c->n_slots * 32, 256, c->launch_sms), 256, 0, s>>>(
-          phi, c->n_slots, c->k, c->kwp, c->mask, c->ab_slot_edge);
-      ++c->kernel_launches;
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  if (c->m > 0 && phi && (e = launch_count_phi(c, part, phi, Gate{})) != cudaSuccess) return e;
   if (c->n > 0) {
     const int g = grid_for(c->n, 1024, c->launch_sms, 4);
     const long long share = ((c->n - 1ll) / (1024ll * g) + 1) * 1024;  // vertices of a block, at most
@@ -769,7 +789,7 @@ cudaError_t launch_pincounts(jet_ctx *c, const int32_t *part, int32_t *phi, int6
 cudaError_t launch_masks_from_phi(jet_ctx *c, const int32_t *phi) {
   if (c->m > 0) {
     k_masks_from_phi<<<grid_for((int64_t)c->m * 32, 256, c->launch_sms), 256, 0, c->stream>>>(phi, c->m, c->k, c->kwp,
-                                                                                            c->mask, nullptr);
+                                                                                            c->mask, nullptr, Gate{});
     ++c->kernel_launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
