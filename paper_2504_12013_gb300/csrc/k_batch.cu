@@ -134,11 +134,44 @@ __device__ __forceinline__ void block_add(long long x, long long *dst, long long
 
 template <bool MULTI, int KWP>
 __device__ __forceinline__ void load_rows_m(const uint32_t *row, uint32_t (&M)[KWP], uint32_t (&M2)[KWP]) {
+  if constexpr (KWP == 1) {
+    const uint2 x = ldm<MULTI>(reinterpret_cast<const uint2 *>(row));
+    M[0] = x.x;
+    M2[0] = x.y;
+  } else if constexpr (KWP == 2) {
+    const uint4 x = ldm<MULTI>(reinterpret_cast<const uint4 *>(row));
+    M[0] = x.x; M[1] = x.y;
+    M2[0] = x.z; M2[1] = x.w;
+  } else {
 #pragma unroll
-  for (int q = 0; q < KWP; ++q) {
-    M[q] = ldm<MULTI>(row + q);
-    M2[q] = ldm<MULTI>(row + KWP + q);
+    for (int h = 0; h < KWP / 4; ++h) {
+      const uint4 x = ldm<MULTI>(reinterpret_cast<const uint4 *>(row) + h);
+      const uint4 y = ldm<MULTI>(reinterpret_cast<const uint4 *>(row + KWP) + h);
+      M[4 * h] = x.x; M[4 * h + 1] = x.y; M[4 * h + 2] = x.z; M[4 * h + 3] = x.w;
+      M2[4 * h] = y.x; M2[4 * h + 1] = y.y; M2[4 * h + 2] = y.z; M2[4 * h + 3] = y.w;
+    }
   }
+}
+
+// max_i c(V_i), the same in every lane: one load per lane and 32 blocks, and a warp maximum (a loop over the blocks
+// in every thread cost a load latency every few blocks, several times per iteration).
+template <bool MULTI>
+__device__ __forceinline__ long long team_max_weight(const TeamInst &I) {
+  long long mx = 0;
+  for (int b = threadIdx.x & 31; b < I.k; b += 32) mx = max(mx, (long long)ldm<MULTI>(I.bw + b));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, o));
+  return mx;
+}
+
+// Append by the warp: each lane with `sel` gets a distinct slot; one atomic per warp that has any (the whole warp
+// calls it).  The block-wide append has three barriers of 1,024 threads per call.
+__device__ __forceinline__ unsigned long long warp_append(bool sel, unsigned long long *counter) {
+  const int lane = threadIdx.x & 31;
+  const unsigned bal = __ballot_sync(kFull, sel);
+  unsigned long long at = 0;
+  if (bal && lane == 0) at = atomicAdd(counter, (unsigned long long)__popc(bal));
+  return __shfl_sync(kFull, at, 0) + __popc(bal & ((1u << lane) - 1));
 }
 
 // Adds the block's shared-memory block-weight deltas to c(V_i) and clears them (every thread of the block).
@@ -209,11 +242,7 @@ __device__ void team_objective(const TeamInst &I, const Team &tm, long long *s_r
   block_add(part, &I.tc->obj, s_red);
   team_sync<MULTI>();
   obj = ldm<MULTI>(&I.tc->obj);
-  maxbw = 0;
-  for (int b = 0; b < I.k; ++b) {
-    const long long w = ldm<MULTI>(I.bw + b);
-    maxbw = w > maxbw ? w : maxbw;
-  }
+  maxbw = team_max_weight<MULTI>(I);
 }
 
 // ------------------------------------------------------------ gains (Section 4.1, 4.3)
@@ -459,9 +488,55 @@ __device__ void team_afterburner(const TeamInst &I, const Team &tm, unsigned lon
   unsigned long long *maxd = s_tab + (size_t)(threadIdx.x >> 5) * (2 * I.k + (KWP + 1) / 2);
   unsigned long long *mina = maxd + I.k;
   uint32_t *nm = reinterpret_cast<uint32_t *>(mina + I.k);
+  int en = tm.wid < I.n_rest ? I.e_rest[tm.wid] : -1;  // the next edge and its offsets, loaded ahead
+  int64_t p0n = en >= 0 ? I.eptr[en] : 0, p1n = en >= 0 ? I.eptr[en + 1] : 0;
   for (long long i = tm.wid; i < I.n_rest; i += tm.nwarps) {
-    const int e = I.e_rest[i];
-    const int64_t p0 = I.eptr[e], p1 = I.eptr[e + 1];
+    const int e = en;
+    const int64_t p0 = p0n, p1 = p1n;
+    en = i + tm.nwarps < I.n_rest ? I.e_rest[i + tm.nwarps] : -1;
+    if (en >= 0) {
+      p0n = I.eptr[en];
+      p1n = I.eptr[en + 1];
+    }
+    if (p1 - p0 <= 32) {  // one pin per lane, read once; the keys' words by 32-bit atomics, as in k_ab_warp_small
+      uint32_t *dh = reinterpret_cast<uint32_t *>(maxd), *dl = dh + I.k, *ah = dl + I.k, *al = ah + I.k;
+      const int v = lane < p1 - p0 ? I.pins[p0 + lane] : -1;
+      const uint64_t r = v >= 0 ? ldm<MULTI>(I.cand + v) : 0ull;
+      const int pb = v >= 0 ? ldm<MULTI>(I.part + v) : 0;
+      if (!__any_sync(kFull, r != 0)) continue;
+      const int s = cand_s(r), t = cand_t(r);
+      if (r) {
+        dh[s] = 0u; dl[s] = 0u; ah[s] = ~0u; al[s] = ~0u;
+        dh[t] = 0u; dl[t] = 0u; ah[t] = ~0u; al[t] = ~0u;
+      }
+      if (lane < KWP) nm[lane] = 0u;
+      __syncwarp();
+      const uint64_t K = cand_key(r, v);
+      const uint32_t kh = (uint32_t)(K >> 32), kl = (uint32_t)K;
+      if (r) {
+        atomicMax(&dh[s], kh);
+        atomicMin(&ah[t], kh);
+      } else if (v >= 0) {
+        atomicOr(&nm[pb >> 5], 1u << (pb & 31));
+      }
+      __syncwarp();
+      if (r) {  // the low words among the keys with the extreme high word
+        if (dh[s] == kh) atomicMax(&dl[s], kl);
+        if (ah[t] == kh) atomicMin(&al[t], kl);
+      }
+      __syncwarp();
+      if (r) {
+        const int wt = I.unit_ewgt ? 1 : I.ewgt[e];
+        const uint64_t maxd_s = ((uint64_t)dh[s] << 32) | dl[s], mina_s = ((uint64_t)ah[s] << 32) | al[s];
+        const uint64_t maxd_t = ((uint64_t)dh[t] << 32) | dl[t], mina_t = ((uint64_t)ah[t] << 32) | al[t];
+        int delta = 0;
+        if (maxd_s == K && !((nm[s >> 5] >> (s & 31)) & 1u) && (mina_s == ~0ull || K < mina_s)) delta += wt;
+        if (mina_t == K && !((nm[t >> 5] >> (t & 31)) & 1u) && maxd_t < K) delta -= wt;
+        if (delta) atomicAdd(&I.rg[v], delta);
+      }
+      __syncwarp();
+      continue;
+    }
     bool any = false;
     for (int64_t p = p0 + lane; p < p1; p += 32) {  // reset the entries of the candidates' blocks
       const uint64_t r = ldm<MULTI>(I.cand + I.pins[p]);
@@ -507,7 +582,7 @@ __device__ void team_afterburner(const TeamInst &I, const Team &tm, unsigned lon
 
 // Approval (recomputed gain > 0), locks, and the move list; clears rg.  The loop is uniform over the block.
 template <bool MULTI>
-__device__ void team_approve(const TeamInst &I, const Team &tm, unsigned *s_wc, unsigned long long *s_base) {
+__device__ void team_approve(const TeamInst &I, const Team &tm) {
   for (long long base = (long long)tm.rank * blockDim.x; base < I.n; base += tm.nthr) {
     const long long v = base + threadIdx.x;
     bool ok = false;
@@ -519,7 +594,7 @@ __device__ void team_approve(const TeamInst &I, const Team &tm, unsigned *s_wc, 
       ok = r != 0 && g > 0;
       I.locked[v] = ok ? 1 : 0;
     }
-    const unsigned long long pos = block_append(ok, &I.tc->n_moves, s_wc, s_base);
+    const unsigned long long pos = warp_append(ok, &I.tc->n_moves);
     if (ok) {
       I.mv_v[pos] = (int32_t)v;
       I.mv_st[pos] = (uint32_t)cand_s(r) | ((uint32_t)cand_t(r) << 16);
@@ -537,15 +612,28 @@ __device__ __forceinline__ void move_vertex(const TeamInst &I, int v, int s, int
   atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c);
   const uint32_t sbit = 1u << (s & 31), tbit = 1u << (t & 31);
   const int64_t j1 = I.vptr[v + 1];
-  for (int64_t j = I.vptr[v]; j < j1; ++j) {
-    const int64_t e = I.inc[j];
-    const int os = atomicSub(&I.phi[e * I.k + s], 1);
-    const int ot = atomicAdd(&I.phi[e * I.k + t], 1);
-    uint32_t *row = I.mask + e * 2 * KWP;
-    if (os == 1) atomicXor(&row[s >> 5], sbit);
-    if (os == 2) atomicXor(&row[KWP + (s >> 5)], sbit);
-    if (ot == 0) atomicXor(&row[t >> 5], tbit);
-    if (ot == 1) atomicXor(&row[KWP + (t >> 5)], tbit);
+  for (int64_t j = I.vptr[v]; j < j1; j += 4) {  // four incidences' atomics in flight
+    int e[4], os[4], ot[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) e[q] = j + q < j1 ? I.inc[j + q] : -1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      os[q] = 0;  // no crossing for an absent incidence
+      ot[q] = 2;
+      if (e[q] >= 0) {
+        os[q] = atomicSub(&I.phi[(int64_t)e[q] * I.k + s], 1);
+        ot[q] = atomicAdd(&I.phi[(int64_t)e[q] * I.k + t], 1);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (e[q] < 0) continue;
+      uint32_t *row = I.mask + (int64_t)e[q] * 2 * KWP;
+      if (os[q] == 1) atomicXor(&row[s >> 5], sbit);
+      if (os[q] == 2) atomicXor(&row[KWP + (s >> 5)], sbit);
+      if (ot[q] == 0) atomicXor(&row[t >> 5], tbit);
+      if (ot[q] == 1) atomicXor(&row[KWP + (t >> 5)], tbit);
+    }
   }
 }
 
@@ -568,8 +656,7 @@ typedef unsigned __int128 u128;
 // block is overloaded (the same answer in every thread of the team).
 template <bool MULTI>
 __device__ bool round_state(const TeamInst &I, long long *s_cap, long long *s_bw, int *s_over) {
-  bool any = false;
-  for (int b = 0; b < I.k; ++b) any |= ldm<MULTI>(I.bw + b) > I.Lmax;
+  const bool any = team_max_weight<MULTI>(I) > I.Lmax;
   for (int b = threadIdx.x; b < I.k; b += blockDim.x) {
     const long long w = ldm<MULTI>(I.bw + b);
     s_bw[b] = w;
@@ -593,11 +680,27 @@ __device__ __forceinline__ void eligible_set(const long long *s_cap, int k, int3
   }
 }
 
+// The eligible sets of c(v) = 1 .. kEligTab, tabulated once per round (a warp per c): the loop over the blocks per
+// vertex was most of a target's instructions.
+constexpr int kEligTab = 32;
+template <int KWP>
+__device__ void eligible_table(const TeamInst &I, const long long *s_cap, uint32_t (*s_elig)[KWP]) {
+  const int lane = threadIdx.x & 31;
+  for (int c = (threadIdx.x >> 5) + 1; c <= kEligTab; c += blockDim.x >> 5) {
+#pragma unroll
+    for (int q = 0; q < KWP; ++q) {
+      const int b = 32 * q + lane;
+      const unsigned bal = __ballot_sync(kFull, b < I.k && s_cap[b] >= c);
+      if (lane == 0) s_elig[c - 1][q] = bal;
+    }
+  }
+}
+
 // Records of the round: every vertex v of an overloaded block s with 2c(v) <= 3(c(V_s) - ceil(c(V)/k)) and an
 // eligible target gets its best eligible target (ties to the smaller block) and its priority key.
 template <bool MULTI, int KWP>
 __device__ void team_targets(const TeamInst &I, const Team &tm, const long long *s_cap, const long long *s_bw,
-                             const int *s_over, unsigned *s_wc, unsigned long long *s_base) {
+                             const int *s_over, const uint32_t (*s_elig)[KWP]) {
   // the next vertex's id, block and weight are loaded while the current one is evaluated
   const long long i0 = (long long)tm.rank * blockDim.x + threadIdx.x;
   int nv = i0 < I.n_light ? I.v_light[i0] : -1;
@@ -615,7 +718,12 @@ __device__ void team_targets(const TeamInst &I, const Team &tm, const long long 
     if (i < I.n_light) {
       if (s_over[s] && 2ll * c <= 3ll * (s_bw[s] - I.A)) {
         uint32_t C[KWP], nz = 0;
-        eligible_set<KWP>(s_cap, I.k, c, C);
+        if (c <= kEligTab) {
+#pragma unroll
+          for (int q = 0; q < KWP; ++q) C[q] = s_elig[c - 1][q];
+        } else {
+          eligible_set<KWP>(s_cap, I.k, c, C);
+        }
 #pragma unroll
         for (int q = 0; q < KWP; ++q) nz |= C[q];
         if (nz) {
@@ -628,7 +736,7 @@ __device__ void team_targets(const TeamInst &I, const Team &tm, const long long 
         }
       }
     }
-    const unsigned long long pos = block_append(rec, &I.tc->n_rec, s_wc, s_base);
+    const unsigned long long pos = warp_append(rec, &I.tc->n_rec);
     if (rec) {
       I.rb_hi[pos] = hi;
       I.rb_v[pos] = v;
@@ -671,32 +779,53 @@ __device__ void team_targets(const TeamInst &I, const Team &tm, const long long 
   }
 }
 
+// The selection state of the blocks (threshold prefix, all-flag) in shared memory, read once per level: per record it
+// cost three dependent L2 loads.
+template <class KT>
+struct SelState {
+  KT pre[kMaxK];
+  int all[kMaxK];
+};
+
+template <bool MULTI, class KT>
+__device__ __forceinline__ void load_select_state(const TeamInst &I, const int *s_over, SelState<KT> &st) {
+  for (int b = threadIdx.x; b < I.k; b += blockDim.x) {
+    if (!s_over[b]) continue;
+    st.all[b] = ldm<MULTI>(&I.rbb[b].all);
+    if constexpr (sizeof(KT) > 8)
+      st.pre[b] = ((KT)ldm<MULTI>(&I.rbb[b].pre_hi) << 64) | (KT)ldm<MULTI>(&I.rbb[b].pre_lo);
+    else
+      st.pre[b] = (KT)ldm<MULTI>(&I.rbb[b].pre_lo);
+  }
+  __syncthreads();
+}
+
 // Selection: per overloaded block the minimal prefix of its records in key order whose weight reaches the
 // excess (all records if they never do), by a radix select over 8-bit digits of the key from the top.  The
 // per-block threshold (prefix), the weight below the fixed prefix (before) and the all-flag live in rbb.
-template <bool MULTI>
-__device__ void team_select(const TeamInst &I, const Team &tm, long long nrec, const int *s_over) {
+// KT: a type that holds the key.
+template <bool MULTI, class KT>
+__device__ void team_select(const TeamInst &I, const Team &tm, long long nrec, const int *s_over, SelState<KT> &st) {
   const int tb = I.rb_tbits;
   const int lane = threadIdx.x & 31;
   for (int hi_bit = tb, level = 0; hi_bit > 0; ++level) {
     const int lo = hi_bit > 8 ? hi_bit - 8 : 0;
     const int up = hi_bit;
+    load_select_state<MULTI, KT>(I, s_over, st);
     for (long long i = tm.tid; i < nrec; i += tm.nthr) {  // histogram of this digit
       const int32_t ct = ldm<MULTI>(I.rb_ct + i);
+      const KT K = ((KT)ldm<MULTI>(I.rb_hi + i) << I.rb_vbits) | (KT)(uint32_t)ldm<MULTI>(I.rb_v + i);
       const int b = (ct >> 8) & 255;
-      if (ldm<MULTI>(&I.rbb[b].all)) continue;
-      const u128 K = ((u128)ldm<MULTI>(I.rb_hi + i) << I.rb_vbits) | (u128)(uint32_t)ldm<MULTI>(I.rb_v + i);
-      const u128 pre = ((u128)ldm<MULTI>(&I.rbb[b].pre_hi) << 64) | (u128)ldm<MULTI>(&I.rbb[b].pre_lo);
-      if (up < tb && (K >> up) != (pre >> up)) continue;
-      const int d = (int)((K >> lo) & (u128)255);
-      atomicAdd(&I.hist[(int64_t)b * 256 + d], (unsigned long long)(ct >> 16));
+      if (st.all[b] || (up < tb && (K >> up) != (st.pre[b] >> up))) continue;
+      atomicAdd(&I.hist[(int64_t)b * 256 + (int)((unsigned)(K >> lo) & 255u)], (unsigned long long)(ct >> 16));
     }
     team_sync<MULTI>();
     for (long long b = tm.wid; b < I.k; b += tm.nwarps) {  // one warp per overloaded block picks the digit
       if (!s_over[b]) continue;
+      if (st.all[b]) continue;
       RbBlock *r = &I.rbb[b];
-      if (ldm<MULTI>(&r->all)) continue;
       unsigned long long *row = I.hist + b * 256;
+      const long long before = ldm<MULTI>(&r->before), need = ldm<MULTI>(&r->excess);
       long long w[8], tot = 0;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
@@ -710,7 +839,6 @@ __device__ void team_select(const TeamInst &I, const Team &tm, long long nrec, c
         if (lane >= o) incl += y;
       }
       const long long total = __shfl_sync(kFull, incl, 31);
-      const long long before = ldm<MULTI>(&r->before), need = ldm<MULTI>(&r->excess);
       __syncwarp();
       if (level == 0 && total < need) {
         if (lane == 0) r->all = 1;
@@ -725,9 +853,8 @@ __device__ void team_select(const TeamInst &I, const Team &tm, long long nrec, c
             run += w[q];
           }
           r->before = run;
-          const u128 pre = (((u128)ldm<MULTI>(&r->pre_hi) << 64) | ldm<MULTI>(&r->pre_lo)) |
-                           ((u128)(unsigned)(lane * 8 + q) << lo);
-          r->pre_hi = (unsigned long long)(pre >> 64);
+          const KT pre = st.pre[b] | ((KT)(unsigned)(lane * 8 + q) << lo);
+          if constexpr (sizeof(KT) > 8) r->pre_hi = (unsigned long long)(pre >> 64);
           r->pre_lo = (unsigned long long)pre;
         }
       }
@@ -740,21 +867,17 @@ __device__ void team_select(const TeamInst &I, const Team &tm, long long nrec, c
 }
 
 // Every record up to its block's threshold (or of an `all` block) moves.
-template <bool MULTI, int KWP>
-__device__ void team_apply_selection(const TeamInst &I, const Team &tm, long long nrec, long long *s_dw,
-                                     long long *s_red) {
+template <bool MULTI, int KWP, class KT>
+__device__ void team_apply_selection(const TeamInst &I, const Team &tm, long long nrec, const int *s_over,
+                                     SelState<KT> &st, long long *s_dw, long long *s_red) {
   long long moved = 0;
+  load_select_state<MULTI, KT>(I, s_over, st);
   for (long long i = tm.tid; i < nrec; i += tm.nthr) {
     const int32_t ct = ldm<MULTI>(I.rb_ct + i);
-    const int b = (ct >> 8) & 255;
     const int v = ldm<MULTI>(I.rb_v + i);
-    bool sel = ldm<MULTI>(&I.rbb[b].all) != 0;
-    if (!sel) {
-      const u128 K = ((u128)ldm<MULTI>(I.rb_hi + i) << I.rb_vbits) | (u128)(uint32_t)v;
-      const u128 pre = ((u128)ldm<MULTI>(&I.rbb[b].pre_hi) << 64) | (u128)ldm<MULTI>(&I.rbb[b].pre_lo);
-      sel = K <= pre;
-    }
-    if (sel) {
+    const KT K = ((KT)ldm<MULTI>(I.rb_hi + i) << I.rb_vbits) | (KT)(uint32_t)v;
+    const int b = (ct >> 8) & 255;
+    if (st.all[b] || K <= st.pre[b]) {
       move_vertex<KWP>(I, v, b, ct & 255, (ct >> 16) & 0xffff, s_dw);
       ++moved;
     }
@@ -766,13 +889,14 @@ __device__ void team_apply_selection(const TeamInst &I, const Team &tm, long lon
 struct SmemPtrs {
   long long *s_dw, *s_cap, *s_bw, *s_red;
   int *s_over;
-  unsigned *s_wc;
-  unsigned long long *s_base, *s_tab;
+  unsigned long long *s_tab;
 };
 
 // Rebalancing rounds until balanced, a round moves nothing, or the round cap.  Returns the rounds; moves in *mv.
 template <bool MULTI, int KWP>
 __device__ long long team_rebalance(const TeamInst &I, const Team &tm, const SmemPtrs &sm, long long *mv) {
+  __shared__ SelState<u128> s_sel;  // or, in its first bytes, the state of 64-bit keys
+  __shared__ uint32_t s_elig[kEligTab][KWP];
   long long rounds = 0, moves = 0;
   for (;;) {
     const bool any = round_state<MULTI>(I, sm.s_cap, sm.s_bw, sm.s_over);
@@ -794,12 +918,19 @@ __device__ long long team_rebalance(const TeamInst &I, const Team &tm, const Sme
       r.all = 0;
       I.rbb[b] = r;
     }
+    eligible_table<KWP>(I, sm.s_cap, s_elig);
     team_sync<MULTI>();
-    team_targets<MULTI, KWP>(I, tm, sm.s_cap, sm.s_bw, sm.s_over, sm.s_wc, sm.s_base);
+    team_targets<MULTI, KWP>(I, tm, sm.s_cap, sm.s_bw, sm.s_over, s_elig);
     team_sync<MULTI>();
     const long long nrec = (long long)ldm<MULTI>(&I.tc->n_rec);
-    team_select<MULTI>(I, tm, nrec, sm.s_over);
-    team_apply_selection<MULTI, KWP>(I, tm, nrec, sm.s_dw, sm.s_red);
+    if (I.rb_tbits <= 64) {
+      SelState<unsigned long long> &st = *reinterpret_cast<SelState<unsigned long long> *>(&s_sel);
+      team_select<MULTI, unsigned long long>(I, tm, nrec, sm.s_over, st);
+      team_apply_selection<MULTI, KWP, unsigned long long>(I, tm, nrec, sm.s_over, st, sm.s_dw, sm.s_red);
+    } else {
+      team_select<MULTI, u128>(I, tm, nrec, sm.s_over, s_sel);
+      team_apply_selection<MULTI, KWP, u128>(I, tm, nrec, sm.s_over, s_sel, sm.s_dw, sm.s_red);
+    }
     team_sync<MULTI>();
     const long long moved = (long long)ldm<MULTI>(&I.tc->moved);
     rounds += 1;
@@ -851,7 +982,7 @@ __device__ void team_refine(const TeamInst &I, const Team &tm, const TeamArgs &a
       team_sync<MULTI>();
       team_afterburner<MULTI, KWP>(I, tm, sm.s_tab);
       team_sync<MULTI>();
-      team_approve<MULTI>(I, tm, sm.s_wc, sm.s_base);
+      team_approve<MULTI>(I, tm);
       team_sync<MULTI>();
       team_apply_list<MULTI, KWP>(I, tm, (long long)ldm<MULTI>(&I.tc->n_moves), sm.s_dw);
       team_sync<MULTI>();
@@ -882,7 +1013,7 @@ __device__ void team_refine(const TeamInst &I, const Team &tm, const TeamArgs &a
           t = ldm<MULTI>(I.best + v);
           mvd = s != t;
         }
-        const unsigned long long pos = block_append(mvd, &I.tc->n_moves, sm.s_wc, sm.s_base);
+        const unsigned long long pos = warp_append(mvd, &I.tc->n_moves);
         if (mvd) {
           I.mv_v[pos] = (int32_t)v;
           I.mv_st[pos] = (uint32_t)s | ((uint32_t)t << 16);
@@ -905,8 +1036,6 @@ __device__ void team_refine(const TeamInst &I, const Team &tm, const TeamArgs &a
 template <bool MULTI, int KWP>
 __global__ void __launch_bounds__(kTeamMaxThreads) k_batch_teams(TeamArgs a, int kmax) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned s_wc[kTeamMaxThreads / 32];
-  __shared__ unsigned long long s_base;
   __shared__ long long s_red[kTeamMaxThreads / 32];
   SmemPtrs sm;
   sm.s_dw = reinterpret_cast<long long *>(smem);
@@ -914,8 +1043,6 @@ __global__ void __launch_bounds__(kTeamMaxThreads) k_batch_teams(TeamArgs a, int
   sm.s_bw = sm.s_cap + kmax;
   sm.s_over = reinterpret_cast<int *>(sm.s_bw + kmax);
   sm.s_tab = reinterpret_cast<unsigned long long *>(sm.s_over + kmax + (kmax & 1));
-  sm.s_wc = s_wc;
-  sm.s_base = &s_base;
   sm.s_red = s_red;
   Team tm;
   if constexpr (MULTI) {
