@@ -24,6 +24,7 @@
 #include <cstdio>
 #include <cstring>
 #include <numeric>
+#include <type_traits>
 #include <new>
 #include <vector>
 
@@ -457,32 +458,43 @@ __device__ void team_afterburner(const TeamInst &I, const Team &tm, unsigned lon
     }
     if (nin == 0) continue;
     const int w = I.unit_ewgt ? 1 : I.ewgt[e];
+    // the pairs of the edge's own size (the list is ordered by size): with 32 warps per SM the comparisons of eight
+    // slots for every edge bound this phase
+    auto decide = [&](auto size) {
+      constexpr int N = decltype(size)::value;
 #pragma unroll
-    for (int q = 0; q < kTinyEdge; ++q) {
-      if (!(st[q] & 0x10000u)) continue;
-      const int s = st[q] & 255, t = (st[q] >> 8) & 255;
-      const uint64_t K = key[q];
-      bool last_dep = true, no_arr_before = true, first_arr = true, no_dep_after = true, nm_s = false, nm_t = false;
+      for (int q = 0; q < N; ++q) {
+        if (!(st[q] & 0x10000u)) continue;
+        const int s = st[q] & 255, t = (st[q] >> 8) & 255;
+        const uint64_t K = key[q];
+        bool last_dep = true, no_arr_before = true, first_arr = true, no_dep_after = true, nm_s = false, nm_t = false;
 #pragma unroll
-      for (int r = 0; r < kTinyEdge; ++r) {
-        if (st[r] & 0x20000u) {
-          const int br = st[r] & 255;
-          nm_s |= br == s;
-          nm_t |= br == t;
+        for (int r = 0; r < N; ++r) {
+          if (r == q) continue;
+          if (st[r] & 0x20000u) {
+            const int br = st[r] & 255;
+            nm_s |= br == s;
+            nm_t |= br == t;
+          }
+          if (!(st[r] & 0x10000u)) continue;
+          const int sr = st[r] & 255, tr = (st[r] >> 8) & 255;
+          const uint64_t Kr = key[r];
+          if (sr == s && Kr > K) last_dep = false;
+          if (tr == s && Kr < K) no_arr_before = false;
+          if (tr == t && Kr < K) first_arr = false;
+          if (sr == t && Kr > K) no_dep_after = false;
         }
-        if (!(st[r] & 0x10000u)) continue;
-        const int sr = st[r] & 255, tr = (st[r] >> 8) & 255;
-        const uint64_t Kr = key[r];
-        if (sr == s && Kr > K) last_dep = false;
-        if (tr == s && Kr < K) no_arr_before = false;
-        if (tr == t && Kr < K) first_arr = false;
-        if (sr == t && Kr > K) no_dep_after = false;
+        int delta = 0;
+        if (last_dep && no_arr_before && !nm_s) delta += w;
+        if (first_arr && no_dep_after && !nm_t) delta -= w;
+        if (delta) atomicAdd(&I.rg[(int)(K & 0xffffffffu)], delta);
       }
-      int delta = 0;
-      if (last_dep && no_arr_before && !nm_s) delta += w;
-      if (first_arr && no_dep_after && !nm_t) delta -= w;
-      if (delta) atomicAdd(&I.rg[(int)(K & 0xffffffffu)], delta);
-    }
+    };
+    if (sz <= 2) decide(std::integral_constant<int, 2>());
+    else if (sz == 3) decide(std::integral_constant<int, 3>());
+    else if (sz == 4) decide(std::integral_constant<int, 4>());
+    else if (sz <= 6) decide(std::integral_constant<int, 6>());
+    else decide(std::integral_constant<int, kTinyEdge>());
   }
   const int lane = threadIdx.x & 31;
   unsigned long long *maxd = s_tab + (size_t)(threadIdx.x >> 5) * (2 * I.k + (KWP + 1) / 2);
@@ -698,51 +710,106 @@ __device__ void eligible_table(const TeamInst &I, const long long *s_cap, uint32
 
 // Records of the round: every vertex v of an overloaded block s with 2c(v) <= 3(c(V_s) - ceil(c(V)/k)) and an
 // eligible target gets its best eligible target (ties to the smaller block) and its priority key.
+// A warp scans its vertices and queues the ones to evaluate, which it evaluates
+// 32 at a time: about one vertex in six lies in an overloaded block, and
+// evaluating where they lay left most lanes idle behind them (29 us per round
+// of 60,000 vertices).
+struct TeamQueue {
+  int v[64], sc[64];  // vertex; block | c(v) << 8
+};
+
+// Counts the records of each block (RbBlock::room, for team_select_local), one atomic per warp and block.
+__device__ __forceinline__ void count_records(const TeamInst &I, bool rec, int s) {
+  const unsigned peers = match_bits<9>(rec ? (unsigned)s : 256u);
+  if (rec && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&I.rbb[s].room, __popc(peers));
+}
+
+template <bool MULTI, int KWP>
+__device__ __forceinline__ void evaluate_targets(const TeamInst &I, const TeamQueue &q, int cnt, const long long *s_cap,
+                                                 const uint32_t (*s_elig)[KWP]) {
+  const int lane = threadIdx.x & 31;
+  const bool rec = lane < cnt;
+  const int v = rec ? q.v[lane] : 0, sc = rec ? q.sc[lane] : 0;
+  const int s = sc & 255;
+  const int32_t c = sc >> 8;
+  int t = 0;
+  uint64_t hi = 0;
+  if (rec) {
+    uint32_t C[KWP];
+    if (c <= kEligTab) {
+#pragma unroll
+      for (int w = 0; w < KWP; ++w) C[w] = s_elig[c - 1][w];
+    } else {
+      eligible_set<KWP>(s_cap, I.k, c, C);
+    }
+    uint32_t pl[kLightPlanes][KWP], any[KWP];
+    const int32_t A = light_planes<MULTI, KWP>(I, v, s, pl, any);
+    int32_t conn;
+    t = argmax_planes<KWP, kLightPlanes>(pl, C, conn);
+    hi = rb_priority_key(I.rb_compact, I.rb_L, I.rb_Pmax, conn - A, c);
+  }
+  const unsigned long long pos = warp_append(rec, &I.tc->n_rec);
+  if (MULTI) count_records(I, rec, s);
+  if (rec) {
+    I.rb_hi[pos] = hi;
+    I.rb_v[pos] = v;
+    I.rb_ct[pos] = (c << 16) | (s << 8) | t;
+  }
+}
+
 template <bool MULTI, int KWP>
 __device__ void team_targets(const TeamInst &I, const Team &tm, const long long *s_cap, const long long *s_bw,
-                             const int *s_over, const uint32_t (*s_elig)[KWP]) {
-  // the next vertex's id, block and weight are loaded while the current one is evaluated
+                             const int *s_over, const uint32_t (*s_elig)[KWP], TeamQueue *s_queue) {
+  TeamQueue &q = s_queue[threadIdx.x >> 5];
+  int qn = 0;
+  // the next vertex's id, block and weight are loaded while the current one is looked at
   const long long i0 = (long long)tm.rank * blockDim.x + threadIdx.x;
   int nv = i0 < I.n_light ? I.v_light[i0] : -1;
   int ns = nv >= 0 ? ldm<MULTI>(I.part + nv) : 0;
   int32_t nc = nv >= 0 ? I.vwgt[nv] : 0;
   for (long long base = (long long)tm.rank * blockDim.x; base < I.n_light; base += tm.nthr) {
     const long long i = base + threadIdx.x;
-    bool rec = false;
-    int v = nv, s = ns, t = 0;
-    int32_t c = nc;
-    uint64_t hi = 0;
+    const int v = nv, s = ns;
+    const int32_t c = nc;
     nv = i + tm.nthr < I.n_light ? I.v_light[i + tm.nthr] : -1;
     ns = nv >= 0 ? ldm<MULTI>(I.part + nv) : 0;
     nc = nv >= 0 ? I.vwgt[nv] : 0;
-    if (i < I.n_light) {
-      if (s_over[s] && 2ll * c <= 3ll * (s_bw[s] - I.A)) {
-        uint32_t C[KWP], nz = 0;
-        if (c <= kEligTab) {
+    bool act = false;
+    if (i < I.n_light && s_over[s] && 2ll * c <= 3ll * (s_bw[s] - I.A)) {
+      uint32_t C[KWP], nz = 0;
+      if (c <= kEligTab) {
 #pragma unroll
-          for (int q = 0; q < KWP; ++q) C[q] = s_elig[c - 1][q];
-        } else {
-          eligible_set<KWP>(s_cap, I.k, c, C);
-        }
-#pragma unroll
-        for (int q = 0; q < KWP; ++q) nz |= C[q];
-        if (nz) {
-          uint32_t pl[kLightPlanes][KWP], any[KWP];
-          const int32_t A = light_planes<MULTI, KWP>(I, v, s, pl, any);
-          int32_t conn;
-          t = argmax_planes<KWP, kLightPlanes>(pl, C, conn);
-          hi = rb_priority_key(I.rb_compact, I.rb_L, I.rb_Pmax, conn - A, c);
-          rec = true;
-        }
+        for (int w = 0; w < KWP; ++w) C[w] = s_elig[c - 1][w];
+      } else {
+        eligible_set<KWP>(s_cap, I.k, c, C);
       }
+#pragma unroll
+      for (int w = 0; w < KWP; ++w) nz |= C[w];
+      act = nz != 0;
     }
-    const unsigned long long pos = warp_append(rec, &I.tc->n_rec);
-    if (rec) {
-      I.rb_hi[pos] = hi;
-      I.rb_v[pos] = v;
-      I.rb_ct[pos] = (c << 16) | (s << 8) | t;
+    const int ln = threadIdx.x & 31;
+    const unsigned bal = __ballot_sync(kFull, act);
+    if (act) {
+      const int at = qn + __popc(bal & ((1u << ln) - 1));
+      q.v[at] = v;
+      q.sc[at] = s | (c << 8);
+    }
+    qn += __popc(bal);
+    __syncwarp();
+    if (qn >= 32) {
+      evaluate_targets<MULTI, KWP>(I, q, 32, s_cap, s_elig);
+      const int rest = qn - 32;
+      const int mv = ln < rest ? q.v[32 + ln] : 0, ms = ln < rest ? q.sc[32 + ln] : 0;
+      __syncwarp();
+      if (ln < rest) {
+        q.v[ln] = mv;
+        q.sc[ln] = ms;
+      }
+      __syncwarp();
+      qn = rest;
     }
   }
+  if (qn > 0) evaluate_targets<MULTI, KWP>(I, q, qn, s_cap, s_elig);
   const int lane = threadIdx.x & 31;
   for (long long i = tm.wid; i < I.n_heavy; i += tm.nwarps) {
     const int v = I.v_heavy[i];
@@ -772,6 +839,7 @@ __device__ void team_targets(const TeamInst &I, const Team &tm, const long long 
     warp_argmax(bc, bb);
     if (lane == 0) {
       const unsigned long long pos = atomicAdd(&I.tc->n_rec, 1ull);
+      if (MULTI) atomicAdd(&I.rbb[s].room, 1);
       I.rb_hi[pos] = rb_priority_key(I.rb_compact, I.rb_L, I.rb_Pmax, bc - A, c);
       I.rb_v[pos] = v;
       I.rb_ct[pos] = (c << 16) | (s << 8) | bb;
@@ -886,17 +954,142 @@ __device__ void team_apply_selection(const TeamInst &I, const Team &tm, long lon
   block_add(moved, reinterpret_cast<long long *>(&I.tc->moved), s_red);
 }
 
+// The selection of a multi-block team where no block of the team owns more than kLocalRecords records (block b of the
+// partition belongs to the team's block b mod size): each reads all records, keeps its own in shared memory, does
+// every level of the radix select for all its blocks of the partition there, with block barriers only, and moves
+// them.  The team-wide form has two team barriers and a chain of global loads per level: 14 to 17 us per round, and
+// 6 to 9 for the moves after it.
+constexpr int kLocalRecords = 4096;
+constexpr int kLocalBlocks = 32;  // blocks of the partition per block of the team
+constexpr size_t kLocalSmem = sizeof(RbRec) * kLocalRecords + sizeof(unsigned) * 256 * kLocalBlocks;
+
+// Whether every thread of the team may take the local form (the same answer in all).
+template <bool MULTI>
+__device__ bool select_is_local(const TeamInst &I, const Team &tm) {
+  const int size = (int)tm.size;  // a power of two up to 8
+  if (!MULTI || size < 2 || (I.k + size - 1) / size > kLocalBlocks) return false;
+  int mine = 0;  // lane l: records of the blocks l, l + 32, ...: all of the team's block l mod size
+  for (int b = threadIdx.x & 31; b < I.k; b += 32) mine += ldm<MULTI>(&I.rbb[b].room);
+  for (int o = size; o < 32; o <<= 1) mine += __shfl_xor_sync(kFull, mine, o);
+  return __reduce_max_sync(kFull, mine) <= kLocalRecords;
+}
+
+template <int KWP, class KT>
+__device__ void team_select_local(const TeamInst &I, const Team &tm, long long nrec, const int *s_over,
+                                  const long long *s_bw, SelState<KT> &st, RbRec *list, long long *s_dw,
+                                  long long *s_red) {
+  __shared__ int s_n;
+  __shared__ long long s_before[kLocalBlocks];
+  unsigned *hist = reinterpret_cast<unsigned *>(list + kLocalRecords);  // 256 bins per own block
+  const int t = threadIdx.x, T = blockDim.x, lane = t & 31, size = (int)tm.size, shift = __ffs(size) - 1;
+  const int own = (I.k - (int)tm.rank + size - 1) / size;  // blocks rank, rank + size, ...
+  for (int x = t; x < 256 * own; x += T) hist[x] = 0;
+  for (int x = t; x < own; x += T) {
+    s_before[x] = 0;
+    st.pre[x] = 0;
+    st.all[x] = 0;
+  }
+  if (t == 0) s_n = 0;
+  __syncthreads();
+  for (long long i0 = 0; i0 < nrec; i0 += 4 * T) {
+    int32_t ct[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const long long i = i0 + q * T + t;
+      ct[q] = i < nrec ? __ldcg(I.rb_ct + i) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const long long i = i0 + q * T + t;
+      const bool mine = ct[q] && (((ct[q] >> 8) & 255) & (size - 1)) == (int)tm.rank;  // c(v) >= 1: no record is 0
+      const unsigned bal = __ballot_sync(kFull, mine);
+      if (!bal) continue;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&s_n, __popc(bal));
+      at = __shfl_sync(kFull, at, 0) + __popc(bal & ((1u << lane) - 1));
+      if (mine) list[at] = RbRec{__ldcg(I.rb_hi + i), __ldcg(I.rb_v + i), ct[q]};
+    }
+  }
+  __syncthreads();
+  const int n = s_n;
+  for (int up = I.rb_tbits; up > 0;) {
+    const int lo = up > 8 ? up - 8 : 0;
+    const bool first = up >= I.rb_tbits;
+    for (int i = t; i < n; i += T) {
+      const RbRec r = list[i];
+      const int x = ((r.ct >> 8) & 255) >> shift;
+      const KT K = ((KT)r.hi << I.rb_vbits) | (KT)(uint32_t)r.v;
+      if (!st.all[x] && (first || (K >> up) == (st.pre[x] >> up)))
+        atomicAdd(&hist[x * 256 + (int)((unsigned)(K >> lo) & 255u)], (unsigned)(r.ct >> 16));
+    }
+    __syncthreads();
+    for (int x = t >> 5; x < own; x += T >> 5) {  // a warp per own block picks the digit
+      const int b = (x << shift) + (int)tm.rank;
+      if (!s_over[b] || st.all[x]) continue;
+      const long long need = s_bw[b] - I.Lmax, before = s_before[x];
+      unsigned *row = hist + x * 256;
+      unsigned w[8];
+      long long tot = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        w[q] = row[lane * 8 + q];
+        tot += w[q];
+      }
+      long long incl = tot;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) row[lane * 8 + q] = 0u;
+      if (first && __shfl_sync(kFull, incl, 31) < need) {
+        if (lane == 0) st.all[x] = 1;
+        continue;
+      }
+      long long run = before + incl - tot;
+      const unsigned hit = __ballot_sync(kFull, run < need && run + tot >= need);
+      if (lane == __ffs(hit) - 1) {
+        int q = 0;
+        for (; q < 7; ++q) {
+          if (run + w[q] >= need) break;
+          run += w[q];
+        }
+        s_before[x] = run;
+        st.pre[x] |= (KT)(unsigned)(lane * 8 + q) << lo;
+      }
+    }
+    __syncthreads();
+    up = lo;
+  }
+  long long moved = 0;
+  for (int i = t; i < n; i += T) {
+    const RbRec r = list[i];
+    const int b = (r.ct >> 8) & 255, x = b >> shift;
+    const KT K = ((KT)r.hi << I.rb_vbits) | (KT)(uint32_t)r.v;
+    if (st.all[x] || K <= st.pre[x]) {
+      move_vertex<KWP>(I, r.v, b, r.ct & 255, (r.ct >> 16) & 0xffff, s_dw);
+      ++moved;
+    }
+  }
+  flush_bw(I, s_dw);
+  block_add(moved, reinterpret_cast<long long *>(&I.tc->moved), s_red);
+}
+
 struct SmemPtrs {
   long long *s_dw, *s_cap, *s_bw, *s_red;
   int *s_over;
-  unsigned long long *s_tab;
+  unsigned long long *s_tab;  // the afterburner's tables; multi-block teams: also the local selection's records
+  void *s_sel;                // SelState<u128>, or in its first bytes the state of 64-bit keys
+  void *s_elig;               // kEligTab x KWP words
+  TeamQueue *s_queue;
 };
 
 // Rebalancing rounds until balanced, a round moves nothing, or the round cap.  Returns the rounds; moves in *mv.
 template <bool MULTI, int KWP>
 __device__ long long team_rebalance(const TeamInst &I, const Team &tm, const SmemPtrs &sm, long long *mv) {
-  __shared__ SelState<u128> s_sel;  // or, in its first bytes, the state of 64-bit keys
-  __shared__ uint32_t s_elig[kEligTab][KWP];
+  uint32_t (*s_elig)[KWP] = reinterpret_cast<uint32_t (*)[KWP]>(sm.s_elig);
   long long rounds = 0, moves = 0;
   for (;;) {
     const bool any = round_state<MULTI>(I, sm.s_cap, sm.s_bw, sm.s_over);
@@ -916,20 +1109,28 @@ __device__ long long team_rebalance(const TeamInst &I, const Team &tm, const Sme
       r.pre_hi = 0;
       r.pre_lo = 0;
       r.all = 0;
+      r.room = 0;
       I.rbb[b] = r;
     }
     eligible_table<KWP>(I, sm.s_cap, s_elig);
     team_sync<MULTI>();
-    team_targets<MULTI, KWP>(I, tm, sm.s_cap, sm.s_bw, sm.s_over, s_elig);
+    team_targets<MULTI, KWP>(I, tm, sm.s_cap, sm.s_bw, sm.s_over, s_elig, sm.s_queue);
     team_sync<MULTI>();
     const long long nrec = (long long)ldm<MULTI>(&I.tc->n_rec);
-    if (I.rb_tbits <= 64) {
-      SelState<unsigned long long> &st = *reinterpret_cast<SelState<unsigned long long> *>(&s_sel);
-      team_select<MULTI, unsigned long long>(I, tm, nrec, sm.s_over, st);
-      team_apply_selection<MULTI, KWP, unsigned long long>(I, tm, nrec, sm.s_over, st, sm.s_dw, sm.s_red);
+    SelState<unsigned long long> &st64 = *static_cast<SelState<unsigned long long> *>(sm.s_sel);
+    SelState<u128> &st128 = *static_cast<SelState<u128> *>(sm.s_sel);
+    if (select_is_local<MULTI>(I, tm)) {
+      RbRec *list = reinterpret_cast<RbRec *>(sm.s_tab);
+      if (I.rb_tbits <= 64)
+        team_select_local<KWP, unsigned long long>(I, tm, nrec, sm.s_over, sm.s_bw, st64, list, sm.s_dw, sm.s_red);
+      else
+        team_select_local<KWP, u128>(I, tm, nrec, sm.s_over, sm.s_bw, st128, list, sm.s_dw, sm.s_red);
+    } else if (I.rb_tbits <= 64) {
+      team_select<MULTI, unsigned long long>(I, tm, nrec, sm.s_over, st64);
+      team_apply_selection<MULTI, KWP, unsigned long long>(I, tm, nrec, sm.s_over, st64, sm.s_dw, sm.s_red);
     } else {
-      team_select<MULTI, u128>(I, tm, nrec, sm.s_over, s_sel);
-      team_apply_selection<MULTI, KWP, u128>(I, tm, nrec, sm.s_over, s_sel, sm.s_dw, sm.s_red);
+      team_select<MULTI, u128>(I, tm, nrec, sm.s_over, st128);
+      team_apply_selection<MULTI, KWP, u128>(I, tm, nrec, sm.s_over, st128, sm.s_dw, sm.s_red);
     }
     team_sync<MULTI>();
     const long long moved = (long long)ldm<MULTI>(&I.tc->moved);
@@ -1032,18 +1233,33 @@ __device__ void team_refine(const TeamInst &I, const Team &tm, const TeamArgs &a
   team_sync<MULTI>();
 }
 
+// Dynamic shared memory: the per-block arrays of the partition, then (16-byte aligned) the afterburner's tables, in
+// multi-block teams with room for the local selection.
+__host__ __device__ constexpr size_t team_smem_head(int kmax) { return ((size_t)kmax * (8 + 8 + 8 + 4) + 15) & ~15ull; }
+template <bool MULTI, int KWP>
+constexpr size_t team_smem(int kmax, int threads) {
+  const size_t tab = (size_t)(threads / 32) * (2 * kmax + (KWP + 1) / 2) * 8;
+  return team_smem_head(kmax) + (MULTI && tab < kLocalSmem ? kLocalSmem : tab);
+}
+
 // The persistent kernel: teams of gridDim.x / clusterDim blocks loop over the work queue.
 template <bool MULTI, int KWP>
-__global__ void __launch_bounds__(kTeamMaxThreads) k_batch_teams(TeamArgs a, int kmax) {
+__global__ void __launch_bounds__(kTeamMaxThreads, 1) k_batch_teams(TeamArgs a, int kmax) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_red[kTeamMaxThreads / 32];
+  __shared__ __align__(16) SelState<u128> s_sel;
+  __shared__ uint32_t s_elig[kEligTab][KWP];
+  __shared__ TeamQueue s_queue[kTeamMaxThreads / 32];
   SmemPtrs sm;
   sm.s_dw = reinterpret_cast<long long *>(smem);
   sm.s_cap = sm.s_dw + kmax;
   sm.s_bw = sm.s_cap + kmax;
   sm.s_over = reinterpret_cast<int *>(sm.s_bw + kmax);
-  sm.s_tab = reinterpret_cast<unsigned long long *>(sm.s_over + kmax + (kmax & 1));
+  sm.s_tab = reinterpret_cast<unsigned long long *>(smem + team_smem_head(kmax));
   sm.s_red = s_red;
+  sm.s_sel = &s_sel;
+  sm.s_elig = s_elig;
+  sm.s_queue = s_queue;
   Team tm;
   if constexpr (MULTI) {
     unsigned r, sz;
@@ -1131,14 +1347,13 @@ template <bool MULTI, int KWP>
 cudaError_t launch_group(const TeamArgs &a, int kmax, int ctas, int threads, int num_sms, cudaStream_t s,
                          int max_teams) {
   auto kern = k_batch_teams<MULTI, KWP>;
-  const size_t smem = (size_t)kmax * (8 + 8 + 8 + 4) + 8 * (size_t)(kmax & 1) +
-                      (size_t)(threads / 32) * (2 * kmax + (KWP + 1) / 2) * 8;
+  const size_t smem = team_smem<MULTI, KWP>(kmax, threads);
   // The limit is a property of the kernel, shared by every batch and graph that launches it: set it for
   // the largest instance this mask width allows (k = 32 KWP) and 1,024 threads, so it never shrinks
   // under an earlier launch.
-  constexpr size_t kSmemMax =
-      (size_t)(32 * KWP) * (8 + 8 + 8 + 4) + 8 + (size_t)32 * (2 * 32 * KWP + (KWP + 1) / 2) * 8;
-  static_assert(kSmemMax <= 227 * 1024, "the team kernel's shared memory must fit one block");
+  constexpr size_t kSmemMax = team_smem<MULTI, KWP>(32 * KWP, kTeamMaxThreads);
+  static_assert(kSmemMax + 32 * 1024 <= 227 * 1024, "the team kernel's shared memory (with its static part) must fit "
+                                                    "one block");
   if (smem > kSmemMax) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
   if (e != cudaSuccess) return e;
