@@ -44,23 +44,22 @@ __device__ __forceinline__ bool mask_bit(const uint32_t (&M)[KWP], int b) {
   return (x >> (b & 31)) & 1u;
 }
 
-// planes += w * M  (w < 2^NP, no overflow past the top plane by construction)
+// planes += w * M  (w < 2^NP, no overflow past the top plane by construction): one full adder per plane, whose
+// addend is M where w has the plane's bit.  Three operations per plane and word whatever w is; a ripple from every set
+// bit of w cost up to that per bit, and the warp the most of any of its lanes.
 template <int KWP, int NP>
 __device__ __forceinline__ void add_weighted(uint32_t (&pl)[NP][KWP], const uint32_t (&M)[KWP], uint32_t w) {
-  while (w) {
-    const int p0 = __ffs(w) - 1;
-    w &= w - 1;
+  uint32_t carry[KWP];
+#pragma unroll
+  for (int q = 0; q < KWP; ++q) carry[q] = 0;
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const uint32_t on = 0u - ((w >> p) & 1u);
 #pragma unroll
     for (int q = 0; q < KWP; ++q) {
-      uint32_t carry = M[q];
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        if (p >= p0) {
-          uint32_t c2 = pl[p][q] & carry;
-          pl[p][q] ^= carry;
-          carry = c2;
-        }
-      }
+      const uint32_t x = M[q] & on, y = pl[p][q], c = carry[q];
+      pl[p][q] = x ^ y ^ c;
+      carry[q] = (x & y) | (c & (x | y));
     }
   }
 }

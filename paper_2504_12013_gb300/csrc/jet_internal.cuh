@@ -49,8 +49,8 @@ __host__ __device__ inline uint64_t cand_key(uint64_t r, int32_t v) { return (r 
 
 // Device-side counters of one call (one cache line each group).
 struct Counters {
-  // |V_b|, recounted from the partition in every call that may rebalance (they size the blocks'
-  // segments of rebalancing records) and kept up by the apply kernels
+  // |V_b| where rebalancing records are segmented (they size the segments): recounted from the
+  // partition in every call that may rebalance, and kept up by the apply kernels
   int vcount[kMaxK];
   unsigned long long n_moves;     // entries in the move list
   unsigned long long n_cand;      // |M|
@@ -308,7 +308,7 @@ cudaError_t launch_rebalance_candidates(jet_ctx *c, const int32_t *part, const i
 cudaError_t prepare_afterburner(jet_ctx *c);
 cudaError_t prepare_afterburner_kernels(jet_ctx *c);  // ab_bps
 cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi);
-// part (with build_moves): the partition, whose blocks' vertices are counted.  rs (may be NULL): if the last
+// part (with build_moves): the partition, whose blocks' vertices are counted where records are segmented.  rs (may be NULL): if the last
 // iteration improved (rs->snap), the partition is also copied to c->best_part.
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
                            bool build_moves, const RefineState *rs = nullptr);

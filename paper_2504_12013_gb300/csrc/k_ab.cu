@@ -52,6 +52,12 @@ struct AbArgs {
 // Thread per edge (|e| <= 8), software-pipelined over the thread's edges:
 // while edge j is decided, the pins of edge j+1, the offsets of edge j+2 and
 // the id of edge j+3 are in flight.
+// AHEAD: calls of up to kAheadEdges such edges wait for their loads, not for
+// the memory: blocks and omega come with the records.  Larger ones load the
+// blocks of the few pins that are no candidates after them (and need the
+// registers for a fourth resident block).
+constexpr int kAheadEdges = 1 << 19;
+template <bool AHEAD>
 __global__ void __launch_bounds__(256) k_ab_tiny(AbArgs a) {
   const int stride = gridDim.x * blockDim.x;
   const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -84,31 +90,33 @@ __global__ void __launch_bounds__(256) k_ab_tiny(AbArgs a) {
     e3 = e4;
     uint64_t key[kTinyEdge];
     uint32_t st[kTinyEdge];  // s | t << 8 | 1 << 16 for a candidate; block | 1 << 17 for another pin
-    int vid[kTinyEdge];
     int nin = 0;
+    int w = AHEAD && sz > 0 ? a.ewgt[e] : 0;
 #pragma unroll
     for (int q = 0; q < kTinyEdge; ++q) {
-      key[q] = 0;
-      st[q] = 0;
-      vid[q] = 0;
+      key[q] = q < sz ? a.cand[pin[q]] : 0ull;
+      st[q] = AHEAD && q < sz ? (uint32_t)(a.part[pin[q]] & 255) : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < kTinyEdge; ++q) {
+      const uint64_t r = key[q];
       if (q < sz) {
-        const int v = pin[q];
-        const uint64_t r = a.cand[v];
-        vid[q] = v;
         if (r) {
           ++nin;
-          key[q] = cand_key(r, v);
+          key[q] = cand_key(r, pin[q]);
           st[q] = (uint32_t)cand_s(r) | ((uint32_t)cand_t(r) << 8) | 0x10000u;
         } else {
-          st[q] = 0x20000u;
+          st[q] |= 0x20000u;
         }
       }
     }
     if (nin == 0) continue;
+    if constexpr (!AHEAD) {
 #pragma unroll
-    for (int q = 0; q < kTinyEdge; ++q)
-      if (st[q] & 0x20000u) st[q] |= (uint32_t)(a.part[vid[q]] & 255);  // block of a non-candidate pin
-    const int w = a.ewgt[e];
+      for (int q = 0; q < kTinyEdge; ++q)
+        if (st[q] & 0x20000u) st[q] |= (uint32_t)(a.part[pin[q]] & 255);  // block of a non-candidate pin
+      w = a.ewgt[e];
+    }
     // Every pair of pins is compared, so the comparisons are made for the edge's size: the list is ordered by
     // size, so a warp's edges mostly take one of these branches together (comparing eight slots for every edge
     // bound the kernel by its instructions: 76 us for 2 M edges of 3 pins on average).
@@ -496,6 +504,7 @@ struct ApArgs {
   const int32_t *part;  // with build_moves
   const RefineState *rs;  // may be NULL
   int32_t *best;
+  int count;              // count the blocks' vertices (for segmented rebalancing records)
   const uint64_t *cand;
   int32_t *rg;
   uint8_t *locked;
@@ -516,7 +525,7 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   __shared__ unsigned long long s_base;
   __shared__ unsigned long long s_cand[kWarps];
   __shared__ int s_vc[kMaxK];  // vertices per block of the partition
-  if (a.build_moves)
+  if (a.count)
     for (int b = threadIdx.x; b < a.k; b += blockDim.x) s_vc[b] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -538,9 +547,9 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     }
     ncand += __popc(__ballot_sync(kFull, in));
     if (a.build_moves) {
-      if (valid) {
+      if (valid && (a.count || snap)) {
         const int b = a.part[v];
-        if ((unsigned)b < (unsigned)a.k) atomicAdd(&s_vc[b], 1);
+        if (a.count && (unsigned)b < (unsigned)a.k) atomicAdd(&s_vc[b], 1);
         if (snap) a.best[v] = b;
       }
       const unsigned bap = __ballot_sync(kFull, ap);
@@ -572,7 +581,7 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     for (int i = 0; i < kWarps; ++i) t += s_cand[i];
     if (t) atomicAdd(&a.cnt->n_cand, t);
   }
-  if (a.build_moves)
+  if (a.count)
     for (int b = threadIdx.x; b < a.k; b += blockDim.x)
       if (s_vc[b]) atomicAdd(&a.cnt->vcount[b], s_vc[b]);
 }
@@ -682,8 +691,9 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
   if (c->n_tiny > 0) {
     a.elist = c->e_tiny;
     a.nlist = c->n_tiny;
-    k_ab_tiny<<<grid_for(c->n_tiny, 256, c->launch_sms, c->ab_bps[0]), 256, 0,
-                fork.stream(branch++)>>>(a);
+    const int g = grid_for(c->n_tiny, 256, c->launch_sms, c->ab_bps[0]);
+    if (c->n_tiny <= kAheadEdges) k_ab_tiny<true><<<g, 256, 0, fork.stream(branch++)>>>(a);
+    else k_ab_tiny<false><<<g, 256, 0, fork.stream(branch++)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_mid_half > 0) {
@@ -749,7 +759,7 @@ cudaError_t prepare_afterburner_kernels(jet_ctx *c) {
   // of the kernel, shared by every context, so it is set for the largest k, not for this context's.
   cudaError_t e = cudaFuncSetAttribute(k_ab_warp_small<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)((size_t)kAbWarps * 2 * 2 * kMaxK * sizeof(unsigned long long)));
-  if (e == cudaSuccess) e = resident_blocks(k_ab_tiny, 256, 0, &c->ab_bps[0]);
+  if (e == cudaSuccess) e = resident_blocks(k_ab_tiny<false>, 256, 0, &c->ab_bps[0]);
   if (e == cudaSuccess) e = resident_blocks(k_ab_warp_small<16>, kAbWarps * 32, 2 * warp_tab, &c->ab_bps[1]);
   if (e == cudaSuccess) e = resident_blocks(k_ab_warp_small<32>, kAbWarps * 32, warp_tab, &c->ab_bps[2]);
   if (e == cudaSuccess) e = resident_blocks(k_ab_warp<4>, kAbWarps * 32, warp_tab, &c->ab_bps[3]);
@@ -822,6 +832,7 @@ cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int
   ApArgs a{};
   a.rs = rs;
   a.best = c->best_part;
+  a.count = build_moves && c->rb_segments;
   a.n = c->n;
   a.k = c->k;
   a.part = part;

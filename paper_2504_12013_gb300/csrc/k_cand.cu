@@ -39,7 +39,7 @@ struct CandArgs {
   uint64_t *rb_hi;
   int32_t *rb_v, *rb_ct;
   long long A;
-  int32_t n;
+  int32_t n, cmax;
   Counters *cnt;
   int rb_compact;
   long long rb_L, rb_Pmax;
@@ -141,27 +141,23 @@ __device__ __forceinline__ uint64_t rb_hi_of(const CandArgs &a, int32_t g, int32
 
 // Adds the thread's work counts to the call's totals: one atomic per thread
 // block and counter (every thread of the block calls it).
-__device__ __forceinline__ void count_work(Counters *cnt, unsigned long long over, unsigned long long eval,
-                                           unsigned long long pins) {
-  __shared__ unsigned long long s_w[3];
-  if (threadIdx.x < 3) s_w[threadIdx.x] = 0;
-  __syncthreads();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    over += __shfl_xor_sync(kFull, over, o);
-    eval += __shfl_xor_sync(kFull, eval, o);
-    pins += __shfl_xor_sync(kFull, pins, o);
-  }
+__device__ __forceinline__ void count_work(Counters *cnt, unsigned over, unsigned eval, unsigned pins) {
+  __shared__ unsigned s_w[256 / 32][3];  // per warp
+  const int w = threadIdx.x >> 5;
+  over = __reduce_add_sync(kFull, over);
+  eval = __reduce_add_sync(kFull, eval);
+  pins = __reduce_add_sync(kFull, pins);
   if ((threadIdx.x & 31) == 0) {
-    if (over) atomicAdd(&s_w[0], over);
-    if (eval) atomicAdd(&s_w[1], eval);
-    if (pins) atomicAdd(&s_w[2], pins);
+    s_w[w][0] = over;
+    s_w[w][1] = eval;
+    s_w[w][2] = pins;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (s_w[0]) atomicAdd(&cnt->w_over, s_w[0]);
-    if (s_w[1]) atomicAdd(&cnt->w_eval, s_w[1]);
-    if (s_w[2]) atomicAdd(&cnt->w_eval_pins, s_w[2]);
+  if (threadIdx.x < 3) {
+    unsigned long long x = 0;
+#pragma unroll
+    for (int i = 0; i < 256 / 32; ++i) x += s_w[i][threadIdx.x];
+    if (x) atomicAdd(threadIdx.x == 0 ? &cnt->w_over : threadIdx.x == 1 ? &cnt->w_eval : &cnt->w_eval_pins, x);
   }
 }
 
@@ -585,14 +581,13 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
     s_base[b] = a.rbb[b].base;
   }
   __syncthreads();
-  for (int x = threadIdx.x; x < kTab * KWP; x += blockDim.x) {
-    const int c = x / KWP + 1, qq = x % KWP;
-    uint32_t wd = 0;
-    for (int bit = 0; bit < 32; ++bit) {
-      const int b = qq * 32 + bit;
-      if (b < a.k && s_cap[b] >= c) wd |= 1u << bit;
+  for (int c = w + 1; c <= kTab && c <= a.cmax; c += warps) {  // a warp per c(v), a block per lane
+#pragma unroll
+    for (int qq = 0; qq < KWP; ++qq) {
+      const int b = qq * 32 + lane;
+      const uint32_t wd = __ballot_sync(kFull, b < a.k && s_cap[b] >= c);
+      if (lane == 0) s_elig[c - 1][qq] = wd;
     }
-    s_elig[c - 1][qq] = wd;
   }
   __syncthreads();
   int qn = 0;
@@ -652,7 +647,8 @@ __global__ void __launch_bounds__(256) k_rbcand_heavy(CandArgs a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  unsigned long long w_over = 0, w_eval = 0, w_pins = 0;
+  unsigned w_over = 0, w_eval = 0;
+  unsigned long long w_pins = 0;  // heavy vertices can have any degree
   for (int i = gw; i < a.nlist; i += nw) {
     const int v = a.vlist[i];
     const int s = a.part[v];
@@ -698,7 +694,12 @@ __global__ void __launch_bounds__(256) k_rbcand_heavy(CandArgs a) {
       a.rb_ct[pos] = (c << 16) | (s << 8) | bb;
     }
   }
-  count_work(a.cnt, w_over, w_eval, w_pins);
+  // a block's sum has to fit 32 bits
+  if (lane == 0 && w_pins >= (1u << 24)) {
+    atomicAdd(&a.cnt->w_eval_pins, w_pins);
+    w_pins = 0;
+  }
+  count_work(a.cnt, w_over, w_eval, (unsigned)w_pins);
 }
 
 template <int KWP>
@@ -764,6 +765,7 @@ CandArgs make_args(jet_ctx *c, const int32_t *part, const int32_t *phi) {
   a.rb_ct = c->rb_ct;
   a.A = c->A;
   a.n = c->n;
+  a.cmax = c->cmax;
   a.cnt = c->cnt;
   a.rb_compact = c->rb_compact;
   a.rb_L = c->rb_L;

@@ -803,7 +803,7 @@ cudaError_t select_segments(jet_ctx *c, const RbArgs &a) {
 }
 
 cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
-  if (c->n == 0) return cudaSuccess;
+  if (c->n == 0 || !c->rb_segments) return cudaSuccess;
   k_count_blocks<<<grid_for(c->n, 1024, c->launch_sms, 4), kMaxK, 0, c->stream>>>(part, c->n, c->k, c->cnt);
   ++c->kernel_launches;
   return cudaGetLastError();
