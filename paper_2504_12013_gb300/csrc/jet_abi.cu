@@ -169,7 +169,7 @@ int rebalance_loop(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) { 
   if (!c->cnt_host->rb_any || c->params.max_rebalance_rounds <= 0) return JET_OK;
   for (;;) {
     CKP(F_RB_TGT, launch_rebalance_candidates(c, part, phi), "rebalance targets");
-    CKP(F_RB_SEL, launch_rb_select(c, part), "rebalance select");
+    CKP(F_RB_SEL, launch_rb_select(c, part, block_w), "rebalance select");
     CKP(F_APPLY, launch_rb_apply(c, part, phi, block_w), "rebalance apply");
     CKP(F_RB_CTL, launch_rb_post(c, block_w), "rebalance post");
     rc = sync_counters(c);
@@ -234,9 +234,16 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     if ((e = launch_candidates(c, tn, td, part, phi, locked)) != cudaSuccess) return e;
     if (ev1 && (e = cudaEventRecordWithFlags(ev1, s_main, cudaEventRecordExternal)) != cudaSuccess) return e;
     if ((e = launch_afterburner(c, part, phi)) != cudaSuccess) return e;
-    if ((e = launch_approve(c, part, locked, nullptr, nullptr, true, rs)) != cudaSuccess) return e;
-    if ((e = launch_apply_jet(c, part, phi, bw)) != cudaSuccess) return e;
-    if ((e = launch_rb_check(c, bw, h, 1)) != cudaSuccess) return e;
+    if ((e = launch_approve(c, part, locked, nullptr, nullptr, true, bw, rs)) != cudaSuccess) return e;
+    {
+      // segmented records: the block weights are known before the apply, and the check runs beside it
+      Fork fork(c, c->rb_segments ? 2 : 1);
+      if ((e = launch_apply_jet(c, part, phi, bw)) != cudaSuccess) return e;
+      c->stream = fork.stream(1);
+      e = launch_rb_check(c, bw, h, 1);
+      c->stream = s_main;
+      if (e != cudaSuccess || (e = fork.join()) != cudaSuccess) return e;
+    }
     // WHILE node: rebalancing rounds
     if ((e = cudaStreamGetCaptureInfo(s_main, &st, nullptr, &cg, &deps, &ed, &nd)) != cudaSuccess) return e;
     cudaGraphNodeParams cp{};
@@ -257,9 +264,16 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     c->side_first = 2;
     c->side_count = 1;
     cudaError_t eb = launch_rebalance_candidates(c, part, phi);
-    if (eb == cudaSuccess) eb = launch_rb_select(c, part);
-    if (eb == cudaSuccess) eb = launch_rb_apply(c, part, phi, bw);
-    if (eb == cudaSuccess) eb = launch_rb_post(c, bw, h, 1);
+    if (eb == cudaSuccess) eb = launch_rb_select(c, part, bw);
+    {
+      Fork fork(c, c->rb_segments ? 2 : 1);  // as above: the end of the round beside its apply
+      if (eb == cudaSuccess) eb = launch_rb_apply(c, part, phi, bw);
+      c->stream = fork.stream(1);
+      if (eb == cudaSuccess) eb = launch_rb_post(c, bw, h, 1);
+      c->stream = s_body;
+      const cudaError_t ej = fork.join();
+      if (eb == cudaSuccess) eb = ej;
+    }
     cudaGraph_t tmp = nullptr;
     e = cudaStreamEndCapture(s_body, &tmp);
     c->stream = s_main;
@@ -629,7 +643,7 @@ int jet_refine_round(jet_ctx *c, int32_t tau_num, int32_t tau_den, int32_t *part
   CK(reset_counters(c), "counters");
   CKP(F_CAND, launch_candidates(c, tau_num, tau_den, part, phi, locked), "candidates");
   CKP(F_AB, launch_afterburner(c, part, phi), "afterburner");
-  CKP(F_APPROVE, launch_approve(c, part, locked, nullptr, nullptr, true), "approve");
+  CKP(F_APPROVE, launch_approve(c, part, locked, nullptr, nullptr, true, block_w), "approve");
   CKP(F_APPLY, launch_apply_jet(c, part, phi, block_w), "apply");
   CKP(F_RB_CTL, launch_rb_check(c, block_w), "rebalance check");
   if ((rc = rebalance_loop(c, part, phi, block_w))) return rc;

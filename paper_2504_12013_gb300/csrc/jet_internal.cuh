@@ -309,9 +309,10 @@ cudaError_t prepare_afterburner(jet_ctx *c);
 cudaError_t prepare_afterburner_kernels(jet_ctx *c);  // ab_bps
 cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi);
 // part (with build_moves): the partition, whose blocks' vertices are counted where records are segmented.  rs (may be NULL): if the last
-// iteration improved (rs->snap), the partition is also copied to c->best_part.
+// iteration improved (rs->snap), the partition is also copied to c->best_part.  block_w (with build_moves): where
+// records are segmented, the moves' weights are added here and not by launch_apply_jet.
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
-                           bool build_moves, const RefineState *rs = nullptr);
+                           bool build_moves, int64_t *block_w = nullptr, const RefineState *rs = nullptr);
 cudaError_t launch_export_candidates(jet_ctx *c, int32_t *target, int32_t *gain, uint8_t *in_m);
 // moves, rebalancing, loop control (k_moves.cu)
 cudaError_t prepare_move_kernels(jet_ctx *c);  // move_bps
@@ -320,7 +321,8 @@ cudaError_t launch_apply_jet(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *b
 cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part);  // cnt->vcount (zeroed by reset_counters)
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                             int use_cond = 0);
-cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part);
+// the selection of a round (where records are segmented, block_w takes its weights here and not in launch_rb_apply)
+cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w);
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // applies the selection
 cudaError_t launch_rb_post(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                            int use_cond = 0);

@@ -504,7 +504,11 @@ struct ApArgs {
   const int32_t *part;  // with build_moves
   const RefineState *rs;  // may be NULL
   int32_t *best;
-  int count;              // count the blocks' vertices (for segmented rebalancing records)
+  // segmented rebalancing records: the vertices of each block after the moves, and the block weights, are kept here,
+  // so that the balance check need not wait for the apply
+  int count;
+  const int32_t *vwgt;
+  int64_t *bw;
   const uint64_t *cand;
   int32_t *rg;
   uint8_t *locked;
@@ -524,9 +528,13 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   __shared__ unsigned s_wc[kWarps];
   __shared__ unsigned long long s_base;
   __shared__ unsigned long long s_cand[kWarps];
-  __shared__ int s_vc[kMaxK];  // vertices per block of the partition
+  __shared__ int s_vc[kMaxK];  // vertices per block after the moves
+  __shared__ long long s_dw[kMaxK];
   if (a.count)
-    for (int b = threadIdx.x; b < a.k; b += blockDim.x) s_vc[b] = 0;
+    for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
+      s_vc[b] = 0;
+      s_dw[b] = 0;
+    }
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   // the snapshot of an improved partition, taken here, before the next moves, and not by a launch of its own
@@ -549,7 +557,15 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     if (a.build_moves) {
       if (valid && (a.count || snap)) {
         const int b = a.part[v];
-        if (a.count && (unsigned)b < (unsigned)a.k) atomicAdd(&s_vc[b], 1);
+        if (a.count) {
+          const int c = a.vwgt[v];
+          if (ap) {
+            atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_s(r)]), (unsigned long long)(-(long long)c));
+            atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_t(r)]), (unsigned long long)c);
+          }
+          const int to = ap ? cand_t(r) : b;
+          if ((unsigned)to < (unsigned)a.k) atomicAdd(&s_vc[to], 1);
+        }
         if (snap) a.best[v] = b;
       }
       const unsigned bap = __ballot_sync(kFull, ap);
@@ -582,8 +598,10 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     if (t) atomicAdd(&a.cnt->n_cand, t);
   }
   if (a.count)
-    for (int b = threadIdx.x; b < a.k; b += blockDim.x)
+    for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
       if (s_vc[b]) atomicAdd(&a.cnt->vcount[b], s_vc[b]);
+      if (s_dw[b]) atomicAdd(reinterpret_cast<unsigned long long *>(&a.bw[b]), (unsigned long long)s_dw[b]);
+    }
 }
 
 __global__ void k_export_cand(const uint64_t *cand, int32_t n, int32_t *target, int32_t *gain, uint8_t *in_m) {
@@ -827,12 +845,14 @@ cudaError_t prepare_afterburner(jet_ctx *c) {
 }
 
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
-                           bool build_moves, const RefineState *rs) {
+                           bool build_moves, int64_t *block_w, const RefineState *rs) {
   if (c->n == 0) return cudaSuccess;
   ApArgs a{};
   a.rs = rs;
   a.best = c->best_part;
   a.count = build_moves && c->rb_segments;
+  a.vwgt = c->vwgt;
+  a.bw = block_w;
   a.n = c->n;
   a.k = c->k;
   a.part = part;

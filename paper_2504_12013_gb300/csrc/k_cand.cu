@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
   const int64_t stride = (int64_t)gridDim.x * warps * 32;
   int64_t base = ((int64_t)blockIdx.x * warps + w) * 32;
   GroupRaw cur = fetch_group(a, base + lane, false);  // on its way while the tables are made
+  if (a.rb_rec && blockIdx.x == 0 && threadIdx.x == 0) a.cnt->n_moves = 0;  // the last round's apply has ended
   for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
     s_cap[b] = a.rbb[b].cap;
     s_bw[b] = a.rbb[b].bw;
@@ -638,6 +639,7 @@ template <int KWP>
 __global__ void __launch_bounds__(256) k_rbcand_heavy(CandArgs a) {
   __shared__ long long s_cap[kMaxK], s_bw[kMaxK];
   __shared__ int s_over[kMaxK];
+  if (a.rb_rec && blockIdx.x == 0 && threadIdx.x == 0) a.cnt->n_moves = 0;
   for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
     s_cap[b] = a.rbb[b].cap;
     s_bw[b] = a.rbb[b].bw;

@@ -27,6 +27,7 @@ struct MoveArgs {
   const uint32_t *mv_st;
   int32_t k, kwp;
   int graph;  // graph path: phi and the bitmasks are not kept, a move changes Pi and c(V_i) only
+  int weights;  // c(V_i) and |V_i| are kept here (0: the kernel that made the list has done it)
   unsigned long long rebuild_min;  // from this many moves on, phi is counted anew (launch_apply_jet)
   Counters *cnt;
 };
@@ -109,6 +110,7 @@ struct RbArgs {
   int32_t *mv_v;
   uint32_t *mv_st;
   int32_t n, k;
+  int segments;
   int vbits, tbits;
   int digit, bins;               // radix-select digit width and bins per block row
   long long Lmax, dz_min;
@@ -158,7 +160,8 @@ __device__ __forceinline__ void rb_prep_blocks(const RbArgs &a) {
     a.cur[b * kCurStride] = 0;
   }
   if (b == 0) {
-    a.cnt->n_moves = 0;
+    // segmented: an apply that reads the count may be running beside this; the target kernels reset it
+    if (!a.segments) a.cnt->n_moves = 0;
     a.cnt->n_rec = 0;
   }
 }
@@ -227,11 +230,13 @@ __global__ void __launch_bounds__(256) k_apply(MoveArgs a) {
     const int s = st & 0xffff, t = st >> 16;
     if (sub == 0) {
       a.part[v] = t;
-      const int c = a.vwgt[v];
-      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[s]), (unsigned long long)(-(long long)c));
-      atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c);
-      atomicSub(&s_dc[s], 1);
-      atomicAdd(&s_dc[t], 1);
+      if (a.weights) {
+        const int c = a.vwgt[v];
+        atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[s]), (unsigned long long)(-(long long)c));
+        atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c);
+        atomicSub(&s_dc[s], 1);
+        atomicAdd(&s_dc[t], 1);
+      }
     }
     const int64_t j1 = a.vptr[v + 1];
     if (sub == 0) pins += (unsigned long long)(j1 - a.vptr[v]);
@@ -278,7 +283,7 @@ __global__ void __launch_bounds__(256) k_apply_part(MoveArgs a) {
     for (int q = 0; q < 2; ++q) {
       c[q] = 0;
       if (v[q] < 0) continue;
-      c[q] = a.vwgt[v[q]];
+      if (a.weights) c[q] = a.vwgt[v[q]];
       pins += (unsigned long long)(a.vptr[v[q] + 1] - a.vptr[v[q]]);
     }
 #pragma unroll
@@ -286,6 +291,7 @@ __global__ void __launch_bounds__(256) k_apply_part(MoveArgs a) {
       if (v[q] < 0) continue;
       const int s = st[q] & 0xffff, t = st[q] >> 16;
       a.part[v[q]] = t;
+      if (!a.weights) continue;
       atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[s]), (unsigned long long)(-(long long)c[q]));
       atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[t]), (unsigned long long)c[q]);
       atomicSub(&s_dc[s], 1);
@@ -455,10 +461,12 @@ struct SelRec<u128> {
 
 // WT: unsigned when c(V) < 2^32 (no sum of weights leaves it), else unsigned long long.
 template <class KT, class WT>
-__global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a) {
+__global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw) {
   typedef SelRec<KT> Rec;
   constexpr int kPer = kSelBins / 32;  // bins per lane
   __shared__ __align__(16) WT s_hist[2][kSelBins];
+  __shared__ long long s_dw[kMaxK];  // weight and vertices that move to each block
+  __shared__ int s_dc[kMaxK];
   const int t = threadIdx.x, lane = t & 31, b = blockIdx.x;
   const RbBlock &blk = a.rbb[b];
   const int over = blk.over, room = blk.room, count = a.cur[b * kCurStride];
@@ -471,6 +479,10 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a) {
   for (int q = 0; q < kSelHeld; ++q)
     held[q] = t + q * kSelThreads < cnt ? Rec(rec[t + q * kSelThreads]) : Rec();
   if (t < kSelBins) s_hist[0][t] = s_hist[1][t] = 0;
+  if (t < kMaxK) {
+    s_dw[t] = 0;
+    s_dc[t] = 0;
+  }
   __syncthreads();
   KT pre = 0;  // the fixed digits of the threshold key
   WT before = 0;
@@ -548,8 +560,11 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a) {
       if (q < n) {
         if ((bal[q] >> lane) & 1u) {
           const unsigned long long x = at + __popc(bal[q] & ((1u << lane) - 1));
+          const int to = r[q].ct & 255;
           a.mv_v[x] = r[q].v;
-          a.mv_st[x] = (uint32_t)b | ((uint32_t)(r[q].ct & 255) << 16);
+          a.mv_st[x] = (uint32_t)b | ((uint32_t)to << 16);
+          atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[to]), (unsigned long long)(r[q].ct >> 16));
+          atomicAdd(&s_dc[to], 1);
         }
         at += __popc(bal[q]);
       }
@@ -562,6 +577,23 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) r[q] = i + q * kSelThreads < cnt ? Rec(rec[i + q * kSelThreads]) : Rec();
     emit(r, 4);
+  }
+  __syncthreads();
+  // the block weights already, so that the end of the round need not wait for the apply
+  if (t < kMaxK) {
+    long long dw = s_dw[t];
+    int dc = s_dc[t];
+    if (dc) {
+      add_i64(reinterpret_cast<long long *>(&bw[t]), dw);
+      atomicAdd(&a.cnt->vcount[t], dc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dw += __shfl_xor_sync(kFull, dw, o);
+    dc = __reduce_add_sync(kFull, dc);
+    if (lane == 0 && dc) {
+      add_i64(reinterpret_cast<long long *>(&bw[b]), -dw);
+      atomicSub(&a.cnt->vcount[b], dc);
+    }
   }
 }
 
@@ -690,6 +722,7 @@ MoveArgs move_args(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   a.mask = c->mask;
   a.graph = c->graph_path;
   a.rebuild_min = c->graph_path ? 0 : ~0ull;
+  a.weights = 1;
   a.mv_v = c->mv_v;
   a.mv_st = c->mv_st;
   a.k = c->k;
@@ -702,6 +735,7 @@ RbArgs rb_args(jet_ctx *c, const int64_t *block_w, const int32_t *part) {
   RbArgs a{};
   a.bw = block_w;
   a.rbb = c->rbb;
+  a.segments = c->rb_segments;
   a.rec = c->rb_rec;
   a.cur = c->rb_cur;
   a.rb_hi = c->rb_hi;
@@ -756,9 +790,15 @@ static cudaError_t apply_part(jet_ctx *c, const MoveArgs &a) {
 // eight iterations of rownet_4m took 42.6 ms with the apply alone and 39.1 so (vlsi_2m 7.99 and 7.94).
 cudaError_t launch_apply_jet(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   const double phi_bytes = 4.0 * c->m * c->k;
-  if (c->n == 0 || c->graph_path || phi_bytes < 256e6) return launch_apply(c, part, phi, block_w);
+  if (c->n == 0) return cudaSuccess;
+  if (c->graph_path || phi_bytes < 256e6) {
+    MoveArgs a = move_args(c, part, phi, block_w);
+    a.weights = !c->rb_segments;  // launch_approve has done it
+    return c->graph_path ? apply_part(c, a) : apply_phi(c, a);
+  }
   const double bytes = phi_bytes + 8.0 * c->m * c->kwp + 8.0 * c->m + 8.0 * c->P;
   MoveArgs a = move_args(c, part, phi, block_w);
+  a.weights = !c->rb_segments;
   a.rebuild_min = (unsigned long long)(bytes / (4.2e3 * 0.075) * c->n / std::max<int64_t>(c->P, 1)) + 1;
   cudaError_t e = apply_phi(c, a);
   if (e == cudaSuccess) e = apply_part(c, a);
@@ -795,9 +835,9 @@ void rb_select_levels(jet_ctx *c, const RbArgs &a) {
 }
 
 template <class KT>
-cudaError_t select_segments(jet_ctx *c, const RbArgs &a) {
-  if (c->W < (1ll << 32)) k_rb_select<KT, unsigned><<<c->k, kSelThreads, 0, c->stream>>>(a);
-  else k_rb_select<KT, unsigned long long><<<c->k, kSelThreads, 0, c->stream>>>(a);
+cudaError_t select_segments(jet_ctx *c, const RbArgs &a, int64_t *bw) {
+  if (c->W < (1ll << 32)) k_rb_select<KT, unsigned><<<c->k, kSelThreads, 0, c->stream>>>(a, bw);
+  else k_rb_select<KT, unsigned long long><<<c->k, kSelThreads, 0, c->stream>>>(a, bw);
   ++c->kernel_launches;
   return cudaGetLastError();
 }
@@ -809,10 +849,11 @@ cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part) {
+cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w) {
   if (c->n == 0) return cudaSuccess;
   const RbArgs a = rb_args(c, nullptr, part);
-  if (c->rb_segments) return a.tbits <= 64 ? select_segments<unsigned long long>(c, a) : select_segments<u128>(c, a);
+  if (c->rb_segments)
+    return a.tbits <= 64 ? select_segments<unsigned long long>(c, a, block_w) : select_segments<u128>(c, a, block_w);
   if (a.tbits <= 64) rb_select_levels<unsigned long long>(c, a);
   else rb_select_levels<u128>(c, a);
   return cudaGetLastError();
@@ -820,7 +861,11 @@ cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part) {
 
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   if (c->n == 0) return cudaSuccess;
-  if (c->rb_segments) return launch_apply(c, part, phi, block_w);  // the selection is a move list
+  if (c->rb_segments) {  // the selection is a move list, its weights are in place
+    MoveArgs a = move_args(c, part, phi, block_w);
+    a.weights = 0;
+    return c->graph_path ? apply_part(c, a) : apply_phi(c, a);
+  }
   const RbArgs r = rb_args(c, block_w, part);
   const MoveArgs a = move_args(c, part, phi, block_w);
   if (r.tbits <= 64)
