@@ -514,16 +514,66 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_cand_light(CandArgs 
   if (qn > 0) cand_batch<KWP, UNIT>(a, stage, q, qn);
 }
 
-// Evaluates queue entries 0..cnt-1 for rebalancing and appends their records.
+// The targets' queue holds the vertices of overloaded blocks only; their
+// weights and offsets are loaded when a batch of 32 is evaluated.  Loaded
+// where the vertices were found, they put a memory latency into every group of
+// the scan that had one of them.
+struct TargetQueue {
+  static constexpr int kCap = 64;
+  int v[kCap], s[kCap];
+};
+
+__device__ __forceinline__ int enqueue(TargetQueue *q, int qn, bool act, int v, int s) {
+  const int lane = threadIdx.x & 31;
+  const unsigned bal = __ballot_sync(kFull, act);
+  if (act) {
+    const int pos = qn + __popc(bal & ((1u << lane) - 1));
+    q->v[pos] = v;
+    q->s[pos] = s;
+  }
+  __syncwarp();
+  return qn + __popc(bal);
+}
+
+__device__ __forceinline__ int dequeue32(TargetQueue *q, int qn) {
+  const int lane = threadIdx.x & 31, rest = qn - 32;
+  const int v = lane < rest ? q->v[32 + lane] : 0, s = lane < rest ? q->s[32 + lane] : 0;
+  __syncwarp();
+  if (lane < rest) {
+    q->v[lane] = v;
+    q->s[lane] = s;
+  }
+  __syncwarp();
+  return rest;
+}
+
+// Evaluates queue entries 0..cnt-1 for rebalancing and appends their records (heavy vertices of Section 4.3, which
+// are never moved, and vertices without an eligible target have none).
 template <int KWP, bool UNIT, int kTab>
-__device__ __forceinline__ void rb_batch(const CandArgs &a, uint8_t *stage, const WarpQueue *q, int cnt,
-                                         const long long *s_cap, const int *s_base, const uint32_t (*s_elig)[KWP]) {
+__device__ __forceinline__ void rb_batch(const CandArgs &a, uint8_t *stage, const TargetQueue *q, int cnt,
+                                         const long long *s_cap, const long long *s_bw, const int *s_base,
+                                         const uint32_t (*s_elig)[KWP], unsigned &w_eval, unsigned &w_pins) {
   constexpr int NP = kLightPlanes;
   const int lane = threadIdx.x & 31;
-  const bool mine = lane < cnt;
-  const int v = mine ? q->v[lane] : 0, s = mine ? q->s[lane] : 0, deg = mine ? q->deg[lane] : 0;
-  const int32_t c = mine ? q->c[lane] : 0;
-  const int64_t j0 = mine ? q->j0[lane] : 0;
+  bool mine = lane < cnt;
+  const int v = mine ? q->v[lane] : 0, s = mine ? q->s[lane] : 0;
+  const int32_t c = mine ? a.vwgt[v] : 1;
+  const int64_t j0 = mine ? a.vptr[v] : 0;
+  int deg = mine ? (int)(a.vptr[v + 1] - j0) : 0;
+  uint32_t nz = 0;
+  if (c <= kTab) {
+#pragma unroll
+    for (int qq = 0; qq < KWP; ++qq) nz |= s_elig[c - 1][qq];
+  } else {
+    uint32_t C[KWP];
+    eligible_words<KWP>(s_cap, a.k, c, C);
+#pragma unroll
+    for (int qq = 0; qq < KWP; ++qq) nz |= C[qq];
+  }
+  mine = mine && nz && 2ll * c <= 3ll * (s_bw[s] - a.A);
+  if (!mine) deg = 0;
+  w_eval += mine;
+  w_pins += deg;
   uint32_t pl[NP][KWP], any[KWP];
   const int32_t A = stage_accumulate<KWP, NP, UNIT>(a, stage, j0, deg, s, pl, any);
   uint64_t hi = 0;
@@ -551,7 +601,7 @@ __device__ __forceinline__ void rb_batch(const CandArgs &a, uint8_t *stage, cons
   if (lane == 0) pos0 = atomicAdd(&a.cnt->n_rec, (unsigned long long)__popc(bal));
   pos0 = __shfl_sync(kFull, pos0, 0);
   if (mine) {
-    const unsigned long long pos = pos0 + lane;
+    const unsigned long long pos = pos0 + __popc(bal & ((1u << lane) - 1));
     a.rb_hi[pos] = hi;
     a.rb_v[pos] = v;
     a.rb_ct[pos] = ct;
@@ -564,11 +614,11 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
   __shared__ long long s_cap[kMaxK], s_bw[kMaxK];
   __shared__ int s_over[kMaxK], s_base[kMaxK];
   __shared__ uint32_t s_elig[kTab][KWP];
-  __shared__ WarpQueue s_q[8];
+  __shared__ TargetQueue s_q[8];
   extern __shared__ __align__(16) uint8_t dyn_smem[];
   const int w = threadIdx.x >> 5;
   uint8_t *stage = dyn_smem + w * Stage<KWP>::template bytes<UNIT>();
-  WarpQueue *q = &s_q[w];
+  TargetQueue *q = &s_q[w];
   const int lane = threadIdx.x & 31;
   const int warps = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * warps * 32;
@@ -597,41 +647,16 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_rbcand_light(CandArg
     const GroupRaw nxt = fetch_group(a, base + stride + lane, false);
     const int64_t v = base + lane;
     const int s = cur.s;
-    bool act = false;
-    int32_t c = 0;
-    int64_t j0 = 0;
-    int deg = 0;
-    if (v < a.n && !cur.hv && (unsigned)s < (unsigned)a.k && s_over[s]) {
-      ++w_over;
-      c = a.vwgt[v];
-      j0 = a.vptr[v];  // loaded together
-      deg = (int)(a.vptr[v + 1] - j0);
-      if (2ll * c <= 3ll * (s_bw[s] - a.A)) {  // heavy vertices (Section 4.3) are never moved
-        uint32_t nz = 0;
-        if (c <= kTab) {
-#pragma unroll
-          for (int qq = 0; qq < KWP; ++qq) nz |= s_elig[c - 1][qq];
-        } else {
-          uint32_t C[KWP];
-          eligible_words<KWP>(s_cap, a.k, c, C);
-#pragma unroll
-          for (int qq = 0; qq < KWP; ++qq) nz |= C[qq];
-        }
-        if (nz) {
-          act = true;
-          ++w_eval;
-          w_pins += deg;
-        }
-      }
-    }
-    qn = enqueue(q, qn, act, (int)v, s, c, j0, deg);
+    const bool act = v < a.n && !cur.hv && (unsigned)s < (unsigned)a.k && s_over[s];
+    w_over += act;
+    qn = enqueue(q, qn, act, (int)v, s);
     if (qn >= 32) {
-      rb_batch<KWP, UNIT, kTab>(a, stage, q, 32, s_cap, s_base, s_elig);
+      rb_batch<KWP, UNIT, kTab>(a, stage, q, 32, s_cap, s_bw, s_base, s_elig, w_eval, w_pins);
       qn = dequeue32(q, qn);
     }
     cur = nxt;
   }
-  if (qn > 0) rb_batch<KWP, UNIT, kTab>(a, stage, q, qn, s_cap, s_base, s_elig);
+  if (qn > 0) rb_batch<KWP, UNIT, kTab>(a, stage, q, qn, s_cap, s_bw, s_base, s_elig, w_eval, w_pins);
   count_work(a.cnt, w_over, w_eval, w_pins);
 }
 
