@@ -17,7 +17,7 @@
 //
 //   k_cl_serial   the leading one-vertex sub-rounds, one block, in order
 //   k_cl_rate     the rating of vertices with few rated pins, a warp each;
-//   k_cl_rate_block  of those with more, a thread block each (two sizes): the
+//   k_cl_rate_block  of those with more, a thread block each (three sizes): the
 //                 (edge, pin) pairs are spread evenly over the threads, a
 //                 hash set of (edge, cluster) pairs counts a cluster once per
 //                 edge and a hash table of clusters sums, both in shared memory
@@ -43,10 +43,12 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kTile = 2048;        // scan / radix tile: 256 threads x 8 items
-// Classes of vertices by table size (entries, at least twice the rated pins): a warp, a small and a large block,
-// the pool.
-constexpr int kWarpTab = 128, kMidTab = 2048, kBlockTab = 8192;
-constexpr int kMidThreads = 256, kBigThreads = 512;
+// Classes of vertices by table size (entries, at least twice the rated pins): a warp, a block of three sizes, the
+// pool.  The blocks' shared memory is their table, so most of a sub-round's vertices are resident at once (with one
+// class for 65 to 1,024 rated pins, 43 KB each, that class took 45 us on 5,000 VLSI vertices: several waves).
+constexpr int kWarpTab = 128, kSmallTab = 512, kMidTab = 2048, kBlockTab = 8192;
+constexpr int kSmallThreads = 128, kMidThreads = 256, kBigThreads = 512;
+constexpr int kLists = 4;  // classes with a list of positions: the blocks and the pool
 constexpr int kSettleSize = 16384;  // sub-rounds up to this size are settled by one cluster
 constexpr int kSettleBlocks = 8, kSettleThreads = 1024;
 constexpr int kHeavyWarps = 16;    // warps of a block that rates one vertex with a table in the pool
@@ -347,32 +349,47 @@ __device__ __forceinline__ int round_of(const int32_t *bounds, int32_t rounds, i
   return lo;
 }
 
-// Class of a vertex by its table: 0 a warp, 1 a small block, 2 a large block, 3 the pool.
+// Class of a vertex by its table: 0 a warp, 1..3 a block, 4 the pool.
 __device__ __forceinline__ int rate_class(int32_t cap) {
-  return cap <= kWarpTab ? 0 : cap <= kMidTab ? 1 : cap <= kBlockTab ? 2 : 3;
+  return cap <= kWarpTab ? 0 : cap <= kSmallTab ? 1 : cap <= kMidTab ? 2 : cap <= kBlockTab ? 3 : 4;
 }
 
-// Per sub-round: vertices of classes 1..3 (counts[(class - 1) * rounds + r]) and the pool entries of class 3.
+// The list of position x (class - 1, sub-round), -1 for class 0.
+__device__ __forceinline__ int list_of(int32_t cap, const int32_t *bounds, int32_t rounds, int64_t x) {
+  const int cl = rate_class(cap);
+  return cl == 0 ? -1 : (cl - 1) * rounds + round_of(bounds, rounds, x);
+}
+
+// Per list: its length (counts), and per sub-round the pool entries of its class-4 vertices.  Neighbouring positions
+// share their lists: one atomic per warp and list.
 __global__ void k_cl_need(const int32_t *order, int32_t n, const int32_t *bounds, int32_t rounds, const int32_t *cap,
                           unsigned long long *need, unsigned long long *counts) {
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t c = cap[order[x]];
-    const int cl = rate_class(c);
-    if (cl == 0) continue;
-    const int r = round_of(bounds, rounds, x);
-    atomicAdd(&counts[(int64_t)(cl - 1) * rounds + r], 1ull);
-    if (cl == 3) atomicAdd(&need[r], (unsigned long long)c);
+  const int lane = threadIdx.x & 31;
+  for (int64_t x0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); x0 < n;
+       x0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t x = x0 + lane;
+    const int32_t c = x < n ? cap[order[x]] : 0;
+    const int l = list_of(c, bounds, rounds, x);
+    const unsigned peers = __match_any_sync(kFull, l);
+    if (l >= 0 && lane == __ffs(peers) - 1) atomicAdd(&counts[l], (unsigned long long)__popc(peers));
+    if (l >= 3 * rounds) atomicAdd(&need[l - 3 * rounds], (unsigned long long)c);
   }
 }
 
-// The positions of classes 1..3 of every sub-round, at off[(class - 1) * rounds + r] onwards (any order within).
+// The positions of every list, at off[list] onwards (any order within).
 __global__ void k_cl_class_list(const int32_t *order, int32_t n, const int32_t *bounds, int32_t rounds,
                                 const int32_t *cap, const int64_t *off, unsigned long long *cur, int32_t *pos) {
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-    const int cl = rate_class(cap[order[x]]);
-    if (cl == 0) continue;
-    const int64_t i = (int64_t)(cl - 1) * rounds + round_of(bounds, rounds, x);
-    pos[off[i] + (int64_t)atomicAdd(&cur[i], 1ull)] = (int32_t)x;
+  const int lane = threadIdx.x & 31;
+  for (int64_t x0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); x0 < n;
+       x0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t x = x0 + lane;
+    const int l = list_of(x < n ? cap[order[x]] : 0, bounds, rounds, x);
+    const unsigned peers = __match_any_sync(kFull, l);
+    const int first = __ffs(peers) - 1;
+    unsigned long long at = 0;
+    if (l >= 0 && lane == first) at = atomicAdd(&cur[l], (unsigned long long)__popc(peers));
+    at = __shfl_sync(kFull, at, first) + __popc(peers & ((1u << lane) - 1));
+    if (l >= 0) pos[off[l] + (int64_t)at] = (int32_t)x;
   }
 }
 
@@ -835,7 +852,7 @@ __global__ void __launch_bounds__(T) k_cl_rate_block(jet_hypergraph g, const int
   if (threadIdx.x == 0 && j >= 0) propose(g, cl, u, j);
 }
 
-// Block per position of class 3.  Dynamic shared memory: kHeavySmem.
+// Block per position of class 4.  Dynamic shared memory: kHeavySmem.
 __global__ void __launch_bounds__(kHeavyWarps * 32) k_cl_rate_pool(jet_hypergraph g, const int32_t *order,
                                                                    const int32_t *pos, long long cmax, int32_t rmax,
                                                                    Cl cl, Tab *pool, unsigned long long *ctr) {
@@ -1163,28 +1180,28 @@ struct Scratch {
   }
 };
 
-// Two streams beside a call's own, for launches that may overlap with its next one.
+// Three streams beside a call's own, for launches that may overlap with its next one.
 struct Side {
-  cudaStream_t main, s[2] = {nullptr, nullptr};
-  cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+  static constexpr int N = 3;
+  cudaStream_t main, s[N] = {nullptr, nullptr, nullptr};
+  cudaEvent_t ev[N + 1] = {nullptr, nullptr, nullptr, nullptr};
   explicit Side(cudaStream_t m) : main(m) {}
   cudaError_t open() {
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking);
-    for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+    for (int i = 0; i < N && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking);
+    for (int i = 0; i <= N && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
     return e;
   }
   // what follows on the used side streams comes after everything on the main stream so far
-  cudaError_t fork(bool use0, bool use1) {
-    cudaError_t e = cudaEventRecord(ev[2], main);
-    if (e == cudaSuccess && use0) e = cudaStreamWaitEvent(s[0], ev[2], 0);
-    if (e == cudaSuccess && use1) e = cudaStreamWaitEvent(s[1], ev[2], 0);
+  cudaError_t fork(const bool (&use)[N]) {
+    cudaError_t e = cudaEventRecord(ev[N], main);
+    for (int i = 0; i < N && e == cudaSuccess; ++i)
+      if (use[i]) e = cudaStreamWaitEvent(s[i], ev[N], 0);
     return e;
   }
-  cudaError_t join(bool use0, bool use1) {
-    const bool use[2] = {use0, use1};
+  cudaError_t join(const bool (&use)[N]) {
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+    for (int i = 0; i < N && e == cudaSuccess; ++i) {
       if (!use[i]) continue;
       e = cudaEventRecord(ev[i], s[i]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(main, ev[i], 0);
@@ -1193,12 +1210,12 @@ struct Side {
   }
   // waits for its own work first: after an error a launch on a side stream may not have been joined
   ~Side() {
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < N; ++i)
       if (s[i]) {
         cudaStreamSynchronize(s[i]);
         cudaStreamDestroy(s[i]);
       }
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i <= N; ++i)
       if (ev[i]) cudaEventDestroy(ev[i]);
   }
 };
@@ -1287,14 +1304,14 @@ int jet_cluster(const jet_hypergraph *hg, const jet_coarsen_params *p, const int
   const std::vector<int32_t> bounds = subround_bounds(n, p->single_subrounds, p->subround_cap_div);
   const int32_t rounds = (int32_t)bounds.size() - 1;
   int32_t *d_bounds = sc.get<int32_t>((int64_t)bounds.size());
-  // per sub-round: pool entries, pool cursor; then the sizes and the list cursors of classes 1..3
+  // per sub-round: pool entries, pool cursor; then the sizes and the cursors of the lists
   const int64_t R = rounds;
-  unsigned long long *d_need = sc.get<unsigned long long>(8 * R);
-  int64_t *d_off = sc.get<int64_t>(3 * R);
+  unsigned long long *d_need = sc.get<unsigned long long>((2 + 2 * kLists) * R);
+  int64_t *d_off = sc.get<int64_t>(kLists * R);
   if (sc.err != cudaSuccess) return cuda_error(sc.err, "jet_cluster: workspace");
-  unsigned long long *d_ctr = d_need + R, *d_counts = d_need + 2 * R, *d_cur = d_need + 5 * R;
+  unsigned long long *d_ctr = d_need + R, *d_counts = d_need + 2 * R, *d_cur = d_need + (2 + kLists) * R;
   cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_need, 0, sizeof(unsigned long long) * 8 * (size_t)rounds, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_need, 0, sizeof(unsigned long long) * (2 + 2 * kLists) * (size_t)rounds, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_bounds, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(cl.T, 0, sizeof(int32_t) * (size_t)n, s);  // "seen" of the order check
@@ -1316,12 +1333,12 @@ int jet_cluster(const jet_hypergraph *hg, const jet_coarsen_params *p, const int
   k_cl_setup<<<g, 256, 0, s>>>(*hg, p->rating_max_edge, cl, d_err);
   k_cl_need<<<g, 256, 0, s>>>(order, n, d_bounds, rounds, cl.cap, d_need, d_counts);
   int h_err = 0;
-  std::vector<unsigned long long> need(rounds), counts(3 * R);
+  std::vector<unsigned long long> need(rounds), counts(kLists * R);
   e = cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(need.data(), d_need, sizeof(unsigned long long) * (size_t)rounds, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(counts.data(), d_counts, sizeof(unsigned long long) * 3 * (size_t)rounds,
+    e = cudaMemcpyAsync(counts.data(), d_counts, sizeof(unsigned long long) * kLists * (size_t)rounds,
                         cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_error(e, "jet_cluster: set-up");
@@ -1330,16 +1347,16 @@ int jet_cluster(const jet_hypergraph *hg, const jet_coarsen_params *p, const int
   if (h_err & 8) return gfail(JET_ERR_OVERFLOW, "%s", "a vertex's rated neighbourhood exceeds 2^27 pins");
   unsigned long long pool_entries = 1;
   for (unsigned long long x : need) pool_entries = std::max(pool_entries, x);
-  std::vector<int64_t> off(3 * R);
+  std::vector<int64_t> off(kLists * R);
   int64_t listed = 0;
-  for (int64_t i = 0; i < 3 * R; ++i) {
+  for (int64_t i = 0; i < kLists * R; ++i) {
     off[i] = listed;
     listed += (int64_t)counts[i];
   }
   Tab *pool = sc.get<Tab>((int64_t)pool_entries);
   int32_t *pos = sc.get<int32_t>(listed);
   if (sc.err != cudaSuccess) return cuda_error(sc.err, "jet_cluster: rating tables");
-  e = cudaMemcpyAsync(d_off, off.data(), sizeof(int64_t) * 3 * (size_t)rounds, cudaMemcpyHostToDevice, s);
+  e = cudaMemcpyAsync(d_off, off.data(), sizeof(int64_t) * kLists * (size_t)rounds, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return cuda_error(e, "jet_cluster");
   if (listed > 0) k_cl_class_list<<<g, 256, 0, s>>>(order, n, d_bounds, rounds, cl.cap, d_off, d_cur, pos);
   // leading one-vertex sub-rounds: one block, in order
@@ -1354,19 +1371,29 @@ int jet_cluster(const jet_hypergraph *hg, const jet_coarsen_params *p, const int
   if (r < rounds && listed > 0 && (e = side.open()) != cudaSuccess) return cuda_error(e, "jet_cluster: streams");
   for (; r < rounds && e == cudaSuccess; ++r) {
     const int32_t a = bounds[r], b = bounds[r + 1];
-    const unsigned n1 = (unsigned)counts[r], n2 = (unsigned)counts[R + r], n3 = (unsigned)counts[2 * R + r];
-    if (n1 || n2 || n3) e = side.fork(n1 > 0, n2 || n3);
-    if (n3 > 0)
-      k_cl_rate_pool<<<n3, kHeavyWarps * 32, kHeavySmem, side.s[1]>>>(*hg, order, pos + off[2 * R + r], cmax, rmax, cl,
-                                                                      pool, d_ctr + r);
-    if (n2 > 0)
-      k_cl_rate_block<kBigThreads><<<n2, kBigThreads, rate_smem(kBlockTab, kBigThreads), side.s[1]>>>(
-          *hg, order, pos + off[R + r], cmax, rmax, cl);
-    if (n1 > 0)
-      k_cl_rate_block<kMidThreads><<<n1, kMidThreads, rate_smem(kMidTab, kMidThreads), side.s[0]>>>(
-          *hg, order, pos + off[r], cmax, rmax, cl);
+    unsigned len[kLists];
+    const int32_t *list[kLists];
+    for (int i = 0; i < kLists; ++i) {
+      len[i] = (unsigned)counts[i * R + r];
+      list[i] = pos + off[i * R + r];
+    }
+    // the largest tables on one side stream, the two smaller blocks' classes on one each
+    const bool use[3] = {len[0] > 0, len[1] > 0, len[2] > 0 || len[3] > 0};
+    if (use[0] || use[1] || use[2]) e = side.fork(use);
+    if (len[3] > 0)
+      k_cl_rate_pool<<<len[3], kHeavyWarps * 32, kHeavySmem, side.s[2]>>>(*hg, order, list[3], cmax, rmax, cl, pool,
+                                                                          d_ctr + r);
+    if (len[2] > 0)
+      k_cl_rate_block<kBigThreads><<<len[2], kBigThreads, rate_smem(kBlockTab, kBigThreads), side.s[2]>>>(
+          *hg, order, list[2], cmax, rmax, cl);
+    if (len[1] > 0)
+      k_cl_rate_block<kMidThreads><<<len[1], kMidThreads, rate_smem(kMidTab, kMidThreads), side.s[1]>>>(
+          *hg, order, list[1], cmax, rmax, cl);
+    if (len[0] > 0)
+      k_cl_rate_block<kSmallThreads><<<len[0], kSmallThreads, rate_smem(kSmallTab, kSmallThreads), side.s[0]>>>(
+          *hg, order, list[0], cmax, rmax, cl);
     k_cl_rate<<<(unsigned)((b - a + 7) / 8), 256, 0, s>>>(*hg, order, a, b, cmax, rmax, cl);
-    if (e == cudaSuccess && (n1 || n2 || n3)) e = side.join(n1 > 0, n2 || n3);
+    if (e == cudaSuccess && (use[0] || use[1] || use[2])) e = side.join(use);
     if (b - a <= kSettleSize) {
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3(kSettleBlocks);

@@ -1,8 +1,8 @@
 """Clustering on the GPU vs the oracle at the edges of the rating classes.
 
-A vertex is rated by a warp (up to 64 rated pins), a small block (1,024), a
-large block (4,096) or with its table in the pool; its edges go through the
-kernels 32, 256 or 512 at a time.  The instance has vertices on both sides of
+A vertex is rated by a warp (up to 64 rated pins), a block of three sizes (256,
+1,024, 4,096) or with its table in the pool; its edges go through the kernels
+32, 128, 256 or 512 at a time.  The instance has vertices on both sides of
 each of these bounds, made of two-pin edges and of edges of up to 1,000 pins.
 """
 import numpy as np
@@ -20,7 +20,7 @@ if not torch.cuda.is_available():
 from paper_2504_12013_gb300 import jet  # noqa: E402
 
 # two-pin edges and edges of the given sizes of one vertex: rated pins = two + sum(size - 1)
-SHAPES = [(31, ()), (32, ()), (33, ()), (64, ()), (65, ()), (25, (40,)), (26, (40,)), (255, (770,)), (257, (768,)),
+SHAPES = [(127, ()), (129, ()), (256, ()), (257, ()), (31, ()), (32, ()), (33, ()), (64, ()), (65, ()), (25, (40,)), (26, (40,)), (255, (770,)), (257, (768,)),
           (1024, ()), (1025, ()), (25, (1000,)), (26, (1000,)), (513, (1000, 1000, 1000, 587)),
           (513, (1000, 1000, 1000, 588)), (4096, ()), (4097, ()), (600, (1000,) * 5), (3, (1001, 1500))]
 
