@@ -236,8 +236,8 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     if ((e = launch_afterburner(c, part, phi)) != cudaSuccess) return e;
     if ((e = launch_approve(c, part, locked, nullptr, nullptr, true, bw, rs)) != cudaSuccess) return e;
     {
-      // segmented records: the block weights are known before the apply, and the check runs beside it
-      Fork fork(c, c->rb_segments ? 2 : 1);
+      // rb_early: the block weights are known before the apply, and the check runs beside it
+      Fork fork(c, c->rb_early ? 2 : 1);
       if ((e = launch_apply_jet(c, part, phi, bw)) != cudaSuccess) return e;
       c->stream = fork.stream(1);
       e = launch_rb_check(c, bw, h, 1);
@@ -266,7 +266,7 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     cudaError_t eb = launch_rebalance_candidates(c, part, phi);
     if (eb == cudaSuccess) eb = launch_rb_select(c, part, bw);
     {
-      Fork fork(c, c->rb_segments ? 2 : 1);  // as above: the end of the round beside its apply
+      Fork fork(c, c->rb_early ? 2 : 1);  // as above: the end of the round beside its apply
       if (eb == cudaSuccess) eb = launch_rb_apply(c, part, phi, bw);
       c->stream = fork.stream(1);
       if (eb == cudaSuccess) eb = launch_rb_post(c, bw, h, 1);

@@ -108,6 +108,11 @@ struct __align__(16) RbRec {
 // Up to this many vertices per block on average, the records of a block are kept in a segment of their own and
 // selected by one thread block (k_rb_select, where the line is explained).
 constexpr int kSegVertices = 4096;
+// Up to this many vertices (and with segments) the block weights are kept by the approval and the selection, not by
+// the apply kernels, so that the balance checks run beside those: it takes a link out of a chain of short kernels
+// (refine 100k weighted 36.6 -> 34.7 ms).  With more vertices the extra atomics cost more than the link (four
+// iterations of 300k vertices at k = 200: 2.12 -> 2.24 ms).
+constexpr int kEarlyVertices = 1 << 17;
 constexpr int kCurStride = 32;  // ints between the blocks' record cursors (a line each)
 
 }  // namespace jet
@@ -168,6 +173,7 @@ struct jet_ctx {
   jet::Counters *cnt_host = nullptr;  // pinned mirror
   jet::RbBlock *rbb = nullptr;
   int rb_segments = 0;                // records in a segment per block
+  int rb_early = 0;                   // and the block weights kept by the kernels that make the move lists
   jet::RbRec *rb_rec = nullptr;       // segmented records; else the same memory holds the three arrays below
   int32_t *rb_cur = nullptr;          // segmented: records of each block (kCurStride ints apart)
   uint64_t *rb_hi = nullptr;          // per record: priority part of the rebalancing key
@@ -310,7 +316,7 @@ cudaError_t prepare_afterburner_kernels(jet_ctx *c);  // ab_bps
 cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi);
 // part (with build_moves): the partition, whose blocks' vertices are counted where records are segmented.  rs (may be NULL): if the last
 // iteration improved (rs->snap), the partition is also copied to c->best_part.  block_w (with build_moves): where
-// records are segmented, the moves' weights are added here and not by launch_apply_jet.
+// rb_early, the moves' weights are added here and not by launch_apply_jet.
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
                            bool build_moves, int64_t *block_w = nullptr, const RefineState *rs = nullptr);
 cudaError_t launch_export_candidates(jet_ctx *c, int32_t *target, int32_t *gain, uint8_t *in_m);
@@ -321,7 +327,7 @@ cudaError_t launch_apply_jet(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *b
 cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part);  // cnt->vcount (zeroed by reset_counters)
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                             int use_cond = 0);
-// the selection of a round (where records are segmented, block_w takes its weights here and not in launch_rb_apply)
+// the selection of a round (with rb_early, block_w takes its weights here and not in launch_rb_apply)
 cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w);
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // applies the selection
 cudaError_t launch_rb_post(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,

@@ -504,9 +504,8 @@ struct ApArgs {
   const int32_t *part;  // with build_moves
   const RefineState *rs;  // may be NULL
   int32_t *best;
-  // segmented rebalancing records: the vertices of each block after the moves, and the block weights, are kept here,
-  // so that the balance check need not wait for the apply
-  int count;
+  int count;  // segmented rebalancing records: count the vertices of each block
+  // rb_early (else NULL): the count is of the blocks after the moves, and the block weights are kept here
   const int32_t *vwgt;
   int64_t *bw;
   const uint64_t *cand;
@@ -528,7 +527,7 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   __shared__ unsigned s_wc[kWarps];
   __shared__ unsigned long long s_base;
   __shared__ unsigned long long s_cand[kWarps];
-  __shared__ int s_vc[kMaxK];  // vertices per block after the moves
+  __shared__ int s_vc[kMaxK];  // vertices per block
   __shared__ long long s_dw[kMaxK];
   if (a.count)
     for (int b = threadIdx.x; b < a.k; b += blockDim.x) {
@@ -545,6 +544,8 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     const bool valid = v < a.n;
     const uint64_t r = valid ? a.cand[v] : 0;
     const int32_t g = valid ? a.rg[v] : 0;
+    const bool blocks = valid && (a.count || snap);
+    const int b = blocks ? a.part[v] : 0, c = blocks && a.bw ? a.vwgt[v] : 0;  // beside the loads above
     const bool in = r != 0;
     const bool ap = in && g > 0;
     if (valid) {
@@ -555,15 +556,13 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
     }
     ncand += __popc(__ballot_sync(kFull, in));
     if (a.build_moves) {
-      if (valid && (a.count || snap)) {
-        const int b = a.part[v];
+      if (blocks) {
         if (a.count) {
-          const int c = a.vwgt[v];
-          if (ap) {
+          if (a.bw && ap) {
             atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_s(r)]), (unsigned long long)(-(long long)c));
             atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_t(r)]), (unsigned long long)c);
           }
-          const int to = ap ? cand_t(r) : b;
+          const int to = a.bw && ap ? cand_t(r) : b;
           if ((unsigned)to < (unsigned)a.k) atomicAdd(&s_vc[to], 1);
         }
         if (snap) a.best[v] = b;
@@ -852,7 +851,7 @@ cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int
   a.best = c->best_part;
   a.count = build_moves && c->rb_segments;
   a.vwgt = c->vwgt;
-  a.bw = block_w;
+  a.bw = c->rb_early ? block_w : nullptr;
   a.n = c->n;
   a.k = c->k;
   a.part = part;
@@ -865,7 +864,8 @@ cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int
   a.mv_v = c->mv_v;
   a.mv_st = c->mv_st;
   a.cnt = c->cnt;
-  k_approve<<<grid_for(c->n, 256, c->launch_sms), 256, 0, c->stream>>>(a);
+  // every block adds its counts and weights of up to k blocks to the same few lines: fewer blocks then
+  k_approve<<<grid_for(c->n, 256, c->launch_sms, a.count ? 4 : 8), 256, 0, c->stream>>>(a);
   ++c->kernel_launches;
   return cudaGetLastError();
 }

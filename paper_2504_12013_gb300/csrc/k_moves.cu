@@ -563,8 +563,10 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw
           const int to = r[q].ct & 255;
           a.mv_v[x] = r[q].v;
           a.mv_st[x] = (uint32_t)b | ((uint32_t)to << 16);
-          atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[to]), (unsigned long long)(r[q].ct >> 16));
-          atomicAdd(&s_dc[to], 1);
+          if (bw) {
+            atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[to]), (unsigned long long)(r[q].ct >> 16));
+            atomicAdd(&s_dc[to], 1);
+          }
         }
         at += __popc(bal[q]);
       }
@@ -578,6 +580,7 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw
     for (int q = 0; q < 4; ++q) r[q] = i + q * kSelThreads < cnt ? Rec(rec[i + q * kSelThreads]) : Rec();
     emit(r, 4);
   }
+  if (!bw) return;
   __syncthreads();
   // the block weights already, so that the end of the round need not wait for the apply
   if (t < kMaxK) {
@@ -762,6 +765,7 @@ RbArgs rb_args(jet_ctx *c, const int64_t *block_w, const int32_t *part) {
 
 cudaError_t prepare_move_kernels(jet_ctx *c) {
   c->rb_segments = c->n / c->k <= kSegVertices ? 1 : 0;
+  c->rb_early = c->rb_segments && c->n <= kEarlyVertices ? 1 : 0;
   cudaError_t e = resident_blocks(k_apply, 256, 0, &c->move_bps[0]);
   if (e == cudaSuccess) e = resident_blocks(k_rb_apply<unsigned long long>, 256, 0, &c->move_bps[1]);
   if (e == cudaSuccess) e = resident_blocks(k_rb_apply<u128>, 256, 0, &c->move_bps[2]);
@@ -793,12 +797,12 @@ cudaError_t launch_apply_jet(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *b
   if (c->n == 0) return cudaSuccess;
   if (c->graph_path || phi_bytes < 256e6) {
     MoveArgs a = move_args(c, part, phi, block_w);
-    a.weights = !c->rb_segments;  // launch_approve has done it
+    a.weights = !c->rb_early;  // else launch_approve has done it
     return c->graph_path ? apply_part(c, a) : apply_phi(c, a);
   }
   const double bytes = phi_bytes + 8.0 * c->m * c->kwp + 8.0 * c->m + 8.0 * c->P;
   MoveArgs a = move_args(c, part, phi, block_w);
-  a.weights = !c->rb_segments;
+  a.weights = !c->rb_early;
   a.rebuild_min = (unsigned long long)(bytes / (4.2e3 * 0.075) * c->n / std::max<int64_t>(c->P, 1)) + 1;
   cudaError_t e = apply_phi(c, a);
   if (e == cudaSuccess) e = apply_part(c, a);
@@ -852,8 +856,10 @@ cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
 cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w) {
   if (c->n == 0) return cudaSuccess;
   const RbArgs a = rb_args(c, nullptr, part);
-  if (c->rb_segments)
-    return a.tbits <= 64 ? select_segments<unsigned long long>(c, a, block_w) : select_segments<u128>(c, a, block_w);
+  if (c->rb_segments) {
+    int64_t *bw = c->rb_early ? block_w : nullptr;
+    return a.tbits <= 64 ? select_segments<unsigned long long>(c, a, bw) : select_segments<u128>(c, a, bw);
+  }
   if (a.tbits <= 64) rb_select_levels<unsigned long long>(c, a);
   else rb_select_levels<u128>(c, a);
   return cudaGetLastError();
@@ -861,9 +867,9 @@ cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w) 
 
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   if (c->n == 0) return cudaSuccess;
-  if (c->rb_segments) {  // the selection is a move list, its weights are in place
+  if (c->rb_segments) {  // the selection is a move list
     MoveArgs a = move_args(c, part, phi, block_w);
-    a.weights = 0;
+    a.weights = !c->rb_early;
     return c->graph_path ? apply_part(c, a) : apply_phi(c, a);
   }
   const RbArgs r = rb_args(c, block_w, part);
