@@ -521,7 +521,13 @@ struct ApArgs {
 
 // Counters and move-list slots are aggregated per thread block (one atomic
 // per block and iteration) rather than per warp, which would serialize on
-// the few counter addresses.
+// the few counter addresses.  R vertices per thread and step: their loads
+// overlap and share the append's barriers.  Bound by those loads: with R = 4
+// eight iterations of 2 M VLSI vertices took 7.89 against 7.98 ms, of a graph
+// of 4 M vertices 8.53 against 8.70; small calls (launch_approve) lose to the
+// longer chain of a step and to blocks left idle: refine of 10k vertices 7.67
+// against 7.52 ms.
+template <int R>
 __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   constexpr int kWarps = 256 / 32;
   __shared__ unsigned s_wc[kWarps];
@@ -539,36 +545,48 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   // the snapshot of an improved partition, taken here, before the next moves, and not by a launch of its own
   const bool snap = a.rs && a.rs->snap;
   unsigned long long ncand = 0;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = base + threadIdx.x;
-    const bool valid = v < a.n;
-    const uint64_t r = valid ? a.cand[v] : 0;
-    const int32_t g = valid ? a.rg[v] : 0;
-    const bool blocks = valid && (a.count || snap);
-    const int b = blocks ? a.part[v] : 0, c = blocks && a.bw ? a.vwgt[v] : 0;  // beside the loads above
-    const bool in = r != 0;
-    const bool ap = in && g > 0;
-    if (valid) {
-      a.rg[v] = 0;
-      if (a.locked) a.locked[v] = ap ? 1 : 0;
-      if (a.rg_out) a.rg_out[v] = g;
-      if (a.approved_out) a.approved_out[v] = ap ? 1 : 0;
+  for (int64_t base = (int64_t)blockIdx.x * R * 256; base < a.n; base += (int64_t)gridDim.x * R * 256) {
+    uint64_t r[R];
+    int32_t g[R];
+    int b[R], c[R];
+    bool ap[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int64_t v = base + q * 256 + threadIdx.x;
+      const bool valid = v < a.n, blocks = valid && (a.count || snap);
+      r[q] = valid ? a.cand[v] : 0;
+      g[q] = valid ? a.rg[v] : 0;
+      b[q] = blocks ? a.part[v] : -1;
+      c[q] = blocks && a.bw ? a.vwgt[v] : 0;
     }
-    ncand += __popc(__ballot_sync(kFull, in));
-    if (a.build_moves) {
-      if (blocks) {
-        if (a.count) {
-          if (a.bw && ap) {
-            atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_s(r)]), (unsigned long long)(-(long long)c));
-            atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_t(r)]), (unsigned long long)c);
+    unsigned mine = 0;  // approved vertices of the warp
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int64_t v = base + q * 256 + threadIdx.x;
+      ap[q] = r[q] != 0 && g[q] > 0;
+      if (v < a.n) {
+        if (g[q]) a.rg[v] = 0;
+        if (a.locked) a.locked[v] = ap[q] ? 1 : 0;
+        if (a.rg_out) a.rg_out[v] = g[q];
+        if (a.approved_out) a.approved_out[v] = ap[q] ? 1 : 0;
+        if (a.build_moves) {
+          if (a.count) {
+            if (a.bw && ap[q]) {
+              atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_s(r[q])]),
+                        (unsigned long long)(-(long long)c[q]));
+              atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[cand_t(r[q])]), (unsigned long long)c[q]);
+            }
+            const int to = a.bw && ap[q] ? cand_t(r[q]) : b[q];
+            if ((unsigned)to < (unsigned)a.k) atomicAdd(&s_vc[to], 1);
           }
-          const int to = a.bw && ap ? cand_t(r) : b;
-          if ((unsigned)to < (unsigned)a.k) atomicAdd(&s_vc[to], 1);
+          if (snap) a.best[v] = b[q];
         }
-        if (snap) a.best[v] = b;
       }
-      const unsigned bap = __ballot_sync(kFull, ap);
-      if (lane == 0) s_wc[wid] = __popc(bap);
+      ncand += __popc(__ballot_sync(kFull, r[q] != 0));
+      mine += __popc(__ballot_sync(kFull, ap[q]));
+    }
+    if (a.build_moves) {
+      if (lane == 0) s_wc[wid] = mine;
       __syncthreads();
       if (threadIdx.x == 0) {
         unsigned tot = 0;
@@ -581,10 +599,16 @@ __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
         if (tot) atomicAdd(&a.cnt->approved, (unsigned long long)tot);
       }
       __syncthreads();
-      if (ap) {
-        const unsigned long long pos = s_base + s_wc[wid] + __popc(bap & ((1u << lane) - 1));
-        a.mv_v[pos] = (int32_t)v;
-        a.mv_st[pos] = (uint32_t)cand_s(r) | ((uint32_t)cand_t(r) << 16);
+      unsigned long long pos = s_base + s_wc[wid];
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const unsigned bap = __ballot_sync(kFull, ap[q]);
+        if (ap[q]) {
+          const unsigned long long at = pos + __popc(bap & ((1u << lane) - 1));
+          a.mv_v[at] = (int32_t)(base + q * 256 + threadIdx.x);
+          a.mv_st[at] = (uint32_t)cand_s(r[q]) | ((uint32_t)cand_t(r[q]) << 16);
+        }
+        pos += __popc(bap);
       }
       __syncthreads();
     }
@@ -865,7 +889,10 @@ cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int
   a.mv_st = c->mv_st;
   a.cnt = c->cnt;
   // every block adds its counts and weights of up to k blocks to the same few lines: fewer blocks then
-  k_approve<<<grid_for(c->n, 256, c->launch_sms, a.count ? 4 : 8), 256, 0, c->stream>>>(a);
+  if (c->n <= kEarlyVertices)  // 100k vertices: refine in 35.9 against 36.0 ms; 300k: R = 4 by 0.8 % of a round
+    k_approve<1><<<grid_for(c->n, 256, c->launch_sms, a.count ? 4 : 8), 256, 0, c->stream>>>(a);
+  else
+    k_approve<4><<<grid_for(c->n, 1024, c->launch_sms, a.count ? 2 : 8), 256, 0, c->stream>>>(a);
   ++c->kernel_launches;
   return cudaGetLastError();
 }
