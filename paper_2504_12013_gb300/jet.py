@@ -178,6 +178,31 @@ def _ptr(t, dtype=None, name="tensor"):
     return t.data_ptr()
 
 
+def _need(t, count, name):
+    """The C entry points take pointers and trust the lengths: an array shorter than the call reads or writes is
+    refused here, before any launch (None is left to the C entry, which reports a NULL argument)."""
+    if t is not None and t.numel() < count:
+        raise ValueError(f"{name} has {t.numel()} entries, the call needs at least {count}")
+
+
+def _need_state(ctx, part, phi, block_w, phi_used=True):
+    """part, phi and block_w of a context; phi_used: the call touches phi."""
+    _need(part, ctx.hg.n, "part")
+    if phi_used:
+        _need(phi, ctx.hg.m * ctx.k, "phi")
+    _need(block_w, ctx.k, "block_w")
+
+
+def _host_hg(hg):
+    """The arrays of a host hypergraph, contiguous and long enough, and the C struct that points at them."""
+    arrs = [np.ascontiguousarray(a) for a in (hg.eptr, hg.pins, hg.vptr, hg.inc, hg.vwgt, hg.ewgt)]
+    for name, a, size in zip(("eptr", "pins", "vptr", "inc", "vwgt", "ewgt"), arrs,
+                             (8 * (hg.m + 1), 4 * hg.P, 8 * (hg.n + 1), 4 * hg.P, 4 * hg.n, 4 * hg.m)):
+        if a.nbytes < size:
+            raise ValueError(f"{name} has {a.nbytes} bytes, the call needs at least {size}")
+    return arrs, JetHypergraph(hg.n, hg.m, hg.P, *[a.ctypes.data for a in arrs])
+
+
 def _check(rc, ctx=None):
     if rc != JET_OK:
         raise JetError(rc, jet_last_error(ctx))
@@ -219,6 +244,10 @@ class DeviceHypergraph:
 
     def c(self) -> JetHypergraph:
         import torch
+        for t, count, name in ((self.eptr, self.m + 1, "eptr"), (self.pins, self.P, "pins"),
+                               (self.vptr, self.n + 1, "vptr"), (self.inc, self.P, "inc"),
+                               (self.vwgt, self.n, "vwgt"), (self.ewgt, self.m, "ewgt")):
+            _need(t, count, name)
         return JetHypergraph(self.n, self.m, self.P, _ptr(self.eptr, torch.int64), _ptr(self.pins, torch.int32),
                              _ptr(self.vptr, torch.int64), _ptr(self.inc, torch.int32),
                              _ptr(self.vwgt, torch.int32), _ptr(self.ewgt, torch.int32))
@@ -233,6 +262,7 @@ def jet_cluster(dh, cmax, order, rmax=RATING_MAX_EDGE, n_single=SINGLE_SUBROUNDS
                 stream=None):
     """One level of synchronous clustering (Section 6, Algorithm 4): the label tensor (int32, n)."""
     import torch
+    _need(order, dh.n, "order")
     label = torch.empty(max(dh.n, 1), dtype=torch.int32, device=dh.eptr.device)
     prm = JetCoarsenParams(int(cmax), int(rmax), int(n_single), int(cap_div))
     _check(load_library().jet_cluster(ctypes.byref(dh.c()), ctypes.byref(prm), _ptr(order, torch.int32, "order"),
@@ -243,6 +273,7 @@ def jet_cluster(dh, cmax, order, rmax=RATING_MAX_EDGE, n_single=SINGLE_SUBROUNDS
 def jet_contract(dh, label, stream=None):
     """Contraction of the label classes: (coarse DeviceHypergraph, map tensor)."""
     import torch
+    _need(label, dh.n, "label")
     dev = dh.eptr.device
     e = lambda n, dt: torch.empty(max(n, 1), dtype=dt, device=dev)
     eptr, pins, vptr, inc = e(dh.m + 1, torch.int64), e(dh.P, torch.int32), e(dh.n + 1, torch.int64), e(dh.P, torch.int32)
@@ -274,6 +305,7 @@ class Ctx:
         self.handle = handle
         self.hg = hg
         self.params = params_
+        self.graph_path = False
 
     @property
     def k(self):
@@ -313,6 +345,7 @@ def jet_ctx_destroy(ctx: Ctx):
 
 def jet_build_pincounts(ctx: Ctx, part, phi, block_w):
     import torch
+    _need_state(ctx, part, phi, block_w)
     _check(load_library().jet_build_pincounts(ctx.handle, _ptr(part, torch.int32, "part"),
                                               _ptr(phi, torch.int32, "phi"), _ptr(block_w, torch.int64, "block_w")),
            ctx)
@@ -320,12 +353,17 @@ def jet_build_pincounts(ctx: Ctx, part, phi, block_w):
 
 def jet_connectivity(ctx: Ctx, phi, objective_out):
     import torch
+    _need(phi, ctx.hg.m * ctx.k, "phi")
+    _need(objective_out, 1, "objective_out")
     _check(load_library().jet_connectivity(ctx.handle, _ptr(phi, torch.int32, "phi"),
                                            _ptr(objective_out, torch.int64, "objective_out")), ctx)
 
 
 def jet_refine_round(ctx: Ctx, tau, part, phi, block_w, locked, stats=None):
     import torch
+    _need_state(ctx, part, phi, block_w, not ctx.graph_path)
+    _need(locked, ctx.hg.n, "locked")
+    _need(stats, len(STATS_FIELDS), "stats")
     _check(load_library().jet_refine_round(ctx.handle, int(tau[0]), int(tau[1]), _ptr(part, torch.int32, "part"),
                                            _ptr(phi, torch.int32, "phi"), _ptr(block_w, torch.int64, "block_w"),
                                            _ptr(locked, torch.uint8, "locked"), _ptr(stats, torch.int64, "stats")),
@@ -334,6 +372,8 @@ def jet_refine_round(ctx: Ctx, tau, part, phi, block_w, locked, stats=None):
 
 def jet_rebalance(ctx: Ctx, part, phi, block_w, stats=None):
     import torch
+    _need_state(ctx, part, phi, block_w, not ctx.graph_path)
+    _need(stats, len(STATS_FIELDS), "stats")
     _check(load_library().jet_rebalance(ctx.handle, _ptr(part, torch.int32, "part"), _ptr(phi, torch.int32, "phi"),
                                         _ptr(block_w, torch.int64, "block_w"), _ptr(stats, torch.int64, "stats")),
            ctx)
@@ -341,6 +381,7 @@ def jet_rebalance(ctx: Ctx, part, phi, block_w, stats=None):
 
 def jet_refine(ctx: Ctx, schedule, limit, part, phi, block_w) -> dict:
     import torch
+    _need_state(ctx, part, phi, block_w)
     pairs = (ctypes.c_int32 * (2 * len(schedule)))(*[int(x) for t in schedule for x in t])
     res = JetRefineResult()
     _check(load_library().jet_refine(ctx.handle, pairs, len(schedule), int(limit), _ptr(part, torch.int32, "part"),
@@ -351,6 +392,9 @@ def jet_refine(ctx: Ctx, schedule, limit, part, phi, block_w) -> dict:
 
 def jet_candidates(ctx: Ctx, tau, part, phi, locked, target, gain, in_m):
     import torch
+    _need_state(ctx, part, phi, None, not ctx.graph_path)
+    for t, name in ((locked, "locked"), (target, "target"), (gain, "gain"), (in_m, "in_m")):
+        _need(t, ctx.hg.n, name)
     _check(load_library().jet_candidates(ctx.handle, int(tau[0]), int(tau[1]), _ptr(part, torch.int32, "part"),
                                          _ptr(phi, torch.int32, "phi"), _ptr(locked, torch.uint8, "locked"),
                                          _ptr(target, torch.int32, "target"), _ptr(gain, torch.int32, "gain"),
@@ -359,6 +403,9 @@ def jet_candidates(ctx: Ctx, tau, part, phi, locked, target, gain, in_m):
 
 def jet_afterburner(ctx: Ctx, part, phi, rg, approved):
     import torch
+    _need_state(ctx, part, phi, None, not ctx.graph_path)
+    _need(rg, ctx.hg.n, "rg")
+    _need(approved, ctx.hg.n, "approved")
     _check(load_library().jet_afterburner(ctx.handle, _ptr(part, torch.int32, "part"), _ptr(phi, torch.int32, "phi"),
                                           _ptr(rg, torch.int32, "rg"), _ptr(approved, torch.uint8, "approved")), ctx)
 
@@ -366,8 +413,9 @@ def jet_afterburner(ctx: Ctx, part, phi, rg, approved):
 def jet_refine_host(hg, p: JetParams, schedule, limit, part: np.ndarray) -> dict:
     """Host buffers in and out: ``hg`` is a ``synth.Hypergraph`` (numpy), ``part`` int32[n] is refined in place."""
     assert part.dtype == np.int32 and part.flags.c_contiguous
-    arrs = [np.ascontiguousarray(a) for a in (hg.eptr, hg.pins, hg.vptr, hg.inc, hg.vwgt, hg.ewgt)]
-    ch = JetHypergraph(hg.n, hg.m, hg.P, *[a.ctypes.data for a in arrs])
+    if part.size < hg.n:
+        raise ValueError(f"part has {part.size} entries, the call needs at least {hg.n}")
+    arrs, ch = _host_hg(hg)  # arrs: kept alive over the call
     pairs = (ctypes.c_int32 * (2 * len(schedule)))(*[int(x) for t in schedule for x in t])
     res = JetRefineResult()
     rc = load_library().jet_refine_host(ctypes.byref(ch), ctypes.byref(p), pairs, len(schedule), int(limit),
@@ -380,8 +428,9 @@ def jet_rounds_host(hg, p: JetParams, tau, n_rounds, part: np.ndarray) -> dict:
     """Host buffers in and out: n_rounds Jet iterations at temperature tau from ``part`` (int32[n], updated in
     place); returns the last iteration's statistics."""
     assert part.dtype == np.int32 and part.flags.c_contiguous
-    arrs = [np.ascontiguousarray(a) for a in (hg.eptr, hg.pins, hg.vptr, hg.inc, hg.vwgt, hg.ewgt)]
-    ch = JetHypergraph(hg.n, hg.m, hg.P, *[a.ctypes.data for a in arrs])
+    if part.size < hg.n:
+        raise ValueError(f"part has {part.size} entries, the call needs at least {hg.n}")
+    arrs, ch = _host_hg(hg)  # arrs: kept alive over the call
     st = JetRoundStats()
     _check(load_library().jet_rounds_host(ctypes.byref(ch), ctypes.byref(p), int(tau[0]), int(tau[1]),
                                           int(n_rounds), part.ctypes.data, ctypes.byref(st)))
@@ -395,6 +444,7 @@ def jet_set_graph_mode(ctx: Ctx, enable: bool = True):
 def jet_set_graph_path(ctx: Ctx, enable: bool = True):
     """Graph path (every edge two distinct pins): neighbour blocks instead of phi; phi is not maintained."""
     _check(load_library().jet_set_graph_path(ctx.handle, 1 if enable else 0), ctx)
+    ctx.graph_path = bool(enable)
 
 
 def jet_release_memory():
@@ -421,6 +471,9 @@ def jet_uncoarsen(ctxs, maps, schedule, limit, states, stream=None) -> list:
     maps[l] (int32 tensor) maps the vertices of level l+1 to level l.  One graph launch."""
     import torch
     n = len(ctxs)
+    for c, m in zip(ctxs[1:], maps):
+        _need(m, c.hg.n, "map of a level")
+    _need_states(ctxs, states)
     hs = (_P * n)(*[c.handle for c in ctxs])
     mp = (_P * max(n - 1, 1))(*([_ptr(m, torch.int32, "map") for m in maps] or [None]))
     part, phi, bw = _state_arrays(states)
@@ -436,6 +489,7 @@ def jet_quotient_schedule(ctx: Ctx, phi):
     """Matching schedule of the quotient graph: (pairs int32[p, 2], round int32[p], rounds) on the host."""
     import torch
     k = ctx.k
+    _need(phi, ctx.hg.m * k, "phi")
     cap = max(k * (k - 1) // 2, 1)
     dev = phi.device
     pairs = torch.zeros(2 * cap, dtype=torch.int32, device=dev)
@@ -460,6 +514,9 @@ def jet_block_weights_noalloc(part, vwgt, k, block_w, block_count=None, stream=N
     """c(V_i) (and |V_i|) with no device allocation; scratch is a static device array (k <= 256)."""
     import torch
     n = part.numel()
+    _need(vwgt, n, "vwgt")
+    _need(block_w, k, "block_w")
+    _need(block_count, k, "block_count")
     _check(load_library().jet_block_weights_noalloc(_ptr(part, torch.int32, "part"), _ptr(vwgt, torch.int32, "vwgt"),
                                                     n, int(k), _ptr(block_w, torch.int64, "block_w"),
                                                     _ptr(block_count, torch.int32, "block_count"),
@@ -502,6 +559,13 @@ def jet_batch_destroy(batch: Batch):
     batch.close()
 
 
+def _need_states(ctxs, states):
+    if len(states) < len(ctxs):
+        raise ValueError(f"{len(states)} states for {len(ctxs)} contexts")
+    for c, s in zip(ctxs, states):
+        _need_state(c, s.part, s.phi, s.block_w)
+
+
 def _state_arrays(states):
     import torch
     part = (_P * len(states))(*[_ptr(s.part, torch.int32, "part") for s in states])
@@ -516,6 +580,7 @@ def _pairs(schedule):
 
 def jet_batch_refine(batch: Batch, schedule, limit, states) -> list:
     """Refine every instance (states[i]: a JetState of batch.ctxs[i]) with one graph launch."""
+    _need_states(batch.ctxs, states)
     part, phi, bw = _state_arrays(states)
     res = (JetRefineResult * len(states))()
     _batch_check(load_library().jet_batch_refine(batch.handle, _pairs(schedule), len(schedule), int(limit), part, phi,
@@ -533,6 +598,7 @@ def jet_batch_get_split(batch: Batch) -> int:
 
 def jet_batch_tune(batch: Batch, schedule, limit, states, splits) -> tuple:
     """Time the batch under each split; keep the fastest.  Returns (chosen split, {split: ms})."""
+    _need_states(batch.ctxs, states)
     part, phi, bw = _state_arrays(states)
     sp = (ctypes.c_int32 * len(splits))(*[int(x) for x in splits])
     ms = (ctypes.c_float * len(splits))()
@@ -577,6 +643,7 @@ def team_candidates(batch: Batch, shapes=TEAM_SHAPES, quantiles=TEAM_SPLIT_QUANT
 def jet_batch_autotune(batch: Batch, schedule, limit, states, shapes=None, sample=24, trial_iterations=8):
     """Choose the persistent form's team shape from short trials on a sample; returns
     ((blocks, threads, split_pins), {shape: (ms, rate)})."""
+    _need_states(batch.ctxs, states)
     shapes = [tuple(s) if len(s) == 3 else (s[0], s[1], 0) for s in (shapes or team_candidates(batch))]
     part, phi, bw = _state_arrays(states)
     sh = (ctypes.c_int32 * (3 * len(shapes)))(*[int(x) for p in shapes for x in p])
@@ -631,8 +698,7 @@ def jet_server_submit(server: Server, hg, p: JetParams, schedule, limit, part: n
     """Submit a job on host arrays (hg: synth.Hypergraph; part: int32[n], refined in place)."""
     if part.dtype != np.int32 or not part.flags["C_CONTIGUOUS"] or part.shape[0] != hg.n:
         raise ValueError("part must be a contiguous int32 array of n entries")
-    arrs = [np.ascontiguousarray(a) for a in (hg.eptr, hg.pins, hg.vptr, hg.inc, hg.vwgt, hg.ewgt)]
-    hh = JetHypergraph(hg.n, hg.m, hg.P, *[a.ctypes.data for a in arrs])
+    arrs, hh = _host_hg(hg)
     pairs = (ctypes.c_int32 * max(2 * len(schedule), 1))(*[int(x) for t in schedule for x in t])
     jid = ctypes.c_int64()
     _server_check(load_library().jet_server_submit(server.handle, ctypes.byref(hh), ctypes.byref(p), pairs,
