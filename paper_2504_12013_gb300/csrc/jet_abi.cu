@@ -684,7 +684,9 @@ int jet_set_graph_path(jet_ctx *c, int enable) {
     if (g.graph) cudaGraphDestroy(g.graph);
     g = jet_ctx::RoundGraph{};
   }
-  destroy_refine_graph(c);
+  // the loop state stays: a batch's graph holds its address
+  if (c->refine_graph.exec) cudaGraphExecDestroy(c->refine_graph.exec);
+  c->refine_graph.exec = nullptr;
   c->graph_path = enable;
   c->phi_owner = nullptr;  // the bitmasks are stale after the graph path ran
   return JET_OK;
