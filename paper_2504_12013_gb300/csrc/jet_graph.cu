@@ -196,6 +196,7 @@ int refine_graph(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, int32_t li
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
       G.exec = nullptr;
+      c->phi_owner = nullptr;  // the capture named phi, and nothing has run
       return cuda_fail(c, e, "refine graph");
     }
     G.tau.assign(tau_pairs, tau_pairs + 2 * n_tau);
@@ -206,6 +207,7 @@ int refine_graph(jet_ctx *c, const int32_t *tau_pairs, int32_t n_tau, int32_t li
     G.res = c->res_host;
   }
   CK(cudaGraphLaunch(G.exec, c->stream), "refine graph launch");
+  c->phi_owner = phi;  // a graph launched again leaves phi's bitmasks too, whatever was counted since its capture
   int rc = sync_counters(c);  // synchronizes; reports data errors found on the device
   if (rc) return rc;
   *result = *c->res_host;
@@ -308,6 +310,7 @@ int build_batch(jet_batch *b, const int32_t *tau, int32_t n_tau, int32_t limit, 
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
     b->exec = nullptr;
+    for (jet_ctx *c : b->ctx) c->phi_owner = nullptr;  // named by the capture, and nothing has run
     return rc != JET_OK ? rc : bfail(b, JET_ERR_CUDA, "batch graph", e);
   }
   b->tau.assign(tau, tau + 2 * n_tau);
@@ -402,6 +405,7 @@ int run_team(jet_batch *b, int32_t limit, jet_refine_result *results) {
     b->team_exec_split = b->team_split;
   }
   cudaError_t e = cudaGraphLaunch(b->team_exec, b->stream);
+  for (size_t i = 0; i < b->ctx.size(); ++i) b->ctx[i]->phi_owner = static_cast<const int32_t *>(b->plan_args[3 * i + 1]);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, JET_ERR_CUDA, "persistent batch launch", e);
   const int bad = jet::team_first_error(b->plan, b->stream);
@@ -411,7 +415,6 @@ int run_team(jet_batch *b, int32_t limit, jet_refine_result *results) {
     snprintf(msg, sizeof(msg), "instance %d: a partition value is outside [0, k)", bad);
     return bfail(b, JET_ERR_DATA, msg);
   }
-  for (size_t i = 0; i < b->ctx.size(); ++i) b->ctx[i]->phi_owner = static_cast<const int32_t *>(b->plan_args[3 * i + 1]);
   if (results) memcpy(results, b->res_host, sizeof(jet_refine_result) * b->ctx.size());
   return JET_OK;
 }
@@ -419,6 +422,7 @@ int run_team(jet_batch *b, int32_t limit, jet_refine_result *results) {
 // Launch the batch graph on b->stream and wait; report per-instance errors.
 int run_batch(jet_batch *b, jet_refine_result *results) {
   cudaError_t e = cudaGraphLaunch(b->exec, b->stream);
+  for (size_t i = 0; i < b->ctx.size(); ++i) b->ctx[i]->phi_owner = static_cast<const int32_t *>(b->args[3 * i + 1]);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, JET_ERR_CUDA, "batch launch", e);
   for (size_t i = 0; i < b->ctx.size(); ++i) {
@@ -548,6 +552,7 @@ int jet_batch_autotune(jet_batch *b, const int32_t *tau_pairs, int32_t n_tau, in
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);
+  for (int32_t i : smp) b->ctx[i]->phi_owner = phi[i];  // the trials count and move it
   std::vector<jet_refine_result> res(b->ctx.size());
   int best = -1;
   double best_rate = 0.0;
@@ -726,6 +731,8 @@ int jet_uncoarsen(jet_ctx *const *levels, int32_t n_levels, const int32_t *const
   }
   if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
   if (e == cudaSuccess) e = cudaGraphLaunch(exec, s);
+  if (e != cudaSuccess)
+    for (int l = 0; l < n_levels; ++l) levels[l]->phi_owner = nullptr;  // named by the capture, and nothing has run
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   int rc = e == cudaSuccess ? JET_OK : bfail(nullptr, JET_ERR_CUDA, "uncoarsening graph", e);
   for (int l = 0; l < n_levels && rc == JET_OK; ++l) {
