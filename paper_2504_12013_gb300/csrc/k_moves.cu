@@ -463,25 +463,61 @@ struct SelRec<u128> {
   __device__ __forceinline__ explicit SelRec(const RbRec &r) : hi(r.hi), v(r.v), ct(r.ct) {}
 };
 
+// Segments of more than kSelLarge records go to a cluster of kSelCluster thread
+// blocks, each with its share of the records and a histogram of its own; the
+// sums over the cluster go through distributed shared memory.  A partition may
+// have a block of nearly all vertices (a seed partition, or the round after
+// many small blocks moved to one).  Bound by the reads of the records, once
+// per level beyond those in registers: jet_rebalance with every vertex in one
+// block, 32 rounds, took 49.1 ms by one thread block at n = 100,003, k = 37
+// (most of it 64-bit shared-memory atomics on the one target's weight) and
+// 54.9 ms at n = 1,000,000, k = 256; so 1.93 and 16.5 ms (grid-wide passes:
+// 2.52 and 20.7).  The line: up to it one block reads the records beyond its
+// registers in about the time of the grid-wide passes (20,000 vertices in one
+// block, k = 8: 0.38 against 0.47 ms), and clusters lose to them where every
+// block of the partition is that large (above).
+constexpr int kSelCluster = 8;
+constexpr int kSelLarge = 16384;
+constexpr int kSelGroups = 8;  // clusters for large segments, at most
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+// *p of the cluster's block `rank`.
+template <class T>
+__device__ __forceinline__ T ld_cluster(const T *p, int rank) {
+  uint32_t at = (uint32_t)__cvta_generic_to_shared(p);
+  asm("mapa.shared::cluster.u32 %0, %0, %1;\n" : "+r"(at) : "r"(rank));
+  T x;
+  if constexpr (sizeof(T) == 4) asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(x) : "r"(at) : "memory");
+  else asm volatile("ld.shared::cluster.u64 %0, [%1];\n" : "=l"(x) : "r"(at) : "memory");
+  return x;
+}
+
+// The selection of block b's segment by one thread block, or (CLUSTER) by all of a cluster.
 // WT: unsigned when c(V) < 2^32 (no sum of weights leaves it), else unsigned long long.
-template <class KT, class WT>
-__global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw) {
+template <class KT, class WT, bool CLUSTER>
+__device__ __forceinline__ void select_segment(const RbArgs &a, int64_t *bw, int b, int rank) {
   typedef SelRec<KT> Rec;
   constexpr int kPer = kSelBins / 32;  // bins per lane
+  constexpr int T = kSelThreads * (CLUSTER ? kSelCluster : 1);
   __shared__ __align__(16) WT s_hist[2][kSelBins];
-  __shared__ long long s_dw[kMaxK];  // weight and vertices that move to each block
+  __shared__ __align__(16) WT s_sum[CLUSTER ? kSelBins : 1];
+  // weight and vertices that move to each block.  64-bit shared-memory atomics are retried until they win, and many
+  // records may go to one block; where block weights are kept here (at most kEarlyVertices), c(V) < 2^32
+  __shared__ WT s_dw[kMaxK];
   __shared__ int s_dc[kMaxK];
-  const int t = threadIdx.x, lane = t & 31, b = blockIdx.x;
+  const int t = threadIdx.x, lane = t & 31, tc = rank * kSelThreads + t;  // tc: thread of the cluster
   const RbBlock &blk = a.rbb[b];
-  const int over = blk.over, room = blk.room, count = a.cur[b * kCurStride];
+  const int room = blk.room, count = a.cur[b * kCurStride];
   const WT excess = (WT)blk.excess;
   const RbRec *rec = a.rec + blk.base;
-  if (!over) return;
   const int cnt = min(count, room);
   Rec held[kSelHeld];  // weight 0: no record
 #pragma unroll
-  for (int q = 0; q < kSelHeld; ++q)
-    held[q] = t + q * kSelThreads < cnt ? Rec(rec[t + q * kSelThreads]) : Rec();
+  for (int q = 0; q < kSelHeld; ++q) held[q] = tc + q * T < cnt ? Rec(rec[tc + q * T]) : Rec();
   if (t < kSelBins) s_hist[0][t] = s_hist[1][t] = 0;
   if (t < kMaxK) {
     s_dw[t] = 0;
@@ -502,17 +538,27 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw
     };
 #pragma unroll
     for (int q = 0; q < kSelHeld; ++q)
-      if (q * kSelThreads < cnt) add(held[q]);
-    for (int i = t + kSelHeld * kSelThreads; i < cnt; i += 4 * kSelThreads) {
+      if (q * T < cnt) add(held[q]);
+    for (int i = tc + kSelHeld * T; i < cnt; i += 4 * T) {
       Rec r[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) r[q] = i + q * kSelThreads < cnt ? Rec(rec[i + q * kSelThreads]) : Rec();
+      for (int q = 0; q < 4; ++q) r[q] = i + q * T < cnt ? Rec(rec[i + q * T]) : Rec();
 #pragma unroll
       for (int q = 0; q < 4; ++q) add(r[q]);
     }
-    __syncthreads();
-    if (t < kSelBins) s_hist[buf ^ 1][t] = 0;  // read a level ago
-    const WT *sum = s_hist[buf] + lane * kPer;
+    if constexpr (CLUSTER) {
+      cluster_sync();
+      if (t < kSelBins) {
+        WT x = 0;
+#pragma unroll
+        for (int r = 0; r < kSelCluster; ++r) x += ld_cluster(&s_hist[buf][t], r);
+        s_sum[t] = x;
+      }
+    }
+    if (!CLUSTER) __syncthreads();
+    if (t < kSelBins) s_hist[buf ^ 1][t] = 0;  // read a level ago (by the cluster: before the barrier)
+    if (CLUSTER) __syncthreads();
+    const WT *sum = (CLUSTER ? s_sum : s_hist[buf]) + lane * kPer;
     WT w[kPer], mine = 0;
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
@@ -541,7 +587,7 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw
     before = __shfl_sync(kFull, run, src);
     pre |= (KT)(unsigned)__shfl_sync(kFull, digit, src) << lo;
     up = lo;
-    if (up > 0) __syncthreads();  // the cleared buffer is added to next
+    if (up > 0 && !CLUSTER) __syncthreads();  // the cleared buffer is added to next
   }
   // the records up to the threshold: one atomic per warp (and batch) on the move list
   auto emit = [&](const Rec *r, int n) {
@@ -568,7 +614,7 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw
           a.mv_v[x] = r[q].v;
           a.mv_st[x] = (uint32_t)b | ((uint32_t)to << 16);
           if (bw) {
-            atomicAdd(reinterpret_cast<unsigned long long *>(&s_dw[to]), (unsigned long long)(r[q].ct >> 16));
+            atomicAdd(&s_dw[to], (WT)(unsigned)(r[q].ct >> 16));
             atomicAdd(&s_dc[to], 1);
           }
         }
@@ -578,28 +624,63 @@ __global__ void __launch_bounds__(kSelThreads) k_rb_select(RbArgs a, int64_t *bw
   };
   emit(held, kSelHeld);
   // the warp's lanes go together, from its first record
-  for (int i = t + kSelHeld * kSelThreads, iw = i - lane; iw < cnt; i += 4 * kSelThreads, iw += 4 * kSelThreads) {
+  for (int i = tc + kSelHeld * T, iw = i - lane; iw < cnt; i += 4 * T, iw += 4 * T) {
     Rec r[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) r[q] = i + q * kSelThreads < cnt ? Rec(rec[i + q * kSelThreads]) : Rec();
+    for (int q = 0; q < 4; ++q) r[q] = i + q * T < cnt ? Rec(rec[i + q * T]) : Rec();
     emit(r, 4);
   }
-  if (!bw) return;
-  __syncthreads();
-  // the block weights already, so that the end of the round need not wait for the apply
-  if (t < kMaxK) {
-    long long dw = s_dw[t];
-    int dc = s_dc[t];
-    if (dc) {
-      add_i64(reinterpret_cast<long long *>(&bw[t]), dw);
-      atomicAdd(&a.cnt->vcount[t], dc);
-    }
+  if (bw) {
+    __syncthreads();
+    // the block weights already, so that the end of the round need not wait for the apply
+    if (t < kMaxK) {
+      long long dw = (long long)s_dw[t];
+      int dc = s_dc[t];
+      if (dc) {
+        add_i64(reinterpret_cast<long long *>(&bw[t]), dw);
+        atomicAdd(&a.cnt->vcount[t], dc);
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dw += __shfl_xor_sync(kFull, dw, o);
-    dc = __reduce_add_sync(kFull, dc);
-    if (lane == 0 && dc) {
-      add_i64(reinterpret_cast<long long *>(&bw[b]), -dw);
-      atomicSub(&a.cnt->vcount[b], dc);
+      for (int o = 16; o > 0; o >>= 1) dw += __shfl_xor_sync(kFull, dw, o);
+      dc = __reduce_add_sync(kFull, dc);
+      if (lane == 0 && dc) {
+        add_i64(reinterpret_cast<long long *>(&bw[b]), -dw);
+        atomicSub(&a.cnt->vcount[b], dc);
+      }
+    }
+  }
+  if (CLUSTER) cluster_sync();  // no block leaves or clears a histogram that another still reads
+}
+
+// A thread block per block of the partition; LARGE (a segment may be large): the blocks from `first` on are clusters
+// that take the large segments in turn.
+template <class KT, class WT, bool LARGE>
+__global__ void __launch_bounds__(kSelThreads, 2) k_rb_select(RbArgs a, int64_t *bw, int first, int groups) {
+  const int b = blockIdx.x;
+  if (!LARGE || b < first) {
+    if (b < a.k && a.rbb[b].over && (!LARGE || a.rbb[b].room <= kSelLarge))
+      select_segment<KT, WT, false>(a, bw, b, 0);
+    return;
+  }
+  if constexpr (LARGE) {
+    __shared__ int s_list[kMaxK / 32], s_which;
+    const int t = threadIdx.x, lane = t & 31;
+    const bool large = t < a.k && a.rbb[t].over && a.rbb[t].room > kSelLarge;
+    const unsigned bal = __ballot_sync(kFull, large);
+    if (lane == 0 && t < kMaxK) s_list[t >> 5] = bal;
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kMaxK / 32; ++w) {
+      before += w < (t >> 5) ? __popc(s_list[w]) : 0;
+      total += __popc(s_list[w]);
+    }
+    before += __popc(bal & ((1u << lane) - 1));
+    const int group = (b - first) / kSelCluster, rank = (b - first) % kSelCluster;
+    for (int i = group; i < total; i += groups) {  // the same in every block of the cluster
+      if (large && before == i) s_which = t;
+      __syncthreads();
+      select_segment<KT, WT, true>(a, bw, s_which, rank);
     }
   }
 }
@@ -842,12 +923,27 @@ void rb_select_levels(jet_ctx *c, const RbArgs &a) {
   }
 }
 
-template <class KT>
+template <class KT, class WT>
 cudaError_t select_segments(jet_ctx *c, const RbArgs &a, int64_t *bw) {
-  if (c->W < (1ll << 32)) k_rb_select<KT, unsigned><<<c->k, kSelThreads, 0, c->stream>>>(a, bw);
-  else k_rb_select<KT, unsigned long long><<<c->k, kSelThreads, 0, c->stream>>>(a, bw);
   ++c->kernel_launches;
-  return cudaGetLastError();
+  if (c->n <= kSelLarge) {  // no segment can be large
+    k_rb_select<KT, WT, false><<<c->k, kSelThreads, 0, c->stream>>>(a, bw, 0, 0);
+    return cudaGetLastError();
+  }
+  const int first = (c->k + kSelCluster - 1) / kSelCluster * kSelCluster;
+  const int groups = std::min(c->n / kSelLarge, kSelGroups);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(first + groups * kSelCluster);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kSelCluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_rb_select<KT, WT, true>, a, bw, first, groups);
 }
 
 cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
@@ -862,7 +958,11 @@ cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w) 
   const RbArgs a = rb_args(c, nullptr, part);
   if (c->rb_segments) {
     int64_t *bw = c->rb_early ? block_w : nullptr;
-    return a.tbits <= 64 ? select_segments<unsigned long long>(c, a, bw) : select_segments<u128>(c, a, bw);
+    if (c->W < (1ll << 32))
+      return a.tbits <= 64 ? select_segments<unsigned long long, unsigned>(c, a, bw)
+                           : select_segments<u128, unsigned>(c, a, bw);
+    return a.tbits <= 64 ? select_segments<unsigned long long, unsigned long long>(c, a, bw)
+                         : select_segments<u128, unsigned long long>(c, a, bw);
   }
   if (a.tbits <= 64) rb_select_levels<unsigned long long>(c, a);
   else rb_select_levels<u128>(c, a);
