@@ -954,33 +954,34 @@ __device__ void team_apply_selection(const TeamInst &I, const Team &tm, long lon
   block_add(moved, reinterpret_cast<long long *>(&I.tc->moved), s_red);
 }
 
-// The selection of a multi-block team where no block of the team owns more than kLocalRecords records (block b of the
+// The selection of a multi-block team where every block of the team has room for the records it owns (block b of the
 // partition belongs to the team's block b mod size): each reads all records, keeps its own in shared memory, does
 // every level of the radix select for all its blocks of the partition there, with block barriers only, and moves
 // them.  The team-wide form has two team barriers and a chain of global loads per level: 14 to 17 us per round, and
-// 6 to 9 for the moves after it.
-constexpr int kLocalRecords = 4096;
-constexpr int kLocalBlocks = 32;  // blocks of the partition per block of the team
-constexpr size_t kLocalSmem = sizeof(RbRec) * kLocalRecords + sizeof(unsigned) * 256 * kLocalBlocks;
+// 6 to 9 for the moves after it.  The room comes in units of kUnitRecords records and the histogram of one block of
+// the partition, kUnits at most (launch_group says how many).
+constexpr int kUnitRecords = 128;
+constexpr int kUnits = 32;
+constexpr size_t kUnitSmem = sizeof(RbRec) * kUnitRecords + sizeof(unsigned) * 256;
 
 // Whether every thread of the team may take the local form (the same answer in all).
 template <bool MULTI>
-__device__ bool select_is_local(const TeamInst &I, const Team &tm) {
+__device__ bool select_is_local(const TeamInst &I, const Team &tm, int units) {
   const int size = (int)tm.size;  // a power of two up to 8
-  if (!MULTI || size < 2 || (I.k + size - 1) / size > kLocalBlocks) return false;
+  if (!MULTI || size < 2 || (I.k + size - 1) / size > units) return false;
   int mine = 0;  // lane l: records of the blocks l, l + 32, ...: all of the team's block l mod size
   for (int b = threadIdx.x & 31; b < I.k; b += 32) mine += ldm<MULTI>(&I.rbb[b].room);
   for (int o = size; o < 32; o <<= 1) mine += __shfl_xor_sync(kFull, mine, o);
-  return __reduce_max_sync(kFull, mine) <= kLocalRecords;
+  return __reduce_max_sync(kFull, mine) <= units * kUnitRecords;
 }
 
 template <int KWP, class KT>
 __device__ void team_select_local(const TeamInst &I, const Team &tm, long long nrec, const int *s_over,
-                                  const long long *s_bw, SelState<KT> &st, RbRec *list, long long *s_dw,
+                                  const long long *s_bw, SelState<KT> &st, RbRec *list, int units, long long *s_dw,
                                   long long *s_red) {
   __shared__ int s_n;
-  __shared__ long long s_before[kLocalBlocks];
-  unsigned *hist = reinterpret_cast<unsigned *>(list + kLocalRecords);  // 256 bins per own block
+  __shared__ long long s_before[kUnits];
+  unsigned *hist = reinterpret_cast<unsigned *>(list + units * kUnitRecords);  // 256 bins per own block
   const int t = threadIdx.x, T = blockDim.x, lane = t & 31, size = (int)tm.size, shift = __ffs(size) - 1;
   const int own = (I.k - (int)tm.rank + size - 1) / size;  // blocks rank, rank + size, ...
   for (int x = t; x < 256 * own; x += T) hist[x] = 0;
@@ -1080,10 +1081,11 @@ __device__ void team_select_local(const TeamInst &I, const Team &tm, long long n
 struct SmemPtrs {
   long long *s_dw, *s_cap, *s_bw, *s_red;
   int *s_over;
-  unsigned long long *s_tab;  // the afterburner's tables; multi-block teams: also the local selection's records
+  // the afterburner's tables, in other phases the targets' queues and (multi-block teams) the local selection's records
+  unsigned long long *s_tab;
   void *s_sel;                // SelState<u128>, or in its first bytes the state of 64-bit keys
   void *s_elig;               // kEligTab x KWP words
-  TeamQueue *s_queue;
+  int units;                  // room of the local selection in s_tab
 };
 
 // Rebalancing rounds until balanced, a round moves nothing, or the round cap.  Returns the rounds; moves in *mv.
@@ -1114,17 +1116,19 @@ __device__ long long team_rebalance(const TeamInst &I, const Team &tm, const Sme
     }
     eligible_table<KWP>(I, sm.s_cap, s_elig);
     team_sync<MULTI>();
-    team_targets<MULTI, KWP>(I, tm, sm.s_cap, sm.s_bw, sm.s_over, s_elig, sm.s_queue);
+    team_targets<MULTI, KWP>(I, tm, sm.s_cap, sm.s_bw, sm.s_over, s_elig,
+                             reinterpret_cast<TeamQueue *>(sm.s_tab));
     team_sync<MULTI>();
     const long long nrec = (long long)ldm<MULTI>(&I.tc->n_rec);
     SelState<unsigned long long> &st64 = *static_cast<SelState<unsigned long long> *>(sm.s_sel);
     SelState<u128> &st128 = *static_cast<SelState<u128> *>(sm.s_sel);
-    if (select_is_local<MULTI>(I, tm)) {
+    if (select_is_local<MULTI>(I, tm, sm.units)) {
       RbRec *list = reinterpret_cast<RbRec *>(sm.s_tab);
       if (I.rb_tbits <= 64)
-        team_select_local<KWP, unsigned long long>(I, tm, nrec, sm.s_over, sm.s_bw, st64, list, sm.s_dw, sm.s_red);
+        team_select_local<KWP, unsigned long long>(I, tm, nrec, sm.s_over, sm.s_bw, st64, list, sm.units, sm.s_dw,
+                                                   sm.s_red);
       else
-        team_select_local<KWP, u128>(I, tm, nrec, sm.s_over, sm.s_bw, st128, list, sm.s_dw, sm.s_red);
+        team_select_local<KWP, u128>(I, tm, nrec, sm.s_over, sm.s_bw, st128, list, sm.units, sm.s_dw, sm.s_red);
     } else if (I.rb_tbits <= 64) {
       team_select<MULTI, unsigned long long>(I, tm, nrec, sm.s_over, st64);
       team_apply_selection<MULTI, KWP, unsigned long long>(I, tm, nrec, sm.s_over, st64, sm.s_dw, sm.s_red);
@@ -1233,23 +1237,24 @@ __device__ void team_refine(const TeamInst &I, const Team &tm, const TeamArgs &a
   team_sync<MULTI>();
 }
 
-// Dynamic shared memory: the per-block arrays of the partition, then (16-byte aligned) the afterburner's tables, in
-// multi-block teams with room for the local selection.
+// Dynamic shared memory: the per-block arrays of the partition, then (16-byte aligned) one area for the afterburner's
+// tables, the targets' queues and in multi-block teams the local selection (`units` of room).
 __host__ __device__ constexpr size_t team_smem_head(int kmax) { return ((size_t)kmax * (8 + 8 + 8 + 4) + 15) & ~15ull; }
-template <bool MULTI, int KWP>
-constexpr size_t team_smem(int kmax, int threads) {
+template <int KWP>
+constexpr size_t team_smem(int kmax, int threads, int units) {
   const size_t tab = (size_t)(threads / 32) * (2 * kmax + (KWP + 1) / 2) * 8;
-  return team_smem_head(kmax) + (MULTI && tab < kLocalSmem ? kLocalSmem : tab);
+  const size_t queues = (size_t)(threads / 32) * sizeof(TeamQueue), local = units * kUnitSmem;
+  const size_t other = queues > local ? queues : local;
+  return team_smem_head(kmax) + (tab > other ? tab : other);
 }
 
 // The persistent kernel: teams of gridDim.x / clusterDim blocks loop over the work queue.
 template <bool MULTI, int KWP>
-__global__ void __launch_bounds__(kTeamMaxThreads, 1) k_batch_teams(TeamArgs a, int kmax) {
+__global__ void __launch_bounds__(kTeamMaxThreads, 1) k_batch_teams(TeamArgs a, int kmax, int units) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_red[kTeamMaxThreads / 32];
   __shared__ __align__(16) SelState<u128> s_sel;
   __shared__ uint32_t s_elig[kEligTab][KWP];
-  __shared__ TeamQueue s_queue[kTeamMaxThreads / 32];
   SmemPtrs sm;
   sm.s_dw = reinterpret_cast<long long *>(smem);
   sm.s_cap = sm.s_dw + kmax;
@@ -1259,7 +1264,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_batch_teams(TeamArgs a, 
   sm.s_red = s_red;
   sm.s_sel = &s_sel;
   sm.s_elig = s_elig;
-  sm.s_queue = s_queue;
+  sm.units = units;
   Team tm;
   if constexpr (MULTI) {
     unsigned r, sz;
@@ -1343,19 +1348,52 @@ struct TeamPlan {
 
 namespace {
 
+constexpr int kShareWaves = 4;          // blocks per SM from which they share it
+constexpr int kShareSmem = 128 * 1024;  // shared memory of an SM for blocks that share it
+
 template <bool MULTI, int KWP>
 cudaError_t launch_group(const TeamArgs &a, int kmax, int ctas, int threads, int num_sms, cudaStream_t s,
                          int max_teams) {
   auto kern = k_batch_teams<MULTI, KWP>;
-  const size_t smem = team_smem<MULTI, KWP>(kmax, threads);
+  int units = 0;
+  size_t pad = 0;
+  cudaError_t e = cudaSuccess;
+  if (MULTI) {
+    // Blocks of fewer threads can share an SM, which pays where a launch has many more of them than there are SMs
+    // (200 instances of up to 6,000 vertices at k = 8: teams of 8 x 512 69.4 -> 34.3 ms, 4 x 512 33.1 -> 20.1, 4 x 256
+    // 37.6 -> 24.1).  With fewer, one block per SM is faster: sharing took 100 instances of up to 10,000 vertices at
+    // k = 64 in teams of 4 x 512 (2.6 blocks per SM) from 33.3 to 35.1 ms, 24 of 20,000 at k = 200 in teams of 8 x 512
+    // (1.3) from 35.6 to 38.2; and the scheduler packs two blocks of a cluster into one SM beside idle ones where
+    // they fit, so their shared memory is then made too large for two.  Blocks that share get room for the local
+    // selection from half of the SM's memory, the other half is L1: all of it as room cost 8 to 40 %.
+    cudaFuncAttributes fa{};
+    int dev = 0, per_sm = 0, reserved = 0, regs = 0;
+    e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
+    if (e != cudaSuccess) return e;
+    const int fit = std::max(1, regs / (std::max(fa.numRegs, 1) * threads));  // by registers
+    const long long fixed = reserved + (long long)fa.sharedSizeBytes;
+    units = kUnits;
+    if (fit > 1 && (long long)max_teams * ctas >= kShareWaves * num_sms) {
+      const long long left = kShareSmem / fit - fixed - (long long)team_smem_head(kmax);
+      units = (int)std::min((long long)kUnits, std::max(0ll, left) / (long long)kUnitSmem);
+    } else if (fit > 1) {
+      pad = (size_t)std::max(0ll, per_sm / 2 + 1 - fixed);
+    }
+  }
   // The limit is a property of the kernel, shared by every batch and graph that launches it: set it for
   // the largest instance this mask width allows (k = 32 KWP) and 1,024 threads, so it never shrinks
   // under an earlier launch.
-  constexpr size_t kSmemMax = team_smem<MULTI, KWP>(32 * KWP, kTeamMaxThreads);
-  static_assert(kSmemMax + 32 * 1024 <= 227 * 1024, "the team kernel's shared memory (with its static part) must fit "
+  constexpr size_t kSmemMax =
+      std::max(team_smem<KWP>(32 * KWP, kTeamMaxThreads, MULTI ? kUnits : 0), (size_t)(MULTI ? 114 * 1024 : 0));
+  static_assert(kSmemMax + 16 * 1024 <= 227 * 1024, "the team kernel's shared memory (with its static part) must fit "
                                                     "one block");
+  const size_t smem = std::max(team_smem<KWP>(kmax, threads, units), std::min(pad, kSmemMax));
   if (smem > kSmemMax) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
   if (e != cudaSuccess) return e;
   if (MULTI && ctas > 8) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1386,7 +1424,7 @@ cudaError_t launch_group(const TeamArgs &a, int kmax, int ctas, int threads, int
   if (teams < 1) return cudaErrorInvalidConfiguration;
   if (teams > max_teams) teams = max_teams;
   cfg.gridDim = dim3(teams * ctas);
-  return cudaLaunchKernelEx(&cfg, kern, a, kmax);
+  return cudaLaunchKernelEx(&cfg, kern, a, kmax, units);
 }
 
 template <int KWP>
