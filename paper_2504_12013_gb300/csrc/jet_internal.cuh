@@ -30,6 +30,8 @@ constexpr int kLightPlanes = 6;      // thread-per-vertex gain path: weighted de
 constexpr int kTinyEdge = 8;         // thread-per-edge afterburner: |e| <= 8
 constexpr int kWarpEdge = 128;       // warp-per-edge afterburner: 8 < |e| <= 128
 constexpr int kSegPins = 2048;       // block-class edges are cut into segments of at most this many pins
+constexpr int kSegWarp = 1024;       // pin counts: many segments of at most this many pins go by a warp each
+constexpr int kSegWaves = 16;        // ... many: more than so many waves of thread blocks
 constexpr int kHalfMidEdge = 16;     // warp-class edges of at most 16 pins: a half warp per edge
 constexpr int kSmallMidEdge = 32;    // warp-class edges of at most 32 pins: one pin per lane, pipelined
 constexpr int kPrioShift = 30;       // exact rebalancing priority encoding (needs c(v) <= 2^15)
@@ -157,7 +159,7 @@ struct jet_ctx {
   int32_t n_mid_hi = 0;  // the first n_mid_hi edges of e_mid have 65..128 pins, the rest 33..64
   // block-class edges as segments (largest first): edge, first pin, pins, table slot (-1: the whole edge)
   int4 *ab_seg = nullptr;
-  int32_t n_seg = 0;
+  int32_t n_seg = 0, n_seg_block = 0;        // the first n_seg_block: pins counted by a thread block each
   int32_t n_slots = 0;                       // edges longer than one segment
   int32_t *ab_slot_edge = nullptr;           // edge of each slot
   unsigned long long *ab_tab = nullptr;      // per slot and block: max departure key, min arrival key

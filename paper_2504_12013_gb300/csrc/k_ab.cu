@@ -840,6 +840,10 @@ cudaError_t prepare_afterburner(jet_ctx *c) {
   }
   std::stable_sort(seg.begin(), seg.end(), [](const int4 &x, const int4 &y) { return x.z > y.z; });
   c->n_seg = (int32_t)seg.size();
+  // of the pin counts' two forms (k_state.cu) thread blocks take the segments above kSegWarp pins, and all of them
+  // up to kSegWaves waves of eight blocks per SM
+  const auto warps = std::partition_point(seg.begin(), seg.end(), [](const int4 &x) { return x.z > kSegWarp; });
+  c->n_seg_block = seg.end() - warps > (int64_t)kSegWaves * 8 * c->num_sms ? (int32_t)(warps - seg.begin()) : c->n_seg;
   c->n_slots = (int32_t)slot_edge.size();
   if ((e = jet::pool_alloc(reinterpret_cast<void **>(&c->ab_seg), sizeof(int4) * seg.size(), c->stream)) != cudaSuccess)
     return e;

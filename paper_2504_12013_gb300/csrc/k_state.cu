@@ -187,8 +187,8 @@ struct Gate {
 // of the edge three steps ahead, the pins of the one two ahead and the blocks
 // of the next are in flight while an edge is counted (a warp per edge with
 // nothing in flight took 364 us for 1.1 M edges at k = 128, 563 MB of phi).
-// G = 8 lanes at k <= 32 and 16 at k <= 64: four lanes' counts fill the row
-// in one step, and most edges are that short.  Longer edges are counted by
+// G = 8 lanes at k <= 64, else 16: the row goes out in two steps at most (four
+// at k > 128), and most edges are that short.  Longer edges are counted by
 // k_pincounts_seg; the rows of those longer than one segment are cleared here.
 template <int KWP>
 constexpr int kPinLanes = KWP <= 2 ? 8 : 16;
@@ -293,12 +293,38 @@ __global__ void __launch_bounds__(256) k_pincounts(const int64_t *eptr, const in
   if (err) atomicOr(&cnt->err, err);
 }
 
-// The edges of more than kWarpEdge pins: a thread block per segment of at most
-// kSegPins pins (the afterburner's segment list) counts the blocks of its pins
-// in shared memory.  An edge of one segment (slot < 0) gets its row and mask
-// words from there; the segments of a longer edge add their counts into the
-// row, cleared by k_pincounts (one atomic per block of the partition that the
-// segment touches), and k_masks_from_phi completes it.
+// The edges of more than kWarpEdge pins, by the segments of at most kSegPins
+// pins that the afterburner's list holds (largest first): the blocks of a
+// segment's pins are counted in shared memory, by a thread block
+// (k_pincounts_seg) or a warp (k_pincounts_warp).  An edge of one segment
+// (slot < 0) gets its row and mask words from there; the segments of a longer
+// edge add their counts into the row, cleared by k_pincounts (one atomic per
+// block of the partition that the segment touches), and k_masks_from_phi
+// completes it.  Bound by the chain segment -> offset -> pins -> blocks ->
+// counts where the segments are few, by the gathers of the blocks where they
+// are many.  So a thread block has the shorter time for one segment and waits
+// out three barriers per segment, and warps are the better form of segments of
+// up to kSegWarp pins when there are many (n_seg_block, prepare_afterburner).
+// 80,000 edges of 150 pins, k = 128: 116 us by thread blocks, 85 by warps;
+// 20,000 of them, k = 256: 46.7 and 45; 20,000 of 600 pins 74 and 70, 8,000 of
+// 1,500 pins 65 and 80; 20 of 1,000 pins beside 100,000 small ones 27.5 and
+// 32 us.  Four pins per lane in flight: with eight and the registers for them
+// (40) 92 us in the first of these.
+__device__ __forceinline__ void store_counts(const int4 &sg, int b, int val, int32_t k, int32_t kwp, int32_t *phi,
+                                             uint32_t *mask) {  // by whole warps, blocks b, b + 1, ... in its lanes
+  int32_t *row = phi + (int64_t)sg.x * k;
+  if (sg.w >= 0) {
+    if (b < k && val) atomicAdd(&row[b], val);
+    return;
+  }
+  if (b < k) row[b] = val;
+  const unsigned one = __ballot_sync(kFull, val > 0), two = __ballot_sync(kFull, val > 1);
+  if ((b & 31) == 0 && (b >> 5) < kwp) {
+    mask[(int64_t)sg.x * 2 * kwp + (b >> 5)] = one;
+    mask[(int64_t)sg.x * 2 * kwp + kwp + (b >> 5)] = two;
+  }
+}
+
 __global__ void __launch_bounds__(256) k_pincounts_seg(const int64_t *eptr, const int32_t *pins, const int32_t *part,
                                                        const int4 *seg, int32_t nseg, int32_t k, int32_t kwp,
                                                        int32_t *phi, uint32_t *mask, Counters *cnt, Gate gate) {
@@ -317,19 +343,60 @@ __global__ void __launch_bounds__(256) k_pincounts_seg(const int64_t *eptr, cons
       else err |= kErrPartRange;
     }
     __syncthreads();
-    const int b = threadIdx.x, val = s_h[b];
-    int32_t *row = phi + (int64_t)sg.x * k;
-    if (sg.w >= 0) {
-      if (b < k && val) atomicAdd(&row[b], val);
-    } else {
-      if (b < k) row[b] = val;
-      const unsigned one = __ballot_sync(kFull, val > 0), two = __ballot_sync(kFull, val > 1);
-      if ((b & 31) == 0 && (b >> 5) < kwp) {
-        mask[(int64_t)sg.x * 2 * kwp + (b >> 5)] = one;
-        mask[(int64_t)sg.x * 2 * kwp + kwp + (b >> 5)] = two;
+    store_counts(sg, threadIdx.x, s_h[threadIdx.x], k, kwp, phi, mask);
+    __syncthreads();
+  }
+  if (err) atomicOr(&cnt->err, err);
+}
+
+template <int KWP>
+__global__ void __launch_bounds__(256, 6) k_pincounts_warp(const int64_t *eptr, const int32_t *pins,
+                                                           const int32_t *part, const int4 *seg, int32_t nseg,
+                                                           int32_t k, int32_t *phi, uint32_t *mask, Counters *cnt,
+                                                           Gate gate) {
+  if (gate.closed()) return;
+  constexpr int R = 4;  // pins per lane in flight
+  __shared__ int s_h[256 / 32][32 * KWP];
+  const int lane = threadIdx.x & 31, nw = gridDim.x * (256 / 32);
+  int *h = s_h[threadIdx.x >> 5];
+#pragma unroll
+  for (int w = 0; w < KWP; ++w) h[32 * w + lane] = 0;
+  __syncwarp();
+  int err = 0;
+  int i = blockIdx.x * (256 / 32) + (threadIdx.x >> 5);
+  int4 next = i < nseg ? seg[i] : make_int4(0, 0, 0, -1);
+  int64_t pn = i < nseg ? eptr[next.x] : 0;
+  for (; i < nseg; i += nw) {
+    const int4 sg = next;
+    const int64_t p0 = pn + sg.y;
+    if (i + nw < nseg) {  // used in the next turn
+      next = seg[i + nw];
+      pn = eptr[next.x];
+    }
+    for (int j0 = 0; j0 < sg.z; j0 += 32 * R) {
+      int v[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) v[q] = j0 + 32 * q + lane < sg.z ? pins[p0 + j0 + 32 * q + lane] : -1;
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        if (j0 + 32 * q < sg.z) v[q] = v[q] >= 0 ? part[v[q]] : -2;
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        if (j0 + 32 * q >= sg.z) break;  // the warp's lanes together
+        if ((unsigned)v[q] < (unsigned)k) atomicAdd(&h[v[q]], 1);
+        else if (v[q] != -2) err |= kErrPartRange;
       }
     }
-    __syncthreads();
+    __syncwarp();
+    int c[KWP];
+#pragma unroll
+    for (int w = 0; w < KWP; ++w) {
+      c[w] = h[32 * w + lane];
+      h[32 * w + lane] = 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int w = 0; w < KWP; ++w) store_counts(sg, 32 * w + lane, c[w], k, KWP, phi, mask);
   }
   if (err) atomicOr(&cnt->err, err);
 }
@@ -749,9 +816,21 @@ static cudaError_t launch_count_phi(jet_ctx *c, const int32_t *part, int32_t *ph
   }
   ++c->kernel_launches;
   if (c->n_seg > 0) {  // edges above kWarpEdge pins
-    k_pincounts_seg<<<grid_for(c->n_seg, 1, c->launch_sms), kMaxK, 0, s>>>(c->eptr, c->pins, part, c->ab_seg, c->n_seg,
-                                                                           c->k, c->kwp, phi, c->mask, c->cnt, gate);
-    ++c->kernel_launches;
+    const int nb = c->n_seg_block, nw = c->n_seg - nb;
+    if (nb > 0)
+      k_pincounts_seg<<<grid_for(nb, 1, c->launch_sms), kMaxK, 0, s>>>(c->eptr, c->pins, part, c->ab_seg, nb, c->k, c->kwp,
+                                                                       phi, c->mask, c->cnt, gate);
+    auto warps = [&](auto words) {
+      k_pincounts_warp<decltype(words)::value><<<grid_for((int64_t)nw * 32, 256, c->launch_sms), 256, 0, s>>>(
+          c->eptr, c->pins, part, c->ab_seg + nb, nw, c->k, phi, c->mask, c->cnt, gate);
+    };
+    if (nw > 0) switch (c->kwp) {
+      case 1: warps(std::integral_constant<int, 1>()); break;
+      case 2: warps(std::integral_constant<int, 2>()); break;
+      case 4: warps(std::integral_constant<int, 4>()); break;
+      default: warps(std::integral_constant<int, 8>()); break;
+    }
+    c->kernel_launches += (nb > 0) + (nw > 0);
   }
   if (c->n_slots > 0) {  // edges longer than one segment
     k_masks_from_phi<<<grid_for((int64_t)c->n_slots * 32, 256, c->launch_sms), 256, 0, s>>>(
