@@ -456,13 +456,13 @@ __global__ void __launch_bounds__(256) k_masks_from_phi(const int32_t *phi, int3
   }
 }
 
-// (lambda-1) from a dense phi, read once: a group of G lanes per row (four
-// entries per lane and load), eight rows in flight per group.  A lane adds
-// omega(e) per nonzero entry it sees and the group's first lane takes one
-// omega(e) off if the row has any, so no sum crosses lanes until the end.
-// Bound by the read of phi (a warp per row, one load at a time: 300 us for
-// 563 MB at k = 128).
-template <int G, bool VEC>
+// (lambda-1) from a dense phi of 16-byte aligned rows, read once: a group of G
+// lanes per row (four entries per lane and load), eight rows in flight per
+// group.  A lane adds omega(e) per nonzero entry it sees and the group's first
+// lane takes one omega(e) off if the row has any, so no sum crosses lanes
+// until the end.  Bound by the read of phi (a warp per row, one load at a
+// time: 300 us for 563 MB at k = 128).
+template <int G>
 __global__ void __launch_bounds__(256) k_connectivity_dense(const int32_t *phi, const int32_t *ewgt, int32_t m,
                                                             int32_t k, long long *out) {
   constexpr int kRows = 8;
@@ -481,22 +481,59 @@ __global__ void __launch_bounds__(256) k_connectivity_dense(const int32_t *phi, 
       w[r] = 0;
       if (e < m) {
         w[r] = ewgt[e];
-        const int32_t *row = phi + e * k;
-        if constexpr (VEC) {
-          const int4 *row4 = reinterpret_cast<const int4 *>(row);
+        const int4 *row4 = reinterpret_cast<const int4 *>(phi + e * k);
 #pragma unroll 2
-          for (int x = li; 4 * x < k; x += G) {
-            const int4 y = __ldcs(row4 + x);
-            c[r] += (y.x > 0) + (y.y > 0) + (y.z > 0) + (y.w > 0);
-          }
-        } else {
-#pragma unroll 4
-          for (int x = li; x < k; x += G) c[r] += row[x] > 0;
+        for (int x = li; 4 * x < k; x += G) {
+          const int4 y = __ldcs(row4 + x);
+          c[r] += (y.x > 0) + (y.y > 0) + (y.z > 0) + (y.w > 0);
         }
       }
     }
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
+      const bool any = (__ballot_sync(kFull, c[r] > 0) & group) != 0;
+      acc += (long long)(c[r] - (any && li == 0 ? 1 : 0)) * w[r];
+    }
+  }
+  long long tot = block_sum_ll(acc);
+  if (threadIdx.x == 0 && tot) add_i64(out, tot);
+}
+
+// The same for rows off the 16-byte boundary: one entry per lane and load, so
+// a row takes Q loads per lane, all issued before the first is used.  Such
+// rows share lines with their neighbours, so the loads go through L1, and rows
+// in flight beyond what L1 holds cost more than they hide: 1 M rows at k = 255
+// took 432 us with a loop over the loads of each of eight rows, 600 with four
+// rows of eight loads in flight per warp and 32 warps, 243 with two and 48,
+// and 190 with the grid in one wave.  At k = 61 eight rows and 32 warps take
+// 127 us (177 by the loop), against 144 with 48 warps.
+template <int Q>
+constexpr int kRowsBlocks = Q <= 2 ? 4 : 6;  // resident blocks per SM
+template <int G, int Q>
+__global__ void __launch_bounds__(256, kRowsBlocks<Q>) k_connectivity_rows(const int32_t *phi, const int32_t *ewgt,
+                                                                           int32_t m, int32_t k, long long *out) {
+  constexpr int kRows = Q <= 2 ? 8 : Q <= 4 ? 4 : 2;
+  const int lane = threadIdx.x & 31, li = lane % G;
+  const unsigned group = (G == 32 ? kFull : ((1u << (G % 32)) - 1) << (lane - li));
+  const int64_t ng = (int64_t)gridDim.x * blockDim.x / G;
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const int64_t gfirst = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;  // the warp's first group
+  long long acc = 0;
+  for (int64_t d = 0; gfirst + d < m; d += kRows * ng) {
+    int c[kRows], w[kRows], y[kRows][Q];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int64_t e = g + d + r * ng;
+      const int32_t *row = phi + (e < m ? e : 0) * k;
+      w[r] = e < m ? ewgt[e] : 0;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) y[r][q] = e < m && li + q * G < k ? row[li + q * G] : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      c[r] = 0;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) c[r] += y[r][q] > 0;
       const bool any = (__ballot_sync(kFull, c[r] > 0) & group) != 0;
       acc += (long long)(c[r] - (any && li == 0 ? 1 : 0)) * w[r];
     }
@@ -883,19 +920,27 @@ cudaError_t launch_connectivity_dense(jet_ctx *c, const int32_t *phi, int64_t *o
   const bool vec = c->k % 4 == 0 && ((uintptr_t)phi & 15) == 0;
   const int lanes = vec ? (c->k + 3) / 4 : c->k;  // lanes that one load of a row needs
   const int G = lanes > 16 ? 32 : lanes > 8 ? 16 : lanes > 4 ? 8 : lanes > 2 ? 4 : 2;
-  const int g = grid_for((int64_t)c->m * G, 256, c->launch_sms);
   long long *o = reinterpret_cast<long long *>(out);
-  auto go = [&](auto lanes_c) {
-    constexpr int L = decltype(lanes_c)::value;
-    if (vec) k_connectivity_dense<L, true><<<g, 256, 0, c->stream>>>(phi, c->ewgt, c->m, c->k, o);
-    else k_connectivity_dense<L, false><<<g, 256, 0, c->stream>>>(phi, c->ewgt, c->m, c->k, o);
+  auto go = [&](auto lanes_c, auto loads_c) {  // loads_c: of rows that are not aligned
+    constexpr int L = decltype(lanes_c)::value, Q = decltype(loads_c)::value;
+    const int g = grid_for((int64_t)c->m * G, 256, c->launch_sms, vec ? 8 : kRowsBlocks<Q>);
+    if (vec) k_connectivity_dense<L><<<g, 256, 0, c->stream>>>(phi, c->ewgt, c->m, c->k, o);
+    else k_connectivity_rows<L, Q><<<g, 256, 0, c->stream>>>(phi, c->ewgt, c->m, c->k, o);
   };
+  using std::integral_constant;
   switch (G) {
-    case 2: go(std::integral_constant<int, 2>()); break;
-    case 4: go(std::integral_constant<int, 4>()); break;
-    case 8: go(std::integral_constant<int, 8>()); break;
-    case 16: go(std::integral_constant<int, 16>()); break;
-    default: go(std::integral_constant<int, 32>()); break;
+    case 2: go(integral_constant<int, 2>(), integral_constant<int, 1>()); break;
+    case 4: go(integral_constant<int, 4>(), integral_constant<int, 1>()); break;
+    case 8: go(integral_constant<int, 8>(), integral_constant<int, 1>()); break;
+    case 16: go(integral_constant<int, 16>(), integral_constant<int, 1>()); break;
+    default:
+      switch ((lanes + 31) / 32) {  // 1 .. 8
+        case 1: go(integral_constant<int, 32>(), integral_constant<int, 1>()); break;
+        case 2: go(integral_constant<int, 32>(), integral_constant<int, 2>()); break;
+        case 3:
+        case 4: go(integral_constant<int, 32>(), integral_constant<int, 4>()); break;
+        default: go(integral_constant<int, 32>(), integral_constant<int, 8>()); break;
+      }
   }
   ++c->kernel_launches;
   return cudaGetLastError();
