@@ -184,11 +184,12 @@ def approve_bytes(hg, stats):
     return 17 * hg.n + 8 * stats["approved"]
 
 
-def selection_bytes(work):
-    """Rebalancing selection over one iteration: every record (16 B: key, vertex, weight and blocks) is read
-    once per radix level after the first (the first level's histogram is built by the target kernels).  The
-    per-block histogram rows the pick kernels scan are not counted."""
-    return 16 * max(work["select_levels"] - 1, 0) * work["rebalance_evaluated"]
+def selection_bytes(work, n, k):
+    """Rebalancing selection over one iteration: with more than 4,096 vertices per block every record (16 B: key,
+    vertex, weight and blocks) is read once per radix level after the first (the first level's histogram is built
+    by the target kernels), else once.  The per-block histogram rows the pick kernels scan are not counted."""
+    reads = 1 if n // k <= 4096 else max(work["select_levels"] - 1, 0)
+    return 16 * reads * work["rebalance_evaluated"]
 
 
 def objective_bytes(hg, k, unit):
@@ -323,7 +324,7 @@ def run_gpu(args, rank, world):
         rb_bytes += rb
         apply_bytes += ap
         for f, b in (("candidates", cb), ("afterburner", afterburner_bytes(hg, unit)), ("approve", approve_bytes(hg, s)),
-                     ("apply", ap), ("rebalance_targets", rb), ("rebalance_select", selection_bytes(work)),
+                     ("apply", ap), ("rebalance_targets", rb), ("rebalance_select", selection_bytes(work, hg.n, k)),
                      ("objective", objective_bytes(hg, k, unit))):
             fam_bytes[f] += b
     prof = jet.jet_profile_read(ctx, reset=True)

@@ -547,7 +547,10 @@ int jet_quotient_schedule(jet_ctx *ctx, const int32_t *phi, int32_t *pairs, int3
  * they evaluated (one record each); [2] the incidences of those vertices;
  * [3] incidences of all moved vertices (Jet and rebalancing moves); [4] the
  * levels of the rebalancing selection's radix select (a property of the
- * context: every record is read once per level after the first).
+ * context).  With more than 4,096 vertices per block of the partition every
+ * record is read once per level after the first; with fewer, the records of
+ * a block are read once and stay in registers (those beyond the registers of
+ * its thread block or cluster are read per level).
  */
 int jet_profile_work(jet_ctx *ctx, int64_t *out, int32_t n);
 

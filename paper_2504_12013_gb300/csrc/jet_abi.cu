@@ -815,7 +815,8 @@ int jet_profile_work(jet_ctx *c, int64_t *out, int32_t n) {
      "work counts");
   CK(cudaStreamSynchronize(c->stream), "synchronize");
   const int tb = c->rb_hbits + c->rb_vbits;
-  w[4] = (unsigned long long)((tb + c->rb_digit - 1) / c->rb_digit);  // radix-select levels per round
+  const int digit = c->rb_segments ? kSelBits : c->rb_digit;
+  w[4] = (unsigned long long)((tb + digit - 1) / digit);  // radix-select levels per round, of the form in use
   for (int i = 0; i < n; ++i) out[i] = (int64_t)w[i];
   return JET_OK;
 }

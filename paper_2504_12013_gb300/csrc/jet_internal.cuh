@@ -110,6 +110,7 @@ struct __align__(16) RbRec {
 // Up to this many vertices per block on average, the records of a block are kept in a segment of their own and
 // selected by one thread block (k_rb_select, where the line is explained).
 constexpr int kSegVertices = 4096;
+constexpr int kSelBits = 8;  // digit of that selection's radix select
 // Up to this many vertices (and with segments) the block weights are kept by the approval and the selection, not by
 // the apply kernels, so that the balance checks run beside those: it takes a link out of a chain of short kernels
 // (refine 100k weighted 36.6 -> 34.7 ms).  With more vertices the extra atomics cost more than the link (four

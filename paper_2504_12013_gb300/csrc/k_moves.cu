@@ -432,7 +432,6 @@ __global__ void __launch_bounds__(kPickThreads) k_rb_pick(RbArgs a, int lo, int 
 // more to the segments' cursors than that gives.
 constexpr int kSelThreads = 512;
 constexpr int kSelHeld = 8;  // records per thread held in registers
-constexpr int kSelBits = 8;
 constexpr int kSelBins = 1 << kSelBits;
 static_assert(kSelThreads * kSelHeld == kSegVertices, "a segment of average size fits the registers");
 
