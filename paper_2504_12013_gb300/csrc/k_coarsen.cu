@@ -52,6 +52,8 @@ constexpr int kLists = 4;  // classes with a list of positions: the blocks and t
 constexpr int kSettleSize = 16384;  // sub-rounds up to this size are settled by one cluster
 constexpr int kSettleBlocks = 8, kSettleThreads = 1024;
 constexpr int kHeavyWarps = 16;    // warps of a block that rates one vertex with a table in the pool
+// k_cl_serial calls rate_pool, which has scratch for kHeavyWarps warps, with the threads of the block rating
+static_assert(kBigThreads == 32 * kHeavyWarps, "rate_pool's scratch is per warp of its block");
 constexpr int kFirstEdge = 64;     // a heavy vertex's edges above this size are rated first
 constexpr int kSetCap = 2048;      // per-warp set of the distinct clusters of one edge (heavy vertices)
 constexpr int kSetEdge = kSetCap / 2;  // edges up to this size are deduplicated in that set
