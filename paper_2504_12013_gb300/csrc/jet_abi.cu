@@ -169,7 +169,7 @@ int rebalance_loop(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) { 
   if (!c->cnt_host->rb_any || c->params.max_rebalance_rounds <= 0) return JET_OK;
   for (;;) {
     CKP(F_RB_TGT, launch_rebalance_candidates(c, part, phi), "rebalance targets");
-    CKP(F_RB_SEL, launch_rb_select(c, part, block_w), "rebalance select");
+    CKP(F_RB_SEL, launch_rb_select(c, block_w), "rebalance select");
     CKP(F_APPLY, launch_rb_apply(c, part, phi, block_w), "rebalance apply");
     CKP(F_RB_CTL, launch_rb_post(c, block_w), "rebalance post");
     rc = sync_counters(c);
@@ -264,7 +264,7 @@ cudaError_t capture_iteration(jet_ctx *c, cudaStream_t s_main, cudaStream_t s_bo
     c->side_first = 2;
     c->side_count = 1;
     cudaError_t eb = launch_rebalance_candidates(c, part, phi);
-    if (eb == cudaSuccess) eb = launch_rb_select(c, part, bw);
+    if (eb == cudaSuccess) eb = launch_rb_select(c, bw);
     {
       Fork fork(c, c->rb_early ? 2 : 1);  // as above: the end of the round beside its apply
       if (eb == cudaSuccess) eb = launch_rb_apply(c, part, phi, bw);

@@ -57,7 +57,6 @@ struct Counters {
   unsigned long long n_moves;     // entries in the move list
   unsigned long long n_cand;      // |M|
   unsigned long long approved;    // afterburner-approved moves
-  unsigned long long unused0;
   long long objective;            // (lambda-1), accumulated
   long long rb_rounds;
   long long rb_moves;
@@ -66,7 +65,6 @@ struct Counters {
   unsigned long long w_over, w_eval, w_eval_pins, w_apply_pins;
   unsigned long long n_rec;       // rebalancing records of the current round
   unsigned ob_done;               // blocks of the objective kernel that have finished
-  unsigned unused1;
   int rb_done;                    // rebalancing loop may stop
   int rb_any;                     // an overloaded block exists
   int err;                        // bit flags of data errors found on the device
@@ -116,6 +114,7 @@ constexpr int kSelBits = 8;  // digit of that selection's radix select
 // (refine 100k weighted 36.6 -> 34.7 ms).  With more vertices the extra atomics cost more than the link (four
 // iterations of 300k vertices at k = 200: 2.12 -> 2.24 ms).
 constexpr int kEarlyVertices = 1 << 17;
+constexpr int kApproveVertices = 1 << 17;  // up to this many vertices the approval takes one per thread and step
 constexpr int kCurStride = 32;  // ints between the blocks' record cursors (a line each)
 
 }  // namespace jet
@@ -184,7 +183,7 @@ struct jet_ctx {
   int32_t *rb_ct = nullptr;           // per record: c(v) << 16 | block << 8 | target
   unsigned long long *rb_hist = nullptr;  // k x 2^rb_digit weighted digit histograms (zero between uses)
   int rb_hbits = 0, rb_vbits = 1;     // key = rb_hi << rb_vbits | v, rb_hbits + rb_vbits significant bits
-  int rb_digit = 1;                   // radix-select digit width: the key in as few levels of <= 16 bits
+  int rb_digit = 1;                   // radix-select digit width: the key in as few levels of <= kRbMaxDigit bits
   int32_t *best_part = nullptr;       // best balanced partition of jet_refine
   uint8_t *locked_ws = nullptr;       // locks of jet_refine
   jet_round_stats *stats_scratch = nullptr;
@@ -317,9 +316,9 @@ cudaError_t launch_rebalance_candidates(jet_ctx *c, const int32_t *part, const i
 cudaError_t prepare_afterburner(jet_ctx *c);
 cudaError_t prepare_afterburner_kernels(jet_ctx *c);  // ab_bps
 cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *phi);
-// part (with build_moves): the partition, whose blocks' vertices are counted where records are segmented.  rs (may be NULL): if the last
-// iteration improved (rs->snap), the partition is also copied to c->best_part.  block_w (with build_moves): where
-// rb_early, the moves' weights are added here and not by launch_apply_jet.
+// part (with build_moves): the partition, whose blocks' vertices are counted where records are segmented.  rs (may be
+// NULL): if the last iteration improved (rs->snap), the partition is also copied to c->best_part.  block_w (with
+// build_moves): where rb_early, the moves' weights are added here and not by launch_apply_jet.
 cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int32_t *rg_out, uint8_t *approved_out,
                            bool build_moves, int64_t *block_w = nullptr, const RefineState *rs = nullptr);
 cudaError_t launch_export_candidates(jet_ctx *c, int32_t *target, int32_t *gain, uint8_t *in_m);
@@ -331,7 +330,7 @@ cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part);  // cnt->vcoun
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                             int use_cond = 0);
 // the selection of a round (with rb_early, block_w takes its weights here and not in launch_rb_apply)
-cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w);
+cudaError_t launch_rb_select(jet_ctx *c, int64_t *block_w);
 cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w);  // applies the selection
 cudaError_t launch_rb_post(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond = 0,
                            int use_cond = 0);

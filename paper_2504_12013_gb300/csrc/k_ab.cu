@@ -893,7 +893,7 @@ cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int
   a.mv_st = c->mv_st;
   a.cnt = c->cnt;
   // every block adds its counts and weights of up to k blocks to the same few lines: fewer blocks then
-  if (c->n <= kEarlyVertices)  // 100k vertices: refine in 35.9 against 36.0 ms; 300k: R = 4 by 0.8 % of a round
+  if (c->n <= kApproveVertices)  // 100k vertices: refine in 35.9 against 36.0 ms; 300k: R = 4 by 0.8 % of a round
     k_approve<1><<<grid_for(c->n, 256, c->launch_sms, a.count ? 4 : 8), 256, 0, c->stream>>>(a);
   else
     k_approve<4><<<grid_for(c->n, 1024, c->launch_sms, a.count ? 2 : 8), 256, 0, c->stream>>>(a);

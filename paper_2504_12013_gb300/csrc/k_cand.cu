@@ -140,7 +140,10 @@ __device__ __forceinline__ uint64_t rb_hi_of(const CandArgs &a, int32_t g, int32
 }
 
 // Adds the thread's work counts to the call's totals: one atomic per thread
-// block and counter (every thread of the block calls it).
+// block and counter (every thread of the block calls it).  A warp's sums fit
+// 32 bits: a light vertex has fewer than 64 incidences, so even a grid of one
+// block would have to meet 5.4e8 vertices; the heavy kernel passes at most
+// 2^24 incidences here.
 __device__ __forceinline__ void count_work(Counters *cnt, unsigned over, unsigned eval, unsigned pins) {
   __shared__ unsigned s_w[256 / 32][3];  // per warp
   const int w = threadIdx.x >> 5;
@@ -213,9 +216,9 @@ __device__ __forceinline__ void eligible_words(const long long *s_cap, int k, in
 // ------------------------------------------------------------ light vertices
 // A warp takes 32 consecutive vertex ids; each lane evaluates one light
 // vertex.  Its incidences I(v) are processed in batches of kBatch: the mask
-// rows of a batch are copied into the lane's slots of a double-buffered shared-memory stage with cp.async, so batch b+1's gathers (and
-// batch b+2's incidence loads) are in flight while batch b is added into the
-// bit planes.
+// rows of a batch are copied into the lane's slots of a double-buffered
+// shared-memory stage with cp.async, so batch b+1's gathers (and batch b+2's
+// incidence loads) are in flight while batch b is added into the bit planes.
 // Slot t of lane l is row t*32 + l of a buffer, so the lanes' reads of the
 // stage are bank-conflict free.  Lanes never read each other's slots.
 
@@ -391,7 +394,7 @@ __device__ __forceinline__ int32_t stage_accumulate(const CandArgs &a, uint8_t *
 // Heavy vertices are skipped here and handled by the warp-per-vertex kernels.
 struct WarpQueue {
   static constexpr int kCap = 64;
-  int v[kCap], s[kCap], c[kCap], deg[kCap];
+  int v[kCap], s[kCap], deg[kCap];
   long long j0[kCap];
 };
 
@@ -413,14 +416,13 @@ __device__ __forceinline__ GroupRaw fetch_group(const CandArgs &a, int64_t v, bo
 
 // Appends this lane's vertex (if `act`) to the warp queue; returns the new
 // (warp-uniform) queue length.
-__device__ __forceinline__ int enqueue(WarpQueue *q, int qn, bool act, int v, int s, int c, int64_t j0, int deg) {
+__device__ __forceinline__ int enqueue(WarpQueue *q, int qn, bool act, int v, int s, int64_t j0, int deg) {
   const int lane = threadIdx.x & 31;
   const unsigned bal = __ballot_sync(kFull, act);
   if (act) {
     const int pos = qn + __popc(bal & ((1u << lane) - 1));
     q->v[pos] = v;
     q->s[pos] = s;
-    q->c[pos] = c;
     q->deg[pos] = deg;
     q->j0[pos] = j0;
   }
@@ -432,14 +434,14 @@ __device__ __forceinline__ int enqueue(WarpQueue *q, int qn, bool act, int v, in
 __device__ __forceinline__ int dequeue32(WarpQueue *q, int qn) {
   const int lane = threadIdx.x & 31;
   const int rest = qn - 32;
-  int v = 0, s = 0, c = 0, deg = 0;
+  int v = 0, s = 0, deg = 0;
   long long j0 = 0;
   if (lane < rest) {
-    v = q->v[32 + lane]; s = q->s[32 + lane]; c = q->c[32 + lane]; deg = q->deg[32 + lane]; j0 = q->j0[32 + lane];
+    v = q->v[32 + lane]; s = q->s[32 + lane]; deg = q->deg[32 + lane]; j0 = q->j0[32 + lane];
   }
   __syncwarp();
   if (lane < rest) {
-    q->v[lane] = v; q->s[lane] = s; q->c[lane] = c; q->deg[lane] = deg; q->j0[lane] = j0;
+    q->v[lane] = v; q->s[lane] = s; q->deg[lane] = deg; q->j0[lane] = j0;
   }
   __syncwarp();
   return rest;
@@ -504,7 +506,7 @@ __global__ void __launch_bounds__(256, kLightBlocks<KWP>) k_cand_light(CandArgs 
         deg = (int)(a.vptr[v + 1] - j0);
       }
     }
-    qn = enqueue(q, qn, act, (int)v, cur.s, 0, j0, deg);
+    qn = enqueue(q, qn, act, (int)v, cur.s, j0, deg);
     if (qn >= 32) {
       cand_batch<KWP, UNIT>(a, stage, q, 32);
       qn = dequeue32(q, qn);

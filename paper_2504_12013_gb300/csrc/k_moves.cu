@@ -818,7 +818,7 @@ MoveArgs move_args(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block_w) {
   return a;
 }
 
-RbArgs rb_args(jet_ctx *c, const int64_t *block_w, const int32_t *part) {
+RbArgs rb_args(jet_ctx *c, const int64_t *block_w) {
   RbArgs a{};
   a.bw = block_w;
   a.rbb = c->rbb;
@@ -828,7 +828,6 @@ RbArgs rb_args(jet_ctx *c, const int64_t *block_w, const int32_t *part) {
   a.rb_hi = c->rb_hi;
   a.rb_v = c->rb_v;
   a.rb_ct = c->rb_ct;
-  (void)part;
   a.hist = c->rb_hist;
   a.mv_v = c->mv_v;
   a.mv_st = c->mv_st;
@@ -901,7 +900,7 @@ cudaError_t launch_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *block
 }
 
 cudaError_t launch_rb_check(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond, int use_cond) {
-  k_rb_check<<<1, kMaxK, 0, c->stream>>>(rb_args(c, block_w, nullptr), cond, use_cond);
+  k_rb_check<<<1, kMaxK, 0, c->stream>>>(rb_args(c, block_w), cond, use_cond);
   ++c->kernel_launches;
   return cudaGetLastError();
 }
@@ -952,9 +951,9 @@ cudaError_t launch_count_blocks(jet_ctx *c, const int32_t *part) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_rb_select(jet_ctx *c, const int32_t *part, int64_t *block_w) {
+cudaError_t launch_rb_select(jet_ctx *c, int64_t *block_w) {
   if (c->n == 0) return cudaSuccess;
-  const RbArgs a = rb_args(c, nullptr, part);
+  const RbArgs a = rb_args(c, nullptr);
   if (c->rb_segments) {
     int64_t *bw = c->rb_early ? block_w : nullptr;
     if (c->W < (1ll << 32))
@@ -975,7 +974,7 @@ cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *bl
     a.weights = !c->rb_early;
     return c->graph_path ? apply_part(c, a) : apply_phi(c, a);
   }
-  const RbArgs r = rb_args(c, block_w, part);
+  const RbArgs r = rb_args(c, block_w);
   const MoveArgs a = move_args(c, part, phi, block_w);
   if (r.tbits <= 64)
     k_rb_apply<unsigned long long><<<grid_for(c->n, 256, c->launch_sms, kRbMoveWaves * c->move_bps[1]), 256, 0,
@@ -987,7 +986,7 @@ cudaError_t launch_rb_apply(jet_ctx *c, int32_t *part, int32_t *phi, int64_t *bl
 }
 
 cudaError_t launch_rb_post(jet_ctx *c, const int64_t *block_w, cudaGraphConditionalHandle cond, int use_cond) {
-  k_rb_post<<<1, kMaxK, 0, c->stream>>>(rb_args(c, block_w, nullptr), cond, use_cond);
+  k_rb_post<<<1, kMaxK, 0, c->stream>>>(rb_args(c, block_w), cond, use_cond);
   ++c->kernel_launches;
   return cudaGetLastError();
 }

@@ -32,7 +32,7 @@ static __device__ __align__(256) int32_t g_noalloc_scratch[kScratchInts];
 std::mutex g_setup_mu;
 int32_t *g_scratch_addr[kMaxDevices] = {nullptr};  // device address of the array, per device
 
-// The block-weight kernel of k_state.cu, with its counts and error flag in `scratch`.
+// Block weights as in k_state.cu, with the blocks' vertices counted too and the error flag in `scratch`.
 __global__ void k_block_weights_static(const int32_t *part, const int32_t *vwgt, int32_t n, int32_t k,
                                        int64_t *bw, int32_t *scratch) {
   __shared__ long long s_bw[kNoAllocMaxK];

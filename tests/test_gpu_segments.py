@@ -26,6 +26,7 @@ CASES = [
     (131_072, 200, 1, 1, 0.03), (131_073, 200, 1, 1, 0.03),
     (8_193, 2, 1, 1, 0.4), (8_194, 2, 1, 1, 0.4),        # 4,096 and 4,097 vertices per block
     (16_384, 8, 1, 1, 1.0), (16_385, 8, 1, 1, 1.0),      # no large segment possible; just one
+    (12_000, 4, 1, 900, 1.0), (140_000, 40, 30_000, 32_767, 0.08),  # one block beyond its registers, longer keys
     (20_000, 8, 1, 4, 0.9), (30_000, 8, 1, 1000, 1.0),   # a cluster, the records held; with longer keys
     (90_000, 37, 1, 3, 1.0), (90_000, 37, 1, 900, 1.0),  # beyond the registers of the cluster
     (140_000, 64, 1, 2, 1.0),                            # ... where the apply keeps the block weights
