@@ -111,8 +111,10 @@ constexpr int kSegVertices = 4096;
 constexpr int kSelBits = 8;  // digit of that selection's radix select
 // Up to this many vertices (and with segments) the block weights are kept by the approval and the selection, not by
 // the apply kernels, so that the balance checks run beside those: it takes a link out of a chain of short kernels
-// (refine 100k weighted 36.6 -> 34.7 ms).  With more vertices the extra atomics cost more than the link (four
-// iterations of 300k vertices at k = 200: 2.12 -> 2.24 ms).
+// (refine 100k weighted 36.6 -> 34.7 ms).  The line: up to it c(V) < 2^32 whatever the weights, so that the
+// selection sums them in 32 bits; with 64-bit sums in shared memory the atomics cost more than the link (four
+// iterations of 300k vertices at k = 200: 2.12 -> 2.24 ms).  With 32-bit sums eight iterations of 160,000 to 400,000
+// vertices of small weights at k = 128 are 7 to 8 % faster this way too (at 130,000: 9 %).
 constexpr int kEarlyVertices = 1 << 17;
 constexpr int kApproveVertices = 1 << 17;  // up to this many vertices the approval takes one per thread and step
 constexpr int kCurStride = 32;  // ints between the blocks' record cursors (a line each)

@@ -52,12 +52,11 @@ struct AbArgs {
 // Thread per edge (|e| <= 8), software-pipelined over the thread's edges:
 // while edge j is decided, the pins of edge j+1, the offsets of edge j+2 and
 // the id of edge j+3 are in flight.
-// AHEAD: calls of up to kAheadEdges such edges wait for their loads, not for
-// the memory: blocks and omega come with the records.  Larger ones load the
-// blocks of the few pins that are no candidates after them (and need the
-// registers for a fourth resident block).
-constexpr int kAheadEdges = 1 << 19;
-template <bool AHEAD>
+// The blocks of the few pins that are no candidates, and omega, are loaded
+// after the records of an edge with a candidate.  Loaded with them for every
+// edge they took longer at every size: eight iterations of 20,000 to 2 M
+// vertices of such edges by 0.2 to 1.4 %, refine of 100k weighted vertices
+// 30.1 against 29.9 ms.
 __global__ void __launch_bounds__(256) k_ab_tiny(AbArgs a) {
   const int stride = gridDim.x * blockDim.x;
   const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -91,32 +90,27 @@ __global__ void __launch_bounds__(256) k_ab_tiny(AbArgs a) {
     uint64_t key[kTinyEdge];
     uint32_t st[kTinyEdge];  // s | t << 8 | 1 << 16 for a candidate; block | 1 << 17 for another pin
     int nin = 0;
-    int w = AHEAD && sz > 0 ? a.ewgt[e] : 0;
 #pragma unroll
-    for (int q = 0; q < kTinyEdge; ++q) {
-      key[q] = q < sz ? a.cand[pin[q]] : 0ull;
-      st[q] = AHEAD && q < sz ? (uint32_t)(a.part[pin[q]] & 255) : 0u;
-    }
+    for (int q = 0; q < kTinyEdge; ++q) key[q] = q < sz ? a.cand[pin[q]] : 0ull;
 #pragma unroll
     for (int q = 0; q < kTinyEdge; ++q) {
       const uint64_t r = key[q];
+      st[q] = 0u;
       if (q < sz) {
         if (r) {
           ++nin;
           key[q] = cand_key(r, pin[q]);
           st[q] = (uint32_t)cand_s(r) | ((uint32_t)cand_t(r) << 8) | 0x10000u;
         } else {
-          st[q] |= 0x20000u;
+          st[q] = 0x20000u;
         }
       }
     }
     if (nin == 0) continue;
-    if constexpr (!AHEAD) {
 #pragma unroll
-      for (int q = 0; q < kTinyEdge; ++q)
-        if (st[q] & 0x20000u) st[q] |= (uint32_t)(a.part[pin[q]] & 255);  // block of a non-candidate pin
-      w = a.ewgt[e];
-    }
+    for (int q = 0; q < kTinyEdge; ++q)
+      if (st[q] & 0x20000u) st[q] |= (uint32_t)(a.part[pin[q]] & 255);  // block of a non-candidate pin
+    const int w = a.ewgt[e];
     // Every pair of pins is compared, so the comparisons are made for the edge's size: the list is ordered by
     // size, so a warp's edges mostly take one of these branches together (comparing eight slots for every edge
     // bound the kernel by its instructions: 76 us for 2 M edges of 3 pins on average).
@@ -522,11 +516,12 @@ struct ApArgs {
 // Counters and move-list slots are aggregated per thread block (one atomic
 // per block and iteration) rather than per warp, which would serialize on
 // the few counter addresses.  R vertices per thread and step: their loads
-// overlap and share the append's barriers.  Bound by those loads: with R = 4
-// eight iterations of 2 M VLSI vertices took 7.89 against 7.98 ms, of a graph
-// of 4 M vertices 8.53 against 8.70; small calls (launch_approve) lose to the
-// longer chain of a step and to blocks left idle: refine of 10k vertices 7.67
-// against 7.52 ms.
+// overlap and share the append's barriers, which pays where those loads bound
+// it; small calls lose to the longer chain of a step and to blocks left idle.
+// Eight iterations with R = 4 against R = 1 (k = 37 and 128): 30,000 vertices
+// 1.2 and 1.0 % slower, 100,000 0.5 and 0.1, 130,000 0.2 slower and 0.5 faster,
+// 160,000 0.1 and 0.9 % faster, 600,000 1.5 and 0.9; 2 M VLSI vertices 7.89
+// against 7.98 ms, a graph of 4 M 8.53 against 8.70.
 template <int R>
 __global__ void __launch_bounds__(256) k_approve(ApArgs a) {
   constexpr int kWarps = 256 / 32;
@@ -733,8 +728,7 @@ cudaError_t launch_afterburner(jet_ctx *c, const int32_t *part, const int32_t *p
     a.elist = c->e_tiny;
     a.nlist = c->n_tiny;
     const int g = grid_for(c->n_tiny, 256, c->launch_sms, c->ab_bps[0]);
-    if (c->n_tiny <= kAheadEdges) k_ab_tiny<true><<<g, 256, 0, fork.stream(branch++)>>>(a);
-    else k_ab_tiny<false><<<g, 256, 0, fork.stream(branch++)>>>(a);
+    k_ab_tiny<<<g, 256, 0, fork.stream(branch++)>>>(a);
     ++c->kernel_launches;
   }
   if (c->n_mid_half > 0) {
@@ -800,7 +794,7 @@ cudaError_t prepare_afterburner_kernels(jet_ctx *c) {
   // of the kernel, shared by every context, so it is set for the largest k, not for this context's.
   cudaError_t e = cudaFuncSetAttribute(k_ab_warp_small<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)((size_t)kAbWarps * 2 * 2 * kMaxK * sizeof(unsigned long long)));
-  if (e == cudaSuccess) e = resident_blocks(k_ab_tiny<false>, 256, 0, &c->ab_bps[0]);
+  if (e == cudaSuccess) e = resident_blocks(k_ab_tiny, 256, 0, &c->ab_bps[0]);
   if (e == cudaSuccess) e = resident_blocks(k_ab_warp_small<16>, kAbWarps * 32, 2 * warp_tab, &c->ab_bps[1]);
   if (e == cudaSuccess) e = resident_blocks(k_ab_warp_small<32>, kAbWarps * 32, warp_tab, &c->ab_bps[2]);
   if (e == cudaSuccess) e = resident_blocks(k_ab_warp<4>, kAbWarps * 32, warp_tab, &c->ab_bps[3]);
@@ -893,7 +887,7 @@ cudaError_t launch_approve(jet_ctx *c, const int32_t *part, uint8_t *locked, int
   a.mv_st = c->mv_st;
   a.cnt = c->cnt;
   // every block adds its counts and weights of up to k blocks to the same few lines: fewer blocks then
-  if (c->n <= kApproveVertices)  // 100k vertices: refine in 35.9 against 36.0 ms; 300k: R = 4 by 0.8 % of a round
+  if (c->n <= kApproveVertices)
     k_approve<1><<<grid_for(c->n, 256, c->launch_sms, a.count ? 4 : 8), 256, 0, c->stream>>>(a);
   else
     k_approve<4><<<grid_for(c->n, 1024, c->launch_sms, a.count ? 2 : 8), 256, 0, c->stream>>>(a);
